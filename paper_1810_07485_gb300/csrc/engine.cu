@@ -265,6 +265,8 @@ Engine::~Engine() {
   dfree(s_.dbg);
   if (st_) cudaStreamSynchronize(st_);  // stream-ordered frees done
   if (pool_) cudaMemPoolDestroy(pool_);
+  if (stage_) cudaFreeHost(stage_);
+  if (stage_ch_) cudaFreeHost(stage_ch_);
   if (own_stream_ && st_) cudaStreamDestroy(st_);
 }
 
@@ -303,6 +305,7 @@ int Engine::open(void *stream, const lcqmc_allocator *alloc, int ring_cap, bool 
   std::vector<uint64_t> T(KMAX);
   poisson_table(CELL_MEAN, T.data());
   set_full_table(T.data(), st_);
+  CK(cudaHostAlloc((void **)&stage_, sizeof(HostStage), cudaHostAllocDefault));
   DALLOC(s_.status, int, 1);
   s_.uf_limit = UF_MAX_ITERS;
   // Tests: the most steps a global union-find walk or retry loop of this
@@ -656,6 +659,7 @@ int Engine::update(int64_t n) {
   if (n == 0) return LCQMC_OK;
   NvtxRange range("lcqmc_update");
   if (pending_ == 0) pending_sweep0_ = hch[0].sweep;
+  dirty_ = true;
   if (timing_) {
     const int per = LCQMC_NPHASE + 1;
     while ((int)ev_.size() < (ev_used_ + (int)n) * per) {
@@ -684,11 +688,22 @@ int Engine::update(int64_t n) {
   return LCQMC_OK;
 }
 
-int Engine::pull_chains() {
-  if (hch.empty()) return LCQMC_OK;
-  CK(cudaMemcpyAsync(hch.data(), dch_, sizeof(DevChain) * hch.size(), cudaMemcpyDeviceToHost, st_));
+// Waits for the stream once: the status word and the chains' descriptors come
+// back through page-locked staging by copies enqueued behind the updates.
+int Engine::fetch(int *status) {
+  const size_t nc = hch.size();
+  if (nc > stage_nch_) {
+    if (stage_ch_) cudaFreeHost(stage_ch_);
+    stage_ch_ = nullptr;
+    stage_nch_ = 0;
+    CK(cudaHostAlloc((void **)&stage_ch_, sizeof(DevChain) * nc, cudaHostAllocDefault));
+    stage_nch_ = nc;
+  }
+  CK(cudaMemcpyAsync(&stage_->status, s_.status, sizeof(int), cudaMemcpyDeviceToHost, st_));
+  if (nc) CK(cudaMemcpyAsync(stage_ch_, dch_, sizeof(DevChain) * nc, cudaMemcpyDeviceToHost, st_));
   CK(cudaStreamSynchronize(st_));
-  for (size_t c = 0; c < hch.size(); ++c) cs_[c]->dev = hch[c];
+  *status = stage_->status;
+  for (size_t c = 0; c < nc; ++c) cs_[c]->dev = hch[c] = stage_ch_[c];
   return LCQMC_OK;
 }
 
@@ -726,12 +741,15 @@ int Engine::grow_ops(int64_t c, int64_t need) {
   return LCQMC_OK;
 }
 
-int Engine::sync() {
-  for (int guard = 0; guard < 64; ++guard) {
+int Engine::sync(bool *at_once) {
+  if (at_once) *at_once = true;
+  if (!dirty_) {  // nothing ran since the last clean sync: the descriptors are current
     CK(cudaStreamSynchronize(st_));
+    return LCQMC_OK;
+  }
+  for (int guard = 0; guard < 64; ++guard) {
     int status = 0;
-    CK(cudaMemcpy(&status, s_.status, sizeof(int), cudaMemcpyDeviceToHost));
-    int rc = pull_chains();
+    int rc = fetch(&status);
     if (rc) return rc;
     if (timing_ && ev_used_ > 0) {
       for (int u = 0; u < ev_used_; ++u)
@@ -745,8 +763,10 @@ int Engine::sync() {
     }
     if (status == 0) {
       pending_ = 0;
+      dirty_ = false;
       return LCQMC_OK;
     }
+    if (at_once) *at_once = false;
     const int64_t done = (int64_t)(uint32_t)(hch[0].sweep - pending_sweep0_);
     const int64_t remaining = pending_ - done;
     if (status & (ST_TIMEOUT | ST_INTERNAL | ST_BADSTATE | ST_ID_OVERFLOW)) {
@@ -837,18 +857,43 @@ int Engine::reset_obs(int64_t c) {
 }
 
 int Engine::records(int64_t c, lcqmc_record *out, int64_t max, int64_t *count) {
-  int rc = sync();
+  max = std::max<int64_t>(0, max);
+  int64_t &rd = cs_[c]->rec_read;
+  const lcqmc_record *ring = cs_[c]->buf.ring;
+  const int64_t cap = ring_cap_;
+  // Copies of records [from, from + m) of the ring, in at most two runs.
+  auto copy = [&](lcqmc_record *dst, int64_t from, int64_t m) -> cudaError_t {
+    for (int64_t i = 0; i < m;) {
+      const int64_t slot = (from + i) % cap, run = std::min<int64_t>(m - i, cap - slot);
+      cudaError_t e = cudaMemcpyAsync(dst + i, ring + slot, sizeof(lcqmc_record) * (size_t)run,
+                                      cudaMemcpyDeviceToHost, st_);
+      if (e != cudaSuccess) return e;
+      i += run;
+    }
+    return cudaSuccess;
+  };
+  // The records that the enqueued updates will have written come back behind
+  // them, with the descriptors (one wait); used if no update had to be redone.
+  int64_t from = 0, staged = 0;
+  if (dirty_ && pending_ > 0) {
+    const int64_t n_rec = hch[c].n_rec + pending_;
+    from = std::max<int64_t>(rd, n_rec - cap);
+    staged = std::min<int64_t>(n_rec - from, max);
+    if (staged > kStageRecords) staged = 0;
+    CK(copy(stage_->rec, from, staged));
+  }
+  bool at_once = true;
+  int rc = sync(&at_once);
   if (rc) return rc;
   const DevChain &d = hch[c];
-  int64_t &rd = cs_[c]->rec_read;
-  if (d.n_rec - rd > d.ring_cap) rd = d.n_rec - d.ring_cap;
-  int64_t avail = d.n_rec - rd;
-  const int64_t m = std::min<int64_t>(avail, std::max<int64_t>(0, max));
-  for (int64_t i = 0; i < m; ++i) {
-    const int64_t slot = (rd + i) % d.ring_cap;
-    CK(cudaMemcpyAsync(out + i, cs_[c]->buf.ring + slot, sizeof(lcqmc_record), cudaMemcpyDeviceToHost, st_));
+  if (d.n_rec - rd > cap) rd = d.n_rec - cap;
+  const int64_t m = std::min<int64_t>(d.n_rec - rd, max);
+  if (at_once && m > 0 && m == staged && rd == from) {
+    std::memcpy(out, stage_->rec, sizeof(lcqmc_record) * (size_t)m);
+  } else if (m > 0) {
+    CK(copy(out, rd, m));
+    CK(cudaStreamSynchronize(st_));
   }
-  CK(cudaStreamSynchronize(st_));
   rd += m;
   *count = m;
   return LCQMC_OK;

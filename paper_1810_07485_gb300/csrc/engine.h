@@ -61,8 +61,8 @@ class Engine {
   static size_t state_bytes(const ChainSpec &c, int ring_cap);
   static size_t scratch_bytes(const ChainSpec &c);
   int update(int64_t n);
-  int sync();
-  int pull_chains();  // device descriptors -> hch (after sync)
+  // at_once (optional): whether no update had to be run again
+  int sync(bool *at_once = nullptr);
   int push_chains();  // hch -> device descriptors (after sync)
   int measure(int64_t chain, lcqmc_obs *out);
   int reset_obs(int64_t chain);
@@ -99,6 +99,7 @@ class Engine {
   int alloc_vertex(int64_t vcap);
   void free_vertex();
   int grow_ops(int64_t chain, int64_t need);
+  int fetch(int *status);  // waits for the stream; device descriptors -> hch
   int enqueue_one(bool timed, int slot);
   int capture(int count, cudaGraphExec_t *out);
   void drop_graphs();
@@ -134,6 +135,18 @@ class Engine {
   int64_t pending_ = 0;
   uint32_t pending_sweep0_ = 0;
   int64_t replays_ = 0;  // updates re-run after capacity growth
+  // Read-back: page-locked staging for the status word, the chains'
+  // descriptors and up to kStageRecords records, filled by copies enqueued
+  // behind the updates, so that a call that reads waits for the stream once.
+  static constexpr int64_t kStageRecords = 256;
+  struct HostStage {
+    int status;
+    lcqmc_record rec[kStageRecords];
+  };
+  HostStage *stage_ = nullptr;
+  DevChain *stage_ch_ = nullptr;
+  size_t stage_nch_ = 0;
+  bool dirty_ = true;  // an update was enqueued (or a sync failed) since the last clean sync
 };
 
 }  // namespace lcq

@@ -205,6 +205,15 @@ def records_to_numpy(buf, n):
     return np.frombuffer(bytes(buf), dtype=RECORD_DTYPE, count=n).copy()
 
 
+RING = 4096  # records a chain keeps on the device (a chain of a batch: fewer)
+
+
+def records_buffer(max_n):
+    """Room for the records of one call: untouched memory (zeroing and copying
+    65536 records took 0.85 ms a call), no more of it than a chain can hold."""
+    return np.empty(max(1, min(int(max_n), RING)), dtype=RECORD_DTYPE)
+
+
 class Chain:
     """One Markov chain on the GPU: lcqmc_create ... lcqmc_destroy."""
 
@@ -256,10 +265,10 @@ class Chain:
         _check(lib().lcqmc_reset_obs(self.h))
 
     def records(self, max_n=1 << 16):
-        buf = (Record * max(1, max_n))()
+        buf = records_buffer(max_n)
         cnt = ctypes.c_int64()
-        _check(lib().lcqmc_get_records(self.h, buf, int(max_n), ctypes.byref(cnt)))
-        return records_to_numpy(buf, cnt.value)
+        _check(lib().lcqmc_get_records(self.h, _p(buf), min(int(max_n), RING), ctypes.byref(cnt)))
+        return buf[: cnt.value].copy()
 
     def geometry(self):
         g = Geometry()
@@ -272,9 +281,9 @@ class Chain:
         _check(lib().lcqmc_export_config(self.h, None, None, None, 0, ctypes.byref(n)))
         s0 = np.zeros(g.nsub, np.uint8)
         ptr = np.zeros(g.ncell + 1, np.int32)
-        tau = np.zeros(max(1, n.value), np.float64)
+        tau = np.empty(max(1, n.value), np.float64)
         _check(lib().lcqmc_export_config(self.h, _p(s0), _p(ptr), _p(tau), n.value, ctypes.byref(n)))
-        return s0, ptr, tau[: n.value].copy()
+        return s0, ptr, tau[: n.value]
 
     def import_config(self, s0, op_ptr, op_tau, sweep):
         s0 = np.ascontiguousarray(s0, np.uint8)
@@ -394,10 +403,10 @@ class Batch:
         return o
 
     def records(self, i, max_n=1 << 12):
-        buf = (Record * max(1, max_n))()
+        buf = records_buffer(max_n)
         cnt = ctypes.c_int64()
-        _check(lib().lcqmc_batch_get_records(self.h, int(i), buf, int(max_n), ctypes.byref(cnt)))
-        return records_to_numpy(buf, cnt.value)
+        _check(lib().lcqmc_batch_get_records(self.h, int(i), _p(buf), min(int(max_n), RING), ctypes.byref(cnt)))
+        return buf[: cnt.value].copy()
 
 
 def footprint(L, beta, S=0.5, J=1.0):
