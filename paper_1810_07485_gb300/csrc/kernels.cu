@@ -1152,6 +1152,75 @@ __global__ void __launch_bounds__(TPB_X) k_link_x(const DevChain *__restrict__ c
   }
 }
 
+// The same unions with one block per tile, for launches of few tiles: there
+// the time is the chain of dependent L2 accesses of the slowest warp, not the
+// work.  The block lists the tile's crossing edges (a warp takes a mark word at
+// a time, one bit per lane; S >= 1 tiles have hundreds, 300 to 700 of 1000
+// edges), every thread unites edges of the list and then walks once more from
+// one node of each of its edges: the walks of all threads halve the same long
+// paths (min-root links chain the tiles of a loop), so that the waiting unions
+// and the compression find short ones.  linking + unions / compression, us:
+// S = 2, 65 tiles 213 / 32 -> 90 / 23; S = 3/2, 1024 tiles 244 / 46 -> 122 /
+// 37; S = 1/2, 128 tiles 47 / 28 -> 40 / 20.  Without the second walk the
+// unions got faster but the compression slower (S = 2: 108 / 49).
+constexpr int64_t XT_MAX_TILES = 20 * 152;
+
+__global__ void __launch_bounds__(TPB_X) k_link_xt(const DevChain *__restrict__ ch,
+                                                const int2 *__restrict__ tab, int64_t blk0,
+                                                Scratch s) {
+  __shared__ unsigned short xlist[SMEM_CAP];
+  __shared__ int nx;
+  if (halted(s)) return;
+  const int2 t = tab[blk0 + blockIdx.x];
+  const DevChain &C = ch[t.x];
+  const int c0 = t.y * TILE, c1 = min(C.ncell, c0 + TILE);
+  const int32_t *vp = s.vptr + C.cell_off;
+  const int a = vp[c0], e = vp[c1];
+  const int64_t vb = C.vtx_base;
+  int32_t *par = s.parent + vb;
+  if (e - a > local_cap(C)) {  // every edge of the tile
+    for (int w = a + threadIdx.x; w < e; w += TPB_X)
+      uf_union(par, s.pl[vb + w], s.pr[vb + w], s.status, s.uf_limit);
+    return;
+  }
+  if (threadIdx.x == 0) nx = 0;
+  __syncthreads();
+  constexpr int NW = TPB_X / 32;
+  constexpr int WMAX = (SMEM_CAP / 32 + 1 + NW - 1) / NW;  // mark words per warp
+  static_assert(WMAX <= 32, "one lane loads each mark word of a warp");
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t wfirst = (vb + a) >> 5, wlast = (vb + e - 1) >> 5;
+  uint32_t mine = 0u;
+  {
+    const int64_t wd = wfirst + wid + NW * lane;
+    if (lane < WMAX && e > a && wd <= wlast) {
+      const int64_t v0 = (wd << 5) - vb;
+      mine = __ldcg(s.xmark + wd);
+      if (v0 < a) mine &= ~0u << (a - v0);
+      if (v0 + 32 > e) mine &= (e - v0 >= 32) ? ~0u : ((1u << (e - v0)) - 1u);
+    }
+  }
+  for (int k = 0; k < WMAX; ++k) {
+    const uint32_t bits = __shfl_sync(0xffffffffu, mine, k);
+    if (!bits) continue;
+    int at = 0;
+    if (lane == 0) at = atomicAdd(&nx, __popc(bits));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(bits & ((1u << lane) - 1u));
+    if ((bits >> lane) & 1u)
+      xlist[at] = (unsigned short)(((wfirst + wid + NW * k) << 5) + lane - vb - a);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nx; i += TPB_X) {
+    const int64_t w = vb + a + xlist[i];
+    uf_union(par, s.pl[w], s.pr[w], s.status, s.uf_limit);
+  }
+  for (int i = threadIdx.x; i < nx; i += TPB_X) {
+    const int p = s.pl[vb + a + xlist[i]];
+    const int r = uf_find(par, p, s.status, s.uf_limit);
+    if (r != p) par[p] = r;  // an ancestor, as in the walk itself
+  }
+}
+
 // ---- compression + coins --------------------------------------------------------
 __global__ void __launch_bounds__(TILE) k_compress(const DevChain *__restrict__ ch,
                                                    const int2 *__restrict__ tab, int64_t blk0,
@@ -1794,9 +1863,19 @@ void launch_link(const Launch &L, cudaStream_t st) {
     k_link<Q><<<g1(L.ntile[Q - 1]), L.link_threads, 0, st>>>(L.ch, L.tile_tab, L.tile0[Q - 1], L.s);
   FOR_EACH_Q(LINK_Q)
 #undef LINK_Q
-  const int64_t n = all_tiles(L);
+  // Tile-crossing edges: a block per tile for few tiles, else a warp per tile.
+  // One update in us (block / warp) by tiles: S = 1/2: 1024 207 / 223, 4096 532 /
+  // 541, 8192 954 / 952; S = 1: 1024 232 / 251, 4096 646 / 651, 8192 1188 / 1172;
+  // S = 2: 1024 429 / 557, 2048 701 / 773, 4096 1224 / 1217.
   const int wpb = L.link_x_warps;
-  if (n) k_link_x<<<g1((n + wpb - 1) / wpb), 32 * wpb, 0, st>>>(L.ch, L.tile_tab, n, L.s);
+  for (int q = 0; q < QMAX; ++q) {
+    const int64_t n = L.ntile[q];
+    if (!n) continue;
+    if (n > XT_MAX_TILES)
+      k_link_x<<<g1((n + wpb - 1) / wpb), 32 * wpb, 0, st>>>(L.ch, L.tile_tab + L.tile0[q], n, L.s);
+    else
+      k_link_xt<<<g1(n), TPB_X, 0, st>>>(L.ch, L.tile_tab, L.tile0[q], L.s);
+  }
 }
 
 void launch_compress(const Launch &L, cudaStream_t st) {
