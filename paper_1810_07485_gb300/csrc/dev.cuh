@@ -132,14 +132,13 @@ __device__ __forceinline__ U4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint
 #pragma unroll
   for (int r = 0; r < 10; ++r) {
     const uint32_t m0 = 0xD2511F53u, m1 = 0xCD9E8D57u;
-    uint32_t lo0 = m0 * c0, hi0 = __umulhi(m0, c0);
-    uint32_t lo1 = m1 * c2, hi1 = __umulhi(m1, c2);
-    uint32_t n0 = hi1 ^ c1 ^ k0;
-    uint32_t n2 = hi0 ^ c3 ^ k1;
+    const uint64_t p0 = (uint64_t)m0 * c0, p1 = (uint64_t)m1 * c2;  // one wide multiply each
+    const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ k0;
+    const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3 ^ k1;
     c0 = n0;
-    c1 = lo1;
+    c1 = (uint32_t)p1;
     c2 = n2;
-    c3 = lo0;
+    c3 = (uint32_t)p0;
     k0 += 0x9E3779B9u;
     k1 += 0xBB67AE85u;
   }
@@ -173,10 +172,10 @@ __device__ __forceinline__ int cell_of(const DevChain &C, int b, int j) {
 
 __device__ __forceinline__ void cell_bj(const DevChain &C, int c, int &b, int &j) {
   int per = C.nbond * TW;
-  int blk = c / per;
+  int blk = c < per ? 0 : c / per;
   int r = c - blk * per;
   int tw = min(TW, C.nwin - blk * TW);
-  b = r / tw;
+  b = tw == TW ? r / TW : r / tw;
   j = blk * TW + (r - b * tw);
 }
 

@@ -201,13 +201,6 @@ __global__ void k_clear(Scratch s, int64_t ntile, int64_t nw) {
 // Imaginary times are handled as the int64 bit patterns of non-negative doubles
 // (same order as the values); a candidate's time is the exact integer form of
 // fma(t_end - t0, u, t0).  No fp64 instruction is issued.
-template <int Q>
-struct NbOps {
-  static constexpr int N = 4 * Q - 2;
-  int bond[N];
-  int o0[N], o1[N];
-};
-
 // Single pass: every tile counts its cells' vertices, publishes the count, and
 // gets the chain-local offset of its first vertex by decoupled look-back over
 // the tiles before it (tile order = order in which blocks took their ticket,
@@ -255,241 +248,345 @@ __device__ int64_t lb_lookback(unsigned long long *st, int64_t g, int64_t first,
   }
 }
 
-// Candidate-parallel insertion.  A tile's cells first set up in shared memory
-// (count K of Poisson candidates, parity at the window start, neighbour
-// operator ranges); then the tile's Philox calls are spread over all threads
-// (call 0 of a cell gives K and candidate 0, call m >= 1 candidates 2m-1 and
-// 2m), each candidate's time is formed and the antiparallel test taken; the
-// kept candidates' places inside their cell follow from ranks: among the
-// cell's kept candidates by (u53, draw index), and against its old operators
-// by time (an old operator goes first on a tie).  Every vertex is then written
-// by its own thread (time, flag, cell; the parent forest is set by the linking
-// kernels).  Candidates are staged INS_CAP at a time: a tile whose candidates
-// exceed that (the mean is 8 * TILE) runs its cells in groups, counting in a
-// first pass and drawing again in the writing pass.
-constexpr int INS_CAP = 1280;
-// Threads of an insertion block: one per cell for the set-up and the scans
-// (the upper half only joins the scans with zeros), all of them for the
-// candidates' draws and the vertices' writes.
+// Candidate-parallel insertion, a warp for every 16 cells of the tile.  Lanes l
+// and l + 16 set up cell l together: each takes the neighbour bonds of one of
+// the cell's subsites (operator ranges, spin parity at the window start) and
+// one of the cell's first two Philox calls (call 0 gives the number K of
+// candidates and candidate 0, call m >= 1 candidates 2m-1 and 2m).  The
+// remaining calls are spread over the lanes, then the candidates: each lane
+// forms a candidate's time, takes the antiparallel test, and the kept ones
+// are packed in place by ballots, so that a cell's kept candidates stay
+// contiguous.  A kept candidate's place inside its cell follows from ranks:
+// among the kept candidates by (u53, draw index), and against the old operators
+// by time (an old operator goes first on a tie).  It marks its position; the
+// unmarked positions are the old operators in their order, so the warp writes
+// its vertices in id order (time, flag, cell; the parent forest is set by the
+// linking kernels).
+//
+// The kernel is bound by instruction issue (85 % of the issue slots; 26 of 32
+// lanes active).  Warps work on their own cells, so that the block meets only
+// for the offsets, and packed candidates and marked positions leave no lane
+// walking a list alone: 1.04 -> 0.78 ms at L=16384, beta=4096 (4.65e7
+// vertices), against one thread per cell for the set-up with block-wide scans
+// and lists (eleven barriers, issue 65 %).  Of the 0.78 ms the set-up takes
+// 0.16, the draws 0.08, the decisions 0.22, the places 0.20, the look-back 0.02
+// and the writes 0.13.  Six blocks per SM at 40 registers (five at 48: 0.82).
+// A warp stages INS_CAP candidates (mean 128, sigma 11): one whose cells have
+// more runs them in groups, counting in a first pass and drawing again in the
+// writing pass.
 constexpr int INS_THREADS = 256;
-constexpr int INS_SPAN = INS_CAP - KMAX;  // a group's cells start within INS_SPAN slots
-constexpr int INS_UCAP = INS_CAP / 2 + TILE;
-constexpr int INS_MIN_SPAN = 256;  // smallest group span a chain may ask for (tests)
-constexpr int INS_MAXG = (TILE * (KMAX - 1)) / INS_MIN_SPAN + 2;
-constexpr int INS_OPCAP = 2048;  // old operators of a group mapped to their cell
-constexpr unsigned long long KEY_DROP = 1ull << 63;
+constexpr int INS_WARPS = INS_THREADS / 32;
+constexpr int INS_WC = TILE / INS_WARPS;  // cells of a warp
+static_assert(INS_WC == 16, "a cell per lane of a half warp");
+constexpr int INS_CAP = 168;
+// Vertices a group of cells may have for its positions to be marked in shared
+// memory (mean 177 for a thermalized S = 1/2 warp, sigma 15).
+constexpr int INS_MARKS = 288;
+// Group sizes a chain may ask for (tests), in candidates of a whole tile.
+constexpr int INS_MIN_SPAN = 256, INS_MAX_SPAN = INS_CAP * INS_WARPS;
 
 // Old operator times a tile stages in shared memory: its own cells' and those
 // of the cells up to 8 Q^2 cells away (the neighbour bonds of the same
 // windows), when they fit (about 1230 for a thermalized S = 1 tile).
 template <int Q>
 struct InsStage {
-  static constexpr int N = Q == 1 ? 1024 : (Q == 2 ? 1536 : 2048);
-};
-
-// Where an old operator's time is read: from the staged copy if its index is
-// in [lo, hi), else from global memory.
-struct OpView {
-  const long long *g;   // op_tau of the chain
-  const long long *sv;  // staged copy, indexed like g (valid in [lo, hi))
-  int lo, hi;
-  __device__ __forceinline__ const long long *range(int a, int b) const {
-    return (a >= lo && b <= hi) ? sv : g;
-  }
+  static constexpr int N = Q == 1 ? 896 : (Q == 2 ? 1536 : 2048);
+  static constexpr int PAD = 4;  // entries a search may read past the last one
 };
 
 template <int Q>
 struct InsSmem {
-  long long sop[InsStage<Q>::N];    // staged old operator times (16-byte aligned: first member)
-  unsigned long long key[INS_CAP];  // (u53 << 6) | draw, with bit 63 set if the candidate is not kept
-  long long tau[INS_CAP];           // time bits; LLONG_MAX if not kept
-  short klist[INS_CAP];             // kept candidates' slots (any order)
-  uint8_t scell[INS_CAP];           // slot -> cell in tile
-  uint8_t ucell[INS_UCAP];          // Philox call -> cell in tile
-  uint8_t qcell[INS_OPCAP];         // old operator -> cell in tile
-  NbOps<Q> X[TILE];
-  unsigned long long T[2][KMAX];    // Poisson thresholds: full windows, last window
-  int kpre[TILE + 1], upre[TILE + 1], q[TILE + 1];
-  int K[TILE], nk[TILE], cex[TILE], b[TILE], j[TILE];
+  static constexpr int NB = 4 * Q - 2;  // neighbour bonds of a cell
+  long long sop[InsStage<Q>::N + InsStage<Q>::PAD];  // staged old operator times (16-byte aligned: first member)
+  // Per warp: the candidates' keys (cell in the warp << 59 | u53 << 6 | draw
+  // index), then, for the kept ones, the same and the times' bits.  Two more
+  // entries: a sentinel, and the second half of a pair load.
+  unsigned long long key[INS_WARPS][INS_CAP + 2];
+  long long tau[INS_WARPS][INS_CAP];
+  // Per cell: neighbour and own operator ranges (from the first staged operator
+  // if all of the warp's ranges are staged), window, kept candidates
+  int2 nb[TILE][NB], own[TILE];
+  int j[TILE], cex[TILE];
+  unsigned short less[TILE], kf[TILE], nk[TILE];  // bit k of less: neighbour bond k < the cell's bond
+  // Per warp: a vertex position's kept candidate + 1, 0 for an old operator
+  uint8_t mark[INS_WARPS][INS_MARKS];
   uint8_t par0[TILE];
-  int gfirst[INS_MAXG + 1];
-  int G, nkept;
-  int sm[33];
+  unsigned long long T[2][KMAX];  // Poisson thresholds: full windows, last window
+  int wtot[INS_WARPS];
   int slo, shi;
   uint64_t bar;
   int64_t excl;
   int64_t gt;
 };
 
-// Number of operators of one neighbour bond (times tq[lo..hi), ascending)
-// that act before a candidate at time tau on bond b: order (time, bond).
-__device__ __forceinline__ int ops_before(const long long *__restrict__ tq, int lo, int hi,
-                                          long long tau, int bb, int b) {
-  const long long thr = tau + (bb < b ? 1 : 0);  // t < thr  <=>  (t, bb) < (tau, b)
+static_assert(sizeof(InsSmem<1>) <= 228 * 1024 / 6 - 1024, "six blocks per SM");
+
+// Number of times below thr in t[lo, hi) (ascending).  ST (staged operators):
+// the ranges hold 4.7 operators on average; more than 7 are halved first, then
+// three steps follow without branches, each reading up to PAD - 1 entries past
+// hi (a halving loop took twice the instructions).
+template <bool ST>
+__device__ __forceinline__ int times_below(const long long *t, int lo, int hi, long long thr) {
   const int base = lo;
-  while (lo < hi) {
+  while (hi - lo > (ST ? 7 : 0)) {
     const int mid = lo + ((hi - lo) >> 1);  // no overflow near 2^31
-    if (tq[mid] < thr)
+    if (t[mid] < thr)
       lo = mid + 1;
     else
       hi = mid;
   }
+  if (ST) {
+#pragma unroll
+    for (int d = 4; d > 0; d >>= 1) {
+      const bool in = lo + d <= hi, below = t[lo + d - 1] < thr;
+      lo += (in & below) ? d : 0;
+    }
+  }
   return lo - base;
 }
 
-// Time of a candidate, tau = fma(d, u53 2^-53, t0) (one IEEE fused
-// multiply-add), and whether it is kept: the bond's spins antiparallel at tau
-// (parity at the window start flipped by the neighbour operators before tau).
-template <int Q>
-__device__ __forceinline__ bool ins_decide(const OpView &V, const NbOps<Q> &X, int b, int par0,
-                                           uint64_t u53, double t0, double d, long long teb,
-                                           long long &tau) {
-  tau = __double_as_longlong(__fma_rn(d, __longlong_as_double((long long)unit_bits(u53)), t0));
-  if (!(tau < teb)) return false;
-  int p = par0;
-#pragma unroll
-  for (int k = 0; k < NbOps<Q>::N; ++k)
-    p ^= ops_before(V.range(X.o0[k], X.o1[k]), X.o0[k], X.o1[k], tau, X.bond[k], b);
-  return p & 1;
+// The double u53 2^-53 of a candidate's key (its bits; unit_bits without the
+// case of fewer than 33 significant bits, which is left to it).
+__device__ __forceinline__ double key_unit(unsigned long long key) {
+  const uint32_t hi = (uint32_t)(key >> 38) & 0x1fffffu, lo = (uint32_t)(key >> 6);
+  uint64_t bits;
+  if (hi) {  // u53 in [2^(52-s), 2^(53-s)), s < 21
+    const int sh = __clz((int)hi) - 11;
+    const uint32_t h = __funnelshift_l(lo, hi, sh) + ((uint32_t)(1021 - sh) << 20);
+    bits = ((uint64_t)h << 32) | (lo << sh);
+  } else {
+    bits = unit_bits(lo);
+  }
+  return __longlong_as_double((long long)bits);
 }
 
-// Draw and decide the candidates of the cells of group g.
-template <int Q>
-__device__ void ins_draw(const DevChain &C, InsSmem<Q> &S, const OpView &V, int g, bool count) {
-  const int c0 = S.gfirst[g], c1 = S.gfirst[g + 1];
-  const int kb = S.kpre[c0], ub = S.upre[c0], nu = S.upre[c1] - ub;
-  {
-    const int c = threadIdx.x;
-    if (c >= c0 && c < c1)
-      for (int u = S.upre[c], e = S.upre[c + 1]; u < e; ++u) S.ucell[u - ub] = (uint8_t)c;
-    if (threadIdx.x == 0) S.nkept = 0;
-  }
-  __syncthreads();
-  const uint32_t k0 = (uint32_t)C.seed, k1 = (uint32_t)(C.seed >> 32);
+// A value that every lane holds, in a form the compiler knows to be uniform
+// (loops bounded by it need no divergence handling).
+__device__ __forceinline__ int uniform(int x) { return (int)__reduce_max_sync(0xffffffffu, x); }
+
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __reduce_max_sync(0xffffffffu, x); }
+
+// A warp's cells: lanes l and l + 16 hold cell l.
+struct InsCell {
+  int b, j, K, kpre;  // bond, window, candidates, candidates of the cells before it
+};
+
+// Times, antiparallel tests and packing of the warp's ns staged candidates;
+// returns how many are kept.  ST: every operator range is staged (shared
+// memory loads), else ot is the chain's operator list.  A candidate's time is
+// tau = fma(d, u53 2^-53, t0) (one IEEE fused multiply-add); it is kept if its
+// bond's spins are antiparallel there (parity at the window start flipped by
+// the neighbour operators before it; order (time, bond)).
+template <int Q, bool ST>
+__device__ __forceinline__ int ins_decide(const DevChain &C, InsSmem<Q> &S, const long long *otau, int wid,
+                                          int ns) {
   const int lane = threadIdx.x & 31;
-  for (int u0 = 0; u0 < nu; u0 += INS_THREADS) {  // whole warps, reconverged per step
-    const int u = u0 + threadIdx.x;
-    bool kp[2] = {false, false};
-    int sl[2] = {0, 0}, c = 0;
-    if (u < nu) {
-      c = S.ucell[u];
-      const int m = u + ub - S.upre[c];
-      const int j = S.j[c], K = S.K[c], ks = S.kpre[c] - kb, b = S.b[c], par0 = S.par0[c];
-      const NbOps<Q> X = S.X[c];
-      const double t0 = __longlong_as_double((long long)C.win[3 * j]);
-      const long long teb = (long long)C.win[3 * j + 1];
-      const double d = __longlong_as_double((long long)C.win[3 * j + 2]);
-      const U4 o = philox((TAG_INSERT << 24) | (uint32_t)m, (uint32_t)b, (uint32_t)j, C.sweep, k0, k1);
-      // words (x, y): candidate 2m-1 (for m = 0 the count); words (z, w): candidate 2m
+  const long long *ot = ST ? S.sop : otau;
+  int nkept = 0;
+  for (int i0 = 0; i0 < ns; i0 += 32) {
+    const int slot = i0 + lane;
+    bool keep = false;
+    unsigned long long key = 1;
+    long long tau = 0;
+    int c = 0;
+    if (slot < ns) {
+      key = S.key[wid][slot];
+      c = (int)(key >> 59);
+      const int cw = wid * INS_WC + c;
+      const uint64_t *win = C.win + 3 * S.j[cw];
+      const double t0 = __longlong_as_double((long long)win[0]);
+      const long long teb = (long long)win[1];
+      const double d = __longlong_as_double((long long)win[2]);
+      tau = __double_as_longlong(__fma_rn(d, key_unit(key), t0));
+      if (tau < teb) {
+        int p = S.par0[cw];
+        const int less = S.less[cw];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int k = 2 * m - 1 + h;
-        if (k < 0 || k >= K) continue;
-        const uint64_t u53 = (h ? ((uint64_t)o.z | ((uint64_t)o.w << 32))
-                                : ((uint64_t)o.x | ((uint64_t)o.y << 32))) >> 11;
-        long long tau;
-        const bool keep = ins_decide<Q>(V, X, b, par0, u53, t0, d, teb, tau);
-        const int slot = ks + k;
-        // (u53, draw) packed into one key, unique within the cell
-        S.key[slot] = ((u53 << 6) | (uint64_t)k) | (keep ? 0ull : KEY_DROP);
-        S.tau[slot] = keep ? tau : LLONG_MAX;
-        S.scell[slot] = (uint8_t)c;
-        kp[h] = keep;
-        sl[h] = slot;
+        for (int k = 0; k < InsSmem<Q>::NB; ++k) {
+          const int2 r = S.nb[cw][k];
+          p ^= times_below<ST>(ot, r.x, r.y, tau + ((less >> k) & 1));
+        }
+        keep = p & 1;
       }
     }
-    // kept list: one shared atomic per warp and half
+    const unsigned km = __ballot_sync(0xffffffffu, keep);
+    const int at = nkept + __popc(km & ((1u << lane) - 1u));
+    __syncwarp();  // every lane has read its candidate: pack over the ones read
+    if (slot < ns && (key & 63) == 0) S.kf[wid * INS_WC + c] = (unsigned short)at;
+    if (keep) {
+      S.key[wid][at] = key;
+      S.tau[wid][at] = tau;
+    }
+    nkept += __popc(km);
+  }
+  __syncwarp();
+  if (lane == 0) S.key[wid][nkept] = ~0ull;
+  return nkept;
+}
+
+// Draw and decide the candidates of the warp's cells [c0, c1); o: the lane's
+// output of Philox call (lane >= 16) of its cell.  Sets kf and nk of the cells;
+// returns the number kept.
+template <int Q>
+__device__ __forceinline__ int ins_group(const DevChain &C, InsSmem<Q> &S, const long long *otau, int wid,
+                                         const InsCell &X, const U4 &o, int c0, int c1, bool staged, uint32_t sweep,
+                                         uint32_t k0, uint32_t k1) {
+  const int lane = threadIdx.x & 31, cl = lane & 15, side = lane >> 4;
+  const bool in = cl >= c0 && cl < c1;
+  const int kb = __shfl_sync(0xffffffffu, X.kpre, c0);
+  const int ns = uniform(__shfl_sync(0xffffffffu, X.kpre + X.K, c1 - 1) - kb);
+  auto put = [&](int c, int slot, int k, uint32_t lo, uint32_t hi) {
+    const uint64_t u53 = ((uint64_t)lo | ((uint64_t)hi << 32)) >> 11;
+    S.key[wid][slot] = ((uint64_t)c << 59) | (u53 << 6) | (uint64_t)k;
+  };
+  // calls 0 (lower lanes: candidate 0) and 1 (upper lanes: candidates 1, 2)
+  if (in) {
+    const int ks = X.kpre - kb;
+    if (side && X.K > 1) put(cl, ks + 1, 1, o.x, o.y);
+    if (X.K > 2 * side) put(cl, ks + 2 * side, 2 * side, o.z, o.w);
+  }
+  // calls 2 .. K/2
+  const int P = (in && X.K > 3) ? X.K / 2 - 1 : 0;
+  int pin = P;  // inclusive scan over the cells (both halves alike)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const unsigned km = __ballot_sync(0xffffffffu, kp[h]);
-      if (km) {
-        const int leader = __ffs(km) - 1;
-        int at = 0;
-        if (lane == leader) at = atomicAdd(&S.nkept, __popc(km));
-        at = __shfl_sync(0xffffffffu, at, leader);
-        if (kp[h]) {
-          S.klist[at + __popc(km & ((1u << lane) - 1u))] = (short)sl[h];
-          if (count) atomicAdd(&S.nk[c], 1);
-        }
+  for (int d = 1; d < 16; d <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, pin, d, 16);
+    if (cl >= d) pin += y;
+  }
+  const int nu = uniform(__shfl_sync(0xffffffffu, pin, 15));
+  for (int u0 = 0; u0 < nu; u0 += 32) {
+    const int u = u0 + lane;
+    int c = 0;  // cells whose calls all come before call u
+#pragma unroll
+    for (int d = 8; d > 0; d >>= 1) {
+      const int y = __shfl_sync(0xffffffffu, pin, c + d - 1);
+      if (y <= u) c += d;
+    }
+    // (for u >= nu the search ends at cell 15; those lanes draw nothing)
+    const int first = __shfl_sync(0xffffffffu, pin - P, c), b = __shfl_sync(0xffffffffu, X.b, c);
+    const int j = __shfl_sync(0xffffffffu, X.j, c), K = __shfl_sync(0xffffffffu, X.K, c);
+    const int ks = __shfl_sync(0xffffffffu, X.kpre, c) - kb;
+    if (u < nu) {
+      const int m = 2 + u - first, k = 2 * m - 1;
+      const U4 p = philox((TAG_INSERT << 24) | (uint32_t)m, (uint32_t)b, (uint32_t)j, sweep, k0, k1);
+      if (k < K) put(c, ks + k, k, p.x, p.y);
+      if (k + 1 < K) put(c, ks + k + 1, k + 1, p.z, p.w);
+    }
+  }
+  __syncwarp();
+  const int nkept = staged ? ins_decide<Q, true>(C, S, otau, wid, ns) : ins_decide<Q, false>(C, S, otau, wid, ns);
+  // first kept candidate and number kept per cell; a cell without candidates
+  // starts where the next one with candidates does
+  const unsigned has = __ballot_sync(0xffffffffu, in && lane < 16 && X.K > 0);
+  const unsigned from = has >> cl;
+  const int nx = from ? cl + __ffs(from) - 1 : cl;
+  int kf = (in && X.K > 0) ? S.kf[wid * INS_WC + cl] : nkept;
+  kf = __shfl_sync(0xffffffffu, kf, nx);
+  const int kn = __shfl_down_sync(0xffffffffu, kf, 1, 16);
+  __syncwarp();
+  if (in && lane < 16) {
+    S.kf[wid * INS_WC + cl] = (unsigned short)kf;
+    S.nk[wid * INS_WC + cl] = (unsigned short)((cl == c1 - 1 ? nkept : kn) - kf);
+  }
+  __syncwarp();
+  return nkept;
+}
+
+// Positions of the warp's nkept kept candidates among the vertices of its cells
+// (cell order, then time): marked in shared memory from position `from` on, or,
+// for DIRECT, written to the vertex arrays at once.
+template <int Q, bool ST, bool DIRECT>
+__device__ __forceinline__ void ins_place(const DevChain &C, InsSmem<Q> &S, const long long *otau, int wid,
+                                          int nkept, int from, int64_t base, const Scratch &s) {
+  const int lane = threadIdx.x & 31;
+  const long long *ot = ST ? S.sop : otau;
+  for (int i0 = 0; i0 < nkept; i0 += 32) {
+    const int i = i0 + lane;
+    if (i < nkept) {
+      const unsigned long long key = S.key[wid][i];
+      const long long tau = S.tau[wid][i];
+      const int cw = wid * INS_WC + (int)(key >> 59);
+      // kept candidates ahead, two keys a step from an even place on (one of
+      // the cell before is below the cell's keys, what follows is above them)
+      const int kf = S.kf[cw], k0 = kf & ~1, k1 = kf + S.nk[cw];
+      int r = k0 - kf;
+      for (int x = k0; x < k1; x += 2) {
+        const ulonglong2 kk = *(const ulonglong2 *)&S.key[wid][x];
+        r += (int)(kk.x < key) + (int)(kk.y < key);
+      }
+      const int2 own = S.own[cw];
+      r += times_below<ST>(ot, own.x, own.y, tau + 1);  // old operators at or before tau
+      const int pos = S.cex[cw] + r;
+      if (DIRECT) {
+        const int64_t v = C.vtx_base + base + pos;
+        ((long long *)s.vtau)[v] = tau;
+        s.vflag[v] = 0;
+        s.vcell[v] = (uint8_t)cw;
+      } else {
+        S.mark[wid][pos - from] = (uint8_t)(i + 1);
       }
     }
     __syncwarp();
   }
-  __syncthreads();
 }
 
-// Place and write the vertices of the cells of group g (kept candidates, then
-// old operators); vertex ids are chain-local, base = the tile's first id.
-template <int Q>
-__device__ void ins_write(const DevChain &C, InsSmem<Q> &S, const OpView &V, int g,
-                          int64_t base, const Scratch &s) {
-  const int c0 = S.gfirst[g], c1 = S.gfirst[g + 1];
-  const int kb = S.kpre[c0];
-  const int64_t vb = C.vtx_base;
+// Write the marked vertices [0, n) from tile position `from` on, in id order:
+// the positions without a mark are the old operators from qa on, in their
+// order.  ce: first position of the lane's cell.
+template <int Q, bool ST>
+__device__ __forceinline__ void ins_write(const DevChain &C, InsSmem<Q> &S, const long long *otau, int wid, int n,
+                                          int from, int ce, int qa, int64_t base, const Scratch &s) {
+  const int lane = threadIdx.x & 31;
+  const int64_t vb = C.vtx_base + base + from;
   long long *vt = (long long *)s.vtau + vb;
   uint8_t *vf = s.vflag + vb, *vc = s.vcell + vb;
-  const int nkept = S.nkept;
-  for (int i0 = 0; i0 < nkept; i0 += INS_THREADS) {
-    const int i = i0 + threadIdx.x;
-    if (i >= nkept) {
-      __syncwarp();
-      continue;
+  const long long *ot = ST ? S.sop - S.slo : otau;
+  for (int i0 = 0; i0 < n; i0 += 32) {
+    const int i = i0 + lane, m = i < n ? S.mark[wid][i] : 0;
+    const unsigned old = __ballot_sync(0xffffffffu, i < n && m == 0);
+    int c = 0;  // largest cell with first position <= i
+#pragma unroll
+    for (int d = 8; d > 0; d >>= 1) {
+      const int y = __shfl_sync(0xffffffffu, ce, c + d);
+      if (y <= from + i) c += d;
     }
-    const int slot = S.klist[i];
-    const long long tau = S.tau[slot];
-    const int c = S.scell[slot];
-    const int ks = S.kpre[c] - kb, K = S.K[c];
-    const unsigned long long key = S.key[slot];
-    int r = 0;
-    for (int x = 0; x < K; ++x) r += S.key[ks + x] < key;  // kept keys ahead (a dropped one has bit 63)
-    // old operators at or before tau (ascending times)
-    int lo = S.q[c], hi = S.q[c + 1];
-    const int q0 = lo;
-    const long long *otau = V.range(lo, hi);
-    while (lo < hi) {
-      const int mid = lo + ((hi - lo) >> 1);  // no overflow near 2^31
-      if (otau[mid] <= tau)
-        lo = mid + 1;
-      else
-        hi = mid;
+    if (i < n) {
+      vt[i] = m ? S.tau[wid][m - 1] : ot[qa + __popc(old & ((1u << lane) - 1u))];
+      vf[i] = m ? 0 : VF_OLD;
+      vc[i] = (uint8_t)(wid * INS_WC + c);
     }
-    r += lo - q0;
-    const int64_t pos = base + S.cex[c] + r;
-    vt[pos] = tau;
-    vf[pos] = 0;
-    vc[pos] = (uint8_t)c;
-    __syncwarp();
+    qa += __popc(old);
   }
-  const int qa = S.q[c0], qb = S.q[c1], qt = S.q[0];
-  const bool mapped = qb - qt <= INS_OPCAP;
-  for (int q0 = qa; q0 < qb; q0 += INS_THREADS) {
-    const int q = q0 + threadIdx.x;
-    if (q >= qb) {
-      __syncwarp();
-      continue;
+  __syncwarp();
+}
+
+// The old operators [qa, qb) of a group of cells with too many vertices for the
+// marks: each finds its place by the kept candidates before it.  q0, ce: first
+// operator and first position of the lane's cell.
+template <int Q>
+__device__ __noinline__ void ins_write_old(InsSmem<Q> &S, const long long *otau, int wid, int q0, int ce, int qa,
+                                           int qb, long long *vt, uint8_t *vf, uint8_t *vc) {
+  const int lane = threadIdx.x & 31;
+  for (int qq = qa; qq < qb; qq += 32) {
+    const int q = qq + lane;
+    int c = 0;  // largest cell with first operator <= q
+#pragma unroll
+    for (int d = 8; d > 0; d >>= 1) {
+      const int y = __shfl_sync(0xffffffffu, q0, c + d);
+      if (y <= q) c += d;
     }
-    int c;
-    if (mapped) {
-      c = S.qcell[q - qt];
-    } else {
-      int lo = c0, hi = c1 - 1;  // largest c in [c0, c1) with S.q[c] <= q
-      while (lo < hi) {
-        const int mid = lo + ((hi - lo + 1) >> 1);
-        if (S.q[mid] <= q)
-          lo = mid;
-        else
-          hi = mid - 1;
-      }
-      c = lo;
+    const int qc = __shfl_sync(0xffffffffu, q0, c), pc = __shfl_sync(0xffffffffu, ce, c);
+    if (q < qb) {
+      const int cw = wid * INS_WC + c;
+      const long long t = otau[q];
+      const long long *tt = &S.tau[wid][S.kf[cw]];
+      const int n = S.nk[cw];
+      int r = q - qc;
+      for (int x = 0; x < n; ++x) r += tt[x] < t;
+      vt[pc + r] = t;
+      vf[pc + r] = VF_OLD;
+      vc[pc + r] = (uint8_t)cw;
     }
-    const long long ot = (q >= V.lo && q < V.hi) ? V.sv[q] : V.g[q];
-    const int ks = S.kpre[c] - kb, K = S.K[c];
-    int r = q - S.q[c];
-    for (int x = 0; x < K; ++x) r += S.tau[ks + x] < ot;
-    const int64_t pos = base + S.cex[c] + r;
-    vt[pos] = ot;
-    vf[pos] = VF_OLD;
-    vc[pos] = (uint8_t)c;
     __syncwarp();
   }
 }
@@ -499,20 +596,14 @@ __device__ __forceinline__ void insert_tile(InsSmem<Q> &S, DevChain *__restrict_
                                             const int2 *__restrict__ tab, int64_t blk0, int group,
                                             Scratch s);
 
-// The staging area is static shared memory for Q = 1 and dynamic shared
-// memory (above the 48 KB static limit) for the larger neighbour tables and
-// operator stages of Q = 2, 3, 4.
+// Dynamic shared memory: 36 KB for Q = 1 (six blocks per SM), above the 48 KB
+// static limit for the larger neighbour tables and operator stages of Q >= 3.
 template <int Q>
-__global__ void __launch_bounds__(INS_THREADS, Q == 1 ? 5 : 4) k_insert(DevChain *__restrict__ ch,
+__global__ void __launch_bounds__(INS_THREADS, Q == 1 ? 6 : 4) k_insert(DevChain *__restrict__ ch,
                                                  const int2 *__restrict__ tab, int64_t blk0,
                                                  int group, Scratch s) {
-  if constexpr (Q == 1) {
-    __shared__ __align__(16) InsSmem<Q> S;
-    insert_tile<Q>(S, ch, tab, blk0, group, s);
-  } else {
-    extern __shared__ __align__(16) unsigned char ins_dyn[];
-    insert_tile<Q>(*reinterpret_cast<InsSmem<Q> *>(ins_dyn), ch, tab, blk0, group, s);
-  }
+  extern __shared__ __align__(16) unsigned char ins_dyn[];
+  insert_tile<Q>(*reinterpret_cast<InsSmem<Q> *>(ins_dyn), ch, tab, blk0, group, s);
 }
 
 template <int Q>
@@ -525,10 +616,6 @@ __device__ __forceinline__ void insert_tile(InsSmem<Q> &S, DevChain *__restrict_
   const int64_t gt = S.gt;
   const int2 t = tab[gt];
   DevChain &C = ch[t.x];
-  const int c = threadIdx.x;
-  const bool own = c < TILE;  // this thread's cell (the upper half has none)
-  const int cell = t.y * TILE + c;
-  const bool valid = own && cell < C.ncell;
   const int cur = C.cur;
   const int32_t *op = C.op_ptr[cur];
   const long long *otau = (const long long *)C.op_tau[cur];
@@ -557,117 +644,140 @@ __device__ __forceinline__ void insert_tile(InsSmem<Q> &S, DevChain *__restrict_
   }
   __syncthreads();
 
-  // -- per-cell setup --------------------------------------------------------
-  // The lower half of the block takes the cells' neighbour ranges and spin
-  // parities, the upper half their candidate counts (Philox call 0), side by
-  // side.
-  int q0 = 0, q1 = 0;
+  // -- per-cell set-up ---------------------------------------------------------
+  const int lane = threadIdx.x & 31, wid = uniform((int)threadIdx.x >> 5), cl = lane & 15, side = lane >> 4;
+  const int cw = wid * INS_WC + cl, cell = t.y * TILE + cw;
+  const bool valid = cell < C.ncell;
+  const int slo = S.slo, shi = S.shi;
+  // the keys as uniform values: their schedule leaves the vector pipes
+  const uint32_t k0 = uniform((uint32_t)C.seed), k1 = uniform((uint32_t)(C.seed >> 32)), sweep = uniform(C.sweep);
+  InsCell X{0, 0, 0, 0};
+  int q0, q1, par = 0, less = 0;
+  bool staged = shi > slo;
+  U4 o{0, 0, 0, 0};
   if (valid) {
-    int b, j;
-    cell_bj(C, cell, b, j);
-    const int ul = left_sub<Q>(b), ur = right_sub<Q>(b, C.L);
-    const int blk = j / TW, jb = blk * TW;
+    cell_bj(C, cell, X.b, X.j);
+    o = philox((TAG_INSERT << 24) | (uint32_t)side, (uint32_t)X.b, (uint32_t)X.j, sweep, k0, k1);
+    const int u = side ? right_sub<Q>(X.b, C.L) : left_sub<Q>(X.b);
+    const int blk = X.j / TW, jb = blk * TW;
     const uint8_t *prow = s.bpar + C.bpar_off + (int64_t)blk * C.nbond;
-    int par0 = (s0[ul] ^ s0[ur]) & 1;
-    NbOps<Q> X;
-    int k = 0;
+    int k = side * (2 * Q - 1);
+    par = s0[u] & 1;
 #pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      const int u = side ? ur : ul;
-#pragma unroll
-      for (int m = 0; m < 2 * Q; ++m) {
-        const int bb = inc_bond<Q>(u, m, C.L);
-        if (bb == b) continue;
-        const int cj = cell_of(C, bb, j), cs = cell_of(C, bb, jb);
-        X.bond[k] = bb;
-        X.o0[k] = op[cj];
-        X.o1[k] = op[cj + 1];
-        par0 ^= (prow[bb] ^ (op[cj] - op[cs])) & 1;
-        ++k;
-      }
+    for (int m = 0; m < 2 * Q; ++m) {
+      const int bb = inc_bond<Q>(u, m, C.L);
+      if (bb == X.b) continue;
+      const int cj = cell_of(C, bb, X.j), cs = cell_of(C, bb, jb);
+      const int a = op[cj], e = op[cj + 1];
+      par ^= (prow[bb] ^ (a - op[cs])) & 1;
+      staged &= a >= slo && e <= shi;
+      less |= (bb < X.b ? 1 : 0) << k;
+      S.nb[cw][k] = make_int2(a, e);
+      ++k;
     }
-    S.X[c] = X;
-    S.par0[c] = (uint8_t)par0;
-    S.b[c] = b;
-    S.j[c] = j;
     q0 = op[cell];
     q1 = op[cell + 1];
-  } else if (!own && t.y * TILE + (c - TILE) < C.ncell) {
-    const int cc = c - TILE;  // the cell whose count this thread draws
-    int b, j, K = 0;
-    cell_bj(C, t.y * TILE + cc, b, j);
-    const uint64_t db = C.win[3 * j + 2];
-    const U4 o0 = philox(TAG_INSERT << 24, (uint32_t)b, (uint32_t)j, C.sweep, (uint32_t)C.seed,
-                         (uint32_t)(C.seed >> 32));
-    const uint64_t U = (uint64_t)o0.x | ((uint64_t)o0.y << 32);
-    const unsigned long long *T = S.T[j == C.nwin - 1 ? 1 : 0];
+    staged &= q0 >= slo && q1 <= shi;
+  } else {
+    q0 = q1 = op[C.ncell];  // cells past the chain's end: empty ranges
+  }
+  __syncwarp();
+  par ^= __shfl_xor_sync(0xffffffffu, par, 16);
+  less |= __shfl_xor_sync(0xffffffffu, less, 16);
+  if (valid && !side) {
+    S.par0[cw] = (uint8_t)par;
+    S.less[cw] = (unsigned short)less;
+    S.j[cw] = X.j;
+    S.own[cw] = make_int2(q0, q1);
     // K = number of thresholds T[0..KMAX-2] at or below U (they ascend)
+    const uint64_t U = (uint64_t)o.x | ((uint64_t)o.y << 32);
+    const unsigned long long *T = S.T[X.j == C.nwin - 1 ? 1 : 0];
 #pragma unroll
     for (int step = 32; step > 0; step >>= 1)
-      if (K + step <= KMAX - 1 && T[K + step - 1] <= U) K += step;
-    if ((long long)db <= 0) K = 0;  // empty last window
-    S.K[cc] = K;
-  } else if (!own) {
-    S.K[c - TILE] = 0;  // cells past the chain's end
+      if (X.K + step <= KMAX - 1 && T[X.K + step - 1] <= U) X.K += step;
+    if ((long long)C.win[3 * X.j + 2] <= 0) X.K = 0;  // empty last window
   }
-  if (!valid) q0 = q1 = op[C.ncell];  // cells past the chain's end: empty ranges
-  if (own) {
-    S.nk[c] = 0;
-    S.q[c] = q0;
+  __syncwarp();
+  X.K = __shfl_sync(0xffffffffu, X.K, cl);
+  X.kpre = X.K;
+#pragma unroll
+  for (int d = 1; d < 16; d <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, X.kpre, d, 16);
+    if (cl >= d) X.kpre += y;
   }
-  if (c == TILE - 1) S.q[TILE] = q1;
-  __syncthreads();
-  const int K = own ? S.K[c] : 0, P = K ? K / 2 + 1 : 0;
-  int tot;
-  const int ex = block_excl_scan<int>(K | (P << 16), S.sm, tot);
-  if (own) {
-    // old operator -> cell map (all of the tile's operators, if they fit)
-    const int qa = S.q[0];
-    for (int q = q0; q < q1 && q - qa < INS_OPCAP; ++q) S.qcell[q - qa] = (uint8_t)c;
-    S.kpre[c] = ex & 0xffff;
-    S.upre[c] = ex >> 16;
-  }
-  if (c == TILE - 1) {
-    S.kpre[TILE] = tot & 0xffff;
-    S.upre[TILE] = tot >> 16;
-  }
-  __syncthreads();
-  if (own) {
-    const int span =
-        (C.ins_span >= INS_MIN_SPAN && C.ins_span < INS_SPAN) ? C.ins_span : INS_SPAN;
-    const int gc = S.kpre[c] / span;
-    if (c == 0 || gc != S.kpre[c - 1] / span) S.gfirst[gc] = c;
-    if (c == TILE - 1) {
-      S.G = gc + 1;
-      S.gfirst[gc + 1] = TILE;
+  X.kpre -= X.K;
+  staged = __all_sync(0xffffffffu, staged || !valid) && shi > slo;
+  if (staged && valid) {  // ranges from the first staged operator on
+    const int n0 = side * (2 * Q - 1);
+#pragma unroll
+    for (int k = 0; k < 2 * Q - 1; ++k) {
+      S.nb[cw][n0 + k].x -= slo;
+      S.nb[cw][n0 + k].y -= slo;
     }
+    if (!side) S.own[cw] = make_int2(q0 - slo, q1 - slo);
   }
-  __syncthreads();
-  const int G = S.G;
-  if (S.shi > S.slo) {
-    const bool ok = mbar_wait(&S.bar, 0);
-    if (!__syncthreads_and(ok)) {
-      if (threadIdx.x == 0) atomicOr(s.status, ST_TIMEOUT);
-      return;
-    }
+  __syncwarp();
+  bool ok = true;
+  if (shi > slo) ok = mbar_wait(&S.bar, 0);
+
+  // -- draw, decide, count; then place and write --------------------------------
+  const int cap = (C.ins_span >= INS_MIN_SPAN && C.ins_span < INS_MAX_SPAN)
+                      ? max(KMAX - 1, C.ins_span / INS_WARPS)
+                      : INS_CAP;
+  const bool single = __shfl_sync(0xffffffffu, X.kpre + X.K, 15) <= cap;
+  // Vertices of a group of cells: kept candidates placed (marked), all written.
+  int nkept = 0, nk = 0, cex = 0;
+  auto next = [&](int c0) {  // end of the group that starts at cell c0
+    if (single) return INS_WC;
+    const int kb = __shfl_sync(0xffffffffu, X.kpre, c0);
+    return c0 + __popc(__ballot_sync(0xffffffffu, lane < 16 && cl >= c0 && X.kpre + X.K - kb <= cap));
+  };
+  for (int c0 = 0; c0 < INS_WC;) {
+    const int c1 = next(c0);
+    nkept = uniform(ins_group<Q>(C, S, otau, wid, X, o, c0, c1, staged, sweep, k0, k1));
+    if (cl >= c0 && cl < c1) nk = S.nk[cw];
+    c0 = c1;
   }
-  const OpView V{otau, S.sop - S.slo, S.slo, S.shi};
-
-  // -- draw, decide and count ------------------------------------------------
-  for (int g = 0; g < G; ++g) ins_draw<Q>(C, S, V, g, true);
-  const int cnt = valid ? (q1 - q0) + S.nk[c] : 0;
-  int ctot;
-  const int cex = block_excl_scan<int>(cnt, S.sm, ctot);
-  if (own) S.cex[c] = cex;
-
-  // -- chain-local offset of the tile: decoupled look-back --------------------
+  const int cnt = q1 - q0 + nk;
+  cex = cnt;
+#pragma unroll
+  for (int d = 1; d < 16; d <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, cex, d, 16);
+    if (cl >= d) cex += y;
+  }
+  if (lane == 15) S.wtot[wid] = cex;
+  cex -= cnt;
+  if (!__syncthreads_and(ok)) {  // the bulk copy did not arrive within its bound
+    if (threadIdx.x == 0) atomicOr(s.status, ST_TIMEOUT);
+    return;
+  }
+  int ctot = 0;
+#pragma unroll
+  for (int k = 0; k < INS_WARPS; ++k) {
+    if (k == wid) cex += ctot;
+    ctot += S.wtot[k];
+  }
+  // The tile's count goes out before its candidates are placed, the look-back
+  // for its offset comes after: by then the tiles before it have mostly
+  // published theirs.
+  if (threadIdx.x == 0) lb_publish(s.tile_state, gt, t.y == 0 ? LB_INC : LB_AGG, ctot);
+  if (lane < 16) S.cex[cw] = cex;
+  auto marked = [&](int from, int n) {
+    if (n > INS_MARKS) return false;
+    for (int i = lane; i < (n + 3) / 4; i += 32) ((uint32_t *)S.mark[wid])[i] = 0u;
+    __syncwarp();
+    if (staged)
+      ins_place<Q, true, false>(C, S, otau, wid, nkept, from, 0, s);
+    else
+      ins_place<Q, false, false>(C, S, otau, wid, nkept, from, 0, s);
+    return true;
+  };
+  const int wfrom = __shfl_sync(0xffffffffu, cex, 0), wn = uniform(__shfl_sync(0xffffffffu, cex + cnt, 15) - wfrom);
+  __syncwarp();
+  bool mk = single && marked(wfrom, wn);
   if (threadIdx.x < 32) {
     int64_t excl = 0;
-    if (t.y == 0) {
-      if (threadIdx.x == 0) lb_publish(s.tile_state, gt, LB_INC, ctot);
-    } else {
-      if (threadIdx.x == 0) lb_publish(s.tile_state, gt, LB_AGG, ctot);
-      __syncwarp();
+    if (t.y != 0) {
       excl = lb_lookback(s.tile_state, gt, gt - t.y, s);
       if (threadIdx.x == 0) lb_publish(s.tile_state, gt, LB_INC, excl + ctot);
     }
@@ -685,16 +795,30 @@ __device__ __forceinline__ void insert_tile(InsSmem<Q> &S, DevChain *__restrict_
   __syncthreads();
   const int64_t base = S.excl;
   if (base + ctot > C.vcap) return;  // overflow: the host grows the chain and replays
-  if (valid) {
-    vp[cell] = (int32_t)(base + S.cex[c]);
-    if (cell == C.ncell - 1) vp[C.ncell] = (int32_t)(base + S.cex[c] + cnt);
+  if (valid && !side) {
+    vp[cell] = (int32_t)(base + cex);
+    if (cell == C.ncell - 1) vp[C.ncell] = (int32_t)(base + cex + cnt);
   }
-
-  // -- write -----------------------------------------------------------------
-  for (int g = 0; g < G; ++g) {
-    if (G > 1) ins_draw<Q>(C, S, V, g, false);
-    ins_write<Q>(C, S, V, g, base, s);
-    __syncthreads();
+  if (!single && valid)  // drawn again group by group
+    o = philox((TAG_INSERT << 24) | (uint32_t)side, (uint32_t)X.b, (uint32_t)X.j, sweep, k0, k1);
+  for (int c0 = 0; c0 < INS_WC;) {
+    const int c1 = next(c0);
+    const int qa = __shfl_sync(0xffffffffu, q0, c0), qb = __shfl_sync(0xffffffffu, q1, c1 - 1);
+    const int from = __shfl_sync(0xffffffffu, cex, c0), n = uniform(__shfl_sync(0xffffffffu, cex + cnt, c1 - 1) - from);
+    if (!single) {
+      nkept = ins_group<Q>(C, S, otau, wid, X, o, c0, c1, staged, sweep, k0, k1);
+      mk = marked(from, n);
+    }
+    if (!mk) {
+      ins_place<Q, false, true>(C, S, staged ? S.sop : otau, wid, nkept, 0, base, s);
+      const int64_t vb = C.vtx_base + base;
+      ins_write_old<Q>(S, otau, wid, q0, cex, qa, qb, (long long *)s.vtau + vb, s.vflag + vb, s.vcell + vb);
+    } else if (staged) {
+      ins_write<Q, true>(C, S, otau, wid, n, from, cex, qa, base, s);
+    } else {
+      ins_write<Q, false>(C, S, otau, wid, n, from, cex, qa, base, s);
+    }
+    c0 = c1;
   }
 }
 
@@ -1838,7 +1962,7 @@ void launch_clear(const Launch &L, int64_t ntile, int64_t nw, cudaStream_t st) {
 void launch_insert(const Launch &L, cudaStream_t st) {
 #define INSERT_Q(Q)                                                                                   \
   if (L.ntile[Q - 1])                                                                                 \
-    k_insert<Q><<<g1(L.ntile[Q - 1]), INS_THREADS, Q == 1 ? 0 : sizeof(InsSmem<Q>), st>>>(L.ch,          \
+    k_insert<Q><<<g1(L.ntile[Q - 1]), INS_THREADS, sizeof(InsSmem<Q>), st>>>(L.ch,          \
                                                                                           L.tile_tab,    \
                                                                                           L.tile0[Q - 1], \
                                                                                           Q - 1, L.s);
@@ -1914,13 +2038,12 @@ int init_kernel_attributes() {
     return -1;
   FOR_EACH_Q(EST_ATTR_Q)
 #undef EST_ATTR_Q
-  if (cudaFuncSetAttribute(k_insert<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)sizeof(InsSmem<2>)) != cudaSuccess ||
-      cudaFuncSetAttribute(k_insert<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)sizeof(InsSmem<3>)) != cudaSuccess ||
-      cudaFuncSetAttribute(k_insert<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)sizeof(InsSmem<4>)) != cudaSuccess)
+#define INS_ATTR_Q(Q)                                                          \
+  if (cudaFuncSetAttribute(k_insert<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                           (int)sizeof(InsSmem<Q>)) != cudaSuccess)                  \
     return -1;
+  FOR_EACH_Q(INS_ATTR_Q)
+#undef INS_ATTR_Q
   done[dev] = true;
   return 0;
 }
