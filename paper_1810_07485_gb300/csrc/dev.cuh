@@ -18,7 +18,6 @@ constexpr int ACC_WORDS = 4;    // 64-bit words of an open loop's record (32 byt
 constexpr int PHASE_BITS = 16;  // phase factor table: 2^16 points of the period
 constexpr int TILE = 128;         // cells per tile (one thread block)
 constexpr int SMEM_CAP = 2048;    // vertices a tile can accumulate in shared memory
-constexpr int MAX_COIN_GROUPS = 64;
 constexpr int SITE_BLOCK = 128;   // original sites per block
 constexpr int BOND_BLOCK = 128;   // bonds per block
 constexpr double CELL_MEAN = 8.0; // mean candidate graphs per full window (w = 16/J)
@@ -37,7 +36,7 @@ enum : int {
 };
 
 // Vertex flag bits.
-enum : uint8_t { VF_OLD = 1, VF_WRAP_L = 2, VF_WRAP_R = 4, VF_NEW = 8 };
+enum : uint8_t { VF_OLD = 1, VF_WRAP_L = 2, VF_WRAP_R = 4 };
 
 struct DevChain {
   // geometry
@@ -99,7 +98,9 @@ struct Scratch {
     ulonglong2 *acc2;         // the same records as two 16-byte halves
   };
   unsigned long long *accz;  // per vertex: Zi, open loops only, temporal moment on
-  uint32_t *openmark, *openroot, *flipbits, *xmark;
+  // one bit per vertex: node on a tile-crossing edge; root of a loop that leaves
+  // its tile; loop of the node flips; new operator; edge leaves the tile
+  uint32_t *openmark, *openroot, *flipbits, *newbits, *xmark;
   int64_t vcap;
   unsigned long long *tile_state;  // per tile: insertion look-back word (flag << 62 | count)
   unsigned int *tickets;           // per Q group: next tile of the insertion launch
@@ -259,10 +260,11 @@ __device__ __forceinline__ u128 sq_abs(long long v) {
 // ---- times as bit patterns ------------------------------------------------------
 // GB300 executes fp64 instructions on a handful of lanes per SM, so the hot
 // loops keep imaginary times as the bit patterns of non-negative doubles
-// (ordered like the doubles themselves when read as int64).  The only fp64
-// instruction left is one fused multiply-add per insertion candidate; the
-// conversion of times to integer ticks is done with integer arithmetic,
-// exactly as IEEE 754 defines it (round to nearest, ties to even).
+// (ordered like the doubles themselves when read as int64) and compare those.
+// Two fp64 instructions are left: one fused multiply-add per insertion
+// candidate, and per vertex the conversion of its time to integer ticks (25
+// integer instructions; rounded to nearest, ties to even), with the fp64 pipe
+// otherwise idle.
 
 constexpr uint64_t M52 = (1ull << 52) - 1;
 
@@ -279,7 +281,14 @@ __host__ __device__ __forceinline__ uint64_t unit_bits(uint64_t u53) {
 }
 
 // llrint(ldexp(x, F)) for a non-negative double x given as bits (x 2^F < 2^62).
+// Device: the exponent raised by F and one rounding conversion (25 integer
+// instructions otherwise: k_est 0.82 -> 0.73 ms at L=16384, beta=4096; the fp64
+// pipe stays at a fifth); a denormal x is below half a tick.  Host (self test):
+// the same from the bits.
 __host__ __device__ __forceinline__ long long q_time(uint64_t x_bits, int F) {
+#ifdef __CUDA_ARCH__
+  return (x_bits >> 52) == 0 ? 0 : __double2ll_rn(__longlong_as_double((long long)(x_bits + ((uint64_t)F << 52))));
+#else
   if (x_bits == 0) return 0;
   const int ex = (int)((x_bits >> 52) & 0x7ff);
   const uint64_t m = (x_bits & M52) | (ex ? (1ull << 52) : 0);
@@ -291,6 +300,7 @@ __host__ __device__ __forceinline__ long long q_time(uint64_t x_bits, int F) {
   const uint64_t rem = m & ((1ull << r) - 1), half = 1ull << (r - 1);
   if (rem > half || (rem == half && (q & 1))) ++q;
   return (long long)q;
+#endif
 }
 
 // exp(i 2 pi q / qbeta) in units of 2^-30 (.x cos, .y sin) for a tick count

@@ -123,7 +123,7 @@ size_t Engine::estimate_footprint(const std::vector<ChainSpec> &specs, int ring_
              14 * g.nsub + sizeof(DevChain) + 8 * (g.ntile + g.nsiteblk + g.nbondblk);
     vc += (vertex_estimate(c) + 127) / 128 * 128;
   }
-  bytes += (size_t)vc * (8 + 2 + 12 + 8 * ACC_WORDS + 8) + 4 * (size_t)(vc / 32 + 1) * 4;
+  bytes += (size_t)vc * (8 + 2 + 12 + 8 * ACC_WORDS + 8) + 5 * (size_t)(vc / 32 + 1) * 4;
   return bytes;
 }
 
@@ -177,6 +177,7 @@ void Engine::free_vertex() {
   dfree(s_.openmark);
   dfree(s_.openroot);
   dfree(s_.flipbits);
+  dfree(s_.newbits);
   dfree(s_.xmark);
   s_.vtau = nullptr;
   s_.vflag = nullptr;
@@ -184,7 +185,7 @@ void Engine::free_vertex() {
   s_.pl = s_.pr = s_.parent = nullptr;
   s_.acc = nullptr;
   s_.accz = nullptr;
-  s_.openmark = s_.openroot = s_.flipbits = s_.xmark = nullptr;
+  s_.openmark = s_.openroot = s_.flipbits = s_.newbits = s_.xmark = nullptr;
   vertex_bytes_ = 0;
 }
 
@@ -203,12 +204,13 @@ int Engine::alloc_vertex(int64_t vcap) {
   DALLOC(s_.openmark, uint32_t, nw);
   DALLOC(s_.openroot, uint32_t, nw);
   DALLOC(s_.flipbits, uint32_t, nw);
+  DALLOC(s_.newbits, uint32_t, nw);
   DALLOC(s_.xmark, uint32_t, nw);
   CK(cudaMemsetAsync(s_.acc, 0, ACC_WORDS * sizeof(unsigned long long) * vcap, st_));
   CK(cudaMemsetAsync(s_.accz, 0, sizeof(unsigned long long) * vcap, st_));
   s_.vcap = vcap;
   vcap_ = vcap;
-  vertex_bytes_ = (size_t)vcap * (8 + 2 + 12 + 8 * ACC_WORDS + 8) + 4 * (size_t)nw * 4;
+  vertex_bytes_ = (size_t)vcap * (8 + 2 + 12 + 8 * ACC_WORDS + 8) + 5 * (size_t)nw * 4;
   L_.s = s_;
   drop_graphs();
   return LCQMC_OK;

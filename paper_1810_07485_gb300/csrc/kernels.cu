@@ -139,21 +139,23 @@ __device__ void block_sums(long long &c, u128 &x, u128 &y, u128 &z) {
 __device__ __forceinline__ bool halted(const Scratch &s) { return __ldcg(s.status) != 0; }
 
 // Tile blocks of the vertex-parallel kernels: TPB threads walk the tile's
-// vertices in id order (coalesced); a vertex's cell comes from a binary search
-// in the tile's cell offsets staged in shared memory.
+// vertices in id order (coalesced).
 constexpr int TPB = 256;
 
-__device__ __forceinline__ int tile_cell_of(const int *cvp, int ncl, int w) {
-  // largest i in [0, ncl) with cvp[i] <= w
-  int lo = 0, hi = ncl - 1;
-  while (lo < hi) {
-    const int mid = lo + ((hi - lo + 1) >> 1);
-    if (cvp[mid] <= w)
-      lo = mid;
-    else
-      hi = mid - 1;
-  }
-  return lo;
+// A value that every lane holds, in a form the compiler knows to be uniform
+// (loops bounded by it need no divergence handling).
+__device__ __forceinline__ int uniform(int x) { return (int)__reduce_max_sync(0xffffffffu, x); }
+
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __reduce_max_sync(0xffffffffu, x); }
+
+// Vertex bitmaps are written a word (32 vertices) at a time by the warp that
+// handles them; a tile's first and last words are shared with its neighbours
+// and take an atomic (the bitmap starts the update at zero).
+__device__ __forceinline__ void store_word(uint32_t *bits, int64_t word, uint32_t x, int v0, int a, int e) {
+  if (v0 >= a && v0 + 32 <= e)
+    bits[word] = x;
+  else if (x)
+    atomicOr(bits + word, x);
 }
 
 // ---- bond parity at time-block starts ---------------------------------------
@@ -180,8 +182,8 @@ __global__ void k_bond_parity(const DevChain *__restrict__ ch, const int2 *__res
 }
 
 // ---- per-update scratch reset -------------------------------------------------
-// The insertion's look-back words and tile tickets and the four per-vertex
-// bitmaps (open marks, open roots, coin flips, crossing marks) start each
+// The insertion's look-back words and tile tickets and the five per-vertex
+// bitmaps (open marks, open roots, flips, new operators, crossing marks) start each
 // update at zero: one grid-stride launch instead of one memset each (a small
 // chain's update is a chain of short launches).
 __global__ void k_clear(Scratch s, int64_t ntile, int64_t nw) {
@@ -191,6 +193,7 @@ __global__ void k_clear(Scratch s, int64_t ntile, int64_t nw) {
     s.openmark[i] = 0u;
     s.openroot[i] = 0u;
     s.flipbits[i] = 0u;
+    s.newbits[i] = 0u;
     s.xmark[i] = 0u;
   }
   for (int64_t i = i0; i < ntile; i += step) s.tile_state[i] = 0ull;
@@ -359,12 +362,6 @@ __device__ __forceinline__ double key_unit(unsigned long long key) {
   }
   return __longlong_as_double((long long)bits);
 }
-
-// A value that every lane holds, in a form the compiler knows to be uniform
-// (loops bounded by it need no divergence handling).
-__device__ __forceinline__ int uniform(int x) { return (int)__reduce_max_sync(0xffffffffu, x); }
-
-__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __reduce_max_sync(0xffffffffu, x); }
 
 // A warp's cells: lanes l and l + 16 hold cell l.
 struct InsCell {
@@ -1346,78 +1343,116 @@ __global__ void __launch_bounds__(TPB_X) k_link_xt(const DevChain *__restrict__ 
 }
 
 // ---- compression + coins --------------------------------------------------------
-__global__ void __launch_bounds__(TILE) k_compress(const DevChain *__restrict__ ch,
+// Every node's root, and the flip of its loop (one coin per root) as one bit
+// per node: the later kernels read flips by node, without the root.
+//
+// Only this block writes parent words of [a, e) in this kernel, and every word
+// it writes is an ancestor of the old one: the tile's copy stays a valid forest.
+// Words that point out of the tile (parents are never larger than their
+// children, so outside means below a) are resolved first, each with one global
+// walk to its root and that root's coin, so that the nodes walking through
+// them share both; every other walk then stays in shared memory.  In the
+// tile's copy a word is the parent's index in the tile, or, with the top bit
+// set, the root outside.  The shared copy and the global words agree after
+// that pass, and a node's word is stored only if its root differs from it
+// (linking left most words at their root: 0.31 -> 0.28 ms at L=16384,
+// beta=4096).
+constexpr unsigned OUTSIDE = 0x80000000u;
+constexpr int COIN_GROUPS = SMEM_CAP / 128 + 2;  // Philox blocks of 128 coins a tile in shared memory spans
+
+__global__ void __launch_bounds__(TILE, 16) k_compress(const DevChain *__restrict__ ch,
                                                    const int2 *__restrict__ tab, int64_t blk0,
                                                    Scratch s) {
-  __shared__ U4 coins[MAX_COIN_GROUPS];
+  __shared__ U4 coins[COIN_GROUPS];
   __shared__ int64_t sm[33];
-  __shared__ int spar[SMEM_CAP];  // the tile's parent words: walks stay here until they leave it
+  __shared__ unsigned spar[SMEM_CAP];
+  __shared__ uint32_t ocoin[SMEM_CAP / 32 + 2];  // coins of the outside roots, at the nodes that point there
+  __shared__ unsigned short olist[SMEM_CAP];     // those nodes
+  __shared__ int nout;
   if (halted(s)) return;
   const int64_t gt = blk0 + blockIdx.x;
   const int2 t = tab[gt];
   const DevChain &C = ch[t.x];
   const int c0 = t.y * TILE, c1 = min(C.ncell, c0 + TILE);
   const int32_t *vp = s.vptr + C.cell_off;
-  const int a = vp[c0], e = vp[c1];
+  const int a = uniform(vp[c0]), e = uniform(vp[c1]);
   const int64_t vb = C.vtx_base, wb = vb >> 5;
   int32_t *par = s.parent + vb;
   const bool oversized = (e - a) > local_cap(C);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int step = blockDim.x, first = (a & ~31) + 32 * wid;  // words of 32 vertices, a warp each
   const int g0 = a >> 7;
-  const int ng = (e > a) ? ((e - 1) >> 7) - g0 + 1 : 0;
-  const uint32_t k0 = (uint32_t)C.seed, k1 = (uint32_t)(C.seed >> 32);
-  for (int g = threadIdx.x; g < ng && g < MAX_COIN_GROUPS; g += blockDim.x)
-    coins[g] = philox(TAG_FLIP << 24, (uint32_t)(g0 + g), 0u, C.sweep, k0, k1);
-  // Only this block writes parent words of [a, e) in this kernel, and every
-  // word it writes is an ancestor of the old one: the copy stays a valid forest.
-  // Words that point out of the tile (parents are never larger than their
-  // children, so outside means below a) are resolved first, each with one
-  // global walk to its root, so that the nodes walking through them share
-  // that walk; every other walk then stays in shared memory.  The shared copy
-  // and the global words agree after that pass, and a node's word is stored
-  // only if its root differs from it (linking left most words at their root:
-  // 0.31 -> 0.28 ms at L=16384, beta=4096).
+  const int ng = (e > a && !oversized) ? ((e - 1) >> 7) - g0 + 1 : 0;
+  const uint32_t k0 = uniform((uint32_t)C.seed), k1 = uniform((uint32_t)(C.seed >> 32)), sweep = uniform(C.sweep);
+  for (int g = threadIdx.x; g < ng; g += blockDim.x)
+    coins[g] = philox(TAG_FLIP << 24, (uint32_t)(g0 + g), 0u, sweep, k0, k1);
+  if (threadIdx.x == 0) nout = 0;
+  for (int i = threadIdx.x; i < SMEM_CAP / 32 + 2; i += blockDim.x) ocoin[i] = 0u;
+  __syncthreads();
   if (!oversized) {
-    for (int i = threadIdx.x; i < e - a; i += blockDim.x) {
-      const int p = __ldcg(par + a + i);
-      int q = p;
-      if (p < a) {
-        q = uf_root(par, p, s.status, s.uf_limit);
-        if (q != p) par[a + i] = q;
+    for (int v0 = first; v0 < e; v0 += step) {
+      const int v = v0 + lane;
+      const bool in = v >= a && v < e;
+      const int p = in ? __ldcg(par + v) : a;
+      const unsigned m = __ballot_sync(0xffffffffu, p < a);
+      if (m) {  // about 5 % of the nodes: listed, so that whole warps take them below
+        int at = 0;
+        if (lane == 0) at = atomicAdd(&nout, __popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (p < a) olist[at + __popc(m & ((1u << lane) - 1u))] = (unsigned short)(v - a);
       }
-      spar[i] = q;
+      if (in) spar[v - a] = p < a ? (OUTSIDE | (unsigned)p) : (unsigned)(p - a);
     }
   }
   __syncthreads();
+  for (int k = threadIdx.x; k < nout; k += blockDim.x) {
+    const int i = olist[k], v = a + i, p = (int)(spar[i] & ~OUTSIDE);
+    const int q = uf_root(par, p, s.status, s.uf_limit);
+    if (q != p) {
+      par[v] = q;
+      spar[i] = OUTSIDE | (unsigned)q;
+    }
+    if (coin_from(philox(TAG_FLIP << 24, (uint32_t)q >> 7, 0u, sweep, k0, k1), (uint32_t)q))
+      atomicOr(&ocoin[(v >> 5) - (a >> 5)], 1u << (v & 31));
+  }
+  __syncthreads();
+  const uint32_t *cw = (const uint32_t *)coins;
   int64_t roots = 0;
-  for (int v0 = a; v0 < e; v0 += blockDim.x) {  // whole warps, reconverged per step
-    const int v = v0 + threadIdx.x;
-    if (v >= e) {
-      __syncwarp();
-      continue;
-    }
-    int r;
-    if (oversized) {
-      r = uf_root(par, v, s.status, s.uf_limit);
-    } else {
-      // the walk ends at a root of the tile, or at a resolved outside root
-      r = v;
-      int p = spar[v - a];
-      for (int it = 0; p != r && p >= a && it < SMEM_CAP; ++it) {
-        r = p;
-        p = spar[p - a];
+  for (int v0 = first; v0 < e; v0 += step) {
+    const int v = v0 + lane;
+    const bool in = v >= a && v < e;
+    int r = -1, flip = 0;
+    if (in && !oversized) {
+      // the walk ends at a root of the tile, or at a word that points outside
+      const unsigned x0 = spar[v - a];
+      unsigned k = (unsigned)(v - a), x = x0;
+      for (int it = 0; x != k && !(x & OUTSIDE) && it < SMEM_CAP; ++it) {
+        k = x;
+        x = spar[k];
       }
-      if (p != r) r = (p < a) ? p : uf_root(par, p, s.status, s.uf_limit);
+      if (x & OUTSIDE) {
+        r = (int)(x & ~OUTSIDE);
+        const int y = a + (int)k;
+        flip = (ocoin[(y >> 5) - (a >> 5)] >> (y & 31)) & 1;
+        if (x0 != x) par[v] = r;
+      } else {
+        r = a + (int)k;
+        flip = (int)((cw[(r >> 5) - (g0 << 2)] >> (r & 31)) & 1u);
+        if (x0 != k) par[v] = r;
+      }
+    } else if (in) {
+      r = uf_root(par, v, s.status, s.uf_limit);
+      if (r != v) par[v] = r;
+      flip = coin_from(philox(TAG_FLIP << 24, (uint32_t)r >> 7, 0u, sweep, k0, k1), (uint32_t)r);
     }
-    if (r != (oversized ? v : spar[v - a])) par[v] = r;  // only words that change
-    if (r == v) {
-      ++roots;
-      const int g = (v >> 7) - g0;
-      const int cf = (g < MAX_COIN_GROUPS) ? coin_from(coins[g], (uint32_t)v) : coin(C, TAG_FLIP, v);
-      if (cf) set_bit(s.flipbits, wb, v);
-      if (oversized) set_bit(s.openroot, wb, v);
+    const unsigned fm = __ballot_sync(0xffffffffu, flip), rm = __ballot_sync(0xffffffffu, in && r == v);
+    if (lane == 0) {
+      roots += __popc(rm);
+      store_word(s.flipbits, wb + (v0 >> 5), fm, v0, a, e);
+      if (oversized && rm) atomicOr(s.openroot + wb + (v0 >> 5), rm);
     }
-    if (get_bit(s.openmark, wb, v)) set_bit(s.openroot, wb, r);
-    __syncwarp();
+    const uint32_t om = __ldcg(s.openmark + wb + (v0 >> 5));
+    if (in && ((om >> lane) & 1u)) set_bit(s.openroot, wb, r);
   }
   const int64_t tot = block_sum<int64_t>(roots, sm);
   if (threadIdx.x == 0) s.tile_roots[gt] = tot;
@@ -1502,12 +1537,47 @@ __device__ __forceinline__ void loop_add(int *keys, unsigned *vals, int key, con
   set_bit(s.openroot, vb >> 5, key);
 }
 
+// A 128-bit sum in four 32-bit words, and the square of |v| < 2^62 added to it:
+// ten multiply-adds with carry (the compiler's 64 x 64 -> 128-bit product and
+// 128-bit add took about twice that).
+struct Sum128 {
+  uint32_t a = 0, b = 0, c = 0, d = 0;
+  __device__ __forceinline__ void add_square(long long v) {
+    const unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
+    const uint32_t lo = (uint32_t)m, hi = (uint32_t)(m >> 32), hi2 = hi << 1;
+    asm("mad.lo.cc.u32 %0, %4, %4, %0;\n\t"
+        "madc.hi.cc.u32 %1, %4, %4, %1;\n\t"
+        "madc.lo.cc.u32 %2, %5, %5, %2;\n\t"
+        "madc.hi.u32 %3, %5, %5, %3;\n\t"
+        "mad.lo.cc.u32 %1, %4, %6, %1;\n\t"
+        "madc.hi.cc.u32 %2, %4, %6, %2;\n\t"
+        "addc.u32 %3, %3, 0;"
+        : "+r"(a), "+r"(b), "+r"(c), "+r"(d)
+        : "r"(lo), "r"(hi), "r"(hi2));
+  }
+  __device__ __forceinline__ u128 value() const {
+    return ((u128)(((unsigned long long)d << 32) | c) << 64) | (((unsigned long long)b << 32) | a);
+  }
+};
+
 // Squares of one loop's sums: W^2 to w2, C^2 + S^2 to f2, (T) Zr^2 + Zi^2 to z2.
 template <bool T>
-__device__ __forceinline__ void loop_squares(const long long *v, u128 &w2, u128 &f2, u128 &z2) {
-  w2 += sq_abs(v[0]);
-  f2 += sq_abs(v[1]) + sq_abs(v[2]);
-  if (T) z2 += sq_abs(v[3]) + sq_abs(v[4]);
+__device__ __forceinline__ void loop_squares(const long long *v, Sum128 &w2, Sum128 &f2, Sum128 &z2) {
+  w2.add_square(v[0]);
+  f2.add_square(v[1]);
+  f2.add_square(v[2]);
+  if (T) {
+    z2.add_square(v[3]);
+    z2.add_square(v[4]);
+  }
+}
+
+// mul_q32 for v >= 0 and |c| <= 2^32 (its two 32-bit words, low first): with
+// c = 2^32 M + l, floor((v c + 2^31) / 2^32) = M v + vh l + floor((vl l + 2^31) / 2^32).
+__device__ __forceinline__ long long mul_len(long long v, int l, int M) {
+  const uint32_t vl = (uint32_t)v, vh = (uint32_t)((unsigned long long)v >> 32), ul = (uint32_t)l;
+  const unsigned long long t = (unsigned long long)vl * ul + 0x80000000ull;
+  return (long long)((t >> 32) + (unsigned long long)vh * ul + (unsigned long long)((long long)M * v));
 }
 
 constexpr int TPB_EST = 256;
@@ -1516,6 +1586,14 @@ constexpr int TPB_EST = 256;
 constexpr int EST_STAGE = 1536;
 
 // T: also the temporal moment (phase factors, Zr and Zi); off by default.
+//
+// Bound by instruction issue (74 % of the slots, 21 of 32 lanes active: the
+// loop table's adds and the squares each take the lanes of their kind).  Flips
+// come one bit per node (no root is followed for a flip), new operators leave
+// as one bitmap word per warp and step, ticks take one conversion, lengths and
+// squares 32-bit multiply-adds: 0.86 -> 0.72 ms at L=16384, beta=4096 (790 ->
+// 650 M warp instructions); of the instructions the table takes 22 %, the
+// staging 15 %, the squares 10 %, the Fourier products 7 %.
 template <int Q, bool T>
 __global__ void __launch_bounds__(TPB_EST, T ? 6 : 8) k_est(const DevChain *__restrict__ ch,
                                              const int2 *__restrict__ tab, int64_t blk0,
@@ -1523,9 +1601,8 @@ __global__ void __launch_bounds__(TPB_EST, T ? 6 : 8) k_est(const DevChain *__re
   __shared__ int lkeys[LOOP_SLOTS];
   constexpr int NS = T ? LOOP_SUMS : 3;  // sums carried per loop
   __shared__ unsigned lvals[2 * NS * LOOP_SLOTS];
-  __shared__ int cvp[TILE + 1];
-  __shared__ int cnew[TILE];
-  __shared__ long long ccl[TILE], csl[TILE], ccr[TILE], csr[TILE], cxl[TILE], cxr[TILE];
+  __shared__ int4 csl[TILE], csr[TILE];  // 2^32 cos, 2^32 sin (low, high words) of a cell's two sites
+  __shared__ char2 cx[TILE];             // cuts crossed by a leg that wraps, left and right
   extern __shared__ long long est_dyn[];
   long long *qv = est_dyn;                   // ticks q(tau) of the tile's vertices
   int2 *ev = (int2 *)(est_dyn + EST_STAGE);  // their phase factors exp(i w1 tau)
@@ -1535,7 +1612,7 @@ __global__ void __launch_bounds__(TPB_EST, T ? 6 : 8) k_est(const DevChain *__re
   const DevChain &C = ch[t.x];
   const int c0 = t.y * TILE, c1 = min(C.ncell, c0 + TILE), ncl = c1 - c0;
   const int32_t *vp = s.vptr + C.cell_off;
-  const int a = vp[c0], e = vp[c1];
+  const int a = uniform(vp[c0]), e = uniform(vp[c1]);
   const int64_t vb = C.vtx_base, wb = vb >> 5;
   const int32_t *par = s.parent + vb;
   const uint64_t *vt = (const uint64_t *)s.vtau + vb;
@@ -1558,20 +1635,16 @@ __global__ void __launch_bounds__(TPB_EST, T ? 6 : 8) k_est(const DevChain *__re
     qv[i] = q;
     if (T) ev[i] = phase_of((uint64_t)q, phR, phS, g_phase_tab);
   }
-  for (int i = threadIdx.x; i <= ncl; i += blockDim.x) cvp[i] = vp[c0 + i];
   if (threadIdx.x < ncl) {
-    // per cell: Fourier weights of its two sites, cut crossings (in ticks)
+    // per cell: Fourier weights of its two sites, cut crossings
     int b, j;
     cell_bj(C, c0 + threadIdx.x, b, j);
     const int ul = left_sub<Q>(b), ur = right_sub<Q>(b, C.L);
     const int xl = ul / Q, xr = ur / Q;
-    ccl[threadIdx.x] = C.cosq[xl];
-    csl[threadIdx.x] = C.sinq[xl];
-    ccr[threadIdx.x] = C.cosq[xr];
-    csr[threadIdx.x] = C.sinq[xr];
-    cxl[threadIdx.x] = (long long)s.cut_cross[C.sub_off + ul] * C.qbeta;
-    cxr[threadIdx.x] = (long long)s.cut_cross[C.sub_off + ur] * C.qbeta;
-    cnew[threadIdx.x] = 0;
+    const long long cl = C.cosq[xl], sl = C.sinq[xl], cr = C.cosq[xr], sr = C.sinq[xr];
+    csl[threadIdx.x] = make_int4((int)cl, (int)(cl >> 32), (int)sl, (int)(sl >> 32));
+    csr[threadIdx.x] = make_int4((int)cr, (int)(cr >> 32), (int)sr, (int)(sr >> 32));
+    cx[threadIdx.x] = make_char2(s.cut_cross[C.sub_off + ul], s.cut_cross[C.sub_off + ur]);
   }
   for (int i = threadIdx.x; i < LOOP_SLOTS; i += blockDim.x) {
     lkeys[i] = -1;
@@ -1579,37 +1652,42 @@ __global__ void __launch_bounds__(TPB_EST, T ? 6 : 8) k_est(const DevChain *__re
     for (int k = 0; k < 2 * NS; ++k) lvals[2 * NS * i + k] = 0u;
   }
   __syncthreads();
-  auto inq = [&](int v) { return v >= a && v < a + nq; };
-  auto ticks = [&](int v) { return inq(v) ? qv[v - a] : q_time(vt[v], F); };
+  auto ticks = [&](int v) { return (unsigned)(v - a) < (unsigned)nq ? qv[v - a] : q_time(vt[v], F); };
   auto phase = [&](int v) {
-    return inq(v) ? ev[v - a] : phase_of((uint64_t)q_time(vt[v], F), phR, phS, g_phase_tab);
+    return (unsigned)(v - a) < (unsigned)nq ? ev[v - a]
+                                            : phase_of((uint64_t)q_time(vt[v], F), phR, phS, g_phase_tab);
   };
-  // Whole warps walk the tile (trip count rounded up), reconverging after
-  // every vertex.
-  u128 w2 = 0, f2 = 0, z2 = 0;  // this thread's share of the loops' squared sums
-  for (int w0 = a; w0 < e; w0 += blockDim.x) {
-    const int w = w0 + threadIdx.x;
-    if (w < e) {
+  const uint32_t *flips = s.flipbits + wb;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  // A warp takes a word of 32 vertices at a time and reconverges after it.
+  // The flips and parents were written by an earlier kernel: they are read
+  // through L1.
+  Sum128 w2, f2, z2;  // this thread's share of the loops' squared sums
+  long long newcnt = 0;
+  for (int v0 = (a & ~31) + 32 * wid; v0 < e; v0 += TPB_EST) {
+    const int w = v0 + lane;
+    int nf = 0;
+    if (w >= a && w < e) {
       const int ci = s.vcell[vb + w];
       const int P = s.pl[vb + w], R = s.pr[vb + w];
       const uint8_t f = s.vflag[vb + w];
-      // a node whose two upper legs both end at w is a loop by itself: its
-      // own root
-      const int rb = (P == R) ? P : __ldcg(par + P), ra = __ldcg(par + w);
-      const int nf = (f & VF_OLD) ^ get_bit(s.flipbits, wb, rb) ^ get_bit(s.flipbits, wb, ra);
-      s.vflag[vb + w] = (uint8_t)(f | (nf ? VF_NEW : 0));
-      if (nf) atomicAdd(cnew + ci, 1);
+      // an operator changes if the loops below and above it do not flip alike
+      nf = (f ^ (flips[P >> 5] >> (P & 31)) ^ (flips[v0 >> 5] >> lane)) & VF_OLD;
       // fragment lengths in ticks of 2^-F: q(tau_top) - q(tau_bottom) (+ crossings)
       const long long qw = ticks(w);
       const long long qP = ticks(P);
       long long dl = qw - qP;
-      if (f & VF_WRAP_L) dl += cxl[ci];
       long long dr = qw - (R == P ? qP : ticks(R));
-      if (f & VF_WRAP_R) dr += cxr[ci];
+      if (f & (VF_WRAP_L | VF_WRAP_R)) {
+        const char2 x = cx[ci];
+        if (f & VF_WRAP_L) dl += (long long)x.x * C.qbeta;
+        if (f & VF_WRAP_R) dr += (long long)x.y * C.qbeta;
+      }
       LoopSums x;
       x.v[0] = dl + dr;
-      x.v[1] = mul_q32(dl, ccl[ci]) + mul_q32(dr, ccr[ci]);
-      x.v[2] = mul_q32(dl, csl[ci]) + mul_q32(dr, csr[ci]);
+      const int4 kl = csl[ci], kr = csr[ci];
+      x.v[1] = mul_len(dl, kl.x, kl.y) + mul_len(dr, kr.x, kr.y);
+      x.v[2] = mul_len(dl, kl.z, kl.w) + mul_len(dr, kr.z, kr.w);
       // int over a fragment of e^{i w1 t} dt = (e(top) - e(bottom)) / (i w1),
       // across the cut too (e(t + beta) = e(t)): both fragments end at w
       x.v[3] = x.v[4] = 0;
@@ -1623,17 +1701,16 @@ __global__ void __launch_bounds__(TPB_EST, T ? 6 : 8) k_est(const DevChain *__re
         // two fragments are the two below w: the loop's sums are complete here.
         loop_squares<T>(x.v, w2, f2, z2);
       } else {
-        loop_add<NS>(lkeys, lvals, rb, x, s, vb, slot_mask);
+        loop_add<NS>(lkeys, lvals, par[P], x, s, vb, slot_mask);
       }
     }
-    __syncwarp();
+    const unsigned nm = __ballot_sync(0xffffffffu, nf);
+    if (lane == 0) {
+      newcnt += __popc(nm);
+      store_word(s.newbits, wb + (v0 >> 5), nm, v0, a, e);
+    }
   }
   __syncthreads();
-  long long newcnt = 0;
-  if (threadIdx.x < ncl) {
-    newcnt = cnew[threadIdx.x];
-    C.op_ptr[C.cur ^ 1][c0 + threadIdx.x] = (int32_t)newcnt;
-  }
   // A loop closed in the tile is complete in its slot: square it here.  A loop
   // that leaves the tile adds its slot to the root's global record, squared
   // once every tile has added (next operator list kernel).
@@ -1649,88 +1726,74 @@ __global__ void __launch_bounds__(TPB_EST, T ? 6 : 8) k_est(const DevChain *__re
       loop_squares<T>(v, w2, f2, z2);
     }
   }
-  block_sums<T>(newcnt, w2, f2, z2);
+  u128 tw = w2.value(), tf = f2.value(), tz = T ? z2.value() : (u128)0;
+  block_sums<T>(newcnt, tw, tf, tz);
   if (threadIdx.x == 0) {
     s.tile_sum2[gt] = newcnt;
-    s.tile_sw2[2 * gt] = (unsigned long long)w2;
-    s.tile_sw2[2 * gt + 1] = (unsigned long long)(w2 >> 64);
-    s.tile_sf2[2 * gt] = (unsigned long long)f2;
-    s.tile_sf2[2 * gt + 1] = (unsigned long long)(f2 >> 64);
-    s.tile_sz2[2 * gt] = (unsigned long long)z2;
-    s.tile_sz2[2 * gt + 1] = (unsigned long long)(z2 >> 64);
+    s.tile_sw2[2 * gt] = (unsigned long long)tw;
+    s.tile_sw2[2 * gt + 1] = (unsigned long long)(tw >> 64);
+    s.tile_sf2[2 * gt] = (unsigned long long)tf;
+    s.tile_sf2[2 * gt + 1] = (unsigned long long)(tf >> 64);
+    s.tile_sz2[2 * gt] = (unsigned long long)tz;
+    s.tile_sz2[2 * gt + 1] = (unsigned long long)(tz >> 64);
   }
 }
 
 // ---- next operator list + open loops -------------------------------------------------
-// The tile's flags are read as aligned 32-bit words (four vertices each).
-// Each warp takes a contiguous range of words: a first pass counts its new
-// operators, one barrier exchanges the warp totals, and a second pass places
-// them with warp shuffles (id order = order of the next operator list).  The
-// cell offsets come from a block scan of the per-cell counts.
+// The tile's new operators are a bitmap of its vertices: a scan of the words'
+// counts gives every word's first place, a warp then moves the marked times of
+// a word at a time (id order = order of the next operator list), and a cell's
+// first operator is the count before its first vertex.
 template <bool T>
 __global__ void __launch_bounds__(TPB, T ? 4 : 8) k_compact(const DevChain *__restrict__ ch,
                                                  const int2 *__restrict__ tab, int64_t blk0,
                                                  Scratch s) {
-  __shared__ int64_t sm[33];
-  __shared__ int wtot[TPB / 32];
+  __shared__ int sm[33];
+  __shared__ uint32_t nbits[TPB];
+  __shared__ int npre[TPB];
   if (halted(s)) return;
   const int64_t gt = blk0 + blockIdx.x;
   const int2 t = tab[gt];
   const DevChain &C = ch[t.x];
   const int c0 = t.y * TILE, c1 = min(C.ncell, c0 + TILE), ncl = c1 - c0;
   int32_t *nptr = C.op_ptr[C.cur ^ 1];
-  double *ntau = C.op_tau[C.cur ^ 1];
   const int32_t *vp = s.vptr + C.cell_off;
   const int64_t vb = C.vtx_base;
   const int64_t base = s.tile_pref2[gt];
-  const int a = vp[c0], e = vp[c1];
-  const uint8_t *vf = s.vflag + vb;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = TPB / 32;
-  // words [wa, we) of four flags; warp wid takes [wa + wid*per, ...)
-  const int wa = a >> 2, we = (e + 3) >> 2;
-  const int per = (we - wa + nw - 1) / nw;
-  const int ww0 = min(we, wa + wid * per), ww1 = min(we, ww0 + per);
-  auto newmask = [&](int wd) {  // bit i: vertex 4*wd + i is a new operator of this tile
-    const uint32_t fl = *(const uint32_t *)(vf + 4 * wd);  // vb and 4*wd are multiples of 4
-    int m = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int w = 4 * wd + i;
-      if (w >= a && w < e && ((fl >> (8 * i)) & VF_NEW)) m |= 1 << i;
+  const int a = uniform(vp[c0]), e = uniform(vp[c1]);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int cv = (threadIdx.x < ncl) ? vp[c0 + threadIdx.x] : e;  // first vertex of the thread's cell
+  const int64_t wfirst = (vb + a) >> 5, wlast = (vb + e - 1) >> 5;
+  const int nw = e > a ? (int)(wlast - wfirst) + 1 : 0;
+  double *ntau = C.op_tau[C.cur ^ 1] + base;
+  int run = 0, at = -1;  // new operators before the chunk; before the thread's cell
+  for (int k0 = 0; k0 < nw; k0 += TPB) {  // one chunk but for tiles of more than 8000 vertices
+    const int nk = min(nw - k0, TPB);
+    uint32_t bits = 0u;
+    if (threadIdx.x < nk) {
+      const int64_t wd = wfirst + k0 + threadIdx.x, v0 = (wd << 5) - vb;
+      bits = s.newbits[wd];
+      if (v0 < a) bits &= ~0u << (a - v0);
+      if (v0 + 32 > e) bits &= (e - v0 >= 32) ? ~0u : ((1u << (e - v0)) - 1u);
     }
-    return m;
-  };
-  int cnt = 0;
-  for (int wd = ww0 + lane; wd < ww1; wd += 32) cnt += __popc(newmask(wd));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-  if (lane == 0) wtot[wid] = cnt;
-  {
-    const int cc = (threadIdx.x < ncl) ? nptr[c0 + threadIdx.x] : 0;
-    int64_t tot;
-    const int64_t ex = block_excl_scan<int64_t>((int64_t)cc, sm, tot);  // also publishes wtot
-    if (threadIdx.x < ncl) {
-      nptr[c0 + threadIdx.x] = (int32_t)(base + ex);
-      if (c0 + (int)threadIdx.x == C.ncell - 1) nptr[C.ncell] = (int32_t)C.n_off_new;
+    int tot;
+    const int ex = run + block_excl_scan<int>(__popc(bits), sm, tot);
+    nbits[threadIdx.x] = bits;
+    npre[threadIdx.x] = ex;
+    __syncthreads();
+    for (int k = wid; k < nk; k += TPB / 32) {
+      const uint32_t x = nbits[k];
+      if ((x >> lane) & 1u)
+        ntau[npre[k] + __popc(x & ((1u << lane) - 1u))] = s.vtau[((wfirst + k0 + k) << 5) + lane];
     }
+    const int64_t k = ((vb + cv) >> 5) - wfirst - k0;
+    if (cv < e && k >= 0 && k < nk) at = npre[k] + __popc(nbits[k] & ((1u << (cv & 31)) - 1u));
+    run += tot;
+    __syncthreads();
   }
-  int64_t pos = base;
-  for (int k = 0; k < wid; ++k) pos += wtot[k];
-  for (int s0 = ww0; s0 < ww1; s0 += 32) {
-    const int wd = s0 + lane;
-    const int m = (wd < ww1) ? newmask(wd) : 0;
-    const int c = __popc(m);
-    int inc = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += y;
-    }
-    int64_t p = pos + inc - c;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (m & (1 << i)) ntau[p++] = s.vtau[vb + 4 * wd + i];
-    pos += __shfl_sync(0xffffffffu, inc, 31);
+  if (threadIdx.x < ncl) {
+    nptr[c0 + threadIdx.x] = (int32_t)(base + (at < 0 ? run : at));
+    if (c0 + (int)threadIdx.x == C.ncell - 1) nptr[C.ncell] = (int32_t)C.n_off_new;
   }
   // Loops that left their tile: one 32-byte accumulator record per root (and
   // its Zi word), read and cleared; a thread takes one 32-vertex word of the
@@ -1739,7 +1802,6 @@ __global__ void __launch_bounds__(TPB, T ? 4 : 8) k_compact(const DevChain *__re
   // without them, the plain loop needs fewer registers and more resident
   // warps hide the latency better.
   u128 w2 = 0, f2 = 0, z2 = 0;
-  const int64_t wfirst = (vb + a) >> 5, wlast = (vb + e - 1) >> 5;
   for (int64_t wd = wfirst + threadIdx.x; e > a && wd <= wlast; wd += blockDim.x) {
     uint32_t bits = __ldcg(s.openroot + wd);
     const int64_t v0 = (wd << 5) - vb;
@@ -1825,7 +1887,7 @@ __global__ void __launch_bounds__(SITE_BLOCK) k_sites(const DevChain *__restrict
       const int node = s.cut_node[C.sub_off + u];
       int f;
       if (node >= 0) {
-        f = get_bit(s.flipbits, wb, __ldcg(s.parent + vb + node));
+        f = get_bit(s.flipbits, wb, node);
       } else {
         const int mn = s.free_min[C.sub_off + u];
         f = coin(C, TAG_FREE, (uint32_t)mn);

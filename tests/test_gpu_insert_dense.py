@@ -1,6 +1,7 @@
-"""Insertion on crowded cells: more operators than a tile stages in shared
+"""Crowded cells: more operators than an insertion tile stages in shared
 memory, more vertices than a warp's position marks hold, one cell with most of
-them, against the oracle (vertices, links, roots, new state, records)."""
+them, a tile of more vertices than one pass of the operator rewrite takes
+(8192), against the oracle (vertices, links, roots, new state, records)."""
 import numpy as np
 import pytest
 
@@ -36,6 +37,7 @@ def crowded(L, beta, Q, per_cell, only_bond, seed):
     (64, 40.0, 1, 20, None),
     (40, 64.0, 1, 400, 20),     # one bond holds every operator
     (2, 16.0, 1, 1000, None),
+    (2, 16.0, 1, 9000, None),
     (12, 20.0, 2, 120, None),
     (6, 16.0, 3, 100, None),
     (4, 20.0, 4, 300, None),
