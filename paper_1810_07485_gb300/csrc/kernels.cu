@@ -139,8 +139,14 @@ __device__ void block_sums(long long &c, u128 &x, u128 &y, u128 &z) {
 __device__ __forceinline__ bool halted(const Scratch &s) { return __ldcg(s.status) != 0; }
 
 // Tile blocks of the vertex-parallel kernels: TPB threads walk the tile's
-// vertices in id order (coalesced).
-constexpr int TPB = 256;
+// vertices in id order (coalesced).  A launch of few tiles leaves most of the
+// SMs' warp slots empty and its time is the longest tile's chain of steps:
+// there linking, compression and loop properties take TPB_WIDE threads per tile
+// while two such blocks per SM hold every tile.  One update, us, 256 / 1024
+// threads: S = 1/2, 2 tiles 94 / 74, 152 tiles 117 / 93, 301 tiles 129 / 110,
+// 598 tiles 146 / 149; S = 2, 68 tiles 207 / 166, 294 tiles 254 / 209.
+constexpr int TPB = 256, TPB_WIDE = 1024;
+constexpr int64_t WIDE_TILES = 152 * 2;
 
 // A value that every lane holds, in a form the compiler knows to be uniform
 // (loops bounded by it need no divergence handling).
@@ -1076,8 +1082,8 @@ __device__ __forceinline__ int time_lower_bound(const long long *vt, int lo, int
 // that leave the tile are marked and united in the global forest by k_link_x,
 // after every tile has stored its forest (a tile too large for shared memory
 // leaves all of its edges to k_link_x, with every node its own root).
-template <int Q>
-__global__ void __launch_bounds__(TPB) k_link(const DevChain *__restrict__ ch,
+template <int Q, int NT>
+__global__ void __launch_bounds__(NT) k_link(const DevChain *__restrict__ ch,
                                               const int2 *__restrict__ tab, int64_t blk0,
                                               Scratch s) {
   __shared__ LinkCell<Q> lc[TILE];
@@ -1360,7 +1366,8 @@ __global__ void __launch_bounds__(TPB_X) k_link_xt(const DevChain *__restrict__ 
 constexpr unsigned OUTSIDE = 0x80000000u;
 constexpr int COIN_GROUPS = SMEM_CAP / 128 + 2;  // Philox blocks of 128 coins a tile in shared memory spans
 
-__global__ void __launch_bounds__(TILE, 16) k_compress(const DevChain *__restrict__ ch,
+template <int NT>
+__global__ void __launch_bounds__(NT, 2048 / NT) k_compress(const DevChain *__restrict__ ch,
                                                    const int2 *__restrict__ tab, int64_t blk0,
                                                    Scratch s) {
   __shared__ U4 coins[COIN_GROUPS];
@@ -1580,7 +1587,6 @@ __device__ __forceinline__ long long mul_len(long long v, int l, int M) {
   return (long long)((t >> 32) + (unsigned long long)vh * ul + (unsigned long long)((long long)M * v));
 }
 
-constexpr int TPB_EST = 256;
 // Vertices of a tile whose ticks (and phase factors) the loop-properties
 // kernel stages in shared memory; ticks beyond it are computed where needed.
 constexpr int EST_STAGE = 1536;
@@ -1594,8 +1600,8 @@ constexpr int EST_STAGE = 1536;
 // squares 32-bit multiply-adds: 0.86 -> 0.72 ms at L=16384, beta=4096 (790 ->
 // 650 M warp instructions); of the instructions the table takes 22 %, the
 // staging 15 %, the squares 10 %, the Fourier products 7 %.
-template <int Q, bool T>
-__global__ void __launch_bounds__(TPB_EST, T ? 6 : 8) k_est(const DevChain *__restrict__ ch,
+template <int Q, bool T, int NT>
+__global__ void __launch_bounds__(NT, (T ? 1536 : 2048) / NT) k_est(const DevChain *__restrict__ ch,
                                              const int2 *__restrict__ tab, int64_t blk0,
                                              Scratch s) {
   __shared__ int lkeys[LOOP_SLOTS];
@@ -1664,7 +1670,7 @@ __global__ void __launch_bounds__(TPB_EST, T ? 6 : 8) k_est(const DevChain *__re
   // through L1.
   Sum128 w2, f2, z2;  // this thread's share of the loops' squared sums
   long long newcnt = 0;
-  for (int v0 = (a & ~31) + 32 * wid; v0 < e; v0 += TPB_EST) {
+  for (int v0 = (a & ~31) + 32 * wid; v0 < e; v0 += NT) {
     const int w = v0 + lane;
     int nf = 0;
     if (w >= a && w < e) {
@@ -2044,9 +2050,14 @@ void launch_cut(const Launch &L, cudaStream_t st) {
 }
 
 void launch_link(const Launch &L, cudaStream_t st) {
-#define LINK_Q(Q)     \
-  if (L.ntile[Q - 1]) \
-    k_link<Q><<<g1(L.ntile[Q - 1]), L.link_threads, 0, st>>>(L.ch, L.tile_tab, L.tile0[Q - 1], L.s);
+  const bool wide = all_tiles(L) <= WIDE_TILES;
+#define LINK_Q(Q)                                                                                              \
+  if (L.ntile[Q - 1]) {                                                                                        \
+    if (wide)                                                                                                  \
+      k_link<Q, TPB_WIDE><<<g1(L.ntile[Q - 1]), TPB_WIDE, 0, st>>>(L.ch, L.tile_tab, L.tile0[Q - 1], L.s);      \
+    else                                                                                                       \
+      k_link<Q, TPB><<<g1(L.ntile[Q - 1]), L.link_threads, 0, st>>>(L.ch, L.tile_tab, L.tile0[Q - 1], L.s);     \
+  }
   FOR_EACH_Q(LINK_Q)
 #undef LINK_Q
   // Tile-crossing edges: a block per tile for few tiles, else a warp per tile.
@@ -2066,7 +2077,11 @@ void launch_link(const Launch &L, cudaStream_t st) {
 
 void launch_compress(const Launch &L, cudaStream_t st) {
   const int64_t n = all_tiles(L);
-  if (n) k_compress<<<g1(n), L.compress_threads, 0, st>>>(L.ch, L.tile_tab, 0, L.s);
+  if (!n) return;
+  if (n <= WIDE_TILES)
+    k_compress<TPB_WIDE><<<g1(n), TPB_WIDE, 0, st>>>(L.ch, L.tile_tab, 0, L.s);
+  else
+    k_compress<TILE><<<g1(n), L.compress_threads, 0, st>>>(L.ch, L.tile_tab, 0, L.s);
 }
 
 void launch_check_forest(const Launch &L, cudaStream_t st) {
@@ -2094,9 +2109,12 @@ int init_kernel_attributes() {
                        (int)std::llrint(std::ldexp(std::sin(ang), 30)));
   }
   if (cudaMemcpyToSymbol(g_phase_tab, tab, sizeof(tab)) != cudaSuccess) return -1;
-#define EST_ATTR_Q(Q)                                                                 \
-  if (cudaFuncSetAttribute(k_est<Q, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                           (int)EST_DYN_SMEM) != cudaSuccess)                           \
+#define EST_ATTR_Q(Q)                                                                      \
+  if (cudaFuncSetAttribute(k_est<Q, true, TPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                           (int)EST_DYN_SMEM) != cudaSuccess ||                              \
+      cudaFuncSetAttribute(k_est<Q, true, TPB_WIDE>,                                         \
+                           cudaFuncAttributeMaxDynamicSharedMemorySize,                      \
+                           (int)EST_DYN_SMEM) != cudaSuccess)                                \
     return -1;
   FOR_EACH_Q(EST_ATTR_Q)
 #undef EST_ATTR_Q
@@ -2113,15 +2131,23 @@ int init_kernel_attributes() {
 void launch_est(const Launch &L, cudaStream_t st) {
   // without the temporal moment only the ticks are staged
   const size_t dyn = L.temporal ? EST_DYN_SMEM : EST_STAGE * sizeof(long long);
-#define EST_Q(Q)                                                                                       \
-  if (L.ntile[Q - 1]) {                                                                                \
-    if (L.temporal)                                                                                    \
-      k_est<Q, true><<<g1(L.ntile[Q - 1]), TPB_EST, dyn, st>>>(L.ch, L.tile_tab, L.tile0[Q - 1], L.s);  \
-    else                                                                                               \
-      k_est<Q, false><<<g1(L.ntile[Q - 1]), TPB_EST, dyn, st>>>(L.ch, L.tile_tab, L.tile0[Q - 1], L.s); \
+  const bool wide = all_tiles(L) <= WIDE_TILES;
+#define EST_QTN(Q, T, NT) \
+  k_est<Q, T, NT><<<g1(L.ntile[Q - 1]), NT, dyn, st>>>(L.ch, L.tile_tab, L.tile0[Q - 1], L.s)
+#define EST_Q(Q)                   \
+  if (L.ntile[Q - 1]) {            \
+    if (L.temporal && wide)        \
+      EST_QTN(Q, true, TPB_WIDE);  \
+    else if (L.temporal)           \
+      EST_QTN(Q, true, TPB);       \
+    else if (wide)                 \
+      EST_QTN(Q, false, TPB_WIDE); \
+    else                           \
+      EST_QTN(Q, false, TPB);      \
   }
   FOR_EACH_Q(EST_Q)
 #undef EST_Q
+#undef EST_QTN
 }
 
 void launch_compact(const Launch &L, cudaStream_t st) {
