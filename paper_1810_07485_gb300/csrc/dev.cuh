@@ -12,6 +12,7 @@ namespace lcq {
 constexpr int KMAX = 48;          // Poisson count table length (K <= KMAX-1)
 constexpr int QMAX = 4;           // largest 2S: subspins per site (S <= 2)
 constexpr int TW = LCQMC_TW;      // windows per time block of the cell order
+constexpr int SCAN_PARTS = 152;   // parts of the operator scan over all chains, at most
 constexpr int64_t VTX_ID_LIMIT = 0x7ffff000;  // largest vertex count of one chain
 constexpr int NOBS = 9;         // running averages per chain (lcqmc_obs.sum)
 constexpr int ACC_WORDS = 4;    // 64-bit words of an open loop's record (32 bytes)
@@ -82,12 +83,12 @@ struct DevChain {
 
 struct Scratch {
   int32_t *vptr;
-  int64_t *tile_sum, *tile_pref, *tile_sum2, *tile_pref2, *tile_roots;
+  int64_t *tile_sum2, *tile_pref2, *tile_roots;
   unsigned long long *tile_sw2, *tile_sf2, *tile_sz2;  // 2 words (lo, hi) per tile
   int64_t *site_free;
   unsigned long long *site_sw2, *site_sf2;   // 2 words per site block
   uint8_t *bpar;
-  int32_t *cut_node, *cut_cell, *free_min;
+  int32_t *cut_node, *free_min;
   int8_t *cut_cross, *free_len;
   double *vtau;
   uint8_t *vflag;
@@ -104,9 +105,10 @@ struct Scratch {
   int64_t vcap;
   unsigned long long *tile_state;  // per tile: insertion look-back word (flag << 62 | count)
   unsigned int *tickets;           // per Q group: next tile of the insertion launch
+  unsigned long long *part_state;  // per part of the operator scan: look-back word (SCAN_PARTS)
+  unsigned int *part_done;         // per chain: parts of the record done; 0 between updates
   int *status;
   int uf_limit;   // bound of the global union-find walks and retries (UF_MAX_ITERS)
-  int64_t *need;  // [0] vertex capacity needed by the last update
   long long *dbg; // first failed consistency check: code, then 7 details
 };
 

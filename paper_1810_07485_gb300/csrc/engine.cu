@@ -243,8 +243,6 @@ Engine::~Engine() {
   dfree(site_tab_);
   dfree(bond_tab_);
   dfree(s_.vptr);
-  dfree(s_.tile_sum);
-  dfree(s_.tile_pref);
   dfree(s_.tile_sum2);
   dfree(s_.tile_pref2);
   dfree(s_.tile_roots);
@@ -256,14 +254,14 @@ Engine::~Engine() {
   dfree(s_.site_sf2);
   dfree(s_.bpar);
   dfree(s_.cut_node);
-  dfree(s_.cut_cell);
   dfree(s_.free_min);
   dfree(s_.cut_cross);
   dfree(s_.free_len);
   dfree(s_.status);
   dfree(s_.tickets);
   dfree(s_.tile_state);
-  dfree(s_.need);
+  dfree(s_.part_state);
+  dfree(s_.part_done);
   dfree(s_.dbg);
   if (st_) cudaStreamSynchronize(st_);  // stream-ordered frees done
   if (pool_) cudaMemPoolDestroy(pool_);
@@ -317,7 +315,7 @@ int Engine::open(void *stream, const lcqmc_allocator *alloc, int ring_cap, bool 
     if (v >= 1 && v <= UF_MAX_ITERS) s_.uf_limit = (int)v;
   }
   DALLOC(s_.tickets, unsigned int, QMAX);
-  DALLOC(s_.need, int64_t, 4);
+  DALLOC(s_.part_state, unsigned long long, SCAN_PARTS);
   DALLOC(s_.dbg, long long, 8);
   CK(cudaMemsetAsync(s_.status, 0, sizeof(int), st_));
   CK(cudaMemsetAsync(s_.dbg, 0, 8 * sizeof(long long), st_));
@@ -504,16 +502,16 @@ int Engine::layout() {
   int rc = 0;
 #define GROW(ptr, cap, need, T)                                                     \
   if ((rc = grow_array((void **)&(ptr), &(cap), (need), sizeof(T))) != 0) return rc
+  int64_t cap_done = cap_chains_;
+  GROW(s_.part_done, cap_done, std::max(nc, 1), unsigned int);
   GROW(dch_, cap_chains_, std::max(nc, 1), DevChain);
   GROW(tile_tab_, cap_tt_, nt, int2);
   GROW(site_tab_, cap_st_, ns, int2);
   GROW(bond_tab_, cap_bt_, nb, int2);
   GROW(s_.vptr, cap_cells_, std::max<int64_t>(1, cell_off), int32_t);
-  int64_t c1 = cap_tiles_, c2 = cap_tiles_, c3 = cap_tiles_, c4 = cap_tiles_, c5 = cap_tiles_,
+  int64_t c3 = cap_tiles_, c4 = cap_tiles_, c5 = cap_tiles_,
           c6 = cap_tiles_, c7 = cap_tiles_, c9 = cap_tiles_;
   if (nt > cap_tiles_) {
-    GROW(s_.tile_sum, c1, nt, int64_t);
-    GROW(s_.tile_pref, c2, nt, int64_t);
     GROW(s_.tile_sum2, c3, nt, int64_t);
     GROW(s_.tile_pref2, c4, nt, int64_t);
     GROW(s_.tile_roots, c5, nt, int64_t);
@@ -533,10 +531,9 @@ int Engine::layout() {
   }
   GROW(s_.bpar, cap_bpar_, std::max<int64_t>(1, bpar_off), uint8_t);
   if (sub_off > cap_subs_ || !s_.cut_node) {
-    int64_t a1 = cap_subs_, a2 = cap_subs_, a3 = cap_subs_, a4 = cap_subs_, a5 = cap_subs_;
+    int64_t a1 = cap_subs_, a3 = cap_subs_, a4 = cap_subs_, a5 = cap_subs_;
     const int64_t need = std::max<int64_t>(1, sub_off);
     GROW(s_.cut_node, a1, need, int32_t);
-    GROW(s_.cut_cell, a2, need, int32_t);
     GROW(s_.free_min, a3, need, int32_t);
     GROW(s_.cut_cross, a4, need, int8_t);
     GROW(s_.free_len, a5, need, int8_t);
@@ -544,15 +541,18 @@ int Engine::layout() {
   }
 #undef GROW
   if (nc > 0) {
+    CK(cudaMemsetAsync(s_.part_done, 0, sizeof(unsigned int) * nc, st_));
     CK(cudaMemcpyAsync(dch_, hch.data(), sizeof(DevChain) * nc, cudaMemcpyHostToDevice, st_));
     CK(cudaMemcpyAsync(tile_tab_, ttab.data(), sizeof(int2) * ttab.size(), cudaMemcpyHostToDevice, st_));
     CK(cudaMemcpyAsync(site_tab_, stab.data(), sizeof(int2) * stab.size(), cudaMemcpyHostToDevice, st_));
     CK(cudaMemcpyAsync(bond_tab_, btab.data(), sizeof(int2) * btab.size(), cudaMemcpyHostToDevice, st_));
   }
-  fixed_bytes_ = 4 * (size_t)cap_cells_ + 112 * (size_t)cap_tiles_ + 48 * (size_t)cap_sites_ +
+  fixed_bytes_ = 4 * (size_t)cap_cells_ + 96 * (size_t)cap_tiles_ + 48 * (size_t)cap_sites_ +
                  (size_t)cap_bpar_ + 14 * (size_t)cap_subs_ + sizeof(DevChain) * (size_t)cap_chains_;
   L_.ch = dch_;
   L_.nchains = nc;
+  L_.max_ntile = 0;
+  for (int c = 0; c < nc; ++c) L_.max_ntile = std::max<int64_t>(L_.max_ntile, hch[c].ntile);
   L_.tile_tab = tile_tab_;
   L_.site_tab = site_tab_;
   L_.bond_tab = bond_tab_;

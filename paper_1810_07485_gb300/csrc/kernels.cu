@@ -203,6 +203,7 @@ __global__ void k_clear(Scratch s, int64_t ntile, int64_t nw) {
     s.xmark[i] = 0u;
   }
   for (int64_t i = i0; i < ntile; i += step) s.tile_state[i] = 0ull;
+  for (int64_t i = i0; i < SCAN_PARTS; i += step) s.part_state[i] = 0ull;
   if (i0 < QMAX) s.tickets[i0] = 0u;
 }
 
@@ -826,16 +827,22 @@ __device__ __forceinline__ void insert_tile(InsSmem<Q> &S, DevChain *__restrict_
 }
 
 // ---- per-chain scan of the tiles' new-operator counts ------------------------------
+// A chain's tiles in gridDim.y parts: a part sums its counts, gets the count
+// before it by look-back over the parts (all parts of all chains are resident
+// at once: see launch_scan_ops), then scans its counts.  One part per chain
+// took 0.35 ms of 46 at 2^19 tiles, and 25 us of 3 ms at 2^15.
 __global__ void __launch_bounds__(1024) k_scan_ops(DevChain *__restrict__ ch, Scratch s) {
   // Chunks of 4 x 1024 tiles: each thread loads four consecutive counts
   // (coalesced across the warp), one block scan per chunk; the next chunk's
   // loads are issued before the current chunk's scan.
   __shared__ int64_t sm[33];
+  __shared__ int64_t before;
   if (halted(s)) return;
   DevChain &C = ch[blockIdx.x];
-  const int nt = C.ntile;
-  const int64_t *cnt = s.tile_sum2 + C.tile0;
-  int64_t *pref = s.tile_pref2 + C.tile0;
+  const int per = (C.ntile + gridDim.y - 1) / gridDim.y;
+  const int i0 = min(C.ntile, (int)blockIdx.y * per), nt = min(C.ntile, i0 + per) - i0;
+  const int64_t *cnt = s.tile_sum2 + C.tile0 + i0;
+  int64_t *pref = s.tile_pref2 + C.tile0 + i0;
   constexpr int V = 4;
   const int chunk = V * (int)blockDim.x;
   int64_t v[V], nx[V];
@@ -846,8 +853,28 @@ __global__ void __launch_bounds__(1024) k_scan_ops(DevChain *__restrict__ ch, Sc
       x[k] = (i < nt) ? cnt[i] : 0;
     }
   };
-  load(0, v);
   int64_t run = 0;
+  if (gridDim.y > 1) {
+    int64_t mine = 0;
+    for (int i = threadIdx.x; i < nt; i += blockDim.x) mine += cnt[i];
+    const int64_t sum = block_sum<int64_t>(mine, sm);
+    if (threadIdx.x < 32) {
+      const int64_t p0 = (int64_t)blockIdx.x * gridDim.y, p = p0 + blockIdx.y;
+      int64_t excl = 0;
+      if (blockIdx.y) {
+        if (threadIdx.x == 0) lb_publish(s.part_state, p, LB_AGG, sum);
+        __syncwarp();
+        excl = lb_lookback(s.part_state, p, p0, s);
+      }
+      if (threadIdx.x == 0) {
+        lb_publish(s.part_state, p, LB_INC, excl + sum);
+        before = excl;
+      }
+    }
+    __syncthreads();
+    run = before;
+  }
+  load(0, v);
   for (int base = 0; base < nt; base += chunk) {
     if (base + chunk < nt) load(base + chunk, nx);
     int64_t mine = 0;
@@ -865,67 +892,77 @@ __global__ void __launch_bounds__(1024) k_scan_ops(DevChain *__restrict__ ch, Sc
 #pragma unroll
     for (int k = 0; k < V; ++k) v[k] = nx[k];
   }
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && blockIdx.y == gridDim.y - 1) {
     C.n_off_new = run;
     if (run > C.op_cap) atomicOr(s.status, ST_OP_OVERFLOW);
   }
 }
 
 // ---- tau = 0: last leg per subsite, subspin permutation, cut predecessors -----
+// One thread per subsite: the last vertex on its 2 Q bonds.  The bonds' last
+// windows are read side by side (a thread per site that walked them one after
+// another took 22 us at S = 2, one dependent load after the other); only a bond
+// whose last window is empty is walked further down.
 template <int Q>
-__device__ void last_leg(const DevChain &C, const int32_t *vp, const long long *vtau, int64_t vb,
-                         int bond, int &id, int &cellc, long long &tau) {
-  id = -1;
-  cellc = -1;
-  tau = 0;
-  for (int j = C.nwin - 1; j >= 0; --j) {
-    const int c = cell_of(C, bond, j);
-    const int a = vp[c], e = vp[c + 1];
-    if (e > a) {
-      id = e - 1;
-      cellc = c;
-      tau = vtau[vb + id];
-      return;
-    }
-  }
-}
-
-template <int Q>
-__global__ void __launch_bounds__(SITE_BLOCK) k_cut(const DevChain *__restrict__ ch,
+__global__ void __launch_bounds__(SITE_BLOCK * Q) k_cut(const DevChain *__restrict__ ch,
                                                     const int2 *__restrict__ tab, int64_t blk0,
                                                     Scratch s) {
+  __shared__ int slast[SITE_BLOCK * Q];
+  __shared__ uint8_t stop_[SITE_BLOCK * Q];
   if (halted(s)) return;
   const int2 t = tab[blk0 + blockIdx.x];
   const DevChain &C = ch[t.x];
-  const int i = t.y * SITE_BLOCK + threadIdx.x;
-  if (i >= C.L) return;
+  const int u = t.y * SITE_BLOCK * Q + threadIdx.x, i = u / Q;  // subsite, site
   const int32_t *vp = s.vptr + C.cell_off;
-  const int64_t vb = C.vtx_base;
+  const long long *vt = (const long long *)s.vtau + C.vtx_base;
   const uint8_t *s0 = C.s0[C.cur];
   const uint8_t *ptot = s.bpar + C.bpar_off + (int64_t)C.nblk * C.nbond;
-  int last[Q], lastc[Q], top[Q];
-#pragma unroll
-  for (int a = 0; a < Q; ++a) {
-    const int u = i * Q + a;
-    int best = -1, bestc = -1;
+  if (i < C.L) {
+    int best = -1, par = 0;
     long long bt = 0;
-    int par = 0;
+    int id[2 * Q];
 #pragma unroll
     for (int m = 0; m < 2 * Q; ++m) {
       const int bb = inc_bond<Q>(u, m, C.L);
       par ^= ptot[bb];
-      int id, cc;
-      long long tt;
-      last_leg<Q>(C, vp, (const long long *)s.vtau, vb, bb, id, cc, tt);
-      if (id >= 0 && (best < 0 || tt > bt || (tt == bt && id > best))) {
-        best = id;
-        bt = tt;
-        bestc = cc;
+      const int c = cell_of(C, bb, C.nwin - 1);
+      const int a = vp[c], e = vp[c + 1];
+      id[m] = e > a ? e - 1 : -1;
+    }
+#pragma unroll
+    for (int m = 0; m < 2 * Q; ++m) {
+      if (id[m] >= 0) continue;
+      const int bb = inc_bond<Q>(u, m, C.L);
+      for (int j = C.nwin - 2; j >= 0; --j) {
+        const int c = cell_of(C, bb, j);
+        const int a = vp[c], e = vp[c + 1];
+        if (e > a) {
+          id[m] = e - 1;
+          break;
+        }
       }
     }
-    last[a] = best;
-    lastc[a] = bestc;
-    top[a] = (s0[u] ^ par) & 1;
+    long long tt[2 * Q];
+#pragma unroll
+    for (int m = 0; m < 2 * Q; ++m) tt[m] = id[m] >= 0 ? vt[id[m]] : 0;
+#pragma unroll
+    for (int m = 0; m < 2 * Q; ++m)
+      if (id[m] >= 0 && (best < 0 || tt[m] > bt || (tt[m] == bt && id[m] > best))) {
+        best = id[m];
+        bt = tt[m];
+      }
+    slast[threadIdx.x] = best;
+    stop_[threadIdx.x] = (uint8_t)((s0[u] ^ par) & 1);
+  }
+  __syncthreads();
+  if (i >= C.L) return;
+  // Every subsite's thread takes its site's permutation (the same on all of them).
+  int last[Q], top[Q];
+  const int k0 = (int)threadIdx.x / Q * Q;  // the site's first thread
+#pragma unroll
+  for (int a = 0; a < Q; ++a) {
+    last[a] = slast[k0 + a];
+    top[a] = stop_[k0 + a];
   }
   // perm[a]: the bottom subspin that the top of subspin a continues into.
   int perm[Q];
@@ -983,34 +1020,34 @@ __global__ void __launch_bounds__(SITE_BLOCK) k_cut(const DevChain *__restrict__
     perm[0] = sw ? 1 : 0;
     perm[1] = sw ? 0 : 1;
   }
+  // Walk down through the cut: the bottom of subspin a is entered from the
+  // top of pinv(a), then possibly through empty subspins.
+  const int a = u - i * Q;
+  int x = a, cross = 0, node = -1, mn = a, len = 0;
+  for (int step = 0; step < Q; ++step) {
+    int y = 0;
 #pragma unroll
-  for (int a = 0; a < Q; ++a) {
-    // Walk down through the cut: the bottom of subspin a is entered from the
-    // top of pinv(a), then possibly through empty subspins.
-    int x = a, cross = 0, node = -1, ncell = -1, mn = a, len = 0;
-    for (int step = 0; step < Q; ++step) {
-      int y = 0;
+    for (int z = 0; z < Q; ++z)
+      if (perm[z] == x) y = z;
+    x = y;
+    ++cross;
+    int lx = 0;
 #pragma unroll
-      for (int z = 0; z < Q; ++z)
-        if (perm[z] == x) y = z;
-      x = y;
-      ++cross;
-      if (last[x] >= 0) {
-        node = last[x];
-        ncell = lastc[x];
-        break;
-      }
-      mn = min(mn, x);
-      ++len;
-      if (x == a) break;
+    for (int z = 0; z < Q; ++z)
+      if (z == x) lx = last[z];
+    if (lx >= 0) {
+      node = lx;
+      break;
     }
-    const int64_t u = C.sub_off + i * Q + a;
-    s.cut_node[u] = node;
-    s.cut_cell[u] = ncell;
-    s.cut_cross[u] = (int8_t)cross;
-    s.free_min[u] = (node < 0) ? i * Q + mn : -1;
-    s.free_len[u] = (int8_t)len;
+    mn = min(mn, x);
+    ++len;
+    if (x == a) break;
   }
+  const int64_t v = C.sub_off + u;
+  s.cut_node[v] = node;
+  s.cut_cross[v] = (int8_t)cross;
+  s.free_min[v] = (node < 0) ? i * Q + mn : -1;
+  s.free_len[v] = (int8_t)len;
 }
 
 // ---- linking + union-find -----------------------------------------------------
@@ -1921,79 +1958,177 @@ __global__ void __launch_bounds__(SITE_BLOCK) k_sites(const DevChain *__restrict
 }
 
 // ---- per-chain record -----------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_final(DevChain *__restrict__ ch, Scratch s) {
-  __shared__ int64_t sm[33];
+// A chain's tiles and site blocks in gridDim.y parts; each part leaves its sums
+// at its first tile, and the part that finishes last adds them up and writes
+// the record.  A chain of few tiles is one part, and its time is the chain of
+// fp64 operations behind the sums (they are slow on GB300): the record's values
+// and running sums are taken side by side, one per lane (13 -> 4 us; one thread
+// took them one after another).  One part per chain took 0.34 ms at 2^19 tiles.
+struct ChainSums {
+  long long roots, nfree;
+  u128 w2, f2, z2;
+};
+
+__device__ __forceinline__ void add_sums(ChainSums &x, const ChainSums &y) {
+  x.roots += y.roots;
+  x.nfree += y.nfree;
+  x.w2 += y.w2;
+  x.f2 += y.f2;
+  x.z2 += y.z2;
+}
+
+__device__ __forceinline__ u128 pair128(const unsigned long long *t, int64_t g) {
+  return ((u128)__ldcg(t + 2 * g + 1) << 64) | __ldcg(t + 2 * g);
+}
+
+__device__ __forceinline__ void warp_sums(ChainSums &x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    ChainSums y;
+    y.roots = __shfl_down_sync(0xffffffffu, x.roots, o);
+    y.nfree = __shfl_down_sync(0xffffffffu, x.nfree, o);
+    y.w2 = shfl_down_u128(x.w2, o);
+    y.f2 = shfl_down_u128(x.f2, o);
+    y.z2 = shfl_down_u128(x.z2, o);
+    add_sums(x, y);
+  }
+}
+
+constexpr int FINAL_THREADS = 256;
+
+__global__ void __launch_bounds__(FINAL_THREADS) k_final(DevChain *__restrict__ ch, Scratch s) {
+  __shared__ ChainSums part[FINAL_THREADS / 32];
+  __shared__ int last;
   if (halted(s)) return;
   DevChain &C = ch[blockIdx.x];
-  int64_t roots = 0, nfree = 0;
-  u128 w2 = 0, f2 = 0, z2 = 0;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, np = gridDim.y;
+  const int per = (C.ntile + np - 1) / np, i0 = min(C.ntile, (int)blockIdx.y * per), i1 = min(C.ntile, i0 + per);
+  const int pers = (C.nsiteblk + np - 1) / np, j0 = min(C.nsiteblk, (int)blockIdx.y * pers),
+            j1 = min(C.nsiteblk, j0 + pers);
+  // the running sums, for the block that comes to need them
+  double run = 0.0, run2 = 0.0;
+  if (threadIdx.x < NOBS) {
+    run = C.sum[threadIdx.x];
+    run2 = C.sumsq[threadIdx.x];
+  }
+  ChainSums x{0, 0, 0, 0, 0};  // vertex-free loops are whole periods: no temporal term
 #pragma unroll 4
-  for (int i = threadIdx.x; i < C.ntile; i += blockDim.x) {
+  for (int i = i0 + threadIdx.x; i < i1; i += FINAL_THREADS) {
     const int64_t g = C.tile0 + i;
-    roots += s.tile_roots[g];
-    w2 += ((u128)s.tile_sw2[2 * g + 1] << 64) | s.tile_sw2[2 * g];
-    f2 += ((u128)s.tile_sf2[2 * g + 1] << 64) | s.tile_sf2[2 * g];
-    z2 += ((u128)s.tile_sz2[2 * g + 1] << 64) | s.tile_sz2[2 * g];
+    add_sums(x, ChainSums{s.tile_roots[g], 0, pair128(s.tile_sw2, g), pair128(s.tile_sf2, g), pair128(s.tile_sz2, g)});
   }
-  for (int i = threadIdx.x; i < C.nsiteblk; i += blockDim.x) {
-    const int64_t g = C.site0 + i;
-    nfree += s.site_free[g];
-    w2 += ((u128)s.site_sw2[2 * g + 1] << 64) | s.site_sw2[2 * g];
-    f2 += ((u128)s.site_sf2[2 * g + 1] << 64) | s.site_sf2[2 * g];
+  for (int j = j0 + threadIdx.x; j < j1; j += FINAL_THREADS) {
+    const int64_t g = C.site0 + j;
+    add_sums(x, ChainSums{0, s.site_free[g], pair128(s.site_sw2, g), pair128(s.site_sf2, g), 0});
   }
-  roots = block_sum<int64_t>(roots, sm);
-  nfree = block_sum<int64_t>(nfree, sm);
-  w2 = block_sum_u128(w2);
-  f2 = block_sum_u128(f2);
-  z2 = block_sum_u128(z2);  // vertex-free loops are whole periods: no temporal term
-  if (threadIdx.x != 0) return;
-  lcqmc_record r;
-  r.n = C.n;
-  r.n_off_old = C.op_ptr[C.cur][C.ncell];
-  r.n_off_new = C.n_off_new;
-  r.n_free = nfree;
-  r.n_clusters = roots + nfree;
-  r.n_seg = 2 * C.n + nfree;
-  r.F = C.F;
-  r.pad = 0;
-  r.sw2_lo = (unsigned long long)w2;
-  r.sw2_hi = (unsigned long long)(w2 >> 64);
-  r.sf2_lo = (unsigned long long)f2;
-  r.sf2_hi = (unsigned long long)(f2 >> 64);
-  r.sz2_lo = (unsigned long long)z2;
-  r.sz2_hi = (unsigned long long)(z2 >> 64);
-  const double two64 = 18446744073709551616.0;
-  const double dsw = __dadd_rn(__dmul_rn((double)r.sw2_hi, two64), (double)r.sw2_lo);
-  const double dsf = __dadd_rn(__dmul_rn((double)r.sf2_hi, two64), (double)r.sf2_lo);
-  const double bl = __dmul_rn(__dmul_rn(4.0, C.beta), (double)C.L);
-  r.energy = __dsub_rn(__dmul_rn(__dmul_rn((double)(C.Q * C.Q), C.J), 0.25),
-                       __ddiv_rn((double)C.n, __dmul_rn(C.beta, (double)C.L)));
-  r.chi_s = __ddiv_rn(ldexp(dsw, -2 * C.F), bl);
-  r.chi_q = __ddiv_rn(ldexp(dsf, -2 * C.F), bl);
-  // |int e^{i w1 t} dt|^2 = |Z|^2 2^-60 / w1^2 with w1 = 2 pi / beta:
-  // chi_w = sz2 2^-60 beta / (16 pi^2 L)
-  const double kPi = 3.14159265358979323846;
-  const double dsz = __dadd_rn(__dmul_rn((double)r.sz2_hi, two64), (double)r.sz2_lo);
-  r.chi_w = __ddiv_rn(__dmul_rn(ldexp(dsz, -60), C.beta),
-                      __dmul_rn(__dmul_rn(__dmul_rn(16.0, kPi), kPi), (double)C.L));
-  C.ring[C.n_rec % C.ring_cap] = r;
-  C.n_rec += 1;
-  const double v[NOBS] = {r.energy,
-                          r.chi_s,
-                          r.chi_q,
-                          (double)r.n,
-                          (double)r.n_off_new,
-                          (double)r.n_seg,
-                          (double)r.n_clusters,
-                          (double)(r.n_seg + 2 * r.n),
-                          r.chi_w};
-  for (int k = 0; k < NOBS; ++k) {
-    C.sum[k] += v[k];
-    C.sumsq[k] += v[k] * v[k];
+  warp_sums(x);
+  if (lane == 0) part[wid] = x;
+  __syncthreads();
+  if (wid) return;
+  x = lane < FINAL_THREADS / 32 ? part[lane] : ChainSums{0, 0, 0, 0, 0};
+  warp_sums(x);
+  if (np > 1) {  // this part's sums to its first tile's place (read by this block only)
+    if (lane == 0) {
+      if (i0 < i1) {
+        const int64_t g = C.tile0 + i0;
+        s.tile_roots[g] = x.roots;
+        s.tile_sum2[g] = x.nfree;
+        s.tile_sw2[2 * g] = (unsigned long long)x.w2;
+        s.tile_sw2[2 * g + 1] = (unsigned long long)(x.w2 >> 64);
+        s.tile_sf2[2 * g] = (unsigned long long)x.f2;
+        s.tile_sf2[2 * g + 1] = (unsigned long long)(x.f2 >> 64);
+        s.tile_sz2[2 * g] = (unsigned long long)x.z2;
+        s.tile_sz2[2 * g + 1] = (unsigned long long)(x.z2 >> 64);
+      }
+      __threadfence();
+      last = atomicAdd(s.part_done + blockIdx.x, 1u) == (unsigned)np - 1;
+      __threadfence();
+    }
+    __syncwarp();
+    if (!last) return;
+    x = ChainSums{0, 0, 0, 0, 0};
+    for (int p = lane; p < np; p += 32) {
+      if (p * per >= C.ntile) break;
+      const int64_t g = C.tile0 + (int64_t)p * per;
+      add_sums(x, ChainSums{__ldcg((const long long *)s.tile_roots + g), __ldcg((const long long *)s.tile_sum2 + g),
+                            pair128(s.tile_sw2, g), pair128(s.tile_sf2, g), pair128(s.tile_sz2, g)});
+    }
+    __syncwarp();
+    warp_sums(x);
   }
-  C.n_updates += 1;
-  C.cur ^= 1;
-  C.sweep += 1;
+  // lane 0 holds the chain's sums
+  const int64_t n = C.n, n_new = C.n_off_new, n_free = __shfl_sync(0xffffffffu, x.nfree, 0),
+                clusters = __shfl_sync(0xffffffffu, x.roots, 0) + n_free, n_seg = 2 * n + n_free;
+  lcqmc_record &r = C.ring[C.n_rec % C.ring_cap];
+  if (lane == 0) {
+    r.n = n;
+    r.n_off_old = C.op_ptr[C.cur][C.ncell];
+    r.n_off_new = n_new;
+    r.n_free = n_free;
+    r.n_clusters = clusters;
+    r.n_seg = n_seg;
+    r.F = C.F;
+    r.pad = 0;
+    r.sw2_lo = (unsigned long long)x.w2;
+    r.sw2_hi = (unsigned long long)(x.w2 >> 64);
+    r.sf2_lo = (unsigned long long)x.f2;
+    r.sf2_hi = (unsigned long long)(x.f2 >> 64);
+    r.sz2_lo = (unsigned long long)x.z2;
+    r.sz2_hi = (unsigned long long)(x.z2 >> 64);
+  }
+  // Lanes 0, 1, 2, 8: energy, chi_s, chi_q, chi_w as numerator / denominator;
+  // the other lanes below NOBS: whole numbers.
+  //   energy = Q^2 J / 4 - n / (beta L);  chi = sum 2^-2F / (4 beta L)
+  //   |int e^{i w1 t} dt|^2 = |Z|^2 2^-60 / w1^2 with w1 = 2 pi / beta:
+  //   chi_w = sz2 2^-60 beta / (16 pi^2 L)
+  unsigned long long lo, hi;
+  {
+    const unsigned long long wl = __shfl_sync(0xffffffffu, (unsigned long long)x.w2, 0),
+                             wh = __shfl_sync(0xffffffffu, (unsigned long long)(x.w2 >> 64), 0),
+                             fl = __shfl_sync(0xffffffffu, (unsigned long long)x.f2, 0),
+                             fh = __shfl_sync(0xffffffffu, (unsigned long long)(x.f2 >> 64), 0),
+                             zl = __shfl_sync(0xffffffffu, (unsigned long long)x.z2, 0),
+                             zh = __shfl_sync(0xffffffffu, (unsigned long long)(x.z2 >> 64), 0);
+    lo = lane == 1 ? wl : (lane == 2 ? fl : zl);
+    hi = lane == 1 ? wh : (lane == 2 ? fh : zh);
+  }
+  double v = 0.0;
+  if (lane < 3 || lane == 8) {
+    const double two64 = 18446744073709551616.0, kPi = 3.14159265358979323846;
+    const double L = (double)C.L;
+    // 2^-2F and 2^-60: exact factors
+    const double scale = __longlong_as_double((long long)(1023 - (lane == 8 ? 60 : 2 * C.F)) << 52);
+    double num = (double)n, den = __dmul_rn(C.beta, L);
+    if (lane) {
+      num = __dmul_rn(__dadd_rn(__dmul_rn((double)hi, two64), (double)lo), scale);
+      den = __dmul_rn(__dmul_rn(4.0, C.beta), L);
+    }
+    if (lane == 8) {
+      num = __dmul_rn(num, C.beta);
+      den = __dmul_rn(__dmul_rn(__dmul_rn(16.0, kPi), kPi), L);
+    }
+    v = __ddiv_rn(num, den);
+    if (lane == 0) v = __dsub_rn(__dmul_rn(__dmul_rn((double)(C.Q * C.Q), C.J), 0.25), v);
+  } else if (lane < NOBS) {
+    const int64_t k = lane == 3 ? n : lane == 4 ? n_new : lane == 5 ? n_seg : lane == 6 ? clusters : n_seg + 2 * n;
+    v = (double)k;
+  }
+  if (lane == 0) r.energy = v;
+  if (lane == 1) r.chi_s = v;
+  if (lane == 2) r.chi_q = v;
+  if (lane == 8) r.chi_w = v;
+  if (lane < NOBS) {
+    C.sum[lane] = __dadd_rn(run, v);
+    C.sumsq[lane] = __dadd_rn(run2, __dmul_rn(v, v));
+  }
+  __syncwarp();
+  if (lane == 0) {
+    if (np > 1) s.part_done[blockIdx.x] = 0;
+    C.n_rec += 1;
+    C.n_updates += 1;
+    C.cur ^= 1;
+    C.sweep += 1;
+  }
 }
 
 // ---- host-side launchers ----------------------------------------------------------------
@@ -2039,12 +2174,15 @@ void launch_insert(const Launch &L, cudaStream_t st) {
 }
 
 void launch_scan_ops(const Launch &L, cudaStream_t st) {
-  k_scan_ops<<<L.nchains, 1024, 0, st>>>(L.ch, L.s);
+  // Parts of at least 1024 tiles, and no more than one block per SM in all, so
+  // that every part is resident while others wait for it.
+  const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(L.max_ntile / 1024, SCAN_PARTS / L.nchains));
+  k_scan_ops<<<dim3(L.nchains, parts), 1024, 0, st>>>(L.ch, L.s);
 }
 
 void launch_cut(const Launch &L, cudaStream_t st) {
 #define CUT_Q(Q) \
-  if (L.nsiteblk[Q - 1]) k_cut<Q><<<g1(L.nsiteblk[Q - 1]), SITE_BLOCK, 0, st>>>(L.ch, L.site_tab, L.site0[Q - 1], L.s);
+  if (L.nsiteblk[Q - 1]) k_cut<Q><<<g1(L.nsiteblk[Q - 1]), SITE_BLOCK * Q, 0, st>>>(L.ch, L.site_tab, L.site0[Q - 1], L.s);
   FOR_EACH_Q(CUT_Q)
 #undef CUT_Q
 }
@@ -2168,7 +2306,8 @@ void launch_sites(const Launch &L, cudaStream_t st) {
 }
 
 void launch_final(const Launch &L, cudaStream_t st) {
-  k_final<<<L.nchains, 1024, 0, st>>>(L.ch, L.s);
+  const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(L.max_ntile / 2048, 64));
+  k_final<<<dim3(L.nchains, parts), FINAL_THREADS, 0, st>>>(L.ch, L.s);
 }
 
 }  // namespace lcq

@@ -10,6 +10,7 @@ namespace lcq {
 struct Launch {
   DevChain *ch;
   int nchains;
+  int64_t max_ntile;  // tiles of the largest chain
   Scratch s;
   const int2 *tile_tab, *site_tab, *bond_tab;
   int64_t ntile[QMAX], tile0[QMAX];

@@ -1,14 +1,17 @@
 """Launches that change form with the number of tiles (1024 or 256 threads per
 tile in linking, compression and loop properties; a block or a warp per tile in
-the unions of tile-crossing edges) against the oracle's roots and records, at
-the sizes where the form changes."""
+the unions of tile-crossing edges; one or several parts per chain in the
+operator scan and the record) against the oracle's roots and records, at the
+sizes where the form changes."""
+import numpy as np
 import pytest
 
 from test_gpu_parity import run_parity
 
 pytestmark = pytest.mark.gpu
 
-# tiles = L Q^2 ceil(beta / 16) / 128; the launches change above 304 and 3040
+# tiles = L Q^2 ceil(beta / 16) / 128; the launches change above 304, at 2048
+# (scan in parts), above 3040 and at 4096 (record in parts)
 CASES = [
     (1216, 16.0 * 32, 1),      # 304 tiles: the last with 1024 threads per tile
     (1218, 16.0 * 32, 1),      # 305 tiles
@@ -21,6 +24,7 @@ CASES = [
     (1522, 16.0 * 256, 1),     # 3044 tiles: the first warp-per-tile launch
     (760, 16.0 * 128, 2),      # 3040 tiles, S = 1
     (762, 16.0 * 128, 2),      # 3048 tiles
+    (2054, 16.0 * 256, 1),     # 4108 tiles: 4 scan parts, 2 record parts
     (80, 16.0 * 4, 3),         # S = 3/2: most edges cross
     (70, 16.0 * 4 + 3.0, 4),   # S = 2, ragged last window
 ]
@@ -29,3 +33,18 @@ CASES = [
 @pytest.mark.parametrize("L,beta,Q", CASES)
 def test_crossing_unions(L, beta, Q):
     run_parity(L, beta, Q=Q, seed=31 + L, nup=3)
+
+
+def test_parts_in_an_uneven_batch():
+    # a chain of several parts beside chains whose later parts are empty
+    from paper_1810_07485_gb300 import lcqmc
+    specs = [dict(L=2, beta=3.0, seed=1), dict(L=2054, beta=4096.0, seed=2), dict(L=34, beta=40.0, S=1.0, seed=3),
+             dict(L=1030, beta=4096.0, seed=4)]
+    b = lcqmc.Batch(specs)
+    b.update(3)
+    for i, sp in enumerate(specs):
+        ch = lcqmc.Chain(sp["L"], sp["beta"], S=sp.get("S", 0.5), seed=sp["seed"])
+        ch.update(3)
+        assert np.array_equal(b.records(i), ch.records()), i
+        ch.close()
+    b.close()
