@@ -53,7 +53,7 @@ BATCH_CHAINS, BATCH_UPDATES, BATCH_BUDGET_GB = 4096, 100, 150.0
 # The served form beside them: request streams at a light and at a saturating
 # rate (latency per update block, p50 / p99, and V+E/s).
 SERVED_RATES, SERVED_SECONDS, SERVED_LMAX = (20.0, 50.0), 10.0, 4096
-KERNELS_PER_UPDATE = 12
+KERNELS_PER_UPDATE = 11
 # DRAM bytes per vertex of each phase's kernels (DRAM bytes of one ncu
 # capture at L=16384, beta=4096 -- dram__bytes.sum.per_second x
 # gpu__time_duration.sum -- divided by that update's vertex count;

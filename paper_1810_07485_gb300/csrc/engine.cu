@@ -602,8 +602,7 @@ int Engine::enqueue_one(bool timed, int slot) {
     if (k < LCQMC_NPHASE) nvtxRangePushA(kPhase[k]);
   };
   mark(0);  // [0] labeling: random numbers, insertion, vertex offsets (one pass)
-  launch_bond_parity(L_, st_);
-  launch_clear(L_, cap_tiles_, nw, st_);
+  launch_start(L_, cap_tiles_, nw, st_);
   launch_insert(L_, st_);
   mark(1);  // [1] tau = 0 cut
   launch_cut(L_, st_);
@@ -617,9 +616,9 @@ int Engine::enqueue_one(bool timed, int slot) {
   mark(5);  // [5] operator offsets
   launch_scan_ops(L_, st_);
   mark(6);  // [6] operator rewrite
-  launch_compact(L_, st_);
+  launch_compact(L_, !timed, st_);
   mark(7);  // [7] spin rewrite + record
-  launch_sites(L_, st_);
+  if (timed) launch_sites(L_, st_);  // on its own, for the phase's time
   launch_final(L_, st_);
   mark(8);
   CK(cudaGetLastError());
@@ -803,6 +802,9 @@ int Engine::sync(bool *at_once) {
       if (rc) return rc;
     }
     if (status & ST_OP_OVERFLOW) {
+      // the open loops' records were added to but not all squared and cleared
+      CK(cudaMemsetAsync(s_.acc, 0, ACC_WORDS * sizeof(unsigned long long) * vcap_, st_));
+      CK(cudaMemsetAsync(s_.accz, 0, sizeof(unsigned long long) * vcap_, st_));
       for (int64_t c = 0; c < (int64_t)hch.size(); ++c)
         if (hch[c].n_off_new > hch[c].op_cap) {
           rc = grow_ops(c, hch[c].n_off_new);

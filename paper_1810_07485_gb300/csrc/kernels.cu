@@ -3,7 +3,8 @@
 // consecutive cells (bond x time window) of one chain; a tile is one block.
 //
 // Phase order per update (the Sec. 4.3 cost table's rows in brackets):
-//   k_bond_parity    spin parity of every bond at each time-block start
+//   k_start          spin parity of every bond at each time-block start; scratch
+//                    reset
 //   k_insert         per cell: Poisson candidates, keep the antiparallel ones,
 //                    merge with old operators, write vertices; offsets by
 //                    decoupled look-back over the tiles          [1, 2]
@@ -13,9 +14,10 @@
 //   k_compress       root of every node, one coin per loop              [3]
 //   k_est            new operator flags, loop lengths (tile-local loops in
 //                    shared memory, others in global accumulators)      [4]
-//   k_scan_ops       operator offsets per tile
+//   k_scan_ops       operator offsets per tile (chains of many tiles)
 //   k_compact        next operator list, squared lengths of open loops  [8]
-//   k_sites          spins at tau = 0, vertex-free loops                [8]
+//   k_sites          spins at tau = 0, vertex-free loops (chains of few
+//                    tiles: blocks of k_compact's launch)               [8]
 //   k_final          per-chain record, running sums, buffer swap
 #include <algorithm>
 #include <cmath>
@@ -164,16 +166,10 @@ __device__ __forceinline__ void store_word(uint32_t *bits, int64_t word, uint32_
     atomicOr(bits + word, x);
 }
 
-// ---- bond parity at time-block starts ---------------------------------------
+// ---- start of an update: bond parities, scratch reset --------------------------
 // bpar[(blk) * nbond + b] = parity of the operators of bond b in time blocks
 // before blk; row nblk is the parity over the whole period.
-__global__ void k_bond_parity(const DevChain *__restrict__ ch, const int2 *__restrict__ tab,
-                              int64_t blk0, Scratch s) {
-  if (halted(s)) return;
-  const int2 t = tab[blk0 + blockIdx.x];
-  const DevChain &C = ch[t.x];
-  const int b = t.y * BOND_BLOCK + threadIdx.x;
-  if (b >= C.nbond) return;
+__device__ __forceinline__ void bond_parity(const DevChain &C, int b, const Scratch &s) {
   const int32_t *op = C.op_ptr[C.cur];
   uint8_t *row = s.bpar + C.bpar_off;
   uint8_t p = 0;
@@ -187,14 +183,23 @@ __global__ void k_bond_parity(const DevChain *__restrict__ ch, const int2 *__res
   }
 }
 
-// ---- per-update scratch reset -------------------------------------------------
-// The insertion's look-back words and tile tickets and the five per-vertex
-// bitmaps (open marks, open roots, flips, new operators, crossing marks) start each
-// update at zero: one grid-stride launch instead of one memset each (a small
-// chain's update is a chain of short launches).
-__global__ void k_clear(Scratch s, int64_t ntile, int64_t nw) {
-  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+// The first nbb blocks take a block of bonds each; the others reset the
+// insertion's look-back words and tile tickets, the operator scan's part words
+// and the five per-vertex bitmaps (open marks, open roots, flips, new
+// operators, crossing marks), which start each update at zero.  One launch for
+// both: a small chain's update is a chain of short launches.
+__global__ void __launch_bounds__(BOND_BLOCK) k_start(const DevChain *__restrict__ ch,
+                                                      const int2 *__restrict__ tab, int64_t nbb, Scratch s,
+                                                      int64_t ntile, int64_t nw) {
+  if (blockIdx.x < nbb) {
+    if (halted(s)) return;
+    const int2 t = tab[blockIdx.x];
+    const int b = t.y * BOND_BLOCK + threadIdx.x;
+    if (b < ch[t.x].nbond) bond_parity(ch[t.x], b, s);
+    return;
+  }
+  const int64_t i0 = (blockIdx.x - nbb) * blockDim.x + threadIdx.x;
+  const int64_t step = (gridDim.x - nbb) * blockDim.x;
   for (int64_t i = i0; i < nw; i += step) {
     s.openmark[i] = 0u;
     s.openroot[i] = 0u;
@@ -1782,27 +1787,112 @@ __global__ void __launch_bounds__(NT, (T ? 1536 : 2048) / NT) k_est(const DevCha
   }
 }
 
+// ---- spins at tau = 0, vertex-free loops -------------------------------------------
+// Site block gb: one thread per site (the threads past SITE_BLOCK have none).
+// QT: Q = 2S if known at compile time, else 0.
+template <int QT>
+__device__ __forceinline__ void rewrite_sites(const DevChain *__restrict__ ch, const int2 *__restrict__ tab,
+                                              int64_t gb, const Scratch &s) {
+  const int2 t = tab[gb];
+  const DevChain &C = ch[t.x];
+  const int i = t.y * SITE_BLOCK + threadIdx.x, Q = QT ? QT : C.Q;
+  const int64_t wb = C.vtx_base >> 5;
+  long long nfree = 0;
+  u128 w2 = 0, f2 = 0, none = 0;
+  if (threadIdx.x < SITE_BLOCK && i < C.L) {
+    const uint8_t *s0 = C.s0[C.cur];
+    uint8_t *s1 = C.s0[C.cur ^ 1];
+    for (int a = 0; a < Q; ++a) {
+      const int u = i * Q + a;
+      const int node = s.cut_node[C.sub_off + u];
+      int f;
+      if (node >= 0) {
+        f = get_bit(s.flipbits, wb, node);
+      } else {
+        const int mn = s.free_min[C.sub_off + u];
+        f = coin(C, TAG_FREE, (uint32_t)mn);
+        if (mn == u) {
+          ++nfree;
+          const long long len = (long long)s.free_len[C.sub_off + u] * C.qbeta;
+          w2 += sq_abs(len);
+          f2 += sq_abs(mul_q32(len, C.cosq[i])) + sq_abs(mul_q32(len, C.sinq[i]));
+        }
+      }
+      s1[u] = (uint8_t)(s0[u] ^ f);
+    }
+  }
+  block_sums<false>(nfree, w2, f2, none);
+  if (threadIdx.x == 0) {
+    s.site_free[gb] = nfree;
+    s.site_sw2[2 * gb] = (unsigned long long)w2;
+    s.site_sw2[2 * gb + 1] = (unsigned long long)(w2 >> 64);
+    s.site_sf2[2 * gb] = (unsigned long long)f2;
+    s.site_sf2[2 * gb + 1] = (unsigned long long)(f2 >> 64);
+  }
+}
+
+template <int Q>
+__global__ void __launch_bounds__(SITE_BLOCK) k_sites(const DevChain *__restrict__ ch,
+                                                      const int2 *__restrict__ tab, int64_t blk0,
+                                                      Scratch s) {
+  if (halted(s)) return;
+  rewrite_sites<Q>(ch, tab, blk0 + blockIdx.x, s);
+}
+
 // ---- next operator list + open loops -------------------------------------------------
 // The tile's new operators are a bitmap of its vertices: a scan of the words'
 // counts gives every word's first place, a warp then moves the marked times of
 // a word at a time (id order = order of the next operator list), and a cell's
 // first operator is the count before its first vertex.
-template <bool T>
-__global__ void __launch_bounds__(TPB, T ? 4 : 8) k_compact(const DevChain *__restrict__ ch,
-                                                 const int2 *__restrict__ tab, int64_t blk0,
-                                                 Scratch s) {
+//
+// SMALL (every chain has at most OWN_SCAN tiles): two launches less.  A tile
+// adds up the counts before it itself instead of reading them from k_scan_ops,
+// and the blocks past the ntiles tiles rewrite the site blocks' spins (k_sites),
+// which need nothing of the operator list: 55 -> 51 us for an update of the
+// L=64 chain, 93 -> 86 us at L=1024, beta=256, with k_start's two parts in one
+// launch.  Longer chains have the two kernels of their own: the code for both
+// in one kernel cost the operator rewrite 4 % at 2^19 tiles (registers).
+constexpr int OWN_SCAN = 1024;
+
+template <bool T, bool SMALL>
+__global__ void __launch_bounds__(TPB, T || SMALL ? 4 : 8) k_compact(DevChain *__restrict__ ch,
+                                                 const int2 *__restrict__ tab, int64_t ntiles,
+                                                 const int2 *__restrict__ site_tab, Scratch s) {
   __shared__ int sm[33];
   __shared__ uint32_t nbits[TPB];
   __shared__ int npre[TPB];
   if (halted(s)) return;
-  const int64_t gt = blk0 + blockIdx.x;
+  if (SMALL && blockIdx.x >= ntiles) {
+    rewrite_sites<0>(ch, site_tab, blockIdx.x - ntiles, s);
+    return;
+  }
+  const int64_t gt = blockIdx.x;
   const int2 t = tab[gt];
-  const DevChain &C = ch[t.x];
+  DevChain &C = ch[t.x];
   const int c0 = t.y * TILE, c1 = min(C.ncell, c0 + TILE), ncl = c1 - c0;
   int32_t *nptr = C.op_ptr[C.cur ^ 1];
   const int32_t *vp = s.vptr + C.cell_off;
   const int64_t vb = C.vtx_base;
-  const int64_t base = s.tile_pref2[gt];
+  int64_t base;
+  bool fits = true;
+  if (SMALL) {
+    int64_t before = 0, all = 0;
+    for (int i = threadIdx.x; i < C.ntile; i += TPB) {
+      const int64_t x = s.tile_sum2[C.tile0 + i];
+      before += i < t.y ? x : 0;
+      all += x;
+    }
+    __shared__ int64_t sm64[2][33];
+    base = block_sum<int64_t>(before, sm64[0]);
+    all = block_sum<int64_t>(all, sm64[1]);
+    fits = all <= C.op_cap;  // else no list is written: the host grows it and replays
+    if (threadIdx.x == 0 && t.y == C.ntile - 1) {
+      C.n_off_new = all;
+      if (!fits) atomicOr(s.status, ST_OP_OVERFLOW);
+    }
+  } else {
+    base = s.tile_pref2[gt];
+  }
   const int a = uniform(vp[c0]), e = uniform(vp[c1]);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int cv = (threadIdx.x < ncl) ? vp[c0 + threadIdx.x] : e;  // first vertex of the thread's cell
@@ -1826,7 +1916,7 @@ __global__ void __launch_bounds__(TPB, T ? 4 : 8) k_compact(const DevChain *__re
     __syncthreads();
     for (int k = wid; k < nk; k += TPB / 32) {
       const uint32_t x = nbits[k];
-      if ((x >> lane) & 1u)
+      if (((x >> lane) & 1u) && fits)
         ntau[npre[k] + __popc(x & ((1u << lane) - 1u))] = s.vtau[((wfirst + k0 + k) << 5) + lane];
     }
     const int64_t k = ((vb + cv) >> 5) - wfirst - k0;
@@ -1836,7 +1926,8 @@ __global__ void __launch_bounds__(TPB, T ? 4 : 8) k_compact(const DevChain *__re
   }
   if (threadIdx.x < ncl) {
     nptr[c0 + threadIdx.x] = (int32_t)(base + (at < 0 ? run : at));
-    if (c0 + (int)threadIdx.x == C.ncell - 1) nptr[C.ncell] = (int32_t)C.n_off_new;
+    // the last tile's operators end the list
+    if (c0 + (int)threadIdx.x == C.ncell - 1) nptr[C.ncell] = (int32_t)(base + run);
   }
   // Loops that left their tile: one 32-byte accumulator record per root (and
   // its Zi word), read and cleared; a thread takes one 32-vertex word of the
@@ -1904,56 +1995,6 @@ __global__ void __launch_bounds__(TPB, T ? 4 : 8) k_compact(const DevChain *__re
     add(s.tile_sw2, w2);
     add(s.tile_sf2, f2);
     add(s.tile_sz2, z2);
-  }
-}
-
-// ---- spins at tau = 0, vertex-free loops -------------------------------------------
-template <int Q>
-__global__ void __launch_bounds__(SITE_BLOCK) k_sites(const DevChain *__restrict__ ch,
-                                                      const int2 *__restrict__ tab, int64_t blk0,
-                                                      Scratch s) {
-  __shared__ int64_t sm[33];
-  if (halted(s)) return;
-  const int64_t gb = blk0 + blockIdx.x;
-  const int2 t = tab[gb];
-  const DevChain &C = ch[t.x];
-  const int i = t.y * SITE_BLOCK + threadIdx.x;
-  const int64_t vb = C.vtx_base, wb = vb >> 5;
-  int64_t nfree = 0;
-  u128 w2 = 0, f2 = 0;
-  if (i < C.L) {
-    const uint8_t *s0 = C.s0[C.cur];
-    uint8_t *s1 = C.s0[C.cur ^ 1];
-#pragma unroll
-    for (int a = 0; a < Q; ++a) {
-      const int u = i * Q + a;
-      const int node = s.cut_node[C.sub_off + u];
-      int f;
-      if (node >= 0) {
-        f = get_bit(s.flipbits, wb, node);
-      } else {
-        const int mn = s.free_min[C.sub_off + u];
-        f = coin(C, TAG_FREE, (uint32_t)mn);
-        if (mn == u) {
-          ++nfree;
-          const long long len = (long long)s.free_len[C.sub_off + u] * C.qbeta;
-          const int x = u / Q;
-          w2 += sq_abs(len);
-          f2 += sq_abs(mul_q32(len, C.cosq[x])) + sq_abs(mul_q32(len, C.sinq[x]));
-        }
-      }
-      s1[u] = (uint8_t)(s0[u] ^ f);
-    }
-  }
-  const int64_t tf = block_sum<int64_t>(nfree, sm);
-  w2 = block_sum_u128(w2);
-  f2 = block_sum_u128(f2);
-  if (threadIdx.x == 0) {
-    s.site_free[gb] = tf;
-    s.site_sw2[2 * gb] = (unsigned long long)w2;
-    s.site_sw2[2 * gb + 1] = (unsigned long long)(w2 >> 64);
-    s.site_sf2[2 * gb] = (unsigned long long)f2;
-    s.site_sf2[2 * gb + 1] = (unsigned long long)(f2 >> 64);
   }
 }
 
@@ -2149,17 +2190,12 @@ static int64_t all_tiles(const Launch &L) {
   return n;
 }
 
-void launch_bond_parity(const Launch &L, cudaStream_t st) {
-  for (int q = 0; q < QMAX; ++q)
-    if (L.nbondblk[q])
-      k_bond_parity<<<g1(L.nbondblk[q]), BOND_BLOCK, 0, st>>>(L.ch, L.bond_tab, L.bond0[q], L.s);
-}
-
-void launch_clear(const Launch &L, int64_t ntile, int64_t nw, cudaStream_t st) {
-  constexpr int T = 256;
-  const int64_t n = std::max<int64_t>(std::max(ntile, nw), QMAX);
-  const int64_t blocks = std::min<int64_t>((n + T - 1) / T, 152 * 8);
-  k_clear<<<g1(blocks), T, 0, st>>>(L.s, ntile, nw);
+void launch_start(const Launch &L, int64_t ntile, int64_t nw, cudaStream_t st) {
+  int64_t nbb = 0;
+  for (int q = 0; q < QMAX; ++q) nbb += L.nbondblk[q];
+  const int64_t n = std::max<int64_t>(std::max(ntile, nw), SCAN_PARTS);
+  const int64_t blocks = std::min<int64_t>((n + BOND_BLOCK - 1) / BOND_BLOCK, 152 * 16);
+  k_start<<<g1(nbb + blocks), BOND_BLOCK, 0, st>>>(L.ch, L.bond_tab, nbb, L.s, ntile, nw);
 }
 
 void launch_insert(const Launch &L, cudaStream_t st) {
@@ -2173,7 +2209,11 @@ void launch_insert(const Launch &L, cudaStream_t st) {
 #undef INSERT_Q
 }
 
+// Whether the operator rewrite adds up the tiles' counts by itself.
+static bool own_scan(const Launch &L) { return L.max_ntile <= OWN_SCAN; }
+
 void launch_scan_ops(const Launch &L, cudaStream_t st) {
+  if (own_scan(L)) return;
   // Parts of at least 1024 tiles, and no more than one block per SM in all, so
   // that every part is resident while others wait for it.
   const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(L.max_ntile / 1024, SCAN_PARTS / L.nchains));
@@ -2288,14 +2328,22 @@ void launch_est(const Launch &L, cudaStream_t st) {
 #undef EST_QTN
 }
 
-void launch_compact(const Launch &L, cudaStream_t st) {
-  const int64_t n = all_tiles(L);
-  if (n) {
+void launch_compact(const Launch &L, bool sites, cudaStream_t st) {
+  const int64_t nt = all_tiles(L);
+  if (own_scan(L)) {
+    int64_t ns = 0;
+    for (int q = 0; q < QMAX && sites; ++q) ns += L.nsiteblk[q];
     if (L.temporal)
-      k_compact<true><<<g1(n), TPB, 0, st>>>(L.ch, L.tile_tab, 0, L.s);
+      k_compact<true, true><<<g1(nt + ns), TPB, 0, st>>>(L.ch, L.tile_tab, nt, L.site_tab, L.s);
     else
-      k_compact<false><<<g1(n), TPB, 0, st>>>(L.ch, L.tile_tab, 0, L.s);
+      k_compact<false, true><<<g1(nt + ns), TPB, 0, st>>>(L.ch, L.tile_tab, nt, L.site_tab, L.s);
+    return;
   }
+  if (L.temporal)
+    k_compact<true, false><<<g1(nt), TPB, 0, st>>>(L.ch, L.tile_tab, nt, L.site_tab, L.s);
+  else
+    k_compact<false, false><<<g1(nt), TPB, 0, st>>>(L.ch, L.tile_tab, nt, L.site_tab, L.s);
+  if (sites) launch_sites(L, st);
 }
 
 void launch_sites(const Launch &L, cudaStream_t st) {

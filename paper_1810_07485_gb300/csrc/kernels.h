@@ -26,9 +26,9 @@ struct Launch {
 
 void set_full_table(const uint64_t *T, cudaStream_t st);
 int init_kernel_attributes();
-void launch_bond_parity(const Launch &L, cudaStream_t st);
-// zeroes the look-back words of ntile tiles, the tickets and nw words of each bitmap
-void launch_clear(const Launch &L, int64_t ntile, int64_t nw, cudaStream_t st);
+// bond parities; zeroes the look-back words of ntile tiles, the tickets and nw
+// words of each bitmap
+void launch_start(const Launch &L, int64_t ntile, int64_t nw, cudaStream_t st);
 void launch_insert(const Launch &L, cudaStream_t st);
 void launch_scan_ops(const Launch &L, cudaStream_t st);
 void launch_cut(const Launch &L, cudaStream_t st);
@@ -36,7 +36,9 @@ void launch_link(const Launch &L, cudaStream_t st);
 void launch_compress(const Launch &L, cudaStream_t st);
 void launch_check_forest(const Launch &L, cudaStream_t st);
 void launch_est(const Launch &L, cudaStream_t st);
-void launch_compact(const Launch &L, cudaStream_t st);
+// operator rewrite; sites: the spin rewrite too, in the same launch where that
+// is faster (else launch_sites is the caller's)
+void launch_compact(const Launch &L, bool sites, cudaStream_t st);
 void launch_sites(const Launch &L, cudaStream_t st);
 void launch_final(const Launch &L, cudaStream_t st);
 

@@ -39,7 +39,7 @@ def test_parts_in_an_uneven_batch():
     # a chain of several parts beside chains whose later parts are empty
     from paper_1810_07485_gb300 import lcqmc
     specs = [dict(L=2, beta=3.0, seed=1), dict(L=2054, beta=4096.0, seed=2), dict(L=34, beta=40.0, S=1.0, seed=3),
-             dict(L=1030, beta=4096.0, seed=4)]
+             dict(L=1030, beta=4096.0, seed=4), dict(L=6, beta=20.0, S=1.5, seed=5), dict(L=130, beta=7.0, S=2.0, seed=6)]
     b = lcqmc.Batch(specs)
     b.update(3)
     for i, sp in enumerate(specs):
