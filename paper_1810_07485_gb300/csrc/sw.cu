@@ -11,16 +11,22 @@
 //   every cluster flips with the coin bit (r mod 128) of
 //   Philox(ctr = (TAG_SWFLIP << 24, r / 128, 0, sweep)).
 //
-// GPU layout: 64 x 32 site tiles, one 256-thread block each.
-//   k_sw_local  bond draws, union-find of the tile's bonds in shared memory
-//               (min-root hooking, one CAS), flattened; par[i] = the tile-local
-//               root (its smallest site); tile-boundary bonds kept as bit masks
+// GPU layout: 64 x 32 site tiles, one 256-thread block each; spins one bit per
+// site, a 64-bit word per tile row (bytes only at the C interface).  Inside a
+// row the active right bonds form runs of consecutive sites; everything a
+// cluster needs is kept per run, and rows are handled as words.
+//   k_sw_local  bond draws, union-find of the tile's runs in shared memory
+//               (min-root hooking, one CAS), flattened: the local root of every
+//               run start (its cluster's smallest site in the tile); tile-boundary
+//               bonds kept as bit masks
 //   k_sw_merge  boundary bonds united in the global forest (same min-root rule,
 //               path halving), one warp per tile: the paper's two-step
 //               local/global union-find (Sec. 3.2) inside one GPU
-//   k_sw_flip   root of every local root (path halving), one coin per local
-//               root, spins flipped; sizes of clusters closed in the tile
-//               squared here, sizes of open ones added at their global root
+//   k_sw_find   global root of every open component's local root (path
+//               halving) and its coin, one warp per tile
+//   k_sw_flip   one coin per local root, spins flipped; sizes of clusters
+//               closed in the tile squared here, sizes of open ones added at
+//               their global root
 //   k_sw_sizes  open clusters' sizes squared, cleared for the next update
 //   k_sw_final  the update's record and running sums
 #include <cuda_runtime.h>
@@ -64,21 +70,31 @@ struct SwDev {
   double sum[LCQMC_SW_NOBS], sumsq[LCQMC_SW_NOBS];
 };
 
+typedef unsigned long long u64;
+
 struct SwScratch {
   SwDev *dev;
   int *status;
-  uint8_t *spin;                // N
-  int32_t *par;                 // N: local root (non-roots), global forest (local roots)
-  uint32_t *lroot, *openb;      // per tile, SW_WORDS words: local roots; roots of open components
+  uint8_t *bytes;               // N: spins as bytes, for the C interface only
+  u64 *spin;                    // per tile, SW_TY rows: spins of its sites (0 past its edges)
+  u64 *starts;                  // per tile, SW_TY rows: first sites of the runs of active right bonds
+  unsigned short *lroot;        // per tile, SW_TS: local root, at run starts
+  int32_t *par;                 // N: global forest, at the local roots of open components
+  uint32_t *openb;              // per tile, SW_WORDS words: local roots of open components
   uint32_t *edge_r;             // per tile: right-edge bond of row j active (bit j)
-  unsigned long long *edge_d;   // per tile: bottom-edge bond of column j active (bit j)
+  u64 *edge_d;                  // per tile: bottom-edge bond of column j active (bit j)
+  unsigned short *olocal;       // per tile, SW_OPEN_PER_TILE: local roots of open components
+  int32_t *oroot;               // the same: their global roots, the top bit their cluster's coin
+  int *onum;                    // per tile: their number
   int32_t *csize;               // N: size of an open cluster at its root; 0 between updates
-  int32_t *olist;               // roots of open clusters (at most SW_OPEN_PER_TILE per tile)
-  int *ocount;                  // their number; 0 between updates
+  int32_t *olist;               // per tile, SW_OPEN_PER_TILE: roots of open clusters in the tile
+  int *rnum;                    // per tile: their number
   long long *tile_part;         // per tile: n_eq, n_act, closed clusters, mag, largest closed
   unsigned long long *tile_c2;  // per tile: sum of the closed clusters' size^2
-  long long *size_part;         // per size block: open clusters, largest open
-  unsigned long long *size_c2;  // per size block: sum of the open clusters' size^2
+  // per block of k_sw_sizes, over its tiles and its open clusters: n_eq, n_act,
+  // clusters, mag, largest
+  long long *size_part;
+  unsigned long long *size_c2;  // per block of k_sw_sizes: sum of size^2
   lcqmc_sw_record *ring;
   int32_t *roots;               // lcqmc_sw_get_roots output (N), allocated on demand
 };
@@ -163,277 +179,486 @@ __device__ void block_reduce(long long (&v)[NS], long long &mx, unsigned long lo
   __syncthreads();
 }
 
+// ---- rows as 64-bit words -----------------------------------------------------------
+// The word of the first n columns.
+__device__ __forceinline__ u64 low_bits(int n) { return n >= 64 ? ~0ull : ((1ull << n) - 1ull); }
+
+// First column of the run that holds column x, given the row's run starts.
+__device__ __forceinline__ int run_start(u64 starts, int x) { return 63 - __clzll((long long)(starts & (~0ull >> (63 - x)))); }
+
+// Columns of the run that starts at column x.
+__device__ __forceinline__ u64 run_bits(u64 starts, int x, int w) {
+  const u64 above = starts & (~1ull << x);  // later starts
+  return (above ? ((above & (0ull - above)) - 1ull) : low_bits(w)) & (~0ull << x);
+}
+
+// Starts of the runs that hold a bit of x.
+__device__ __forceinline__ u64 runs_with(u64 starts, u64 x) {
+  u64 go = ~starts;  // columns a bit may move down from, o places at a time
+#pragma unroll
+  for (int o = 1; o < 64; o <<= 1) {
+    x |= (x & go) >> o;
+    go &= go << o;
+  }
+  return x & starts;
+}
+
+// Site id of tile-local index l.
+__device__ __forceinline__ int32_t site_of(int x0, int y0, int L, int l) {
+  return (int32_t)((int64_t)(y0 + (l >> 6)) * L + x0 + (l & 63));
+}
+
+// Philox4x32-10 of the counter (TAG_SWBOND << 24, site, 0, sweep), words 0 and
+// 1: the rounds whose inputs do not depend on the site are taken once (15 of
+// the 20 products are left), with the round keys.
+struct SiteDraw {
+  uint32_t k0, k1, b1, d0, e1, f;
+
+  __device__ __forceinline__ SiteDraw(uint32_t key0, uint32_t key1, uint32_t sweep) : k0(key0), k1(key1) {
+    const u64 p0 = (u64)M0 * (TAG_SWBOND << 24);           // round 0: second product zero
+    const uint32_t a = (uint32_t)(p0 >> 32) ^ sweep ^ k1;  // c2 of round 1
+    const u64 p1 = (u64)M1 * a;                            // round 1: c1 = 0
+    const uint32_t c = (uint32_t)(p1 >> 32) ^ (k0 + W0);   // c0 of round 2
+    const u64 p2 = (u64)M0 * c;
+    b1 = (uint32_t)p0 ^ (k1 + W1);
+    d0 = (uint32_t)p1 ^ (k0 + 2 * W0);
+    e1 = (uint32_t)(p2 >> 32) ^ (k1 + 2 * W1);
+    f = (uint32_t)p2;
+  }
+
+  __device__ __forceinline__ void operator()(uint32_t site, uint32_t &x, uint32_t &y) const {
+    const u64 p = (u64)M0 * (site ^ k0);                 // round 1
+    const u64 q = (u64)M1 * ((uint32_t)(p >> 32) ^ b1);  // round 2
+    uint32_t c0 = (uint32_t)(q >> 32) ^ d0, c1 = (uint32_t)q, c2 = e1 ^ (uint32_t)p, c3 = f;
+#pragma unroll
+    for (uint32_t r = 3; r < 10; ++r) {
+      const u64 u = (u64)M0 * c0, v = (u64)M1 * c2;
+      c0 = (uint32_t)(v >> 32) ^ c1 ^ (k0 + r * W0);
+      c1 = (uint32_t)v;
+      c2 = (uint32_t)(u >> 32) ^ c3 ^ (k1 + r * W1);
+      c3 = (uint32_t)u;
+    }
+    x = c0;
+    y = c1;
+  }
+
+  static constexpr uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u, W0 = 0x9E3779B9u, W1 = 0xBB67AE85u;
+};
+
+__device__ __forceinline__ uint32_t same_on_all(uint32_t x) { return __reduce_max_sync(0xffffffffu, x); }
+
 // ---- bonds and tile union-find --------------------------------------------------
-// Bond bits are kept per tile in shared memory, one ballot per warp and step.
-// Inside a row the active right bonds form runs of consecutive sites; a site's
-// run starts at the highest "run start" bit at or below it (bit arithmetic on
-// the row's 64-bit mask), which seeds the forest.  Only the vertical bonds
-// then need unions, and a vertical bond whose left neighbour is also active,
-// with both right bonds between them active, joins runs already joined.
-__global__ void __launch_bounds__(SW_TPB) k_sw_local(SwScratch s) {
-  __shared__ uint8_t sp[SW_TY + 2][SW_TX + 2];  // spins with a one-site periodic halo
-  __shared__ int lp[SW_TS];
-  __shared__ uint32_t bR[SW_WORDS], bD[SW_WORDS], bO[SW_WORDS];  // inner right / down bonds, open sites
-  __shared__ uint32_t ob[SW_WORDS];                              // local roots of open components
-  __shared__ uint32_t er_s;
-  __shared__ unsigned long long ed_s;
+// The draws of a half row are two ballots of a warp; one thread per row then
+// takes the row's bonds as words: active right and down bonds, run starts, and
+// the down bonds that need a union (one whose left neighbour is also active,
+// with both right bonds between them active, joins runs already joined).  Those
+// bonds are listed, about 650 of 2048 sites at K_c, and united by whole warps,
+// run start to run start.
+//
+// Bound by instruction issue: the draws are about a quarter of it, the unions
+// the larger part of the rest.
+__global__ void __launch_bounds__(SW_TPB, 8) k_sw_local(SwScratch s) {
+  __shared__ int lp[SW_TS];               // forest of the run starts
+  __shared__ unsigned short vlist[SW_TS]; // upper ends of the down bonds to unite
+  __shared__ uint32_t drawR[SW_WORDS], drawD[SW_WORDS];  // draws below T, per half row
+  __shared__ u64 start_s[SW_TY], vert_s[SW_TY], open_run[SW_TY];  // open_run: run starts of open sites
+  __shared__ uint32_t open_s[SW_WORDS];   // sites on active tile-boundary bonds
+  __shared__ uint32_t ob[SW_WORDS];       // local roots of open components
+  __shared__ int vbase[SW_TY];
+  __shared__ int nvert, nopen;
   if (__ldcg(s.status)) return;
   const SwDev &D = *s.dev;
   const int t = blockIdx.x, L = D.L;
   int x0, y0, w, h;
   sw_tile(D, t, x0, y0, w, h);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int r = wid; r < h + 2; r += SW_TPB / 32) {  // a warp per row, no division
-    int gy = y0 - 1 + r;
-    gy += (gy < 0) ? L : 0;
-    gy -= (gy >= L) ? L : 0;
-    const uint8_t *row = s.spin + (int64_t)gy * L;
-    for (int c = lane; c < w + 2; c += 32) {
-      int gx = x0 - 1 + c;
-      gx += (gx < 0) ? L : 0;
-      gx -= (gx >= L) ? L : 0;
-      sp[r][c] = row[gx];
-    }
+  const SiteDraw draw(same_on_all((uint32_t)D.seed), same_on_all((uint32_t)(D.seed >> 32)), same_on_all(D.sweep));
+  const bool some = D.T > 0;  // a draw is below T iff T > 0 and it is at most T - 1
+  const uint32_t top = (uint32_t)(D.T - 1);
+  if (threadIdx.x < SW_WORDS) {
+    ob[threadIdx.x] = 0u;
+    open_s[threadIdx.x] = 0u;
+    if (threadIdx.x == 0) nopen = 0;
   }
-  if (threadIdx.x < SW_WORDS) ob[threadIdx.x] = 0u;
-  if (threadIdx.x == 0) {
-    er_s = 0u;
-    ed_s = 0ull;
+  {
+    const int lx = 32 * (wid & 1) + lane;
+    const uint32_t g0 = (uint32_t)((int64_t)y0 * L + x0 + lx);
+#pragma unroll 2
+    for (int k = 0; k < SW_PER; ++k) {
+      const int ly = 4 * k + (wid >> 1), l = ly * SW_TX + lx;
+      uint32_t x, y;
+      draw(g0 + (uint32_t)ly * (uint32_t)L, x, y);
+      const bool in = some && lx < w && ly < h;
+      const uint32_t mr = __ballot_sync(0xffffffffu, in && x <= top);
+      const uint32_t md = __ballot_sync(0xffffffffu, in && y <= top);
+      if (lane == 0) {
+        drawR[l >> 5] = mr;
+        drawD[l >> 5] = md;
+      }
+      lp[l] = l;
+    }
   }
   __syncthreads();
-  const uint32_t k0 = (uint32_t)D.seed, k1 = (uint32_t)(D.seed >> 32), sweep = D.sweep;
-  const uint64_t T = D.T;
-  long long cnt[2] = {0, 0};  // equal bonds, active bonds
-#pragma unroll 2
-  for (int k = 0; k < SW_PER; ++k) {
-    const int l = threadIdx.x + k * SW_TPB, lx = l & (SW_TX - 1), ly = l / SW_TX;
-    bool ar = false, ad = false;
-    if (lx < w && ly < h) {
-      const uint32_t g = (uint32_t)((int64_t)(y0 + ly) * L + x0 + lx);
-      const U4 o = philox(TAG_SWBOND << 24, g, 0u, sweep, k0, k1);
-      const uint8_t sc = sp[ly + 1][lx + 1];
-      const bool eqr = sc == sp[ly + 1][lx + 2], eqd = sc == sp[ly + 2][lx + 1];
-      ar = eqr && (uint64_t)o.x < T;
-      ad = eqd && (uint64_t)o.y < T;
-      cnt[0] += (int)eqr + (int)eqd;
-      cnt[1] += (int)ar + (int)ad;
+  const int tx = t % D.ntx, ty = t / D.ntx;
+  const int left = ty * D.ntx + (tx ? tx - 1 : D.ntx - 1), right = ty * D.ntx + (tx + 1 < D.ntx ? tx + 1 : 0);
+  const int up = (ty ? ty - 1 : D.nty - 1) * D.ntx + tx, down = (ty + 1 < D.nty ? ty + 1 : 0) * D.ntx + tx;
+  if (wid == 0) {  // a thread per row
+    const int j = lane;
+    const u64 *own = s.spin + (int64_t)t * SW_TY;
+    u64 r = 0, d = 0, eq_r = 0, eq_d = 0;
+    if (j < h) {
+      const u64 me = own[j], cols = low_bits(w);
+      const u64 next = (me >> 1) | ((s.spin[(int64_t)right * SW_TY + j] & 1ull) << (w - 1));
+      const u64 below = j + 1 < h ? own[j + 1] : s.spin[(int64_t)down * SW_TY];
+      eq_r = ~(me ^ next) & cols;
+      eq_d = ~(me ^ below) & cols;
+      r = eq_r & (((u64)drawR[2 * j + 1] << 32) | drawR[2 * j]);
+      d = eq_d & (((u64)drawD[2 * j + 1] << 32) | drawD[2 * j]);
     }
-    const bool edge_r = ar && lx + 1 == w, edge_d = ad && ly + 1 == h;
-    const uint32_t mr = __ballot_sync(0xffffffffu, ar && !edge_r);
-    const uint32_t md = __ballot_sync(0xffffffffu, ad && !edge_d);
-    const uint32_t mo = __ballot_sync(0xffffffffu, edge_r || edge_d);
+    const u64 last = 1ull << (w - 1);
+    const uint32_t er = __ballot_sync(0xffffffffu, (r & last) != 0);
+    const u64 open = (r & last) | (j == h - 1 ? d : 0ull);
+    const u64 ri = r & ~last;                  // right bonds inside the tile
+    const u64 di = j < h - 1 ? d : 0ull;       // down bonds inside the tile
+    const u64 r1 = __shfl_down_sync(0xffffffffu, ri, 1);
+    const u64 vert = di & ~((di & ri & r1) << 1);
+    start_s[j] = ~(ri << 1) & (j < h ? low_bits(w) : 0ull);
+    vert_s[j] = vert;
+    if ((uint32_t)open) atomicOr(&open_s[2 * j], (uint32_t)open);
+    if (open >> 32) atomicOr(&open_s[2 * j + 1], (uint32_t)(open >> 32));
+    const int nv = __popcll(vert);
+    int inc = nv;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    vbase[j] = inc - nv;
+    int n_eq = __popcll(eq_r) + __popcll(eq_d), n_act = __popcll(r) + __popcll(d);
+    n_eq = __reduce_add_sync(0xffffffffu, n_eq);
+    n_act = __reduce_add_sync(0xffffffffu, n_act);
+    s.starts[(int64_t)t * SW_TY + j] = start_s[j];
+    if (j == h - 1) s.edge_d[t] = d;
+    if (lane == 31) nvert = inc;
     if (lane == 0) {
-      bR[k * (SW_TPB / 32) + wid] = mr;
-      bD[k * (SW_TPB / 32) + wid] = md;
-      bO[k * (SW_TPB / 32) + wid] = mo;
+      s.edge_r[t] = er;
+      s.tile_part[5 * (int64_t)t] = n_eq;
+      s.tile_part[5 * (int64_t)t + 1] = n_act;
     }
-    if (edge_r) atomicOr(&er_s, 1u << ly);
-    if (edge_d) atomicOr(&ed_s, 1ull << lx);
+  } else if (wid == 1) {
+    // bonds of the neighbouring tiles that end in this one: R of the column to
+    // the left
+    const int j = lane, wl = min(SW_TX, L - (left % D.ntx) * SW_TX);
+    if (j < h) {
+      const uint32_t g = (uint32_t)((int64_t)(y0 + j) * L + (x0 == 0 ? L - 1 : x0 - 1));
+      uint32_t x, y;
+      draw(g, x, y);
+      const u64 a = s.spin[(int64_t)left * SW_TY + j] >> (wl - 1), b = s.spin[(int64_t)t * SW_TY + j];
+      if (some && x <= top && !((a ^ b) & 1ull)) atomicOr(&open_s[2 * j], 1u);
+    }
+  } else if (wid < 4) {  // D of the row above
+    const int c = threadIdx.x - 64, hu = min(SW_TY, L - (up / D.ntx) * SW_TY);
+    bool on = false;
+    if (c < w) {
+      const uint32_t g = (uint32_t)((int64_t)(y0 == 0 ? L - 1 : y0 - 1) * L + x0 + c);
+      uint32_t x, y;
+      draw(g, x, y);
+      const u64 a = s.spin[(int64_t)up * SW_TY + hu - 1], b = s.spin[(int64_t)t * SW_TY];
+      on = some && y <= top && !(((a ^ b) >> c) & 1ull);
+    }
+    const uint32_t m = __ballot_sync(0xffffffffu, on);
+    if (lane == 0 && m) atomicOr(&open_s[wid - 2], m);
   }
   __syncthreads();
-  // bonds of the neighbouring tiles that end in this one: R of the column to
-  // the left (threads 0..h-1), D of the row above (threads 64..64+w-1)
-  if (threadIdx.x < h) {
-    const int j = threadIdx.x;
-    const uint32_t gl = (uint32_t)((int64_t)(y0 + j) * L + (x0 == 0 ? L - 1 : x0 - 1));
-    if (sp[j + 1][0] == sp[j + 1][1] && (uint64_t)philox(TAG_SWBOND << 24, gl, 0u, sweep, k0, k1).x < T)
-      atomicOr(&bO[(j * SW_TX) >> 5], 1u);
-  } else if (threadIdx.x >= 64 && threadIdx.x < 64 + w) {
-    const int c = threadIdx.x - 64;
-    const uint32_t gu = (uint32_t)((int64_t)(y0 == 0 ? L - 1 : y0 - 1) * L + x0 + c);
-    if (sp[0][c + 1] == sp[1][c + 1] && (uint64_t)philox(TAG_SWBOND << 24, gu, 0u, sweep, k0, k1).y < T)
-      atomicOr(&bO[c >> 5], 1u << (c & 31));
+  // the open sites' runs, a thread per row
+  if (wid == 7) {
+    const u64 open = ((u64)open_s[2 * lane + 1] << 32) | open_s[2 * lane];
+    open_run[lane] = runs_with(start_s[lane], open);
   }
-  // forest seeded with the row runs
-  for (int l = threadIdx.x; l < SW_TS; l += SW_TPB) {
-    const int lx = l & (SW_TX - 1), ly = l / SW_TX;
-    const unsigned long long m = ((unsigned long long)bR[2 * ly + 1] << 32) | bR[2 * ly];
-    const unsigned long long starts = ~(m << 1);  // bit x: R(x-1) inactive
-    const unsigned long long upto = (lx == SW_TX - 1) ? ~0ull : ((2ull << lx) - 1ull);
-    lp[l] = ly * SW_TX + (63 - __clzll(starts & upto));
+#pragma unroll
+  for (int k = 0; k < SW_PER; ++k) {
+    const int ly = 4 * k + (wid >> 1), lx = 32 * (wid & 1) + lane;
+    const u64 v = vert_s[ly];
+    if ((v >> lx) & 1ull)
+      vlist[vbase[ly] + __popcll(v & low_bits(lx))] = (unsigned short)(ly * SW_TX + lx);
   }
   __syncthreads();
-  // vertical bonds, skipping those implied by the left neighbour's
+  for (int i = threadIdx.x; i < nvert; i += SW_TPB) {
+    const int l = vlist[i], lx = l & (SW_TX - 1), ly = l / SW_TX;
+    sw_union(lp, ly * SW_TX + run_start(start_s[ly], lx), (ly + 1) * SW_TX + run_start(start_s[ly + 1], lx),
+             s.status);
+  }
+  __syncthreads();
+  // every run's local root (read-only walks: no union is running any more)
 #pragma unroll 2
   for (int k = 0; k < SW_PER; ++k) {
-    const int l = threadIdx.x + k * SW_TPB, lx = l & (SW_TX - 1), ly = l / SW_TX;
-    if (ly + 1 >= SW_TY) continue;
-    const unsigned long long d = ((unsigned long long)bD[2 * ly + 1] << 32) | bD[2 * ly];
-    if (!((d >> lx) & 1ull)) continue;
-    if (lx > 0) {
-      const unsigned long long r0 = ((unsigned long long)bR[2 * ly + 1] << 32) | bR[2 * ly];
-      const unsigned long long r1 = ((unsigned long long)bR[2 * ly + 3] << 32) | bR[2 * ly + 2];
-      if ((d & r0 & r1) >> (lx - 1) & 1ull) continue;  // D(x-1), R(x-1) above and below: joined
-    }
-    sw_union(lp, l, l + SW_TX, s.status);
-  }
-  __syncthreads();
-  // every site's local root (read-only walks: no union is running any more)
-#pragma unroll 2
-  for (int k = 0; k < SW_PER; ++k) {
-    const int l = threadIdx.x + k * SW_TPB, lx = l & (SW_TX - 1), ly = l / SW_TX;
-    const bool valid = lx < w && ly < h;
-    int r = l;
-    if (valid) {
-      r = lp[l];
+    const int ly = 4 * k + (wid >> 1), lx = 32 * (wid & 1) + lane, l = ly * SW_TX + lx;
+    const u64 st = start_s[ly];
+    if ((st >> lx) & 1ull) {
+      int r = lp[l];
       for (int it = 0; it <= SW_TS && lp[r] != r; ++it) r = lp[r];
-      s.par[(int64_t)(y0 + ly) * L + x0 + lx] = (int32_t)((int64_t)(y0 + r / SW_TX) * L + x0 + (r & (SW_TX - 1)));
-      if ((bO[l >> 5] >> (l & 31)) & 1u) atomicOr(&ob[r >> 5], 1u << (r & 31));
+      s.lroot[(int64_t)t * SW_TS + l] = (unsigned short)r;
+      if ((open_run[ly] >> lx) & 1ull) atomicOr(&ob[r >> 5], 1u << (r & 31));
     }
-    const uint32_t m = __ballot_sync(0xffffffffu, valid && r == l);
-    if (lane == 0) s.lroot[(int64_t)t * SW_WORDS + k * (SW_TPB / 32) + wid] = m;
   }
-  long long mx = 0;
-  unsigned long long none = 0;
-  block_reduce<2>(cnt, mx, none);  // its barrier also completes the open marks
-  if (threadIdx.x < SW_WORDS) s.openb[(int64_t)t * SW_WORDS + threadIdx.x] = ob[threadIdx.x];
-  if (threadIdx.x == 0) {
-    s.edge_r[t] = er_s;
-    s.edge_d[t] = ed_s;
-    s.tile_part[5 * (int64_t)t] = cnt[0];
-    s.tile_part[5 * (int64_t)t + 1] = cnt[1];
+  __syncthreads();
+  if (threadIdx.x < SW_WORDS) {
+    uint32_t m = ob[threadIdx.x];
+    s.openb[(int64_t)t * SW_WORDS + threadIdx.x] = m;
+    int at = m ? atomicAdd(&nopen, __popc(m)) : 0;
+    while (m) {  // open components are listed, and enter the global forest as their own roots
+      const int l = 32 * threadIdx.x + __ffs(m) - 1;
+      const int32_t g = site_of(x0, y0, L, l);
+      m &= m - 1;
+      s.par[g] = g;
+      s.olocal[(int64_t)t * SW_OPEN_PER_TILE + at++] = (unsigned short)l;
+    }
   }
+  __syncthreads();
+  if (threadIdx.x == 0) s.onum[t] = nopen;
 }
 
 // ---- tile-boundary bonds in the global forest ------------------------------------
+// Site of the local root of tile t's column x, row y.
+__device__ __forceinline__ int32_t local_root(const SwScratch &s, const SwDev &D, int t, int x, int y) {
+  const int l = y * SW_TX + run_start(s.starts[(int64_t)t * SW_TY + y], x);
+  int x0, y0, w, h;
+  sw_tile(D, t, x0, y0, w, h);
+  return site_of(x0, y0, D.L, s.lroot[(int64_t)t * SW_TS + l]);
+}
+
 __global__ void __launch_bounds__(256) k_sw_merge(SwScratch s) {
   if (__ldcg(s.status)) return;
   const SwDev &D = *s.dev;
   const int t = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (t >= D.ntile) return;
-  const int L = D.L;
   int x0, y0, w, h;
   sw_tile(D, t, x0, y0, w, h);
   const uint32_t er = s.edge_r[t];
-  const unsigned long long ed = s.edge_d[t];
-  const int xr = (x0 + w == L) ? 0 : x0 + w, yd = (y0 + h == L) ? 0 : y0 + h;
+  const u64 ed = s.edge_d[t];
+  const int tx = t % D.ntx, ty = t / D.ntx;
+  const int right = ty * D.ntx + (tx + 1 < D.ntx ? tx + 1 : 0), down = (ty + 1 < D.nty ? ty + 1 : 0) * D.ntx + tx;
   for (int j = lane; j < SW_TY + SW_TX; j += 32) {
-    int64_t a, b;
+    int32_t a, b;
     if (j < SW_TY) {
       if (!((er >> j) & 1u)) continue;
-      a = (int64_t)(y0 + j) * L + x0 + w - 1;
-      b = (int64_t)(y0 + j) * L + xr;
+      a = local_root(s, D, t, w - 1, j);
+      b = local_root(s, D, right, 0, j);
     } else {
       const int c = j - SW_TY;
       if (!((ed >> c) & 1ull)) continue;
-      a = (int64_t)(y0 + h - 1) * L + x0 + c;
-      b = (int64_t)yd * L + x0 + c;
+      a = local_root(s, D, t, c, h - 1);
+      b = local_root(s, D, down, c, 0);
     }
-    // start from the two local roots: only local roots' words change here
-    uf_union(s.par, __ldcg(s.par + a), __ldcg(s.par + b), s.status);
+    uf_union(s.par, a, b, s.status);
+  }
+}
+
+// ---- global roots of the open components --------------------------------------------
+// Chains of dependent loads, about 50 per tile at K_c: a kernel of their own
+// keeps every warp slot of the chip on them (inside k_sw_flip a block's other
+// work waited for them: 0.53 ms there).
+__global__ void __launch_bounds__(256) k_sw_find(SwScratch s) {
+  if (__ldcg(s.status)) return;
+  const SwDev &D = *s.dev;
+  const int t = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (t >= D.ntile) return;
+  int x0, y0, w, h;
+  sw_tile(D, t, x0, y0, w, h);
+  const uint32_t k0 = (uint32_t)D.seed, k1 = (uint32_t)(D.seed >> 32);
+  const int n = s.onum[t];
+  for (int i = lane; i < n; i += 32) {
+    const int64_t k = (int64_t)t * SW_OPEN_PER_TILE + i;
+    const int32_t g = site_of(x0, y0, D.L, s.olocal[k]);
+    // path halving on the way and the root stored at the start: every entry
+    // still points to an ancestor
+    const int gr = uf_find(s.par, g, s.status);
+    if (gr != g) s.par[g] = gr;
+    const int coin = coin_from(philox(TAG_SWFLIP << 24, (uint32_t)gr >> 7, 0u, D.sweep, k0, k1), (uint32_t)gr);
+    s.oroot[k] = (int32_t)((uint32_t)gr | ((uint32_t)coin << 31));
   }
 }
 
 // ---- roots, coins, flips, cluster sizes ---------------------------------------------
-__global__ void __launch_bounds__(SW_TPB, 6) k_sw_flip(SwScratch s) {
+// A site's coin as a root of its own is one bit of at most two Philox blocks per
+// row; the local roots of open components take their global root's coin
+// instead.  A run then flips as its local root's bit says: the coins of the run
+// starts are ballots, spread over the runs by word operations, one thread per
+// row.  Sizes are added once per run.
+__global__ void __launch_bounds__(SW_TPB, 8) k_sw_flip(SwScratch s) {
   __shared__ int cnt[SW_TS];
-  __shared__ uint8_t coin_s[SW_TS];
+  __shared__ uint32_t coin_s[SW_WORDS];               // per half row: coins of its sites as roots
+  __shared__ uint32_t flip_s[SW_WORDS];               // per half row: run starts that flip
+  __shared__ int32_t groot[SW_OPEN_PER_TILE];         // global roots of the open components
+  __shared__ u64 start_s[SW_TY];
+  __shared__ int nroot;
+  __shared__ uint32_t closed[3];
   if (__ldcg(s.status)) return;
   const SwDev &D = *s.dev;
   const int t = blockIdx.x, L = D.L;
   int x0, y0, w, h;
   sw_tile(D, t, x0, y0, w, h);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int nopen = s.onum[t];
+  const unsigned short *olocal = s.olocal + (int64_t)t * SW_OPEN_PER_TILE;
+  const int32_t *oroot = s.oroot + (int64_t)t * SW_OPEN_PER_TILE;
+  const uint32_t k0 = same_on_all((uint32_t)D.seed), k1 = same_on_all((uint32_t)(D.seed >> 32)),
+                 sweep = same_on_all(D.sweep);
+  const unsigned short *lroot = s.lroot + (int64_t)t * SW_TS;
   for (int l = threadIdx.x; l < SW_TS; l += SW_TPB) cnt[l] = 0;
+  if (threadIdx.x < SW_TY) start_s[threadIdx.x] = s.starts[(int64_t)t * SW_TY + threadIdx.x];
+  if (threadIdx.x == 0) nroot = 0;
+  if (threadIdx.x < 3) closed[threadIdx.x] = 0u;
   __syncthreads();
-  const uint32_t k0 = (uint32_t)D.seed, k1 = (uint32_t)(D.seed >> 32), sweep = D.sweep;
-  const uint32_t *lrw = s.lroot + (int64_t)t * SW_WORDS;
-  const float invL = 1.0f / (float)L;
-  int lr[SW_PER], gr[SW_PER];
-  uint32_t isroot = 0u;
+  // local roots of the thread's run starts (0xffff: no start)
+  unsigned short lr[SW_PER];
 #pragma unroll
   for (int k = 0; k < SW_PER; ++k) {
-    const int l = threadIdx.x + k * SW_TPB, lx = l & (SW_TX - 1), ly = l / SW_TX;
-    lr[k] = -1;
-    gr[k] = 0;
-    if (lx >= w || ly >= h) continue;
-    const int64_t g = (int64_t)(y0 + ly) * L + x0 + lx;
-    if ((lrw[l >> 5] >> (l & 31)) & 1u) {
-      isroot |= 1u << k;
-      lr[k] = l;
-      // path halving on the way and the root stored at the start: every
-      // entry still points to an ancestor, and only local roots' entries
-      // change (non-roots keep pointing at their local root)
-      gr[k] = uf_find(s.par, (int)g, s.status);
-      if (gr[k] != (int)g) s.par[g] = gr[k];
-      coin_s[l] = (uint8_t)coin_from(philox(TAG_SWFLIP << 24, (uint32_t)gr[k] >> 7, 0u, sweep, k0, k1),
-                                     (uint32_t)gr[k]);
-    } else {
-      const int p = __ldcg(s.par + g);  // the site's local root, in this tile
-      int py = __float2int_rz((float)p * invL), px = p - py * L;  // quotient within 1, corrected
-      if (px < 0) {
-        --py;
-        px += L;
-      } else if (px >= L) {
-        ++py;
-        px -= L;
-      }
-      if (py < y0 || py >= y0 + h || px < x0 || px >= x0 + w) {  // cannot happen: merges
-        atomicOr(s.status, ST_INTERNAL);                         // write local roots only
-        lr[k] = -1;
-        continue;
-      }
-      lr[k] = (py - y0) * SW_TX + (px - x0);
-    }
-    atomicAdd(&cnt[lr[k]], 1);
+    const int ly = 4 * k + (wid >> 1), lx = 32 * (wid & 1) + lane;
+    lr[k] = (start_s[ly] >> lx) & 1ull ? lroot[ly * SW_TX + lx] : (unsigned short)0xffff;
   }
-  __syncthreads();
-  long long v[2] = {0, 0};  // closed clusters, magnetization
-  long long mx = 0;
-  unsigned long long c2 = 0;
+  if (threadIdx.x < SW_WORDS) {
+    // half row: 32 sites from g on, in one or two blocks of 128 coins
+    const int ly = threadIdx.x >> 1, lx = 32 * (threadIdx.x & 1);
+    uint32_t c = 0u;
+    if (ly < h && lx < w) {
+      const uint32_t g = (uint32_t)site_of(x0, y0, L, ly * SW_TX + lx);
+      const U4 o = philox(TAG_SWFLIP << 24, g >> 7, 0u, sweep, k0, k1);
+      const int i = (g >> 5) & 3;
+      const uint32_t lo = i == 0 ? o.x : i == 1 ? o.y : i == 2 ? o.z : o.w;
+      uint32_t hi = i == 0 ? o.y : i == 1 ? o.z : o.w;
+      if (i == 3 && (g & 31u)) hi = philox(TAG_SWFLIP << 24, (g >> 7) + 1u, 0u, sweep, k0, k1).x;
+      c = __funnelshift_r(lo, hi, g & 31u);
+    }
+    coin_s[threadIdx.x] = c;
+  }
+  // sizes of the local components, a run at a time
 #pragma unroll
   for (int k = 0; k < SW_PER; ++k) {
-    if (lr[k] < 0) continue;
-    const int l = threadIdx.x + k * SW_TPB, lx = l & (SW_TX - 1), ly = l / SW_TX;
-    const int64_t g = (int64_t)(y0 + ly) * L + x0 + lx;
-    const uint8_t ns = (uint8_t)(s.spin[g] ^ coin_s[lr[k]]);
-    s.spin[g] = ns;
-    v[1] += ns ? -1 : 1;
-    if ((isroot >> k) & 1u) {
-      const int c = cnt[l];
-      if ((__ldcg(s.openb + (int64_t)t * SW_WORDS + (l >> 5)) >> (l & 31)) & 1u) {
-        atomicAdd(s.csize + gr[k], c);
-        if (gr[k] == (int)g) {  // the cluster's root: listed once
-          const int i = atomicAdd(s.ocount, 1);
-          if (i < SW_OPEN_PER_TILE * D.ntile)
-            s.olist[i] = gr[k];
-          else
-            atomicOr(s.status, ST_INTERNAL);
-        }
-      } else {
-        v[0] += 1;
-        c2 += (unsigned long long)c * (unsigned long long)c;
-        mx = max(mx, (long long)c);
+    const int ly = 4 * k + (wid >> 1), lx = 32 * (wid & 1) + lane;
+    if (lr[k] != 0xffff) atomicAdd(&cnt[lr[k]], __popcll(run_bits(start_s[ly], lx, w)));
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nopen; i += SW_TPB) {
+    const int l = olocal[i];
+    const uint32_t bit = 1u << (l & 31);
+    const int32_t r = oroot[i];
+    groot[i] = r & 0x7fffffff;
+    if (r < 0)
+      atomicOr(&coin_s[l >> 5], bit);
+    else
+      atomicAnd(&coin_s[l >> 5], ~bit);
+  }
+  __syncthreads();
+  // clusters closed in the tile: their number, sum of squares (at most 2^22) and
+  // largest, in 32 bits
+  uint32_t nc = 0, c2 = 0, mx = 0;
+  const uint32_t *openb = s.openb + (int64_t)t * SW_WORDS;
+#pragma unroll
+  for (int k = 0; k < SW_PER; ++k) {
+    const int ly = 4 * k + (wid >> 1), lx = 32 * (wid & 1) + lane, l = ly * SW_TX + lx;
+    bool f = false;
+    if (lr[k] != 0xffff) {
+      const int r = lr[k];
+      f = (coin_s[r >> 5] >> (r & 31)) & 1u;
+      if (r == l && !((openb[l >> 5] >> (l & 31)) & 1u)) {  // a cluster closed in the tile
+        const uint32_t c = (uint32_t)cnt[l];
+        nc += 1;
+        c2 += c * c;
+        mx = max(mx, c);
+      }
+    }
+    const uint32_t m = __ballot_sync(0xffffffffu, f);
+    if (lane == 0) flip_s[l >> 5] = m;
+  }
+  nc = __reduce_add_sync(0xffffffffu, nc);
+  c2 = __reduce_add_sync(0xffffffffu, c2);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0) {
+    atomicAdd(&closed[0], nc);
+    atomicAdd(&closed[1], c2);
+    atomicMax(&closed[2], mx);
+  }
+  // Open components of one cluster are added up in the tile first (about half of
+  // them belong to the largest cluster at K_c: an atomic for each took 0.35 ms).
+  for (int i = threadIdx.x; i < nopen; i += SW_TPB) {
+    const int32_t gr = groot[i];
+    int size = 0, lead = i;
+    bool root = false;
+    for (int j = 0; j < nopen; ++j)
+      if (groot[j] == gr) {
+        const int l = olocal[j];
+        lead = min(lead, j);
+        size += cnt[l];
+        root |= gr == site_of(x0, y0, L, l);
+      }
+    if (lead == i) {
+      atomicAdd(s.csize + gr, size);
+      if (root) {  // the cluster's root is in this tile: listed once
+        s.olist[(int64_t)t * SW_OPEN_PER_TILE + atomicAdd(&nroot, 1)] = gr;
       }
     }
   }
-  block_reduce<2>(v, mx, c2);
-  if (threadIdx.x == 0) {
-    s.tile_part[5 * (int64_t)t + 2] = v[0];
-    s.tile_part[5 * (int64_t)t + 3] = v[1];
-    s.tile_part[5 * (int64_t)t + 4] = mx;
-    s.tile_c2[t] = c2;
+  __syncthreads();
+  if (wid) return;
+  int mag = 0;
+  if (lane < h) {  // a thread per row: the starts' flips spread over their runs
+    u64 f = ((u64)flip_s[2 * lane + 1] << 32) | flip_s[2 * lane], go = ~start_s[lane] & low_bits(w);
+#pragma unroll
+    for (int o = 1; o < 64; o <<= 1) {
+      f |= go & (f << o);
+      go &= go << o;
+    }
+    u64 *row = s.spin + (int64_t)t * SW_TY + lane;
+    const u64 ns = *row ^ f;
+    *row = ns;
+    mag = w - 2 * __popcll(ns);
+  }
+  mag = __reduce_add_sync(0xffffffffu, mag);
+  if (lane == 0) {
+    s.rnum[t] = nroot;
+    s.tile_part[5 * (int64_t)t + 2] = closed[0];
+    s.tile_part[5 * (int64_t)t + 3] = mag;
+    s.tile_part[5 * (int64_t)t + 4] = closed[2];
+    s.tile_c2[t] = closed[1];
   }
 }
 
-// ---- open clusters: sizes squared and cleared -----------------------------------------
+// ---- open clusters: sizes squared and cleared; the tiles' sums -------------------------
 __global__ void __launch_bounds__(256) k_sw_sizes(SwScratch s) {
   if (__ldcg(s.status)) return;
-  const int n = __ldcg(s.ocount);
-  long long v[1] = {0};
+  const SwDev &D = *s.dev;
+  long long v[4] = {0, 0, 0, 0};  // n_eq, n_act, clusters, magnetization
   long long mx = 0;
   unsigned long long c2 = 0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const int r = __ldcg(s.olist + i);
-    const long long c = __ldcg(s.csize + r);
-    s.csize[r] = 0;
-    v[0] += 1;
-    c2 += (unsigned long long)c * (unsigned long long)c;
-    mx = max(mx, c);
+  const int lane = threadIdx.x & 31, nwarp = gridDim.x * (blockDim.x / 32);
+  for (int t = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); t < D.ntile; t += nwarp) {  // a warp per tile
+    const int n = s.rnum[t];
+    for (int i = lane; i < n; i += 32) {
+      const int r = s.olist[(int64_t)t * SW_OPEN_PER_TILE + i];
+      const long long c = atomicExch(s.csize + r, 0);
+      v[2] += 1;
+      c2 += (unsigned long long)c * (unsigned long long)c;
+      mx = max(mx, c);
+    }
   }
-  block_reduce<1>(v, mx, c2);
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < D.ntile; t += gridDim.x * blockDim.x) {
+    const long long *p = s.tile_part + 5 * (int64_t)t;
+    v[0] += p[0];
+    v[1] += p[1];
+    v[2] += p[2];
+    v[3] += p[3];
+    mx = max(mx, p[4]);
+    c2 += s.tile_c2[t];
+  }
+  block_reduce<4>(v, mx, c2);
   if (threadIdx.x == 0) {
-    s.size_part[2 * blockIdx.x] = v[0];
-    s.size_part[2 * blockIdx.x + 1] = mx;
+    long long *p = s.size_part + 5 * (int64_t)blockIdx.x;
+    p[0] = v[0];
+    p[1] = v[1];
+    p[2] = v[2];
+    p[3] = v[3];
+    p[4] = mx;
     s.size_c2[blockIdx.x] = c2;
   }
 }
@@ -445,18 +670,13 @@ __global__ void __launch_bounds__(1024) k_sw_final(SwScratch s, int nsize) {
   long long v[4] = {0, 0, 0, 0};  // n_eq, n_act, clusters, magnetization
   long long mx = 0;
   unsigned long long c2 = 0;
-  for (int t = threadIdx.x; t < D.ntile; t += blockDim.x) {
-    const long long *p = s.tile_part + 5 * (int64_t)t;
+  for (int b = threadIdx.x; b < nsize; b += blockDim.x) {
+    const long long *p = s.size_part + 5 * (int64_t)b;
     v[0] += p[0];
     v[1] += p[1];
     v[2] += p[2];
     v[3] += p[3];
     mx = max(mx, p[4]);
-    c2 += s.tile_c2[t];
-  }
-  for (int b = threadIdx.x; b < nsize; b += blockDim.x) {
-    v[2] += s.size_part[2 * b];
-    mx = max(mx, s.size_part[2 * b + 1]);
     c2 += s.size_c2[b];
   }
   block_reduce<4>(v, mx, c2);
@@ -481,15 +701,55 @@ __global__ void __launch_bounds__(1024) k_sw_final(SwScratch s, int nsize) {
     }
     D.n_updates += 1;
     D.sweep += 1u;
-    *s.ocount = 0;
   }
+}
+
+// Tile and tile-local index of site g.
+__device__ __forceinline__ void tile_site(const SwDev &D, int64_t g, int &t, int &x, int &y) {
+  const int gy = (int)(g / D.L), gx = (int)(g - (int64_t)gy * D.L);
+  t = (gy / SW_TY) * D.ntx + gx / SW_TX;
+  x = gx % SW_TX;
+  y = gy % SW_TY;
 }
 
 __global__ void k_sw_roots(SwScratch s) {
   if (__ldcg(s.status)) return;
   const SwDev &D = *s.dev;
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < D.N; g += (int64_t)gridDim.x * blockDim.x)
-    s.roots[g] = uf_root(s.par, (int)g, s.status);
+  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < D.N; g += (int64_t)gridDim.x * blockDim.x) {
+    int t, x, y, x0, y0, w, h;
+    tile_site(D, g, t, x, y);
+    sw_tile(D, t, x0, y0, w, h);
+    const int l = s.lroot[(int64_t)t * SW_TS + y * SW_TX + run_start(s.starts[(int64_t)t * SW_TY + y], x)];
+    const int32_t r = site_of(x0, y0, D.L, l);
+    const bool open = (s.openb[(int64_t)t * SW_WORDS + (l >> 5)] >> (l & 31)) & 1u;
+    s.roots[g] = open ? uf_root(s.par, r, s.status) : r;
+  }
+}
+
+// Spins between bytes (row-major) and tile rows, a thread per tile row.
+__global__ void k_sw_pack(SwScratch s) {
+  const SwDev &D = *s.dev;
+  const int64_t n = (int64_t)D.ntile * SW_TY;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    int x0, y0, w, h;
+    sw_tile(D, (int)(i / SW_TY), x0, y0, w, h);
+    const int y = (int)(i % SW_TY);
+    u64 row = 0;
+    if (y < h) {
+      const uint8_t *p = s.bytes + (int64_t)(y0 + y) * D.L + x0;
+      for (int x = 0; x < w; ++x) row |= (u64)(p[x] & 1) << x;
+    }
+    s.spin[i] = row;
+  }
+}
+
+__global__ void k_sw_unpack(SwScratch s) {
+  const SwDev &D = *s.dev;
+  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < D.N; g += (int64_t)gridDim.x * blockDim.x) {
+    int t, x, y;
+    tile_site(D, g, t, x, y);
+    s.bytes[g] = (uint8_t)((s.spin[(int64_t)t * SW_TY + y] >> x) & 1ull);
+  }
 }
 
 #define SWCK(call)                                                                   \
@@ -542,25 +802,29 @@ class SwEngine {
     int rc = 0;
     rc |= dalloc((void **)&s_.dev, sizeof(SwDev));
     rc |= dalloc((void **)&s_.status, sizeof(int));
-    rc |= dalloc((void **)&s_.spin, (size_t)N);
+    rc |= dalloc((void **)&s_.bytes, (size_t)N);
+    rc |= dalloc((void **)&s_.spin, 8 * (size_t)nt * SW_TY);
+    rc |= dalloc((void **)&s_.starts, 8 * (size_t)nt * SW_TY);
+    rc |= dalloc((void **)&s_.lroot, 2 * (size_t)nt * SW_TS);
     rc |= dalloc((void **)&s_.par, 4 * (size_t)N);
-    rc |= dalloc((void **)&s_.lroot, 4 * (size_t)nt * SW_WORDS);
     rc |= dalloc((void **)&s_.openb, 4 * (size_t)nt * SW_WORDS);
     rc |= dalloc((void **)&s_.edge_r, 4 * (size_t)nt);
     rc |= dalloc((void **)&s_.edge_d, 8 * (size_t)nt);
+    rc |= dalloc((void **)&s_.olocal, 2 * (size_t)nt * SW_OPEN_PER_TILE);
+    rc |= dalloc((void **)&s_.oroot, 4 * (size_t)nt * SW_OPEN_PER_TILE);
+    rc |= dalloc((void **)&s_.onum, 4 * (size_t)nt);
     rc |= dalloc((void **)&s_.csize, 4 * (size_t)N);
     rc |= dalloc((void **)&s_.olist, 4 * (size_t)nt * SW_OPEN_PER_TILE);
-    rc |= dalloc((void **)&s_.ocount, sizeof(int));
+    rc |= dalloc((void **)&s_.rnum, 4 * (size_t)nt);
     rc |= dalloc((void **)&s_.tile_part, 5 * 8 * (size_t)nt);
     rc |= dalloc((void **)&s_.tile_c2, 8 * (size_t)nt);
-    rc |= dalloc((void **)&s_.size_part, 2 * 8 * (size_t)SW_SIZE_BLOCKS);
+    rc |= dalloc((void **)&s_.size_part, 5 * 8 * (size_t)SW_SIZE_BLOCKS);
     rc |= dalloc((void **)&s_.size_c2, 8 * (size_t)SW_SIZE_BLOCKS);
     rc |= dalloc((void **)&s_.ring, sizeof(lcqmc_sw_record) * SW_RING);
     if (rc) return LCQMC_E_NOMEM;
     SWCK(cudaMemsetAsync(s_.status, 0, sizeof(int), st_));
-    SWCK(cudaMemsetAsync(s_.spin, 0, (size_t)N, st_));  // ordered start: every sigma = +1
+    SWCK(cudaMemsetAsync(s_.spin, 0, 8 * (size_t)nt * SW_TY, st_));  // ordered start: every sigma = +1
     SWCK(cudaMemsetAsync(s_.csize, 0, 4 * (size_t)N, st_));
-    SWCK(cudaMemsetAsync(s_.ocount, 0, sizeof(int), st_));
     SWCK(cudaMemcpyAsync(s_.dev, &h_, sizeof(SwDev), cudaMemcpyHostToDevice, st_));
     for (int i = 0; i <= 4; ++i) SWCK(cudaEventCreate(&ev_[i]));
     SWCK(cudaStreamSynchronize(st_));
@@ -665,7 +929,10 @@ class SwEngine {
       }
     int rc = sync();
     if (rc) return rc;
-    SWCK(cudaMemcpy(s_.spin, spins, (size_t)h_.N, cudaMemcpyHostToDevice));
+    SWCK(cudaMemcpy(s_.bytes, spins, (size_t)h_.N, cudaMemcpyHostToDevice));
+    k_sw_pack<<<(int)std::min<int64_t>(((int64_t)h_.ntile * SW_TY + 255) / 256, 4096), 256, 0, st_>>>(s_);
+    SWCK(cudaGetLastError());
+    SWCK(cudaStreamSynchronize(st_));
     SWCK(cudaMemcpy((char *)s_.dev + offsetof(SwDev, sweep), &sweep, sizeof(uint32_t),
                     cudaMemcpyHostToDevice));
     return LCQMC_OK;
@@ -678,7 +945,10 @@ class SwEngine {
     }
     int rc = sync();
     if (rc) return rc;
-    SWCK(cudaMemcpy(spins, s_.spin, (size_t)h_.N, cudaMemcpyDeviceToHost));
+    k_sw_unpack<<<(int)std::min<int64_t>((h_.N + 255) / 256, 152 * 64), 256, 0, st_>>>(s_);
+    SWCK(cudaGetLastError());
+    SWCK(cudaMemcpyAsync(spins, s_.bytes, (size_t)h_.N, cudaMemcpyDeviceToHost, st_));
+    SWCK(cudaStreamSynchronize(st_));
     return LCQMC_OK;
   }
 
@@ -768,12 +1038,13 @@ class SwEngine {
     }
     auto mark = [&](int k) -> cudaError_t { return timed ? cudaEventRecord(ev_[k], st_) : cudaSuccess; };
     const int nt = h_.ntile;
-    const int nsize = (int)std::min<int64_t>(SW_SIZE_BLOCKS, ((int64_t)nt * SW_OPEN_PER_TILE + 255) / 256);
+    const int nsize = (int)std::min<int64_t>(SW_SIZE_BLOCKS, ((int64_t)nt + 7) / 8);
     SWCK(mark(0));  // [0] bond draws, tile union-find
     k_sw_local<<<nt, SW_TPB, 0, st_>>>(s_);
     SWCK(mark(1));  // [1] tile-boundary bonds, global union-find
     k_sw_merge<<<(nt * 32 + 255) / 256, 256, 0, st_>>>(s_);
     SWCK(mark(2));  // [2] roots, coins, flips
+    k_sw_find<<<(nt * 32 + 255) / 256, 256, 0, st_>>>(s_);
     k_sw_flip<<<nt, SW_TPB, 0, st_>>>(s_);
     SWCK(mark(3));  // [3] open clusters' sizes, record
     k_sw_sizes<<<nsize, 256, 0, st_>>>(s_);
