@@ -620,15 +620,16 @@ SW_TILE = (64, 32)
 
 def sw_phase_bytes(L):
     """Algorithmic bytes of each phase of one update (every datum read or
-    written once): spins and the local-root word per site, the tile bitmaps,
-    edge masks and partial sums per tile, the open-root bitmap per 32 sites."""
+    written once): a spin bit and a run-start bit per site, two bytes of local
+    root per run start (about half of the sites at K_c), per tile the
+    open-component bitmap and list, edge masks and partial sums."""
     N = L * L
     nt = -(-L // SW_TILE[0]) * -(-L // SW_TILE[1])
-    tile_bits = 2 * 64 * 4  # local-root and open-component bitmaps
-    return {"tile_bonds_uf": N * (1 + 4) + nt * (tile_bits + 4 + 8 + 16),
+    bits, roots, opens = N // 8, N, nt * (64 * 4 + 50 * 2)
+    return {"tile_bonds_uf": 2 * bits + roots + opens + nt * (4 + 8 + 16),
             "boundary_merge": nt * (4 + 8),
-            "roots_flip": N * (4 + 1 + 1) + nt * (tile_bits + 24),
-            "open_sizes_record": (N // 32 + 1) * 4 + nt * 48}
+            "roots_flip": 3 * bits + roots + opens + nt * (50 * 8 + 24),
+            "open_sizes_record": nt * (48 + 30 * 8)}
 
 
 def sw_oracle_sample(steps=5, warmup=2, L=SW_ORACLE_L):

@@ -27,8 +27,8 @@
 //   k_sw_flip   one coin per local root, spins flipped; sizes of clusters
 //               closed in the tile squared here, sizes of open ones added at
 //               their global root
-//   k_sw_sizes  open clusters' sizes squared, cleared for the next update
-//   k_sw_final  the update's record and running sums
+//   k_sw_sizes  open clusters' sizes squared, cleared for the next update; the
+//               update's record and running sums
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -49,8 +49,11 @@ namespace lcq {
 namespace {
 
 constexpr int SW_TX = 64, SW_TY = 32, SW_TS = SW_TX * SW_TY;  // tile of 64 x 32 sites
-constexpr int SW_TPB = 256;
-constexpr int SW_PER = SW_TS / SW_TPB;  // sites per thread
+// Threads of a tile's block: SW_TPB, or SW_TPB_WIDE for lattices of up to two
+// tiles per SM, whose update lasts as long as one tile's steps (us per update,
+// 256 / 1024 threads: L=48 29 / 24, L=333 43 / 34, L=700, 242 tiles, 48 / 43,
+// L=800, 325 tiles, 50 / 52, L=1500 75 / 90).
+constexpr int SW_TPB = 256, SW_TPB_WIDE = 1024, SW_WIDE_TILES = 152 * 2;
 constexpr int SW_WORDS = SW_TS / 32;    // bitmap words per tile
 constexpr int SW_SIZE_BLOCKS = 1216;    // blocks of the open-cluster pass: 8 per SM
 // An open cluster's root is the smallest site of a tile component that holds
@@ -95,6 +98,7 @@ struct SwScratch {
   // clusters, mag, largest
   long long *size_part;
   unsigned long long *size_c2;  // per block of k_sw_sizes: sum of size^2
+  unsigned *done;               // blocks of k_sw_sizes done; 0 between updates
   lcqmc_sw_record *ring;
   int32_t *roots;               // lcqmc_sw_get_roots output (N), allocated on demand
 };
@@ -257,7 +261,9 @@ __device__ __forceinline__ uint32_t same_on_all(uint32_t x) { return __reduce_ma
 //
 // Bound by instruction issue: the draws are about a quarter of it, the unions
 // the larger part of the rest.
-__global__ void __launch_bounds__(SW_TPB, 8) k_sw_local(SwScratch s) {
+template <int NT>
+__global__ void __launch_bounds__(NT, 2048 / NT) k_sw_local(SwScratch s) {
+  constexpr int PER = SW_TS / NT, ROWS = NT / SW_TX;  // sites per thread, rows per step
   __shared__ int lp[SW_TS];               // forest of the run starts
   __shared__ unsigned short vlist[SW_TS]; // upper ends of the down bonds to unite
   __shared__ uint32_t drawR[SW_WORDS], drawD[SW_WORDS];  // draws below T, per half row
@@ -284,8 +290,8 @@ __global__ void __launch_bounds__(SW_TPB, 8) k_sw_local(SwScratch s) {
     const int lx = 32 * (wid & 1) + lane;
     const uint32_t g0 = (uint32_t)((int64_t)y0 * L + x0 + lx);
 #pragma unroll 2
-    for (int k = 0; k < SW_PER; ++k) {
-      const int ly = 4 * k + (wid >> 1), l = ly * SW_TX + lx;
+    for (int k = 0; k < PER; ++k) {
+      const int ly = ROWS * k + (wid >> 1), l = ly * SW_TX + lx;
       uint32_t x, y;
       draw(g0 + (uint32_t)ly * (uint32_t)L, x, y);
       const bool in = some && lx < w && ly < h;
@@ -371,19 +377,19 @@ __global__ void __launch_bounds__(SW_TPB, 8) k_sw_local(SwScratch s) {
   }
   __syncthreads();
   // the open sites' runs, a thread per row
-  if (wid == 7) {
+  if (wid == NT / 32 - 1) {
     const u64 open = ((u64)open_s[2 * lane + 1] << 32) | open_s[2 * lane];
     open_run[lane] = runs_with(start_s[lane], open);
   }
 #pragma unroll
-  for (int k = 0; k < SW_PER; ++k) {
-    const int ly = 4 * k + (wid >> 1), lx = 32 * (wid & 1) + lane;
+  for (int k = 0; k < PER; ++k) {
+    const int ly = ROWS * k + (wid >> 1), lx = 32 * (wid & 1) + lane;
     const u64 v = vert_s[ly];
     if ((v >> lx) & 1ull)
       vlist[vbase[ly] + __popcll(v & low_bits(lx))] = (unsigned short)(ly * SW_TX + lx);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < nvert; i += SW_TPB) {
+  for (int i = threadIdx.x; i < nvert; i += NT) {
     const int l = vlist[i], lx = l & (SW_TX - 1), ly = l / SW_TX;
     sw_union(lp, ly * SW_TX + run_start(start_s[ly], lx), (ly + 1) * SW_TX + run_start(start_s[ly + 1], lx),
              s.status);
@@ -391,8 +397,8 @@ __global__ void __launch_bounds__(SW_TPB, 8) k_sw_local(SwScratch s) {
   __syncthreads();
   // every run's local root (read-only walks: no union is running any more)
 #pragma unroll 2
-  for (int k = 0; k < SW_PER; ++k) {
-    const int ly = 4 * k + (wid >> 1), lx = 32 * (wid & 1) + lane, l = ly * SW_TX + lx;
+  for (int k = 0; k < PER; ++k) {
+    const int ly = ROWS * k + (wid >> 1), lx = 32 * (wid & 1) + lane, l = ly * SW_TX + lx;
     const u64 st = start_s[ly];
     if ((st >> lx) & 1ull) {
       int r = lp[l];
@@ -427,31 +433,39 @@ __device__ __forceinline__ int32_t local_root(const SwScratch &s, const SwDev &D
   return site_of(x0, y0, D.L, s.lroot[(int64_t)t * SW_TS + l]);
 }
 
-__global__ void __launch_bounds__(256) k_sw_merge(SwScratch s) {
+// One thread per edge bond.  Up to SW_WALK_TILES tiles every thread walks once
+// more after its union: the time there is the longest chain of dependent
+// accesses, and all threads' walks halve the same paths for the waiting unions
+// and for k_sw_find (update, us, without / with: L=333 48 / 43, L=1500, 1128
+// tiles, 91 / 75, L=3000, 4418 tiles, 178 / 177, L=8192 977 / 1005).
+constexpr int SW_WALK_TILES = 2048;
+constexpr int SW_EDGE = SW_TX + SW_TY;
+
+__global__ void __launch_bounds__(SW_EDGE) k_sw_merge(SwScratch s) {
   if (__ldcg(s.status)) return;
   const SwDev &D = *s.dev;
-  const int t = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (t >= D.ntile) return;
+  const int t = blockIdx.x, j = threadIdx.x;
   int x0, y0, w, h;
   sw_tile(D, t, x0, y0, w, h);
   const uint32_t er = s.edge_r[t];
   const u64 ed = s.edge_d[t];
   const int tx = t % D.ntx, ty = t / D.ntx;
   const int right = ty * D.ntx + (tx + 1 < D.ntx ? tx + 1 : 0), down = (ty + 1 < D.nty ? ty + 1 : 0) * D.ntx + tx;
-  for (int j = lane; j < SW_TY + SW_TX; j += 32) {
-    int32_t a, b;
-    if (j < SW_TY) {
-      if (!((er >> j) & 1u)) continue;
-      a = local_root(s, D, t, w - 1, j);
-      b = local_root(s, D, right, 0, j);
-    } else {
-      const int c = j - SW_TY;
-      if (!((ed >> c) & 1ull)) continue;
-      a = local_root(s, D, t, c, h - 1);
-      b = local_root(s, D, down, c, 0);
-    }
-    uf_union(s.par, a, b, s.status);
+  int32_t a, b;
+  if (j < SW_TY) {
+    if (!((er >> j) & 1u)) return;
+    a = local_root(s, D, t, w - 1, j);
+    b = local_root(s, D, right, 0, j);
+  } else {
+    const int c = j - SW_TY;
+    if (!((ed >> c) & 1ull)) return;
+    a = local_root(s, D, t, c, h - 1);
+    b = local_root(s, D, down, c, 0);
   }
+  uf_union(s.par, a, b, s.status);
+  if (D.ntile > SW_WALK_TILES) return;
+  const int r = uf_find(s.par, a, s.status);
+  if (r != a) s.par[a] = r;
 }
 
 // ---- global roots of the open components --------------------------------------------
@@ -485,7 +499,9 @@ __global__ void __launch_bounds__(256) k_sw_find(SwScratch s) {
 // instead.  A run then flips as its local root's bit says: the coins of the run
 // starts are ballots, spread over the runs by word operations, one thread per
 // row.  Sizes are added once per run.
-__global__ void __launch_bounds__(SW_TPB, 8) k_sw_flip(SwScratch s) {
+template <int NT>
+__global__ void __launch_bounds__(NT, 2048 / NT) k_sw_flip(SwScratch s) {
+  constexpr int PER = SW_TS / NT, ROWS = NT / SW_TX;  // sites per thread, rows per step
   __shared__ int cnt[SW_TS];
   __shared__ uint32_t coin_s[SW_WORDS];               // per half row: coins of its sites as roots
   __shared__ uint32_t flip_s[SW_WORDS];               // per half row: run starts that flip
@@ -505,16 +521,16 @@ __global__ void __launch_bounds__(SW_TPB, 8) k_sw_flip(SwScratch s) {
   const uint32_t k0 = same_on_all((uint32_t)D.seed), k1 = same_on_all((uint32_t)(D.seed >> 32)),
                  sweep = same_on_all(D.sweep);
   const unsigned short *lroot = s.lroot + (int64_t)t * SW_TS;
-  for (int l = threadIdx.x; l < SW_TS; l += SW_TPB) cnt[l] = 0;
+  for (int l = threadIdx.x; l < SW_TS; l += NT) cnt[l] = 0;
   if (threadIdx.x < SW_TY) start_s[threadIdx.x] = s.starts[(int64_t)t * SW_TY + threadIdx.x];
   if (threadIdx.x == 0) nroot = 0;
   if (threadIdx.x < 3) closed[threadIdx.x] = 0u;
   __syncthreads();
   // local roots of the thread's run starts (0xffff: no start)
-  unsigned short lr[SW_PER];
+  unsigned short lr[PER];
 #pragma unroll
-  for (int k = 0; k < SW_PER; ++k) {
-    const int ly = 4 * k + (wid >> 1), lx = 32 * (wid & 1) + lane;
+  for (int k = 0; k < PER; ++k) {
+    const int ly = ROWS * k + (wid >> 1), lx = 32 * (wid & 1) + lane;
     lr[k] = (start_s[ly] >> lx) & 1ull ? lroot[ly * SW_TX + lx] : (unsigned short)0xffff;
   }
   if (threadIdx.x < SW_WORDS) {
@@ -534,12 +550,12 @@ __global__ void __launch_bounds__(SW_TPB, 8) k_sw_flip(SwScratch s) {
   }
   // sizes of the local components, a run at a time
 #pragma unroll
-  for (int k = 0; k < SW_PER; ++k) {
-    const int ly = 4 * k + (wid >> 1), lx = 32 * (wid & 1) + lane;
+  for (int k = 0; k < PER; ++k) {
+    const int ly = ROWS * k + (wid >> 1), lx = 32 * (wid & 1) + lane;
     if (lr[k] != 0xffff) atomicAdd(&cnt[lr[k]], __popcll(run_bits(start_s[ly], lx, w)));
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < nopen; i += SW_TPB) {
+  for (int i = threadIdx.x; i < nopen; i += NT) {
     const int l = olocal[i];
     const uint32_t bit = 1u << (l & 31);
     const int32_t r = oroot[i];
@@ -555,8 +571,8 @@ __global__ void __launch_bounds__(SW_TPB, 8) k_sw_flip(SwScratch s) {
   uint32_t nc = 0, c2 = 0, mx = 0;
   const uint32_t *openb = s.openb + (int64_t)t * SW_WORDS;
 #pragma unroll
-  for (int k = 0; k < SW_PER; ++k) {
-    const int ly = 4 * k + (wid >> 1), lx = 32 * (wid & 1) + lane, l = ly * SW_TX + lx;
+  for (int k = 0; k < PER; ++k) {
+    const int ly = ROWS * k + (wid >> 1), lx = 32 * (wid & 1) + lane, l = ly * SW_TX + lx;
     bool f = false;
     if (lr[k] != 0xffff) {
       const int r = lr[k];
@@ -581,7 +597,7 @@ __global__ void __launch_bounds__(SW_TPB, 8) k_sw_flip(SwScratch s) {
   }
   // Open components of one cluster are added up in the tile first (about half of
   // them belong to the largest cluster at K_c: an atomic for each took 0.35 ms).
-  for (int i = threadIdx.x; i < nopen; i += SW_TPB) {
+  for (int i = threadIdx.x; i < nopen; i += NT) {
     const int32_t gr = groot[i];
     int size = 0, lead = i;
     bool root = false;
@@ -624,10 +640,14 @@ __global__ void __launch_bounds__(SW_TPB, 8) k_sw_flip(SwScratch s) {
   }
 }
 
-// ---- open clusters: sizes squared and cleared; the tiles' sums -------------------------
+// ---- open clusters: sizes squared and cleared; the tiles' sums; the record --------------
+// A size is taken and cleared by one exchange (a load followed by a store to the
+// same word waits for the load at L2: 0.2 ms).  The block that finishes last
+// adds up the blocks' sums and writes the record, its fp64 values one per lane.
 __global__ void __launch_bounds__(256) k_sw_sizes(SwScratch s) {
+  __shared__ int last;
   if (__ldcg(s.status)) return;
-  const SwDev &D = *s.dev;
+  SwDev &D = *s.dev;
   long long v[4] = {0, 0, 0, 0};  // n_eq, n_act, clusters, magnetization
   long long mx = 0;
   unsigned long long c2 = 0;
@@ -652,37 +672,53 @@ __global__ void __launch_bounds__(256) k_sw_sizes(SwScratch s) {
     c2 += s.tile_c2[t];
   }
   block_reduce<4>(v, mx, c2);
-  if (threadIdx.x == 0) {
-    long long *p = s.size_part + 5 * (int64_t)blockIdx.x;
-    p[0] = v[0];
-    p[1] = v[1];
-    p[2] = v[2];
-    p[3] = v[3];
-    p[4] = mx;
-    s.size_c2[blockIdx.x] = c2;
+  if (gridDim.x > 1) {
+    if (threadIdx.x == 0) {
+      long long *p = s.size_part + 5 * (int64_t)blockIdx.x;
+      p[0] = v[0];
+      p[1] = v[1];
+      p[2] = v[2];
+      p[3] = v[3];
+      p[4] = mx;
+      s.size_c2[blockIdx.x] = c2;
+      __threadfence();
+      last = atomicAdd(s.done, 1u) == gridDim.x - 1;
+      __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    v[0] = v[1] = v[2] = v[3] = mx = 0;
+    c2 = 0;
+    for (int b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
+      const long long *p = s.size_part + 5 * (int64_t)b;
+      v[0] += __ldcg(p);
+      v[1] += __ldcg(p + 1);
+      v[2] += __ldcg(p + 2);
+      v[3] += __ldcg(p + 3);
+      mx = max(mx, __ldcg(p + 4));
+      c2 += __ldcg(s.size_c2 + b);
+    }
+    block_reduce<4>(v, mx, c2);
   }
-}
-
-// ---- record --------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_sw_final(SwScratch s, int nsize) {
-  if (__ldcg(s.status)) return;
-  SwDev &D = *s.dev;
-  long long v[4] = {0, 0, 0, 0};  // n_eq, n_act, clusters, magnetization
-  long long mx = 0;
-  unsigned long long c2 = 0;
-  for (int b = threadIdx.x; b < nsize; b += blockDim.x) {
-    const long long *p = s.size_part + 5 * (int64_t)b;
-    v[0] += p[0];
-    v[1] += p[1];
-    v[2] += p[2];
-    v[3] += p[3];
-    mx = max(mx, p[4]);
-    c2 += s.size_c2[b];
+  if (threadIdx.x >= 32) return;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) v[k] = __shfl_sync(0xffffffffu, v[k], 0);
+  c2 = __shfl_sync(0xffffffffu, c2, 0);
+  const int64_t N = D.N;
+  // lane 0: energy = -(1/N) sum_bonds sigma sigma; 1: chi = sum_c |c|^2 / N;
+  // 2: M^2 / N; 3: |M| / N
+  const double m = (double)v[3];
+  const double num = lane == 0 ? (double)(2 * N - 2 * v[0]) : lane == 1 ? (double)c2 : lane == 2 ? m * m : fabs(m);
+  const double x = num / (double)N;
+  lcqmc_sw_record &r = s.ring[D.n_updates % D.ring_cap];
+  if (lane < LCQMC_SW_NOBS) {
+    D.sum[lane] += x;
+    D.sumsq[lane] += x * x;
   }
-  block_reduce<4>(v, mx, c2);
-  if (threadIdx.x == 0) {
-    const int64_t N = D.N;
-    lcqmc_sw_record r;
+  if (lane == 0) r.energy = x;
+  if (lane == 1) r.chi = x;
+  __syncwarp();
+  if (lane == 0) {
     r.sweep = D.sweep;
     r.n_eq = v[0];
     r.n_act = v[1];
@@ -690,17 +726,9 @@ __global__ void __launch_bounds__(1024) k_sw_final(SwScratch s, int nsize) {
     r.max_cluster = mx;
     r.sum_c2 = c2;
     r.mag = v[3];
-    r.energy = (double)(2 * N - 2 * v[0]) / (double)N;  // -(1/N) sum_bonds sigma sigma
-    r.chi = (double)c2 / (double)N;                      // sum_c |c|^2 / N
-    s.ring[D.n_updates % D.ring_cap] = r;
-    const double m = (double)v[3];
-    const double x[LCQMC_SW_NOBS] = {r.energy, r.chi, m * m / (double)N, fabs(m) / (double)N};
-    for (int k = 0; k < LCQMC_SW_NOBS; ++k) {
-      D.sum[k] += x[k];
-      D.sumsq[k] += x[k] * x[k];
-    }
     D.n_updates += 1;
     D.sweep += 1u;
+    *s.done = 0u;
   }
 }
 
@@ -726,30 +754,32 @@ __global__ void k_sw_roots(SwScratch s) {
   }
 }
 
-// Spins between bytes (row-major) and tile rows, a thread per tile row.
+// Spins between bytes (row-major) and tile rows, a warp per tile row.
 __global__ void k_sw_pack(SwScratch s) {
   const SwDev &D = *s.dev;
-  const int64_t n = (int64_t)D.ntile * SW_TY;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    int x0, y0, w, h;
-    sw_tile(D, (int)(i / SW_TY), x0, y0, w, h);
-    const int y = (int)(i % SW_TY);
-    u64 row = 0;
-    if (y < h) {
-      const uint8_t *p = s.bytes + (int64_t)(y0 + y) * D.L + x0;
-      for (int x = 0; x < w; ++x) row |= (u64)(p[x] & 1) << x;
-    }
-    s.spin[i] = row;
-  }
+  const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (i >= (int64_t)D.ntile * SW_TY) return;
+  int x0, y0, w, h;
+  sw_tile(D, (int)(i / SW_TY), x0, y0, w, h);
+  const int y = (int)(i % SW_TY), lane = threadIdx.x & 31;
+  const uint8_t *p = s.bytes + (int64_t)(y0 + y) * D.L + x0;
+  const uint32_t lo = __ballot_sync(0xffffffffu, y < h && lane < w && (p[lane] & 1));
+  const uint32_t hi = __ballot_sync(0xffffffffu, y < h && lane + 32 < w && (p[lane + 32] & 1));
+  if (lane == 0) s.spin[i] = ((u64)hi << 32) | lo;
 }
 
 __global__ void k_sw_unpack(SwScratch s) {
   const SwDev &D = *s.dev;
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < D.N; g += (int64_t)gridDim.x * blockDim.x) {
-    int t, x, y;
-    tile_site(D, g, t, x, y);
-    s.bytes[g] = (uint8_t)((s.spin[(int64_t)t * SW_TY + y] >> x) & 1ull);
-  }
+  const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (i >= (int64_t)D.ntile * SW_TY) return;
+  int x0, y0, w, h;
+  sw_tile(D, (int)(i / SW_TY), x0, y0, w, h);
+  const int y = (int)(i % SW_TY), lane = threadIdx.x & 31;
+  if (y >= h) return;
+  uint8_t *p = s.bytes + (int64_t)(y0 + y) * D.L + x0;
+  const u64 row = s.spin[i];
+  if (lane < w) p[lane] = (uint8_t)((row >> lane) & 1ull);
+  if (lane + 32 < w) p[lane + 32] = (uint8_t)((row >> (lane + 32)) & 1ull);
 }
 
 #define SWCK(call)                                                                   \
@@ -820,9 +850,11 @@ class SwEngine {
     rc |= dalloc((void **)&s_.tile_c2, 8 * (size_t)nt);
     rc |= dalloc((void **)&s_.size_part, 5 * 8 * (size_t)SW_SIZE_BLOCKS);
     rc |= dalloc((void **)&s_.size_c2, 8 * (size_t)SW_SIZE_BLOCKS);
+    rc |= dalloc((void **)&s_.done, sizeof(unsigned));
     rc |= dalloc((void **)&s_.ring, sizeof(lcqmc_sw_record) * SW_RING);
     if (rc) return LCQMC_E_NOMEM;
     SWCK(cudaMemsetAsync(s_.status, 0, sizeof(int), st_));
+    SWCK(cudaMemsetAsync(s_.done, 0, sizeof(unsigned), st_));
     SWCK(cudaMemsetAsync(s_.spin, 0, 8 * (size_t)nt * SW_TY, st_));  // ordered start: every sigma = +1
     SWCK(cudaMemsetAsync(s_.csize, 0, 4 * (size_t)N, st_));
     SWCK(cudaMemcpyAsync(s_.dev, &h_, sizeof(SwDev), cudaMemcpyHostToDevice, st_));
@@ -843,26 +875,26 @@ class SwEngine {
   }
 
   int update_n(int64_t n) {
-    for (int64_t i = 0; i < n; ++i) {
-      if (timing_) {
+    if (timing_) {
+      for (int64_t i = 0; i < n; ++i) {
         int rc = enqueue(true);
         if (rc) return rc;
-      } else {
-        if (!gexec_) {
-          cudaGraph_t g;
-          SWCK(cudaStreamBeginCapture(st_, cudaStreamCaptureModeThreadLocal));
-          int rc = enqueue(false);
-          cudaGraph_t gg = nullptr;
-          cudaError_t e = cudaStreamEndCapture(st_, &gg);
-          if (rc) return rc;
-          SWCK(e);
-          g = gg;
-          e = cudaGraphInstantiate(&gexec_, g, 0);
-          cudaGraphDestroy(g);
-          SWCK(e);
-        }
-        SWCK(cudaGraphLaunch(gexec_, st_));
+        ++enq_;
       }
+      return LCQMC_OK;
+    }
+    // graphs of kGraphBlock updates, then of one (a launch per update left gaps
+    // between the few microseconds of a small lattice's updates)
+    const int64_t nblk = n / kGraphBlock, rest = n % kGraphBlock;
+    int rc = nblk ? capture(kGraphBlock, &gexec_blk_) : LCQMC_OK;
+    if (!rc && rest) rc = capture(1, &gexec_);
+    if (rc) return rc;
+    for (int64_t i = 0; i < nblk; ++i) {
+      SWCK(cudaGraphLaunch(gexec_blk_, st_));
+      enq_ += kGraphBlock;
+    }
+    for (int64_t i = 0; i < rest; ++i) {
+      SWCK(cudaGraphLaunch(gexec_, st_));
       ++enq_;
     }
     return LCQMC_OK;
@@ -930,7 +962,7 @@ class SwEngine {
     int rc = sync();
     if (rc) return rc;
     SWCK(cudaMemcpy(s_.bytes, spins, (size_t)h_.N, cudaMemcpyHostToDevice));
-    k_sw_pack<<<(int)std::min<int64_t>(((int64_t)h_.ntile * SW_TY + 255) / 256, 4096), 256, 0, st_>>>(s_);
+    k_sw_pack<<<h_.ntile * SW_TY / 8, 256, 0, st_>>>(s_);  // a warp per tile row
     SWCK(cudaGetLastError());
     SWCK(cudaStreamSynchronize(st_));
     SWCK(cudaMemcpy((char *)s_.dev + offsetof(SwDev, sweep), &sweep, sizeof(uint32_t),
@@ -945,7 +977,7 @@ class SwEngine {
     }
     int rc = sync();
     if (rc) return rc;
-    k_sw_unpack<<<(int)std::min<int64_t>((h_.N + 255) / 256, 152 * 64), 256, 0, st_>>>(s_);
+    k_sw_unpack<<<h_.ntile * SW_TY / 8, 256, 0, st_>>>(s_);  // a warp per tile row
     SWCK(cudaGetLastError());
     SWCK(cudaMemcpyAsync(spins, s_.bytes, (size_t)h_.N, cudaMemcpyDeviceToHost, st_));
     SWCK(cudaStreamSynchronize(st_));
@@ -1014,7 +1046,8 @@ class SwEngine {
   void release() {
     if (st_) cudaStreamSynchronize(st_);
     if (gexec_) cudaGraphExecDestroy(gexec_);
-    gexec_ = nullptr;
+    if (gexec_blk_) cudaGraphExecDestroy(gexec_blk_);
+    gexec_ = gexec_blk_ = nullptr;
     for (cudaEvent_t &e : ev_)
       if (e) cudaEventDestroy(e);
     for (void *p : allocs_) cudaFree(p);
@@ -1030,6 +1063,24 @@ class SwEngine {
     }
   }
 
+  int capture(int count, cudaGraphExec_t *out) {
+    if (*out) return LCQMC_OK;
+    SWCK(cudaStreamBeginCapture(st_, cudaStreamCaptureModeThreadLocal));
+    int rc = LCQMC_OK;
+    for (int i = 0; i < count && !rc; ++i) rc = enqueue(false);
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamEndCapture(st_, &g);
+    if (rc) {
+      if (e == cudaSuccess) cudaGraphDestroy(g);
+      return rc;
+    }
+    SWCK(e);
+    e = cudaGraphInstantiate(out, g, 0);
+    cudaGraphDestroy(g);
+    SWCK(e);
+    return LCQMC_OK;
+  }
+
   int enqueue(bool timed) {
     if (timed && pending_) {  // the previous timed update's events are complete once it is
       SWCK(cudaEventSynchronize(ev_[LCQMC_SW_NPHASE]));
@@ -1040,15 +1091,20 @@ class SwEngine {
     const int nt = h_.ntile;
     const int nsize = (int)std::min<int64_t>(SW_SIZE_BLOCKS, ((int64_t)nt + 7) / 8);
     SWCK(mark(0));  // [0] bond draws, tile union-find
-    k_sw_local<<<nt, SW_TPB, 0, st_>>>(s_);
+    if (nt <= SW_WIDE_TILES)
+      k_sw_local<SW_TPB_WIDE><<<nt, SW_TPB_WIDE, 0, st_>>>(s_);
+    else
+      k_sw_local<SW_TPB><<<nt, SW_TPB, 0, st_>>>(s_);
     SWCK(mark(1));  // [1] tile-boundary bonds, global union-find
-    k_sw_merge<<<(nt * 32 + 255) / 256, 256, 0, st_>>>(s_);
+    k_sw_merge<<<nt, SW_EDGE, 0, st_>>>(s_);
     SWCK(mark(2));  // [2] roots, coins, flips
     k_sw_find<<<(nt * 32 + 255) / 256, 256, 0, st_>>>(s_);
-    k_sw_flip<<<nt, SW_TPB, 0, st_>>>(s_);
+    if (nt <= SW_WIDE_TILES)
+      k_sw_flip<SW_TPB_WIDE><<<nt, SW_TPB_WIDE, 0, st_>>>(s_);
+    else
+      k_sw_flip<SW_TPB><<<nt, SW_TPB, 0, st_>>>(s_);
     SWCK(mark(3));  // [3] open clusters' sizes, record
     k_sw_sizes<<<nsize, 256, 0, st_>>>(s_);
-    k_sw_final<<<1, 1024, 0, st_>>>(s_, nsize);
     SWCK(mark(4));
     SWCK(cudaGetLastError());
     if (timed) pending_ = true;
@@ -1059,7 +1115,8 @@ class SwEngine {
   SwScratch s_{};
   cudaStream_t st_ = nullptr;
   bool own_stream_ = false;
-  cudaGraphExec_t gexec_ = nullptr;
+  static constexpr int kGraphBlock = 8;
+  cudaGraphExec_t gexec_ = nullptr, gexec_blk_ = nullptr;
   cudaEvent_t ev_[LCQMC_SW_NPHASE + 1] = {};
   bool timing_ = false, pending_ = false;
   double ph_[LCQMC_SW_NPHASE] = {};
