@@ -14,6 +14,7 @@ constexpr int QMAX = 4;           // largest 2S: subspins per site (S <= 2)
 constexpr int TW = LCQMC_TW;      // windows per time block of the cell order
 constexpr int SCAN_PARTS = 152;   // parts of the operator scan over all chains, at most
 constexpr int64_t VTX_ID_LIMIT = 0x7ffff000;  // largest vertex count of one chain
+constexpr int VTX_PAD = 8;       // times a search may read past the last vertex
 constexpr int NOBS = 9;         // running averages per chain (lcqmc_obs.sum)
 constexpr int ACC_WORDS = 4;    // 64-bit words of an open loop's record (32 bytes)
 constexpr int PHASE_BITS = 16;  // phase factor table: 2^16 points of the period

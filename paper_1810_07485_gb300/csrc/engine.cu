@@ -192,7 +192,7 @@ void Engine::free_vertex() {
 int Engine::alloc_vertex(int64_t vcap) {
   free_vertex();
   vcap = (vcap + 127) / 128 * 128;
-  DALLOC(s_.vtau, double, vcap);
+  DALLOC(s_.vtau, double, vcap + VTX_PAD);
   DALLOC(s_.vflag, uint8_t, vcap);
   DALLOC(s_.vcell, uint8_t, vcap);
   DALLOC(s_.pl, int32_t, vcap);
