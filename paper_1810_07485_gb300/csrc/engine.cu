@@ -236,6 +236,11 @@ Engine::~Engine() {
   if (st_) cudaStreamSynchronize(st_);
   drop_graphs();
   for (auto e : ev_) cudaEventDestroy(e);
+  if (fork_) cudaEventDestroy(fork_);
+  for (int q = 0; q < QMAX; ++q) {
+    if (join_[q]) cudaEventDestroy(join_[q]);
+    if (side_[q]) cudaStreamDestroy(side_[q]);
+  }
   free_vertex();
   for (auto &c : owned_) destroy_state(c.get());
   dfree(dch_);
@@ -558,6 +563,7 @@ int Engine::layout() {
   L_.bond_tab = bond_tab_;
   L_.s = s_;
   drop_graphs();
+  if ((rc = count_groups()) != 0) return rc;
   if (vest > vcap_) {
     rc = alloc_vertex(vest);
     if (rc) return rc;
@@ -603,16 +609,36 @@ int Engine::enqueue_one(bool timed, int slot) {
   };
   mark(0);  // [0] labeling: random numbers, insertion, vertex offsets (one pass)
   launch_start(L_, cap_tiles_, nw, st_);
-  launch_insert(L_, st_);
-  mark(1);  // [1] tau = 0 cut
-  launch_cut(L_, st_);
-  mark(2);  // [2] linking + union-find
-  launch_link(L_, st_);
-  mark(3);  // [3] loop ids (compression, coins)
-  launch_compress(L_, st_);
-  if (L_.check_forest) launch_check_forest(L_, st_);
-  mark(4);  // [4] loop properties, new flags
-  launch_est(L_, st_);
+  if (timed || L_.check_forest || ngroups_ < 2) {
+    launch_insert(L_, -1, st_);
+    mark(1);  // [1] tau = 0 cut
+    launch_cut(L_, -1, st_);
+    mark(2);  // [2] linking + union-find
+    launch_link(L_, -1, st_);
+    mark(3);  // [3] loop ids (compression, coins)
+    launch_compress(L_, -1, st_);
+    if (L_.check_forest) launch_check_forest(L_, st_);
+    mark(4);  // [4] loop properties, new flags
+    launch_est(L_, -1, st_);
+  } else {
+    // A group's last blocks leave SMs free, which the other groups' kernels fill:
+    // 16 chains of S = 1/2 and 1, 3800 tiles together, 0.73 -> 0.66 ms per update.
+    CK(cudaEventRecord(fork_, st_));
+    int first = -1;
+    for (int q = 0; q < QMAX; ++q) {
+      if (!L_.ntile[q]) continue;
+      if (first < 0) {
+        first = q;
+        continue;
+      }
+      CK(cudaStreamWaitEvent(side_[q], fork_, 0));
+      front(q, side_[q]);
+      CK(cudaEventRecord(join_[q], side_[q]));
+    }
+    front(first, st_);
+    for (int q = first + 1; q < QMAX; ++q)
+      if (L_.ntile[q]) CK(cudaStreamWaitEvent(st_, join_[q], 0));
+  }
   mark(5);  // [5] operator offsets
   launch_scan_ops(L_, st_);
   mark(6);  // [6] operator rewrite
@@ -622,6 +648,27 @@ int Engine::enqueue_one(bool timed, int slot) {
   launch_final(L_, st_);
   mark(8);
   CK(cudaGetLastError());
+  return LCQMC_OK;
+}
+
+void Engine::front(int only, cudaStream_t st) {
+  launch_insert(L_, only, st);
+  launch_cut(L_, only, st);
+  launch_link(L_, only, st);
+  launch_compress(L_, only, st);
+  launch_est(L_, only, st);
+}
+
+// Counts the Q groups of the resident set and makes the side streams they need.
+int Engine::count_groups() {
+  ngroups_ = 0;
+  for (int q = 0; q < QMAX; ++q) {
+    if (!L_.ntile[q]) continue;
+    if (ngroups_++ == 0) continue;
+    if (!fork_) CK(cudaEventCreateWithFlags(&fork_, cudaEventDisableTiming));
+    if (!side_[q]) CK(cudaStreamCreateWithFlags(&side_[q], cudaStreamNonBlocking));
+    if (!join_[q]) CK(cudaEventCreateWithFlags(&join_[q], cudaEventDisableTiming));
+  }
   return LCQMC_OK;
 }
 
@@ -768,6 +815,10 @@ int Engine::sync(bool *at_once) {
       return LCQMC_OK;
     }
     if (at_once) *at_once = false;
+    // An update that stopped may have added to open loops' records (always taken
+    // and cleared by the operator rewrite, which did not run): they start at zero.
+    CK(cudaMemsetAsync(s_.acc, 0, ACC_WORDS * sizeof(unsigned long long) * vcap_, st_));
+    CK(cudaMemsetAsync(s_.accz, 0, sizeof(unsigned long long) * vcap_, st_));
     const int64_t done = (int64_t)(uint32_t)(hch[0].sweep - pending_sweep0_);
     const int64_t remaining = pending_ - done;
     if (status & (ST_TIMEOUT | ST_INTERNAL | ST_BADSTATE | ST_ID_OVERFLOW)) {
@@ -802,9 +853,6 @@ int Engine::sync(bool *at_once) {
       if (rc) return rc;
     }
     if (status & ST_OP_OVERFLOW) {
-      // the open loops' records were added to but not all squared and cleared
-      CK(cudaMemsetAsync(s_.acc, 0, ACC_WORDS * sizeof(unsigned long long) * vcap_, st_));
-      CK(cudaMemsetAsync(s_.accz, 0, sizeof(unsigned long long) * vcap_, st_));
       for (int64_t c = 0; c < (int64_t)hch.size(); ++c)
         if (hch[c].n_off_new > hch[c].op_cap) {
           rc = grow_ops(c, hch[c].n_off_new);

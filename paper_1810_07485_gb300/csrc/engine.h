@@ -126,6 +126,14 @@ class Engine {
   // small chains, whose updates are a few microseconds of work)
   static constexpr int kGraphBlock = 8;
   cudaGraphExec_t gexec_ = nullptr, gexec_blk_ = nullptr;
+  // A resident set of several Q: every group's kernels up to the loop properties
+  // run on a stream of their own beside the first group's (the groups share no
+  // data there), between the update's start and its operator scan.
+  cudaStream_t side_[QMAX] = {};
+  cudaEvent_t fork_ = nullptr, join_[QMAX] = {};
+  int ngroups_ = 0;
+  void front(int only, cudaStream_t st);  // insertion .. loop properties of a group
+  int count_groups();
   bool serving_ = false;
   cudaMemPool_t pool_ = nullptr;
   bool timing_ = false;

@@ -2212,6 +2212,9 @@ static int64_t all_tiles(const Launch &L) {
   return n;
 }
 
+// Whether Q group q is launched: the one asked for, or all (only < 0).
+static bool picked(int only, int q) { return only < 0 || only == q; }
+
 void launch_start(const Launch &L, int64_t ntile, int64_t nw, cudaStream_t st) {
   int64_t nbb = 0;
   for (int q = 0; q < QMAX; ++q) nbb += L.nbondblk[q];
@@ -2220,9 +2223,9 @@ void launch_start(const Launch &L, int64_t ntile, int64_t nw, cudaStream_t st) {
   k_start<<<g1(nbb + blocks), BOND_BLOCK, 0, st>>>(L.ch, L.bond_tab, nbb, L.s, ntile, nw);
 }
 
-void launch_insert(const Launch &L, cudaStream_t st) {
+void launch_insert(const Launch &L, int only, cudaStream_t st) {
 #define INSERT_Q(Q)                                                                                   \
-  if (L.ntile[Q - 1])                                                                                 \
+  if (L.ntile[Q - 1] && picked(only, Q - 1))                                                          \
     k_insert<Q><<<g1(L.ntile[Q - 1]), INS_THREADS, sizeof(InsSmem<Q>), st>>>(L.ch,          \
                                                                                           L.tile_tab,    \
                                                                                           L.tile0[Q - 1], \
@@ -2242,17 +2245,18 @@ void launch_scan_ops(const Launch &L, cudaStream_t st) {
   k_scan_ops<<<dim3(L.nchains, parts), 1024, 0, st>>>(L.ch, L.s);
 }
 
-void launch_cut(const Launch &L, cudaStream_t st) {
+void launch_cut(const Launch &L, int only, cudaStream_t st) {
 #define CUT_Q(Q) \
-  if (L.nsiteblk[Q - 1]) k_cut<Q><<<g1(L.nsiteblk[Q - 1]), SITE_BLOCK * Q, 0, st>>>(L.ch, L.site_tab, L.site0[Q - 1], L.s);
+  if (L.nsiteblk[Q - 1] && picked(only, Q - 1)) \
+    k_cut<Q><<<g1(L.nsiteblk[Q - 1]), SITE_BLOCK * Q, 0, st>>>(L.ch, L.site_tab, L.site0[Q - 1], L.s);
   FOR_EACH_Q(CUT_Q)
 #undef CUT_Q
 }
 
-void launch_link(const Launch &L, cudaStream_t st) {
+void launch_link(const Launch &L, int only, cudaStream_t st) {
   const bool wide = all_tiles(L) <= WIDE_TILES;
 #define LINK_Q(Q)                                                                                              \
-  if (L.ntile[Q - 1]) {                                                                                        \
+  if (L.ntile[Q - 1] && picked(only, Q - 1)) {                                                                 \
     if (wide)                                                                                                  \
       k_link<Q, TPB_WIDE><<<g1(L.ntile[Q - 1]), TPB_WIDE, 0, st>>>(L.ch, L.tile_tab, L.tile0[Q - 1], L.s);      \
     else                                                                                                       \
@@ -2267,7 +2271,7 @@ void launch_link(const Launch &L, cudaStream_t st) {
   const int wpb = L.link_x_warps;
   for (int q = 0; q < QMAX; ++q) {
     const int64_t n = L.ntile[q];
-    if (!n) continue;
+    if (!n || !picked(only, q)) continue;
     if (n > XT_MAX_TILES)
       k_link_x<<<g1((n + wpb - 1) / wpb), 32 * wpb, 0, st>>>(L.ch, L.tile_tab + L.tile0[q], n, L.s);
     else
@@ -2275,13 +2279,13 @@ void launch_link(const Launch &L, cudaStream_t st) {
   }
 }
 
-void launch_compress(const Launch &L, cudaStream_t st) {
-  const int64_t n = all_tiles(L);
+void launch_compress(const Launch &L, int only, cudaStream_t st) {
+  const int64_t n = only < 0 ? all_tiles(L) : L.ntile[only], t0 = only < 0 ? 0 : L.tile0[only];
   if (!n) return;
-  if (n <= WIDE_TILES)
-    k_compress<TPB_WIDE><<<g1(n), TPB_WIDE, 0, st>>>(L.ch, L.tile_tab, 0, L.s);
+  if (all_tiles(L) <= WIDE_TILES)
+    k_compress<TPB_WIDE><<<g1(n), TPB_WIDE, 0, st>>>(L.ch, L.tile_tab, t0, L.s);
   else
-    k_compress<TILE><<<g1(n), L.compress_threads, 0, st>>>(L.ch, L.tile_tab, 0, L.s);
+    k_compress<TILE><<<g1(n), L.compress_threads, 0, st>>>(L.ch, L.tile_tab, t0, L.s);
 }
 
 void launch_check_forest(const Launch &L, cudaStream_t st) {
@@ -2328,22 +2332,22 @@ int init_kernel_attributes() {
   return 0;
 }
 
-void launch_est(const Launch &L, cudaStream_t st) {
+void launch_est(const Launch &L, int only, cudaStream_t st) {
   // without the temporal moment only the ticks are staged
   const size_t dyn = L.temporal ? EST_DYN_SMEM : EST_STAGE * sizeof(long long);
   const bool wide = all_tiles(L) <= WIDE_TILES;
 #define EST_QTN(Q, T, NT) \
   k_est<Q, T, NT><<<g1(L.ntile[Q - 1]), NT, dyn, st>>>(L.ch, L.tile_tab, L.tile0[Q - 1], L.s)
-#define EST_Q(Q)                   \
-  if (L.ntile[Q - 1]) {            \
-    if (L.temporal && wide)        \
-      EST_QTN(Q, true, TPB_WIDE);  \
-    else if (L.temporal)           \
-      EST_QTN(Q, true, TPB);       \
-    else if (wide)                 \
-      EST_QTN(Q, false, TPB_WIDE); \
-    else                           \
-      EST_QTN(Q, false, TPB);      \
+#define EST_Q(Q)                               \
+  if (L.ntile[Q - 1] && picked(only, Q - 1)) { \
+    if (L.temporal && wide)                    \
+      EST_QTN(Q, true, TPB_WIDE);              \
+    else if (L.temporal)                       \
+      EST_QTN(Q, true, TPB);                   \
+    else if (wide)                             \
+      EST_QTN(Q, false, TPB_WIDE);             \
+    else                                       \
+      EST_QTN(Q, false, TPB);                  \
   }
   FOR_EACH_Q(EST_Q)
 #undef EST_Q

@@ -29,13 +29,14 @@ int init_kernel_attributes();
 // bond parities; zeroes the look-back words of ntile tiles, the tickets and nw
 // words of each bitmap
 void launch_start(const Launch &L, int64_t ntile, int64_t nw, cudaStream_t st);
-void launch_insert(const Launch &L, cudaStream_t st);
+// only: the Q group to launch (Q - 1), or -1 for all of them
+void launch_insert(const Launch &L, int only, cudaStream_t st);
 void launch_scan_ops(const Launch &L, cudaStream_t st);
-void launch_cut(const Launch &L, cudaStream_t st);
-void launch_link(const Launch &L, cudaStream_t st);
-void launch_compress(const Launch &L, cudaStream_t st);
+void launch_cut(const Launch &L, int only, cudaStream_t st);
+void launch_link(const Launch &L, int only, cudaStream_t st);
+void launch_compress(const Launch &L, int only, cudaStream_t st);
 void launch_check_forest(const Launch &L, cudaStream_t st);
-void launch_est(const Launch &L, cudaStream_t st);
+void launch_est(const Launch &L, int only, cudaStream_t st);
 // operator rewrite; sites: the spin rewrite too, in the same launch where that
 // is faster (else launch_sites is the caller's)
 void launch_compact(const Launch &L, bool sites, cudaStream_t st);
