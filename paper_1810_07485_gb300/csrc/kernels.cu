@@ -263,8 +263,8 @@ __device__ int64_t lb_lookback(unsigned long long *st, int64_t g, int64_t first,
   }
 }
 
-// Candidate-parallel insertion, a warp for every 16 cells of the tile.  Lanes l
-// and l + 16 set up cell l together: each takes the neighbour bonds of one of
+// Candidate-parallel insertion, a warp for every 16 (or 8) cells of the tile.
+// Lanes l and l + 16 (l + 8) set up cell l together: each takes the neighbour bonds of one of
 // the cell's subsites (operator ranges, spin parity at the window start) and
 // one of the cell's first two Philox calls (call 0 gives the number K of
 // candidates and candidate 0, call m >= 1 candidates 2m-1 and 2m).  The
@@ -286,19 +286,26 @@ __device__ int64_t lb_lookback(unsigned long long *st, int64_t g, int64_t first,
 // and lists (eleven barriers, issue 65 %).  Of the 0.78 ms the set-up takes
 // 0.16, the draws 0.08, the decisions 0.22, the places 0.20, the look-back 0.02
 // and the writes 0.13.  Six blocks per SM at 40 registers (five at 48: 0.82).
-// A warp stages INS_CAP candidates (mean 128, sigma 11): one whose cells have
+// A warp stages InsWarp::CAP candidates (mean 128 for 16 cells, sigma 11): one whose cells have
 // more runs them in groups, counting in a first pass and drawing again in the
 // writing pass.
-constexpr int INS_THREADS = 256;
-constexpr int INS_WARPS = INS_THREADS / 32;
-constexpr int INS_WC = TILE / INS_WARPS;  // cells of a warp
-static_assert(INS_WC == 16, "a cell per lane of a half warp");
-constexpr int INS_CAP = 168;
-// Vertices a group of cells may have for its positions to be marked in shared
-// memory (mean 177 for a thermalized S = 1/2 warp, sigma 15).
-constexpr int INS_MARKS = 288;
-// Group sizes a chain may ask for (tests), in candidates of a whole tile.
-constexpr int INS_MIN_SPAN = 256, INS_MAX_SPAN = INS_CAP * INS_WARPS;
+//
+// NW warps per tile: 8, or 16 with 8 cells each for launches of few tiles, whose
+// time is one tile's chain of steps (insertion in us, 8 / 16 warps: L=64 20.6 /
+// 18.0, L=1024, 128 tiles, 28.9 / 21.3, S = 2, 65 tiles, 36 / 29).  There lanes
+// l + 16 and l + 24 repeat what l and l + 8 do in the set-up.
+constexpr int INS_WARPS = 8, INS_WARPS_WIDE = 16;
+template <int NW>
+struct InsWarp {
+  static constexpr int WC = TILE / NW;  // cells of a warp
+  // candidates a warp stages, and vertices a group of its cells may have for
+  // their positions to be marked in shared memory (mean 177 for 16 cells of a
+  // thermalized S = 1/2 chain, sigma 15)
+  static constexpr int CAP = NW == 8 ? 168 : 104, MARKS = NW == 8 ? 288 : 160;
+  static_assert(WC <= 16, "two lanes per cell, four bits of a key");
+  static_assert(CAP >= KMAX - 1, "a cell's candidates fit");
+};
+constexpr int INS_MIN_SPAN = 256;  // smallest group a chain may ask for (tests), in candidates of a whole tile
 
 // Old operator times a tile stages in shared memory: its own cells' and those
 // of the cells up to 8 Q^2 cells away (the neighbour bonds of the same
@@ -309,32 +316,33 @@ struct InsStage {
   static constexpr int PAD = 4;  // entries a search may read past the last one
 };
 
-template <int Q>
-struct InsSmem {
+template <int Q, int NW>
+struct InsSmem : InsWarp<NW> {
+  using W = InsWarp<NW>;
   static constexpr int NB = 4 * Q - 2;  // neighbour bonds of a cell
   long long sop[InsStage<Q>::N + InsStage<Q>::PAD];  // staged old operator times (16-byte aligned: first member)
   // Per warp: the candidates' keys (cell in the warp << 59 | u53 << 6 | draw
   // index), then, for the kept ones, the same and the times' bits.  Two more
   // entries: a sentinel, and the second half of a pair load.
-  unsigned long long key[INS_WARPS][INS_CAP + 2];
-  long long tau[INS_WARPS][INS_CAP];
+  unsigned long long key[NW][W::CAP + 2];
+  long long tau[NW][W::CAP];
   // Per cell: neighbour and own operator ranges (from the first staged operator
   // if all of the warp's ranges are staged), window, kept candidates
   int2 nb[TILE][NB], own[TILE];
   int j[TILE], cex[TILE];
   unsigned short less[TILE], kf[TILE], nk[TILE];  // bit k of less: neighbour bond k < the cell's bond
   // Per warp: a vertex position's kept candidate + 1, 0 for an old operator
-  uint8_t mark[INS_WARPS][INS_MARKS];
+  uint8_t mark[NW][W::MARKS];
   uint8_t par0[TILE];
   unsigned long long T[2][KMAX];  // Poisson thresholds: full windows, last window
-  int wtot[INS_WARPS];
+  int wtot[NW];
   int slo, shi;
   uint64_t bar;
   int64_t excl;
   int64_t gt;
 };
 
-static_assert(sizeof(InsSmem<1>) <= 228 * 1024 / 6 - 1024, "six blocks per SM");
+static_assert(sizeof(InsSmem<1, INS_WARPS>) <= 228 * 1024 / 6 - 1024, "six blocks per SM");
 
 // Number of times below thr in t[lo, hi) (ascending).  ST (staged operators):
 // the ranges hold 4.7 operators on average; more than 7 are halved first, then
@@ -375,7 +383,7 @@ __device__ __forceinline__ double key_unit(unsigned long long key) {
   return __longlong_as_double((long long)bits);
 }
 
-// A warp's cells: lanes l and l + 16 hold cell l.
+// A warp's cells: lanes l and l + WC hold cell l.
 struct InsCell {
   int b, j, K, kpre;  // bond, window, candidates, candidates of the cells before it
 };
@@ -386,9 +394,10 @@ struct InsCell {
 // tau = fma(d, u53 2^-53, t0) (one IEEE fused multiply-add); it is kept if its
 // bond's spins are antiparallel there (parity at the window start flipped by
 // the neighbour operators before it; order (time, bond)).
-template <int Q, bool ST>
-__device__ __forceinline__ int ins_decide(const DevChain &C, InsSmem<Q> &S, const long long *otau, int wid,
+template <int Q, int NW, bool ST>
+__device__ __forceinline__ int ins_decide(const DevChain &C, InsSmem<Q, NW> &S, const long long *otau, int wid,
                                           int ns) {
+  constexpr int WC = InsWarp<NW>::WC;
   const int lane = threadIdx.x & 31;
   const long long *ot = ST ? S.sop : otau;
   int nkept = 0;
@@ -401,7 +410,7 @@ __device__ __forceinline__ int ins_decide(const DevChain &C, InsSmem<Q> &S, cons
     if (slot < ns) {
       key = S.key[wid][slot];
       c = (int)(key >> 59);
-      const int cw = wid * INS_WC + c;
+      const int cw = wid * WC + c;
       const uint64_t *win = C.win + 3 * S.j[cw];
       const double t0 = __longlong_as_double((long long)win[0]);
       const long long teb = (long long)win[1];
@@ -411,7 +420,7 @@ __device__ __forceinline__ int ins_decide(const DevChain &C, InsSmem<Q> &S, cons
         int p = S.par0[cw];
         const int less = S.less[cw];
 #pragma unroll
-        for (int k = 0; k < InsSmem<Q>::NB; ++k) {
+        for (int k = 0; k < InsSmem<Q, NW>::NB; ++k) {
           const int2 r = S.nb[cw][k];
           p ^= times_below<ST>(ot, r.x, r.y, tau + ((less >> k) & 1));
         }
@@ -421,7 +430,7 @@ __device__ __forceinline__ int ins_decide(const DevChain &C, InsSmem<Q> &S, cons
     const unsigned km = __ballot_sync(0xffffffffu, keep);
     const int at = nkept + __popc(km & ((1u << lane) - 1u));
     __syncwarp();  // every lane has read its candidate: pack over the ones read
-    if (slot < ns && (key & 63) == 0) S.kf[wid * INS_WC + c] = (unsigned short)at;
+    if (slot < ns && (key & 63) == 0) S.kf[wid * WC + c] = (unsigned short)at;
     if (keep) {
       S.key[wid][at] = key;
       S.tau[wid][at] = tau;
@@ -436,11 +445,12 @@ __device__ __forceinline__ int ins_decide(const DevChain &C, InsSmem<Q> &S, cons
 // Draw and decide the candidates of the warp's cells [c0, c1); o: the lane's
 // output of Philox call (lane >= 16) of its cell.  Sets kf and nk of the cells;
 // returns the number kept.
-template <int Q>
-__device__ __forceinline__ int ins_group(const DevChain &C, InsSmem<Q> &S, const long long *otau, int wid,
+template <int Q, int NW>
+__device__ __forceinline__ int ins_group(const DevChain &C, InsSmem<Q, NW> &S, const long long *otau, int wid,
                                          const InsCell &X, const U4 &o, int c0, int c1, bool staged, uint32_t sweep,
                                          uint32_t k0, uint32_t k1) {
-  const int lane = threadIdx.x & 31, cl = lane & 15, side = lane >> 4;
+  constexpr int WC = InsWarp<NW>::WC;
+  const int lane = threadIdx.x & 31, cl = lane & (WC - 1), side = (lane / WC) & 1;
   const bool in = cl >= c0 && cl < c1;
   const int kb = __shfl_sync(0xffffffffu, X.kpre, c0);
   const int ns = uniform(__shfl_sync(0xffffffffu, X.kpre + X.K, c1 - 1) - kb);
@@ -458,16 +468,16 @@ __device__ __forceinline__ int ins_group(const DevChain &C, InsSmem<Q> &S, const
   const int P = (in && X.K > 3) ? X.K / 2 - 1 : 0;
   int pin = P;  // inclusive scan over the cells (both halves alike)
 #pragma unroll
-  for (int d = 1; d < 16; d <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, pin, d, 16);
+  for (int d = 1; d < WC; d <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, pin, d, WC);
     if (cl >= d) pin += y;
   }
-  const int nu = uniform(__shfl_sync(0xffffffffu, pin, 15));
+  const int nu = uniform(__shfl_sync(0xffffffffu, pin, WC - 1));
   for (int u0 = 0; u0 < nu; u0 += 32) {
     const int u = u0 + lane;
     int c = 0;  // cells whose calls all come before call u
 #pragma unroll
-    for (int d = 8; d > 0; d >>= 1) {
+    for (int d = WC / 2; d > 0; d >>= 1) {
       const int y = __shfl_sync(0xffffffffu, pin, c + d - 1);
       if (y <= u) c += d;
     }
@@ -483,19 +493,19 @@ __device__ __forceinline__ int ins_group(const DevChain &C, InsSmem<Q> &S, const
     }
   }
   __syncwarp();
-  const int nkept = staged ? ins_decide<Q, true>(C, S, otau, wid, ns) : ins_decide<Q, false>(C, S, otau, wid, ns);
+  const int nkept = staged ? ins_decide<Q, NW, true>(C, S, otau, wid, ns) : ins_decide<Q, NW, false>(C, S, otau, wid, ns);
   // first kept candidate and number kept per cell; a cell without candidates
   // starts where the next one with candidates does
-  const unsigned has = __ballot_sync(0xffffffffu, in && lane < 16 && X.K > 0);
+  const unsigned has = __ballot_sync(0xffffffffu, in && lane < WC && X.K > 0);
   const unsigned from = has >> cl;
   const int nx = from ? cl + __ffs(from) - 1 : cl;
-  int kf = (in && X.K > 0) ? S.kf[wid * INS_WC + cl] : nkept;
+  int kf = (in && X.K > 0) ? S.kf[wid * WC + cl] : nkept;
   kf = __shfl_sync(0xffffffffu, kf, nx);
-  const int kn = __shfl_down_sync(0xffffffffu, kf, 1, 16);
+  const int kn = __shfl_down_sync(0xffffffffu, kf, 1, WC);
   __syncwarp();
-  if (in && lane < 16) {
-    S.kf[wid * INS_WC + cl] = (unsigned short)kf;
-    S.nk[wid * INS_WC + cl] = (unsigned short)((cl == c1 - 1 ? nkept : kn) - kf);
+  if (in && lane < WC) {
+    S.kf[wid * WC + cl] = (unsigned short)kf;
+    S.nk[wid * WC + cl] = (unsigned short)((cl == c1 - 1 ? nkept : kn) - kf);
   }
   __syncwarp();
   return nkept;
@@ -504,9 +514,10 @@ __device__ __forceinline__ int ins_group(const DevChain &C, InsSmem<Q> &S, const
 // Positions of the warp's nkept kept candidates among the vertices of its cells
 // (cell order, then time): marked in shared memory from position `from` on, or,
 // for DIRECT, written to the vertex arrays at once.
-template <int Q, bool ST, bool DIRECT>
-__device__ __forceinline__ void ins_place(const DevChain &C, InsSmem<Q> &S, const long long *otau, int wid,
+template <int Q, int NW, bool ST, bool DIRECT>
+__device__ __forceinline__ void ins_place(const DevChain &C, InsSmem<Q, NW> &S, const long long *otau, int wid,
                                           int nkept, int from, int64_t base, const Scratch &s) {
+  constexpr int WC = InsWarp<NW>::WC;
   const int lane = threadIdx.x & 31;
   const long long *ot = ST ? S.sop : otau;
   for (int i0 = 0; i0 < nkept; i0 += 32) {
@@ -514,7 +525,7 @@ __device__ __forceinline__ void ins_place(const DevChain &C, InsSmem<Q> &S, cons
     if (i < nkept) {
       const unsigned long long key = S.key[wid][i];
       const long long tau = S.tau[wid][i];
-      const int cw = wid * INS_WC + (int)(key >> 59);
+      const int cw = wid * WC + (int)(key >> 59);
       // kept candidates ahead, two keys a step from an even place on (one of
       // the cell before is below the cell's keys, what follows is above them)
       const int kf = S.kf[cw], k0 = kf & ~1, k1 = kf + S.nk[cw];
@@ -542,9 +553,10 @@ __device__ __forceinline__ void ins_place(const DevChain &C, InsSmem<Q> &S, cons
 // Write the marked vertices [0, n) from tile position `from` on, in id order:
 // the positions without a mark are the old operators from qa on, in their
 // order.  ce: first position of the lane's cell.
-template <int Q, bool ST>
-__device__ __forceinline__ void ins_write(const DevChain &C, InsSmem<Q> &S, const long long *otau, int wid, int n,
+template <int Q, int NW, bool ST>
+__device__ __forceinline__ void ins_write(const DevChain &C, InsSmem<Q, NW> &S, const long long *otau, int wid, int n,
                                           int from, int ce, int qa, int64_t base, const Scratch &s) {
+  constexpr int WC = InsWarp<NW>::WC;
   const int lane = threadIdx.x & 31;
   const int64_t vb = C.vtx_base + base + from;
   long long *vt = (long long *)s.vtau + vb;
@@ -555,14 +567,14 @@ __device__ __forceinline__ void ins_write(const DevChain &C, InsSmem<Q> &S, cons
     const unsigned old = __ballot_sync(0xffffffffu, i < n && m == 0);
     int c = 0;  // largest cell with first position <= i
 #pragma unroll
-    for (int d = 8; d > 0; d >>= 1) {
+    for (int d = WC / 2; d > 0; d >>= 1) {
       const int y = __shfl_sync(0xffffffffu, ce, c + d);
       if (y <= from + i) c += d;
     }
     if (i < n) {
       vt[i] = m ? S.tau[wid][m - 1] : ot[qa + __popc(old & ((1u << lane) - 1u))];
       vf[i] = m ? 0 : VF_OLD;
-      vc[i] = (uint8_t)(wid * INS_WC + c);
+      vc[i] = (uint8_t)(wid * WC + c);
     }
     qa += __popc(old);
   }
@@ -572,21 +584,22 @@ __device__ __forceinline__ void ins_write(const DevChain &C, InsSmem<Q> &S, cons
 // The old operators [qa, qb) of a group of cells with too many vertices for the
 // marks: each finds its place by the kept candidates before it.  q0, ce: first
 // operator and first position of the lane's cell.
-template <int Q>
-__device__ __noinline__ void ins_write_old(InsSmem<Q> &S, const long long *otau, int wid, int q0, int ce, int qa,
+template <int Q, int NW>
+__device__ __noinline__ void ins_write_old(InsSmem<Q, NW> &S, const long long *otau, int wid, int q0, int ce, int qa,
                                            int qb, long long *vt, uint8_t *vf, uint8_t *vc) {
+  constexpr int WC = InsWarp<NW>::WC;
   const int lane = threadIdx.x & 31;
   for (int qq = qa; qq < qb; qq += 32) {
     const int q = qq + lane;
     int c = 0;  // largest cell with first operator <= q
 #pragma unroll
-    for (int d = 8; d > 0; d >>= 1) {
+    for (int d = WC / 2; d > 0; d >>= 1) {
       const int y = __shfl_sync(0xffffffffu, q0, c + d);
       if (y <= q) c += d;
     }
     const int qc = __shfl_sync(0xffffffffu, q0, c), pc = __shfl_sync(0xffffffffu, ce, c);
     if (q < qb) {
-      const int cw = wid * INS_WC + c;
+      const int cw = wid * WC + c;
       const long long t = otau[q];
       const long long *tt = &S.tau[wid][S.kf[cw]];
       const int n = S.nk[cw];
@@ -600,25 +613,26 @@ __device__ __noinline__ void ins_write_old(InsSmem<Q> &S, const long long *otau,
   }
 }
 
-template <int Q>
-__device__ __forceinline__ void insert_tile(InsSmem<Q> &S, DevChain *__restrict__ ch,
+template <int Q, int NW>
+__device__ __forceinline__ void insert_tile(InsSmem<Q, NW> &S, DevChain *__restrict__ ch,
                                             const int2 *__restrict__ tab, int64_t blk0, int group,
                                             Scratch s);
 
 // Dynamic shared memory: 36 KB for Q = 1 (six blocks per SM), above the 48 KB
 // static limit for the larger neighbour tables and operator stages of Q >= 3.
-template <int Q>
-__global__ void __launch_bounds__(INS_THREADS, Q == 1 ? 6 : 4) k_insert(DevChain *__restrict__ ch,
+template <int Q, int NW>
+__global__ void __launch_bounds__(32 * NW, NW > 8 ? 2 : (Q == 1 ? 6 : 4)) k_insert(DevChain *__restrict__ ch,
                                                  const int2 *__restrict__ tab, int64_t blk0,
                                                  int group, Scratch s) {
   extern __shared__ __align__(16) unsigned char ins_dyn[];
-  insert_tile<Q>(*reinterpret_cast<InsSmem<Q> *>(ins_dyn), ch, tab, blk0, group, s);
+  insert_tile<Q, NW>(*reinterpret_cast<InsSmem<Q, NW> *>(ins_dyn), ch, tab, blk0, group, s);
 }
 
-template <int Q>
-__device__ __forceinline__ void insert_tile(InsSmem<Q> &S, DevChain *__restrict__ ch,
+template <int Q, int NW>
+__device__ __forceinline__ void insert_tile(InsSmem<Q, NW> &S, DevChain *__restrict__ ch,
                                             const int2 *__restrict__ tab, int64_t blk0, int group,
                                             Scratch s) {
+  constexpr int WC = InsWarp<NW>::WC;
   if (halted(s)) return;
   if (threadIdx.x == 0) S.gt = blk0 + (int64_t)atomicAdd(s.tickets + group, 1u);
   __syncthreads();
@@ -654,8 +668,8 @@ __device__ __forceinline__ void insert_tile(InsSmem<Q> &S, DevChain *__restrict_
   __syncthreads();
 
   // -- per-cell set-up ---------------------------------------------------------
-  const int lane = threadIdx.x & 31, wid = uniform((int)threadIdx.x >> 5), cl = lane & 15, side = lane >> 4;
-  const int cw = wid * INS_WC + cl, cell = t.y * TILE + cw;
+  const int lane = threadIdx.x & 31, wid = uniform((int)threadIdx.x >> 5), cl = lane & (WC - 1), side = (lane / WC) & 1;
+  const int cw = wid * WC + cl, cell = t.y * TILE + cw;
   const bool valid = cell < C.ncell;
   const int slo = S.slo, shi = S.shi;
   // the keys as uniform values: their schedule leaves the vector pipes
@@ -691,8 +705,8 @@ __device__ __forceinline__ void insert_tile(InsSmem<Q> &S, DevChain *__restrict_
     q0 = q1 = op[C.ncell];  // cells past the chain's end: empty ranges
   }
   __syncwarp();
-  par ^= __shfl_xor_sync(0xffffffffu, par, 16);
-  less |= __shfl_xor_sync(0xffffffffu, less, 16);
+  par ^= __shfl_xor_sync(0xffffffffu, par, WC);
+  less |= __shfl_xor_sync(0xffffffffu, less, WC);
   if (valid && !side) {
     S.par0[cw] = (uint8_t)par;
     S.less[cw] = (unsigned short)less;
@@ -710,8 +724,8 @@ __device__ __forceinline__ void insert_tile(InsSmem<Q> &S, DevChain *__restrict_
   X.K = __shfl_sync(0xffffffffu, X.K, cl);
   X.kpre = X.K;
 #pragma unroll
-  for (int d = 1; d < 16; d <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, X.kpre, d, 16);
+  for (int d = 1; d < WC; d <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, X.kpre, d, WC);
     if (cl >= d) X.kpre += y;
   }
   X.kpre -= X.K;
@@ -730,31 +744,31 @@ __device__ __forceinline__ void insert_tile(InsSmem<Q> &S, DevChain *__restrict_
   if (shi > slo) ok = mbar_wait(&S.bar, 0);
 
   // -- draw, decide, count; then place and write --------------------------------
-  const int cap = (C.ins_span >= INS_MIN_SPAN && C.ins_span < INS_MAX_SPAN)
-                      ? max(KMAX - 1, C.ins_span / INS_WARPS)
-                      : INS_CAP;
-  const bool single = __shfl_sync(0xffffffffu, X.kpre + X.K, 15) <= cap;
+  const int cap = (C.ins_span >= INS_MIN_SPAN && C.ins_span < InsWarp<NW>::CAP * NW)
+                      ? max(KMAX - 1, C.ins_span / NW)
+                      : InsWarp<NW>::CAP;
+  const bool single = __shfl_sync(0xffffffffu, X.kpre + X.K, WC - 1) <= cap;
   // Vertices of a group of cells: kept candidates placed (marked), all written.
   int nkept = 0, nk = 0, cex = 0;
   auto next = [&](int c0) {  // end of the group that starts at cell c0
-    if (single) return INS_WC;
+    if (single) return WC;
     const int kb = __shfl_sync(0xffffffffu, X.kpre, c0);
-    return c0 + __popc(__ballot_sync(0xffffffffu, lane < 16 && cl >= c0 && X.kpre + X.K - kb <= cap));
+    return c0 + __popc(__ballot_sync(0xffffffffu, lane < WC && cl >= c0 && X.kpre + X.K - kb <= cap));
   };
-  for (int c0 = 0; c0 < INS_WC;) {
+  for (int c0 = 0; c0 < WC;) {
     const int c1 = next(c0);
-    nkept = uniform(ins_group<Q>(C, S, otau, wid, X, o, c0, c1, staged, sweep, k0, k1));
+    nkept = uniform(ins_group<Q, NW>(C, S, otau, wid, X, o, c0, c1, staged, sweep, k0, k1));
     if (cl >= c0 && cl < c1) nk = S.nk[cw];
     c0 = c1;
   }
   const int cnt = q1 - q0 + nk;
   cex = cnt;
 #pragma unroll
-  for (int d = 1; d < 16; d <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, cex, d, 16);
+  for (int d = 1; d < WC; d <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, cex, d, WC);
     if (cl >= d) cex += y;
   }
-  if (lane == 15) S.wtot[wid] = cex;
+  if (lane == WC - 1) S.wtot[wid] = cex;
   cex -= cnt;
   if (!__syncthreads_and(ok)) {  // the bulk copy did not arrive within its bound
     if (threadIdx.x == 0) atomicOr(s.status, ST_TIMEOUT);
@@ -762,7 +776,7 @@ __device__ __forceinline__ void insert_tile(InsSmem<Q> &S, DevChain *__restrict_
   }
   int ctot = 0;
 #pragma unroll
-  for (int k = 0; k < INS_WARPS; ++k) {
+  for (int k = 0; k < NW; ++k) {
     if (k == wid) cex += ctot;
     ctot += S.wtot[k];
   }
@@ -770,18 +784,18 @@ __device__ __forceinline__ void insert_tile(InsSmem<Q> &S, DevChain *__restrict_
   // for its offset comes after: by then the tiles before it have mostly
   // published theirs.
   if (threadIdx.x == 0) lb_publish(s.tile_state, gt, t.y == 0 ? LB_INC : LB_AGG, ctot);
-  if (lane < 16) S.cex[cw] = cex;
+  if (lane < WC) S.cex[cw] = cex;
   auto marked = [&](int from, int n) {
-    if (n > INS_MARKS) return false;
+    if (n > InsWarp<NW>::MARKS) return false;
     for (int i = lane; i < (n + 3) / 4; i += 32) ((uint32_t *)S.mark[wid])[i] = 0u;
     __syncwarp();
     if (staged)
-      ins_place<Q, true, false>(C, S, otau, wid, nkept, from, 0, s);
+      ins_place<Q, NW, true, false>(C, S, otau, wid, nkept, from, 0, s);
     else
-      ins_place<Q, false, false>(C, S, otau, wid, nkept, from, 0, s);
+      ins_place<Q, NW, false, false>(C, S, otau, wid, nkept, from, 0, s);
     return true;
   };
-  const int wfrom = __shfl_sync(0xffffffffu, cex, 0), wn = uniform(__shfl_sync(0xffffffffu, cex + cnt, 15) - wfrom);
+  const int wfrom = __shfl_sync(0xffffffffu, cex, 0), wn = uniform(__shfl_sync(0xffffffffu, cex + cnt, WC - 1) - wfrom);
   __syncwarp();
   bool mk = single && marked(wfrom, wn);
   if (threadIdx.x < 32) {
@@ -810,22 +824,22 @@ __device__ __forceinline__ void insert_tile(InsSmem<Q> &S, DevChain *__restrict_
   }
   if (!single && valid)  // drawn again group by group
     o = philox((TAG_INSERT << 24) | (uint32_t)side, (uint32_t)X.b, (uint32_t)X.j, sweep, k0, k1);
-  for (int c0 = 0; c0 < INS_WC;) {
+  for (int c0 = 0; c0 < WC;) {
     const int c1 = next(c0);
     const int qa = __shfl_sync(0xffffffffu, q0, c0), qb = __shfl_sync(0xffffffffu, q1, c1 - 1);
     const int from = __shfl_sync(0xffffffffu, cex, c0), n = uniform(__shfl_sync(0xffffffffu, cex + cnt, c1 - 1) - from);
     if (!single) {
-      nkept = ins_group<Q>(C, S, otau, wid, X, o, c0, c1, staged, sweep, k0, k1);
+      nkept = ins_group<Q, NW>(C, S, otau, wid, X, o, c0, c1, staged, sweep, k0, k1);
       mk = marked(from, n);
     }
     if (!mk) {
-      ins_place<Q, false, true>(C, S, staged ? S.sop : otau, wid, nkept, 0, base, s);
+      ins_place<Q, NW, false, true>(C, S, staged ? S.sop : otau, wid, nkept, 0, base, s);
       const int64_t vb = C.vtx_base + base;
-      ins_write_old<Q>(S, otau, wid, q0, cex, qa, qb, (long long *)s.vtau + vb, s.vflag + vb, s.vcell + vb);
+      ins_write_old<Q, NW>(S, otau, wid, q0, cex, qa, qb, (long long *)s.vtau + vb, s.vflag + vb, s.vcell + vb);
     } else if (staged) {
-      ins_write<Q, true>(C, S, otau, wid, n, from, cex, qa, base, s);
+      ins_write<Q, NW, true>(C, S, otau, wid, n, from, cex, qa, base, s);
     } else {
-      ins_write<Q, false>(C, S, otau, wid, n, from, cex, qa, base, s);
+      ins_write<Q, NW, false>(C, S, otau, wid, n, from, cex, qa, base, s);
     }
     c0 = c1;
   }
@@ -2224,14 +2238,20 @@ void launch_start(const Launch &L, int64_t ntile, int64_t nw, cudaStream_t st) {
 }
 
 void launch_insert(const Launch &L, int only, cudaStream_t st) {
-#define INSERT_Q(Q)                                                                                   \
-  if (L.ntile[Q - 1] && picked(only, Q - 1))                                                          \
-    k_insert<Q><<<g1(L.ntile[Q - 1]), INS_THREADS, sizeof(InsSmem<Q>), st>>>(L.ch,          \
-                                                                                          L.tile_tab,    \
-                                                                                          L.tile0[Q - 1], \
-                                                                                          Q - 1, L.s);
+  const bool wide = all_tiles(L) <= WIDE_TILES;
+#define INSERT_QW(Q, NW)                                                                            \
+  k_insert<Q, NW><<<g1(L.ntile[Q - 1]), 32 * NW, sizeof(InsSmem<Q, NW>), st>>>(L.ch, L.tile_tab,     \
+                                                                              L.tile0[Q - 1], Q - 1, L.s)
+#define INSERT_Q(Q)                              \
+  if (L.ntile[Q - 1] && picked(only, Q - 1)) {   \
+    if (wide)                                    \
+      INSERT_QW(Q, INS_WARPS_WIDE);              \
+    else                                         \
+      INSERT_QW(Q, INS_WARPS);                   \
+  }
   FOR_EACH_Q(INSERT_Q)
 #undef INSERT_Q
+#undef INSERT_QW
 }
 
 // Whether the operator rewrite adds up the tiles' counts by itself.
@@ -2322,9 +2342,11 @@ int init_kernel_attributes() {
     return -1;
   FOR_EACH_Q(EST_ATTR_Q)
 #undef EST_ATTR_Q
-#define INS_ATTR_Q(Q)                                                          \
-  if (cudaFuncSetAttribute(k_insert<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                           (int)sizeof(InsSmem<Q>)) != cudaSuccess)                  \
+#define INS_ATTR_Q(Q)                                                                                       \
+  if (cudaFuncSetAttribute(k_insert<Q, INS_WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,               \
+                           (int)sizeof(InsSmem<Q, INS_WARPS>)) != cudaSuccess ||                              \
+      cudaFuncSetAttribute(k_insert<Q, INS_WARPS_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,          \
+                           (int)sizeof(InsSmem<Q, INS_WARPS_WIDE>)) != cudaSuccess)                           \
     return -1;
   FOR_EACH_Q(INS_ATTR_Q)
 #undef INS_ATTR_Q
