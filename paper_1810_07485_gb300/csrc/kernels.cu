@@ -2082,28 +2082,44 @@ __global__ void __launch_bounds__(FINAL_THREADS) k_final(DevChain *__restrict__ 
   const int per = (C.ntile + np - 1) / np, i0 = min(C.ntile, (int)blockIdx.y * per), i1 = min(C.ntile, i0 + per);
   const int pers = (C.nsiteblk + np - 1) / np, j0 = min(C.nsiteblk, (int)blockIdx.y * pers),
             j1 = min(C.nsiteblk, j0 + pers);
-  // the running sums, for the block that comes to need them
+  // (nsiteblk <= ntile / k with k = ntile per site block, rounded up: a part
+  // with site blocks has tiles)
+  // What the record needs besides the sums, loaded beside them, for the block
+  // that comes to write it.
   double run = 0.0, run2 = 0.0;
   if (threadIdx.x < NOBS) {
     run = C.sum[threadIdx.x];
     run2 = C.sumsq[threadIdx.x];
   }
+  const int64_t n = C.n, n_new = C.n_off_new;
+  const int32_t n_old = wid ? 0 : C.op_ptr[C.cur][C.ncell];
+  lcqmc_record &r = C.ring[(uint64_t)C.n_rec % (uint32_t)C.ring_cap];
   ChainSums x{0, 0, 0, 0, 0};  // vertex-free loops are whole periods: no temporal term
+  const int nt = i1 - i0, ns = j1 - j0;
+  auto tile = [&](int64_t g) {
+    return ChainSums{s.tile_roots[g], 0, pair128(s.tile_sw2, g), pair128(s.tile_sf2, g), pair128(s.tile_sz2, g)};
+  };
+  auto site = [&](int64_t g) {
+    return ChainSums{0, s.site_free[g], pair128(s.site_sw2, g), pair128(s.site_sf2, g), 0};
+  };
+  if (nt + ns <= 32) {  // one warp takes them all
+    if (wid) return;
+    if (lane < nt)
+      x = tile(C.tile0 + i0 + lane);
+    else if (lane < nt + ns)
+      x = site(C.site0 + j0 + lane - nt);
+    warp_sums(x);
+  } else {
 #pragma unroll 4
-  for (int i = i0 + threadIdx.x; i < i1; i += FINAL_THREADS) {
-    const int64_t g = C.tile0 + i;
-    add_sums(x, ChainSums{s.tile_roots[g], 0, pair128(s.tile_sw2, g), pair128(s.tile_sf2, g), pair128(s.tile_sz2, g)});
+    for (int i = i0 + threadIdx.x; i < i1; i += FINAL_THREADS) add_sums(x, tile(C.tile0 + i));
+    for (int j = j0 + threadIdx.x; j < j1; j += FINAL_THREADS) add_sums(x, site(C.site0 + j));
+    warp_sums(x);
+    if (lane == 0) part[wid] = x;
+    __syncthreads();
+    if (wid) return;
+    x = lane < FINAL_THREADS / 32 ? part[lane] : ChainSums{0, 0, 0, 0, 0};
+    warp_sums(x);
   }
-  for (int j = j0 + threadIdx.x; j < j1; j += FINAL_THREADS) {
-    const int64_t g = C.site0 + j;
-    add_sums(x, ChainSums{0, s.site_free[g], pair128(s.site_sw2, g), pair128(s.site_sf2, g), 0});
-  }
-  warp_sums(x);
-  if (lane == 0) part[wid] = x;
-  __syncthreads();
-  if (wid) return;
-  x = lane < FINAL_THREADS / 32 ? part[lane] : ChainSums{0, 0, 0, 0, 0};
-  warp_sums(x);
   if (np > 1) {  // this part's sums to its first tile's place (read by this block only)
     if (lane == 0) {
       if (i0 < i1) {
@@ -2134,12 +2150,11 @@ __global__ void __launch_bounds__(FINAL_THREADS) k_final(DevChain *__restrict__ 
     warp_sums(x);
   }
   // lane 0 holds the chain's sums
-  const int64_t n = C.n, n_new = C.n_off_new, n_free = __shfl_sync(0xffffffffu, x.nfree, 0),
+  const int64_t n_free = __shfl_sync(0xffffffffu, x.nfree, 0),
                 clusters = __shfl_sync(0xffffffffu, x.roots, 0) + n_free, n_seg = 2 * n + n_free;
-  lcqmc_record &r = C.ring[C.n_rec % C.ring_cap];
   if (lane == 0) {
     r.n = n;
-    r.n_off_old = C.op_ptr[C.cur][C.ncell];
+    r.n_off_old = n_old;
     r.n_off_new = n_new;
     r.n_free = n_free;
     r.n_clusters = clusters;
@@ -2402,7 +2417,7 @@ void launch_sites(const Launch &L, cudaStream_t st) {
 }
 
 void launch_final(const Launch &L, cudaStream_t st) {
-  const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(L.max_ntile / 2048, 64));
+  const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(L.max_ntile / 512, 64));
   k_final<<<dim3(L.nchains, parts), FINAL_THREADS, 0, st>>>(L.ch, L.s);
 }
 

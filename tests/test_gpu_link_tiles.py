@@ -11,7 +11,7 @@ from test_gpu_parity import run_parity
 pytestmark = pytest.mark.gpu
 
 # tiles = L Q^2 ceil(beta / 16) / 128; the launches change above 304, at 2048
-# (scan in parts), above 3040 and at 4096 (record in parts)
+# (scan in parts), above 3040 and at 1024 (record in parts)
 CASES = [
     (1216, 16.0 * 32, 1),      # 304 tiles: the last with 1024 threads per tile
     (1218, 16.0 * 32, 1),      # 305 tiles
@@ -24,7 +24,7 @@ CASES = [
     (1522, 16.0 * 256, 1),     # 3044 tiles: the first warp-per-tile launch
     (760, 16.0 * 128, 2),      # 3040 tiles, S = 1
     (762, 16.0 * 128, 2),      # 3048 tiles
-    (2054, 16.0 * 256, 1),     # 4108 tiles: 4 scan parts, 2 record parts
+    (2054, 16.0 * 256, 1),     # 4108 tiles: 4 scan parts, 8 record parts
     (80, 16.0 * 4, 3),         # S = 3/2: most edges cross
     (70, 16.0 * 4 + 3.0, 4),   # S = 2, ragged last window
 ]
