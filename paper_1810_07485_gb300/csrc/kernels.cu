@@ -72,69 +72,50 @@ __device__ T block_sum(T v, T *sm) {
   return tot;
 }
 
-// Exact block-wide sum of 128-bit values (warp shuffles of both halves).
-__device__ u128 block_sum_u128(u128 v) {
-  __shared__ u128 part[32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  u128 x = v;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    unsigned long long l = __shfl_down_sync(0xffffffffu, (unsigned long long)x, o);
-    unsigned long long h = __shfl_down_sync(0xffffffffu, (unsigned long long)(x >> 64), o);
-    x += ((u128)h << 64) | (u128)l;
-  }
-  if (lane == 0) part[wid] = x;
-  __syncthreads();
-  u128 t = 0;
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < nw; ++i) t += part[i];
-    part[0] = t;
-  }
-  __syncthreads();
-  t = part[0];
-  __syncthreads();
-  return t;
-}
-
 __device__ __forceinline__ u128 shfl_down_u128(u128 v, int o) {
   const unsigned long long l = __shfl_down_sync(0xffffffffu, (unsigned long long)v, o);
   const unsigned long long h = __shfl_down_sync(0xffffffffu, (unsigned long long)(v >> 64), o);
   return ((u128)h << 64) | (u128)l;
 }
 
-// Exact block-wide sums of one int64 and two (Z: three) 128-bit values with a
-// single barrier; the totals are valid in thread 0.  Once per kernel.
+// Exact sum of a 128-bit value over the warp, on every lane: eight warp
+// reductions of 16-bit pieces (32 of them stay below 2^21) instead of five
+// rounds of four shuffles and a 128-bit add.
+__device__ __forceinline__ u128 warp_sum_u128(u128 v) {
+  u128 t = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const uint32_t w = (uint32_t)(v >> (32 * k));
+    const uint32_t lo = __reduce_add_sync(0xffffffffu, w & 0xffffu), hi = __reduce_add_sync(0xffffffffu, w >> 16);
+    t += (u128)(lo + ((unsigned long long)hi << 16)) << (32 * k);
+  }
+  return t;
+}
+
+// Exact block-wide sums of one count (block total below 2^32) and two (Z: three)
+// 128-bit values with a single barrier; the totals are valid in thread 0.  Once
+// per kernel.
 template <bool Z>
 __device__ void block_sums(long long &c, u128 &x, u128 &y, u128 &z) {
-  __shared__ long long pc[32];
+  __shared__ uint32_t pc[32];
   __shared__ u128 px[32], py[32], pz[Z ? 32 : 1];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    c += __shfl_down_sync(0xffffffffu, c, o);
-    x += shfl_down_u128(x, o);
-    y += shfl_down_u128(y, o);
-    if (Z) z += shfl_down_u128(z, o);
-  }
+  const uint32_t n = __reduce_add_sync(0xffffffffu, (uint32_t)c);
+  x = warp_sum_u128(x);
+  y = warp_sum_u128(y);
+  if (Z) z = warp_sum_u128(z);
   if (lane == 0) {
-    pc[wid] = c;
+    pc[wid] = n;
     px[wid] = x;
     py[wid] = y;
     if (Z) pz[wid] = z;
   }
   __syncthreads();
   if (wid == 0) {
-    c = lane < nw ? pc[lane] : 0;
-    x = lane < nw ? px[lane] : (u128)0;
-    y = lane < nw ? py[lane] : (u128)0;
-    if (Z) z = lane < nw ? pz[lane] : (u128)0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      c += __shfl_down_sync(0xffffffffu, c, o);
-      x += shfl_down_u128(x, o);
-      y += shfl_down_u128(y, o);
-      if (Z) z += shfl_down_u128(z, o);
-    }
+    c = __reduce_add_sync(0xffffffffu, lane < nw ? pc[lane] : 0u);
+    x = warp_sum_u128(lane < nw ? px[lane] : (u128)0);
+    y = warp_sum_u128(lane < nw ? py[lane] : (u128)0);
+    if (Z) z = warp_sum_u128(lane < nw ? pz[lane] : (u128)0);
   }
 }
 
