@@ -95,15 +95,17 @@ __device__ __forceinline__ u128 warp_sum_u128(u128 v) {
 // Exact block-wide sums of one count (block total below 2^32) and two (Z: three)
 // 128-bit values with a single barrier; the totals are valid in thread 0.  Once
 // per kernel.
-template <bool Z>
+template <bool Z, bool SPARSE = false>
 __device__ void block_sums(long long &c, u128 &x, u128 &y, u128 &z) {
   __shared__ uint32_t pc[32];
   __shared__ u128 px[32], py[32], pz[Z ? 32 : 1];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const uint32_t n = __reduce_add_sync(0xffffffffu, (uint32_t)c);
-  x = warp_sum_u128(x);
-  y = warp_sum_u128(y);
-  if (Z) z = warp_sum_u128(z);
+  if (!SPARSE || __any_sync(0xffffffffu, (x | y | z) != 0)) {
+    x = warp_sum_u128(x);
+    y = warp_sum_u128(y);
+    if (Z) z = warp_sum_u128(z);
+  }
   if (lane == 0) {
     pc[wid] = n;
     px[wid] = x;
@@ -1862,6 +1864,16 @@ __global__ void __launch_bounds__(SITE_BLOCK) k_sites(const DevChain *__restrict
 // a word at a time (id order = order of the next operator list), and a cell's
 // first operator is the count before its first vertex.
 //
+// Bound by the chain of dependent loads of a tile (table, chain, first vertices,
+// words, then times and open roots), with 8 blocks per SM to hide it; more
+// registers and fewer blocks lose (6 blocks 324 us).  So a tile passes two
+// barriers only: a warp scans consecutive words of its own, which it then moves
+// without a barrier, and the barrier of the final sums also covers the counts
+// that the cells' offsets read.  The tile's own sums come in by cp.async
+// meanwhile, and a warp takes the open roots of its words 32 at a time instead of
+// a word's roots one after another.  L=16384, beta=4096 (32768 tiles): 277 -> 235
+// us (249 with the sums read at the end); with the temporal sums, L=4098, beta=1000.7: 31 -> 25.
+//
 // SMALL (every chain has at most OWN_SCAN tiles): two launches less.  A tile
 // adds up the counts before it itself instead of reading them from k_scan_ops,
 // and the blocks past the ntiles tiles rewrite the site blocks' spins (k_sites),
@@ -1875,143 +1887,160 @@ template <bool T, bool SMALL>
 __global__ void __launch_bounds__(TPB, T || SMALL ? 4 : 8) k_compact(DevChain *__restrict__ ch,
                                                  const int2 *__restrict__ tab, int64_t ntiles,
                                                  const int2 *__restrict__ site_tab, Scratch s) {
-  __shared__ int sm[33];
-  __shared__ uint32_t nbits[TPB];
-  __shared__ int npre[TPB];
+  constexpr int NW = TPB / 32;
+  __shared__ uint32_t nbits[TPB];  // per word: new operators, and their number before it
+  __shared__ int npre[TPB], wtot[NW];
+  __shared__ uint32_t wsum[2][NW];
+  __shared__ unsigned short olist[NW][32];
+  __shared__ ulonglong2 tsum[3];
+  const int2 t = SMALL && blockIdx.x >= ntiles ? make_int2(0, 0) : tab[blockIdx.x];
   if (halted(s)) return;
   if (SMALL && blockIdx.x >= ntiles) {
     rewrite_sites<0>(ch, site_tab, blockIdx.x - ntiles, s);
     return;
   }
   const int64_t gt = blockIdx.x;
-  const int2 t = tab[gt];
   DevChain &C = ch[t.x];
   const int c0 = t.y * TILE, c1 = min(C.ncell, c0 + TILE), ncl = c1 - c0;
-  int32_t *nptr = C.op_ptr[C.cur ^ 1];
   const int32_t *vp = s.vptr + C.cell_off;
   const int64_t vb = C.vtx_base;
-  int64_t base;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int64_t base = SMALL ? 0 : s.tile_pref2[gt];
   bool fits = true;
   if (SMALL) {
-    int64_t before = 0, all = 0;
+    uint32_t before = 0, all = 0;  // a chain has fewer than 2^31 operators
     for (int i = threadIdx.x; i < C.ntile; i += TPB) {
-      const int64_t x = s.tile_sum2[C.tile0 + i];
-      before += i < t.y ? x : 0;
+      const uint32_t x = (uint32_t)s.tile_sum2[C.tile0 + i];
+      before += i < t.y ? x : 0u;
       all += x;
     }
-    __shared__ int64_t sm64[2][33];
-    base = block_sum<int64_t>(before, sm64[0]);
-    all = block_sum<int64_t>(all, sm64[1]);
-    fits = all <= C.op_cap;  // else no list is written: the host grows it and replays
-    if (threadIdx.x == 0 && t.y == C.ntile - 1) {
-      C.n_off_new = all;
-      if (!fits) atomicOr(s.status, ST_OP_OVERFLOW);
+    before = __reduce_add_sync(0xffffffffu, before);
+    all = __reduce_add_sync(0xffffffffu, all);
+    if (lane == 0) {
+      wsum[0][wid] = before;
+      wsum[1][wid] = all;
     }
-  } else {
-    base = s.tile_pref2[gt];
   }
   const int a = uniform(vp[c0]), e = uniform(vp[c1]);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int cv = (threadIdx.x < ncl) ? vp[c0 + threadIdx.x] : e;  // first vertex of the thread's cell
-  const int64_t wfirst = (vb + a) >> 5, wlast = (vb + e - 1) >> 5;
-  const int nw = e > a ? (int)(wlast - wfirst) + 1 : 0;
-  double *ntau = C.op_tau[C.cur ^ 1] + base;
-  int run = 0, at = -1;  // new operators before the chunk; before the thread's cell
-  for (int k0 = 0; k0 < nw; k0 += TPB) {  // one chunk but for tiles of more than 8000 vertices
-    const int nk = min(nw - k0, TPB);
-    uint32_t bits = 0u;
-    if (threadIdx.x < nk) {
-      const int64_t wd = wfirst + k0 + threadIdx.x, v0 = (wd << 5) - vb;
-      bits = s.newbits[wd];
-      if (v0 < a) bits &= ~0u << (a - v0);
-      if (v0 + 32 > e) bits &= (e - v0 >= 32) ? ~0u : ((1u << (e - v0)) - 1u);
-    }
-    int tot;
-    const int ex = run + block_excl_scan<int>(__popc(bits), sm, tot);
-    nbits[threadIdx.x] = bits;
-    npre[threadIdx.x] = ex;
-    __syncthreads();
-    for (int k = wid; k < nk; k += TPB / 32) {
-      const uint32_t x = nbits[k];
-      if (((x >> lane) & 1u) && fits)
-        ntau[npre[k] + __popc(x & ((1u << lane) - 1u))] = s.vtau[((wfirst + k0 + k) << 5) + lane];
-    }
-    const int64_t k = ((vb + cv) >> 5) - wfirst - k0;
-    if (cv < e && k >= 0 && k < nk) at = npre[k] + __popc(nbits[k] & ((1u << (cv & 31)) - 1u));
-    run += tot;
-    __syncthreads();
+  const int64_t wfirst = (vb + a) >> 5;
+  const int nw = e > a ? (int)(((vb + e - 1) >> 5) - wfirst) + 1 : 0;
+  // Words in chunks (one but for tiles of more than 8000 vertices); a warp takes
+  // pw consecutive words of a chunk, one per lane.
+  const int pw = max(1, min(32, (nw + NW - 1) / NW)), chunk = NW * pw;
+  double *ntau = C.op_tau[C.cur ^ 1];
+  if (threadIdx.x < (T ? 3 : 2)) {  // the sums that the tile's own loops left
+    const unsigned long long *p = (threadIdx.x == 0 ? s.tile_sw2 : threadIdx.x == 1 ? s.tile_sf2 : s.tile_sz2) + 2 * gt;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(&tsum[threadIdx.x])), "l"(p) : "memory");
   }
+  Sum128 sw, sf, sz;
+  int run = 0, at = -1;  // new operators before the chunk; before the thread's cell
+  auto cell_start = [&](int k0) {  // new operators before the cell's first vertex, if it lies in the chunk
+    const int64_t k = ((vb + cv) >> 5) - wfirst - k0;
+    if (cv < e && k >= 0 && k < chunk) at = npre[k] + __popc(nbits[k] & ((1u << (cv & 31)) - 1u));
+  };
+  for (int k0 = 0; k0 < nw || (SMALL && k0 == 0); k0 += chunk) {
+    const int k = k0 + wid * pw + lane;
+    const bool in = lane < pw && k < nw;
+    uint32_t bits = 0u, open = 0u;
+    if (in) {
+      const int64_t wd = wfirst + k, v0 = (wd << 5) - vb;
+      uint32_t mask = ~0u;
+      if (v0 < a) mask &= ~0u << (a - v0);
+      if (v0 + 32 > e) mask &= (e - v0 >= 32) ? ~0u : ((1u << (e - v0)) - 1u);
+      bits = s.newbits[wd] & mask;
+      open = __ldcg(s.openroot + wd) & mask;
+    }
+    const int cnt = __popc(bits);
+    int inc = cnt, oinc = __popc(open);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, inc, o), z = __shfl_up_sync(0xffffffffu, oinc, o);
+      if (lane >= o) {
+        inc += y;
+        oinc += z;
+      }
+    }
+    if (lane == 31) wtot[wid] = inc;
+    __syncthreads();
+    if (SMALL && k0 == 0) {
+      base = __reduce_add_sync(0xffffffffu, lane < NW ? wsum[0][lane] : 0u);
+      const int64_t all = __reduce_add_sync(0xffffffffu, lane < NW ? wsum[1][lane] : 0u);
+      fits = all <= C.op_cap;  // else no list is written: the host grows it and replays
+      if (threadIdx.x == 0 && t.y == C.ntile - 1) {
+        C.n_off_new = all;
+        if (!fits) atomicOr(s.status, ST_OP_OVERFLOW);
+      }
+    }
+    const int wt = lane < NW ? wtot[lane] : 0;
+    const int pre = run + __reduce_add_sync(0xffffffffu, lane < wid ? wt : 0) + inc - cnt;
+    run += __reduce_add_sync(0xffffffffu, wt);
+    if (in) {
+      nbits[k - k0] = bits;
+      npre[k - k0] = pre;
+    }
+    const int64_t v0 = (wfirst + k0 + wid * pw) << 5;
+    for (int i = 0; i < pw; ++i) {
+      const uint32_t x = __shfl_sync(0xffffffffu, bits, i);
+      const int p = __shfl_sync(0xffffffffu, pre, i);
+      if (((x >> lane) & 1u) && fits) ntau[base + p + __popc(x & ((1u << lane) - 1u))] = s.vtau[v0 + 32 * i + lane];
+    }
+    // Loops that left their tile: one 32-byte record per root (and its Zi word),
+    // read and cleared.  The roots cluster at a tile's first vertices: the warp
+    // lists those of its words and takes one per lane.
+    const int nopen = __shfl_sync(0xffffffffu, oinc, 31);
+    for (int r0 = 0; r0 < nopen; r0 += 32) {
+      int p = oinc - __popc(open) - r0;
+      for (uint32_t x = open; x; x &= x - 1, ++p)
+        if (p >= 0 && p < 32) olist[wid][p] = (unsigned short)(32 * lane + __ffs(x) - 1);
+      __syncwarp();
+      if (lane < nopen - r0) {
+        const int64_t v = v0 + olist[wid][lane];
+        const ulonglong2 x = s.acc2[2 * v], y = s.acc2[2 * v + 1];
+        const unsigned long long zi = T ? s.accz[v] : 0ull;
+        // The stores follow the loads' arrival (the sums are far below 2^63, so
+        // the test always holds): issued with the loads still on their way to
+        // the same sector, they made this kernel four times slower.
+        if (((long long)x.x >= 0) & (y.x != 1ull << 63) & (zi != 1ull << 63)) {
+          s.acc2[2 * v] = make_ulonglong2(0ull, 0ull);
+          s.acc2[2 * v + 1] = make_ulonglong2(0ull, 0ull);
+          if (T) s.accz[v] = 0ull;
+        }
+        sw.add_square((long long)x.x);
+        sf.add_square((long long)x.y);
+        sf.add_square((long long)y.x);
+        if (T) {
+          sz.add_square((long long)y.y);
+          sz.add_square((long long)zi);
+        }
+      }
+      __syncwarp();
+    }
+    if (nw > chunk) {  // the words' counts are overwritten by the next chunk
+      __syncthreads();
+      cell_start(k0);
+      __syncthreads();
+    }
+  }
+  long long none = 0;
+  u128 w2 = sw.value(), f2 = sf.value(), z2 = T ? sz.value() : (u128)0;
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  block_sums<T, true>(none, w2, f2, z2);  // its barrier also completes the words' counts
+  if (nw && nw <= chunk) cell_start(0);
+  int32_t *nptr = C.op_ptr[C.cur ^ 1];
   if (threadIdx.x < ncl) {
     nptr[c0 + threadIdx.x] = (int32_t)(base + (at < 0 ? run : at));
     // the last tile's operators end the list
     if (c0 + (int)threadIdx.x == C.ncell - 1) nptr[C.ncell] = (int32_t)(base + run);
   }
-  // Loops that left their tile: one 32-byte accumulator record per root (and
-  // its Zi word), read and cleared; a thread takes one 32-vertex word of the
-  // open-root bitmap.  With the Zi words, the next root's reads are issued
-  // before the current root is cleared (two roots in flight per thread);
-  // without them, the plain loop needs fewer registers and more resident
-  // warps hide the latency better.
-  u128 w2 = 0, f2 = 0, z2 = 0;
-  for (int64_t wd = wfirst + threadIdx.x; e > a && wd <= wlast; wd += blockDim.x) {
-    uint32_t bits = __ldcg(s.openroot + wd);
-    const int64_t v0 = (wd << 5) - vb;
-    if (v0 < a) bits &= ~0u << (a - v0);
-    if (v0 + 32 > e) bits &= (e - v0 >= 32) ? ~0u : ((1u << (e - v0)) - 1u);
-    if (!T) {
-      while (bits) {
-        const int64_t v = vb + v0 + __ffs(bits) - 1;
-        bits &= bits - 1;
-        const ulonglong2 x = s.acc2[2 * v], y = s.acc2[2 * v + 1];
-        s.acc2[2 * v] = make_ulonglong2(0ull, 0ull);
-        s.acc2[2 * v + 1] = make_ulonglong2(0ull, 0ull);
-        w2 += sq_abs((long long)x.x);
-        f2 += sq_abs((long long)x.y) + sq_abs((long long)y.x);
-      }
-      continue;
-    }
-    if (!bits) continue;
-    int64_t v = vb + v0 + __ffs(bits) - 1;
-    bits &= bits - 1;
-    ulonglong2 x = s.acc2[2 * v], y = s.acc2[2 * v + 1];
-    unsigned long long zi = s.accz[v];
-    for (;;) {
-      const bool more = bits != 0;
-      int64_t vn = 0;
-      ulonglong2 xn, yn;
-      unsigned long long zn = 0ull;
-      if (more) {
-        vn = vb + v0 + __ffs(bits) - 1;
-        bits &= bits - 1;
-        xn = s.acc2[2 * vn];
-        yn = s.acc2[2 * vn + 1];
-        zn = s.accz[vn];
-      }
-      s.acc2[2 * v] = make_ulonglong2(0ull, 0ull);
-      s.acc2[2 * v + 1] = make_ulonglong2(0ull, 0ull);
-      s.accz[v] = 0ull;
-      w2 += sq_abs((long long)x.x);
-      f2 += sq_abs((long long)x.y) + sq_abs((long long)y.x);
-      z2 += sq_abs((long long)y.y) + sq_abs((long long)zi);
-      if (!more) break;
-      v = vn;
-      x = xn;
-      y = yn;
-      zi = zn;
-    }
-  }
-  long long none = 0;
-  block_sums<T>(none, w2, f2, z2);
   if (threadIdx.x == 0) {
-    auto add = [&](unsigned long long *t, u128 v) {
-      u128 x = ((u128)t[2 * gt + 1] << 64) | t[2 * gt];
-      x += v;
-      t[2 * gt] = (unsigned long long)x;
-      t[2 * gt + 1] = (unsigned long long)(x >> 64);
+    auto add = [&](unsigned long long *t, const ulonglong2 &old, u128 v) {
+      const u128 x = (((u128)old.y << 64) | old.x) + v;
+      *(ulonglong2 *)(t + 2 * gt) = make_ulonglong2((unsigned long long)x, (unsigned long long)(x >> 64));
     };
-    add(s.tile_sw2, w2);
-    add(s.tile_sf2, f2);
-    add(s.tile_sz2, z2);
+    add(s.tile_sw2, tsum[0], w2);
+    add(s.tile_sf2, tsum[1], f2);
+    if (T) add(s.tile_sz2, tsum[2], z2);
   }
 }
 
