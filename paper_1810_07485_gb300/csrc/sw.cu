@@ -187,6 +187,9 @@ __device__ void block_reduce(long long (&v)[NS], long long &mx, unsigned long lo
 // The word of the first n columns.
 __device__ __forceinline__ u64 low_bits(int n) { return n >= 64 ? ~0ull : ((1ull << n) - 1ull); }
 
+// Half row k of rows in shared memory (32 columns).
+__device__ __forceinline__ uint32_t half_row(const u64 *rows, int k) { return reinterpret_cast<const uint32_t *>(rows)[k]; }
+
 // First column of the run that holds column x, given the row's run starts.
 __device__ __forceinline__ int run_start(u64 starts, int x) { return 63 - __clzll((long long)(starts & (~0ull >> (63 - x)))); }
 
@@ -256,21 +259,30 @@ __device__ __forceinline__ uint32_t same_on_all(uint32_t x) { return __reduce_ma
 // takes the row's bonds as words: active right and down bonds, run starts, and
 // the down bonds that need a union (one whose left neighbour is also active,
 // with both right bonds between them active, joins runs already joined).  Those
-// bonds are listed, about 650 of 2048 sites at K_c, and united by whole warps,
-// run start to run start.
+// bonds are listed, about 650 of 2048 sites at K_c, and taken by whole warps, run
+// start to run start.  A run's first bond to the row above hangs the run below
+// the upper one by a plain store: every run has one such bond at most and hangs
+// below a lower index, so the stores make a forest whose roots are their trees'
+// lowest sites.  Only a run's further bonds need find and compare-and-swap.  A
+// run's root is stored when found, so that the rows below walk from there.
 //
-// Bound by instruction issue: the draws are about a quarter of it, the unions
-// the larger part of the rest.
+// Bound by instruction issue (82 % at L=8192): the draws are a fifth of it, the
+// unions a tenth, hanging the runs and finding their roots a fifth, listing and
+// row words the rest.  L=8192: 530 us with a union for every listed bond, 483
+// with the runs hung, 471 with their roots stored, 449 with the list made from
+// half rows in 32 bits.
 template <int NT>
 __global__ void __launch_bounds__(NT, 2048 / NT) k_sw_local(SwScratch s) {
   constexpr int PER = SW_TS / NT, ROWS = NT / SW_TX;  // sites per thread, rows per step
   __shared__ int lp[SW_TS];               // forest of the run starts
   __shared__ unsigned short vlist[SW_TS]; // upper ends of the down bonds to unite
   __shared__ uint32_t drawR[SW_WORDS], drawD[SW_WORDS];  // draws below T, per half row
-  __shared__ u64 start_s[SW_TY], vert_s[SW_TY], open_run[SW_TY];  // open_run: run starts of open sites
+  __shared__ u64 start_s[SW_TY];
+  __shared__ uint32_t vert_s[SW_WORDS], more_s[SW_WORDS];
+  __shared__ u64 open_run[SW_TY];         // run starts of open sites
   __shared__ uint32_t open_s[SW_WORDS];   // sites on active tile-boundary bonds
   __shared__ uint32_t ob[SW_WORDS];       // local roots of open components
-  __shared__ int vbase[SW_TY];
+  __shared__ int vbase[SW_WORDS];
   __shared__ int nvert, nopen;
   if (__ldcg(s.status)) return;
   const SwDev &D = *s.dev;
@@ -328,22 +340,36 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_sw_local(SwScratch s) {
     const u64 di = j < h - 1 ? d : 0ull;       // down bonds inside the tile
     const u64 r1 = __shfl_down_sync(0xffffffffu, ri, 1);
     const u64 vert = di & ~((di & ri & r1) << 1);
-    start_s[j] = ~(ri << 1) & (j < h ? low_bits(w) : 0ull);
-    vert_s[j] = vert;
+    const u64 starts = ~(ri << 1) & (j < h ? low_bits(w) : 0ull);
+    start_s[j] = starts;
+    // the bonds whose lower run has one further left already
+    u64 go = ~__shfl_down_sync(0xffffffffu, starts, 1), more = (vert << 1) & go;
+#pragma unroll
+    for (int o = 1; o < 64; o <<= 1) {
+      more |= go & (more << o);
+      go &= go << o;
+    }
+    more &= vert;
+    vert_s[2 * j] = (uint32_t)vert;
+    vert_s[2 * j + 1] = (uint32_t)(vert >> 32);
+    more_s[2 * j] = (uint32_t)more;
+    more_s[2 * j + 1] = (uint32_t)(more >> 32);
     if ((uint32_t)open) atomicOr(&open_s[2 * j], (uint32_t)open);
     if (open >> 32) atomicOr(&open_s[2 * j + 1], (uint32_t)(open >> 32));
-    const int nv = __popcll(vert);
+    const int nlo = __popc((uint32_t)vert) | __popc((uint32_t)more) << 16;  // at most 2048 each in a tile
+    const int nv = nlo + (__popc((uint32_t)(vert >> 32)) | __popc((uint32_t)(more >> 32)) << 16);
     int inc = nv;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, inc, o);
       if (lane >= o) inc += y;
     }
-    vbase[j] = inc - nv;
+    vbase[2 * j] = inc - nv;
+    vbase[2 * j + 1] = inc - nv + nlo;
     int n_eq = __popcll(eq_r) + __popcll(eq_d), n_act = __popcll(r) + __popcll(d);
     n_eq = __reduce_add_sync(0xffffffffu, n_eq);
     n_act = __reduce_add_sync(0xffffffffu, n_act);
-    s.starts[(int64_t)t * SW_TY + j] = start_s[j];
+    s.starts[(int64_t)t * SW_TY + j] = starts;
     if (j == h - 1) s.edge_d[t] = d;
     if (lane == 31) nvert = inc;
     if (lane == 0) {
@@ -381,30 +407,45 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_sw_local(SwScratch s) {
     const u64 open = ((u64)open_s[2 * lane + 1] << 32) | open_s[2 * lane];
     open_run[lane] = runs_with(start_s[lane], open);
   }
+  const int nall = nvert & 0xffff, nfirst = nall - (nvert >> 16);
 #pragma unroll
   for (int k = 0; k < PER; ++k) {
-    const int ly = ROWS * k + (wid >> 1), lx = 32 * (wid & 1) + lane;
-    const u64 v = vert_s[ly];
-    if ((v >> lx) & 1ull)
-      vlist[vbase[ly] + __popcll(v & low_bits(lx))] = (unsigned short)(ly * SW_TX + lx);
+    const int word = k * (NT / 32) + wid;  // half row
+    const uint32_t v = vert_s[word], m = more_s[word], low = (1u << lane) - 1u;
+    if ((v >> lane) & 1u) {
+      const int b = vbase[word], i = (b >> 16) + __popc(m & low);
+      vlist[(m >> lane) & 1u ? nfirst + i : (b & 0xffff) + __popc(v & low) - i] = (unsigned short)(32 * word + lane);
+    }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < nvert; i += NT) {
+  auto ends = [&](int i, int &a, int &b) {
     const int l = vlist[i], lx = l & (SW_TX - 1), ly = l / SW_TX;
-    sw_union(lp, ly * SW_TX + run_start(start_s[ly], lx), (ly + 1) * SW_TX + run_start(start_s[ly + 1], lx),
-             s.status);
+    a = ly * SW_TX + run_start(start_s[ly], lx);
+    b = (ly + 1) * SW_TX + run_start(start_s[ly + 1], lx);
+  };
+  for (int i = threadIdx.x; i < nfirst; i += NT) {
+    int a, b;
+    ends(i, a, b);
+    lp[b] = a;  // a run's only one of these bonds, and a < b
+  }
+  __syncthreads();
+  for (int i = nfirst + threadIdx.x; i < nall; i += NT) {
+    int a, b;
+    ends(i, a, b);
+    sw_union(lp, a, b, s.status);
   }
   __syncthreads();
   // every run's local root (read-only walks: no union is running any more)
 #pragma unroll 2
   for (int k = 0; k < PER; ++k) {
-    const int ly = ROWS * k + (wid >> 1), lx = 32 * (wid & 1) + lane, l = ly * SW_TX + lx;
-    const u64 st = start_s[ly];
-    if ((st >> lx) & 1ull) {
-      int r = lp[l];
-      for (int it = 0; it <= SW_TS && lp[r] != r; ++it) r = lp[r];
+    const int word = k * (NT / 32) + wid, l = 32 * word + lane;
+    if ((half_row(start_s, word) >> lane) & 1u) {
+      volatile int *f = lp;
+      int r = f[l];
+      for (int it = 0, g; it <= SW_TS && (g = f[r]) != r; ++it) r = g;
+      f[l] = r;
       s.lroot[(int64_t)t * SW_TS + l] = (unsigned short)r;
-      if ((open_run[ly] >> lx) & 1ull) atomicOr(&ob[r >> 5], 1u << (r & 31));
+      if ((half_row(open_run, word) >> lane) & 1u) atomicOr(&ob[r >> 5], 1u << (r & 31));
     }
   }
   __syncthreads();
@@ -531,7 +572,7 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_sw_flip(SwScratch s) {
 #pragma unroll
   for (int k = 0; k < PER; ++k) {
     const int ly = ROWS * k + (wid >> 1), lx = 32 * (wid & 1) + lane;
-    lr[k] = (start_s[ly] >> lx) & 1ull ? lroot[ly * SW_TX + lx] : (unsigned short)0xffff;
+    lr[k] = (half_row(start_s, 2 * ly + (wid & 1)) >> lane) & 1u ? lroot[ly * SW_TX + lx] : (unsigned short)0xffff;
   }
   if (threadIdx.x < SW_WORDS) {
     // half row: 32 sites from g on, in one or two blocks of 128 coins
