@@ -1178,9 +1178,13 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_link(const DevChain *__restri
   const long long *__restrict__ vt = (const long long *)s.vtau + vb;
   int32_t *par = s.parent + vb;
   // Whole warps walk the tile (trip count rounded up).  About half of the
-  // vertices have an edge to unite in the tile; a warp queues them and unites
-  // 32 at a time with all lanes (0.675 -> 0.638 ms at L=16384, beta=4096, against
-  // uniting each step's edges; the branchless search steps took it from 0.698).
+  // vertices have an edge to unite in the tile.  Most find their larger node
+  // still its own parent: one compare-and-swap hangs it below the smaller one
+  // without looking for roots.  Else the node's parent and the smaller node are to
+  // be united; a warp queues these and unites 32 at a time with all lanes.  At
+  // L=16384, beta=4096: 0.607 -> 0.575 ms against queueing every edge (S=1, L=4096:
+  // 0.265 -> 0.255), 0.675 -> 0.638 queueing against uniting each step's edges (both
+  // with k_link_x); a second such try before queueing gains nothing.
   const int lane = threadIdx.x & 31;
   uint32_t *queue = equeue[threadIdx.x >> 5];
   int nqueue = 0;
@@ -1229,7 +1233,9 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_link(const DevChain *__restri
         set_bit(s.openmark, wb, P[0]);
         if (local && P[0] != P[1]) set_bit(s.xmark, wb, w);
       } else if (local && P[0] != P[1]) {
-        edge = (uint32_t)(P[0] - a) | ((uint32_t)(P[1] - a) << 16);
+        const int lo = min(P[0], P[1]) - a, hi = max(P[0], P[1]) - a;
+        const int old = atomicCAS(lp + hi, hi, lo);
+        if (old != hi && old != lo) edge = (uint32_t)lo | ((uint32_t)old << 16);
       }
     }
     const unsigned m = __ballot_sync(0xffffffffu, edge != 0u);
