@@ -1282,6 +1282,18 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_link(const DevChain *__restri
 // tile, eight tiles per block: a tile has about 45 words of marks, and the
 // unions are chains of dependent global loads, so many tiles are kept in
 // flight.
+// Union that tries one compare-and-swap on the nodes' parents (tile roots) before
+// it looks for global roots: L=16384, beta=4096 linking + unions 0.688 -> 0.679 ms,
+// S=1, L=4096 0.312 -> 0.305 (no difference in k_link_xt, whose time is the
+// longest chain).
+__device__ __forceinline__ void uf_union_try(int32_t *par, int a, int b, int *status, int limit) {
+  const int ra = __ldcg(par + a), rb = __ldcg(par + b);
+  if (ra == rb) return;
+  const int lo = min(ra, rb), hi = max(ra, rb);
+  const int old = atomicCAS(par + hi, hi, lo);
+  if (old != hi && old != lo) uf_union(par, lo, old, status, limit);
+}
+
 constexpr int TPB_X = 256;
 constexpr int XLIST = 256;  // crossing edges of a tile listed per warp
 
@@ -1342,7 +1354,7 @@ __global__ void __launch_bounds__(TPB_X) k_link_x(const DevChain *__restrict__ c
   __syncwarp();
   for (int i = lane; i < min(nlist, XLIST); i += 32) {
     const int w = list[i];
-    uf_union(par, s.pl[vb + w], s.pr[vb + w], s.status, s.uf_limit);
+    uf_union_try(par, s.pl[vb + w], s.pr[vb + w], s.status, s.uf_limit);
   }
 }
 
