@@ -212,6 +212,8 @@ int lcqmc_set_wait_limit(lcqmc_handle h, int64_t limit);
  * block of the tile linking and local union-find (128 or 256), warps per block
  * of the union of tile-crossing edges (1..8, one tile each) and threads per
  * block of the compression (32..128 in steps of 32).  Defaults 256, 8, 128.
+ * Launches of few tiles take 1024 threads for the first and third, and a block
+ * per tile for the second, whatever is set here.
  * Any choice gives bit-identical results; only the time changes. */
 typedef struct {
   int32_t link_threads, link_x_warps, compress_threads, pad;

@@ -66,8 +66,9 @@ extern "C" {
 
 const char *lcqmc_last_error(void) { return lcq::last_error(); }
 
-// Host-side check of the integer forms of the method's rounding steps (the
-// same functions the kernels run) against the C library's fma / llrint.
+// Host-side check of the integer forms of the method's rounding steps against
+// the C library's fma / llrint (the kernels take the tick conversion's hardware
+// form, compared with the oracle by the GPU tests).
 int lcqmc_selftest(int which, int64_t n, uint64_t seed, int64_t *mismatches) {
   if (!mismatches || n < 0) return LCQMC_E_INVAL;
   uint64_t x = seed * 0x9E3779B97F4A7C15ull + 1;

@@ -1676,8 +1676,8 @@ constexpr int EST_STAGE = 1536;
 // loop table's adds and the squares each take the lanes of their kind).  Flips
 // come one bit per node (no root is followed for a flip), new operators leave
 // as one bitmap word per warp and step, ticks take one conversion, lengths and
-// squares 32-bit multiply-adds: 0.86 -> 0.72 ms at L=16384, beta=4096 (790 ->
-// 650 M warp instructions); of the instructions the table takes 22 %, the
+// squares 32-bit multiply-adds, the block's 128-bit sums warp reductions of 16-bit
+// pieces: 0.86 -> 0.70 ms at L=16384, beta=4096 (790 -> 640 M warp instructions); of the instructions the table takes 22 %, the
 // staging 15 %, the squares 10 %, the Fourier products 7 %.
 template <int Q, bool T, int NT>
 __global__ void __launch_bounds__(NT, (T ? 1536 : 2048) / NT) k_est(const DevChain *__restrict__ ch,
@@ -1895,9 +1895,9 @@ __global__ void __launch_bounds__(SITE_BLOCK) k_sites(const DevChain *__restrict
 // SMALL (every chain has at most OWN_SCAN tiles): two launches less.  A tile
 // adds up the counts before it itself instead of reading them from k_scan_ops,
 // and the blocks past the ntiles tiles rewrite the site blocks' spins (k_sites),
-// which need nothing of the operator list: 55 -> 51 us for an update of the
-// L=64 chain, 93 -> 86 us at L=1024, beta=256, with k_start's two parts in one
-// launch.  Longer chains have the two kernels of their own: the code for both
+// which need nothing of the operator list (with k_start's two parts in one launch:
+// an update of the L=64 chain 55 -> 51 us, of L=1024, beta=256 93 -> 86 us;
+// later steps brought these to 43 and 75).  Longer chains have the two kernels of their own: the code for both
 // in one kernel cost the operator rewrite 4 % at 2^19 tiles (registers).
 constexpr int OWN_SCAN = 1024;
 
@@ -2067,8 +2067,9 @@ __global__ void __launch_bounds__(TPB, T || SMALL ? 4 : 8) k_compact(DevChain *_
 // at its first tile, and the part that finishes last adds them up and writes
 // the record.  A chain of few tiles is one part, and its time is the chain of
 // fp64 operations behind the sums (they are slow on GB300): the record's values
-// and running sums are taken side by side, one per lane (13 -> 4 us; one thread
-// took them one after another).  One part per chain took 0.34 ms at 2^19 tiles.
+// and running sums are taken side by side, one per lane, with the loads they need
+// issued beside the sums (launch 13 -> 8 us; one thread took them one after
+// another).  One part per chain took 0.34 ms at 2^19 tiles.
 struct ChainSums {
   long long roots, nfree;
   u128 w2, f2, z2;

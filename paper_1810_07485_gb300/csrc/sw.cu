@@ -476,11 +476,12 @@ __device__ __forceinline__ int32_t local_root(const SwScratch &s, const SwDev &D
 
 // One thread per edge bond.  Most find the larger local root still its own parent
 // and hang it below the smaller one (L=3000 update 165 -> 154 us, L=8192 899 -> 895,
-// against a search for both global roots first).  Up to SW_WALK_TILES tiles every thread walks once
-// more after its union: the time there is the longest chain of dependent
-// accesses, and all threads' walks halve the same paths for the waiting unions
-// and for k_sw_find (update, us, without / with: L=333 48 / 43, L=1500, 1128
-// tiles, 91 / 75, L=3000, 4418 tiles, 178 / 177, L=8192 977 / 1005).
+// against a search for both global roots first).  Up to SW_WALK_TILES tiles every
+// thread walks once more after its union: the time there is the longest chain of
+// dependent accesses, and all threads' walks halve the same paths for the waiting
+// unions and for k_sw_find (update, us, without / with, measured before the above:
+// L=333 48 / 43, L=1500, 1128 tiles, 91 / 75, L=3000, 4418 tiles, 178 / 177,
+// L=8192 977 / 1005).
 constexpr int SW_WALK_TILES = 2048;
 constexpr int SW_EDGE = SW_TX + SW_TY;
 
