@@ -239,7 +239,10 @@ Engine::~Engine() {
   if (fork_) cudaEventDestroy(fork_);
   for (int q = 0; q < QMAX; ++q) {
     if (join_[q]) cudaEventDestroy(join_[q]);
-    if (side_[q]) cudaStreamDestroy(side_[q]);
+    if (side_[q]) {
+      cudaStreamSynchronize(side_[q]);  // an update that failed halfway may not have joined it
+      cudaStreamDestroy(side_[q]);
+    }
   }
   free_vertex();
   for (auto &c : owned_) destroy_state(c.get());
