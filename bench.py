@@ -54,34 +54,25 @@ BATCH_CHAINS, BATCH_UPDATES, BATCH_BUDGET_GB = 4096, 100, 150.0
 # rate (latency per update block, p50 / p99, and V+E/s).
 SERVED_RATES, SERVED_SECONDS, SERVED_LMAX = (20.0, 50.0), 10.0, 4096
 KERNELS_PER_UPDATE = 11
-# DRAM bytes per vertex of each phase's kernels (DRAM bytes of one ncu
-# capture at L=16384, beta=4096 -- dram__bytes.sum.per_second x
-# gpu__time_duration.sum -- divided by that update's vertex count;
-# profiles/topkernels_L16384_beta4096.md), valid for the kernel source with
+KERNELS_PER_SHORT_UPDATE = 9  # chains of at most 1024 tiles of 128 cells: operator offsets and spins with the rewrite
+# DRAM bytes per vertex of each phase's kernels (dram__bytes.sum of one ncu
+# capture of an update at L=16384, beta=4096, divided by that update's vertex
+# count; profiles/topkernels_L16384_beta4096.md), valid for the kernel source with
 # this sha1 only.  The same tile shapes and per-vertex work hold at
 # L=2^20, beta=2^10, so the full launch's traffic is this figure times its
 # vertex count.  With the temporal moment on, the loop-properties and
-# operator-rewrite kernels differ and have no entry.  The compression kernel
-# was captured from the first source listed; the other kernels from an
-# earlier one that differs from it only in S >= 1 staging.  The second
-# source flattens the linking kernel's shared-memory forest by root walks
-# instead of pointer jumping (the same global loads and stores); the third
-# also stages the loop-properties kernel's ticks before its first barrier
-# (the same loads).
-TRAFFIC_PER_VERTEX = {"insert": 13.5, "link_union": 26.7, "loop_ids": 6.6, "loop_props": 25.0,
-                      "op_rewrite": 14.8}
+# operator-rewrite kernels differ and have no entry.
+TRAFFIC_PER_VERTEX = {"insert": 13.2, "link_union": 26.5, "loop_ids": 6.6, "loop_props": 23.5,
+                      "op_rewrite": 13.8}
 TRAFFIC_PER_VERTEX_TEMPORAL = {k: v for k, v in TRAFFIC_PER_VERTEX.items() if k not in ("loop_props", "op_rewrite")}
-TRAFFIC_KERNELS_SHA1 = ("2bcd43154d5dbe04227fe45c685d4a3e85f64f03", "7f31eb08d2f1539aba0a26c771a385c99bf920e5",
-                        "fa8691b2a774215fa52e6afef9cb78fd57fd7843")
+TRAFFIC_KERNELS_SHA1 = ("2a9085956a733fbf1087d3164e1e29dfc4790f18",)
 
 
 # DRAM bytes per launch of each Swendsen-Wang phase at L = 8192, K = K_c (one
 # ncu capture; profiles/sw_L8192_Kc.md), valid for sw.cu with this sha1 only.
-SW_TRAFFIC = {"tile_bonds_uf": 294.5e6, "boundary_merge": 173.2e6, "roots_flip": 444.6e6,
-              "open_sizes_record": 24.4e6}
-# the profiled source, and the current one, whose kernels are the same (it
-# only adds an NVTX range around the host's update loop)
-SW_TRAFFIC_SHA1 = ("dadb5c42ae8fdb32d88e4c88ee578722234bd1c4", "e7d41349163f593cc5c0ea1dba9a5d2e5e8bd8bb")
+SW_TRAFFIC = {"tile_bonds_uf": 323.1e6, "boundary_merge": 175.4e6, "roots_flip": 285.8e6,
+              "open_sizes_record": 20.0e6}
+SW_TRAFFIC_SHA1 = ("0d60bfd6c39d312a1fe66898190c3b14d1ce0958",)
 
 
 def kernels_sha1(name="kernels.cu"):
@@ -439,7 +430,7 @@ def run_ours(args, world, rank, local):
                 "note": "each step is lcqmc_update(h, 1) plus the readback of its record; the chain's "
                         "world-line state lives on the device by design (the paper's nodes keep their "
                         "world lines), so no input is copied in per step"},
-        "gpu_launches": KERNELS_PER_UPDATE * args.steps,
+        "gpu_launches": (KERNELS_PER_SHORT_UPDATE if geo.ncell <= 1024 * 128 else KERNELS_PER_UPDATE) * args.steps,
         "clocks": clocks,
     }
     if batched is not None:
