@@ -1369,7 +1369,13 @@ __global__ void __launch_bounds__(TPB_X) k_link_x(const DevChain *__restrict__ c
 // S = 2, 65 tiles 213 / 32 -> 90 / 23; S = 3/2, 1024 tiles 244 / 46 -> 122 /
 // 37; S = 1/2, 128 tiles 47 / 28 -> 40 / 20.  Without the second walk the
 // unions got faster but the compression slower (S = 2: 108 / 49).
-constexpr int64_t XT_MAX_TILES = 20 * 152;
+// Up to how many tiles per launch: where a warp per tile becomes as fast.  One
+// update in us, block / warp per tile: S = 1/2, 64 tiles 71.7 / 75.2, 512 122 / 128,
+// 1024 173 / 179, 1280 206 / 208, 1408 217 / 217, 2048 258 / 257, 3000 344 / 342
+// (beta = 4, loops that span few tiles: 2048 140 / 136, 3072 180 / 175); S = 1, 512
+// 140 / 151, 1024 190 / 199, 2048 305 / 306, 3000 411 / 407; S = 2 crosses
+// between 2048 (701 / 773) and 4096 (1224 / 1217).
+constexpr int64_t xt_max_tiles(int Q) { return 152 * (Q == 1 ? 8 : Q == 2 ? 12 : 20); }
 
 __global__ void __launch_bounds__(TPB_X) k_link_xt(const DevChain *__restrict__ ch,
                                                 const int2 *__restrict__ tab, int64_t blk0,
@@ -2329,14 +2335,11 @@ void launch_link(const Launch &L, int only, cudaStream_t st) {
   FOR_EACH_Q(LINK_Q)
 #undef LINK_Q
   // Tile-crossing edges: a block per tile for few tiles, else a warp per tile.
-  // One update in us (block / warp) by tiles: S = 1/2: 1024 207 / 223, 4096 532 /
-  // 541, 8192 954 / 952; S = 1: 1024 232 / 251, 4096 646 / 651, 8192 1188 / 1172;
-  // S = 2: 1024 429 / 557, 2048 701 / 773, 4096 1224 / 1217.
   const int wpb = L.link_x_warps;
   for (int q = 0; q < QMAX; ++q) {
     const int64_t n = L.ntile[q];
     if (!n || !picked(only, q)) continue;
-    if (n > XT_MAX_TILES)
+    if (n > xt_max_tiles(q + 1))
       k_link_x<<<g1((n + wpb - 1) / wpb), 32 * wpb, 0, st>>>(L.ch, L.tile_tab + L.tile0[q], n, L.s);
     else
       k_link_xt<<<g1(n), TPB_X, 0, st>>>(L.ch, L.tile_tab, L.tile0[q], L.s);

@@ -479,9 +479,9 @@ __device__ __forceinline__ int32_t local_root(const SwScratch &s, const SwDev &D
 // against a search for both global roots first).  Up to SW_WALK_TILES tiles every
 // thread walks once more after its union: the time there is the longest chain of
 // dependent accesses, and all threads' walks halve the same paths for the waiting
-// unions and for k_sw_find (update, us, without / with, measured before the above:
-// L=333 48 / 43, L=1500, 1128 tiles, 91 / 75, L=3000, 4418 tiles, 178 / 177,
-// L=8192 977 / 1005).
+// unions and for k_sw_find (update, us, without / with: L=48 24.2 / 25.0, L=333
+// 34.7 / 34.7, L=1000 50.7 / 49.4, L=1500, 1128 tiles, 70.9 / 68.0, L=3000, 4418
+// tiles, 153.8 / 154.0, L=8192 890 / 890).
 constexpr int SW_WALK_TILES = 2048;
 constexpr int SW_EDGE = SW_TX + SW_TY;
 

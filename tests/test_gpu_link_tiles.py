@@ -11,7 +11,8 @@ from test_gpu_parity import run_parity
 pytestmark = pytest.mark.gpu
 
 # tiles = L Q^2 ceil(beta / 16) / 128; the launches change above 304, at 2048
-# (scan in parts), above 3040 and at 1024 (record in parts)
+# (scan in parts), at 1024 (record in parts) and above 1216 (S = 1/2), 1824 (S = 1)
+# and 3040 (a warp per tile for the crossing edges)
 CASES = [
     (1216, 16.0 * 32, 1),      # 304 tiles: the last with 1024 threads per tile
     (1218, 16.0 * 32, 1),      # 305 tiles
@@ -20,10 +21,16 @@ CASES = [
     (136, 16.0 * 32, 3),       # 306 tiles, S = 3/2
     (78, 16.0 * 32, 4),        # 312 tiles, S = 2
     (2, 16.0 * 64, 1),         # one tile, time blocks only
-    (1520, 16.0 * 256, 1),     # 3040 tiles: the last block-per-tile launch
-    (1522, 16.0 * 256, 1),     # 3044 tiles: the first warp-per-tile launch
+    (1520, 16.0 * 256, 1),     # 3040 tiles
+    (1522, 16.0 * 256, 1),     # 3044 tiles
     (760, 16.0 * 128, 2),      # 3040 tiles, S = 1
     (762, 16.0 * 128, 2),      # 3048 tiles
+    (608, 16.0 * 256, 1),      # 1216 tiles: the last block-per-tile launch of S = 1/2
+    (610, 16.0 * 256, 1),      # 1220 tiles: the first warp-per-tile launch
+    (456, 16.0 * 128, 2),      # 1824 tiles, S = 1: the last
+    (458, 16.0 * 128, 2),      # 1832 tiles: the first
+    (336, 16.0 * 128, 3),      # 3024 tiles, S = 3/2
+    (338, 16.0 * 128, 3),      # 3042 tiles
     (2054, 16.0 * 256, 1),     # 4108 tiles: 4 scan parts, 8 record parts
     (80, 16.0 * 4, 3),         # S = 3/2: most edges cross
     (70, 16.0 * 4 + 3.0, 4),   # S = 2, ragged last window
