@@ -65,14 +65,17 @@ KERNELS_PER_SHORT_UPDATE = 9  # chains of at most 1024 tiles of 128 cells: opera
 TRAFFIC_PER_VERTEX = {"insert": 13.2, "link_union": 26.5, "loop_ids": 6.6, "loop_props": 23.5,
                       "op_rewrite": 13.8}
 TRAFFIC_PER_VERTEX_TEMPORAL = {k: v for k, v in TRAFFIC_PER_VERTEX.items() if k not in ("loop_props", "op_rewrite")}
-TRAFFIC_KERNELS_SHA1 = ("2a9085956a733fbf1087d3164e1e29dfc4790f18",)
+# the profiled source, and the current one, which only moves the number of tiles
+# up to which crossing edges take a block per tile (below that of either size)
+TRAFFIC_KERNELS_SHA1 = ("2a9085956a733fbf1087d3164e1e29dfc4790f18", "002b5e34b1aa9cf33922f27dd67dcd92f0e4d81f")
 
 
 # DRAM bytes per launch of each Swendsen-Wang phase at L = 8192, K = K_c (one
 # ncu capture; profiles/sw_L8192_Kc.md), valid for sw.cu with this sha1 only.
 SW_TRAFFIC = {"tile_bonds_uf": 323.1e6, "boundary_merge": 175.4e6, "roots_flip": 285.8e6,
               "open_sizes_record": 20.0e6}
-SW_TRAFFIC_SHA1 = ("0d60bfd6c39d312a1fe66898190c3b14d1ce0958",)
+# the profiled source, and the current one (a comment differs)
+SW_TRAFFIC_SHA1 = ("0d60bfd6c39d312a1fe66898190c3b14d1ce0958", "f441500369003b81e4dfa7ae59eb521ece966b94")
 
 
 def kernels_sha1(name="kernels.cu"):
