@@ -288,6 +288,24 @@ struct InsWarp {
   static_assert(WC <= 16, "two lanes per cell, four bits of a key");
   static_assert(CAP >= KMAX - 1, "a cell's candidates fit");
 };
+// The lanes that move their cell's staged ranges (the neighbours' of their side):
+// one per cell and side, since a range is moved in place and a lane that repeats
+// another would move it a second time.  With 8 cells lanes 16 to 31 repeat.
+template <int NW>
+__host__ __device__ constexpr bool ins_moves(int lane) {
+  return lane < 2 * InsWarp<NW>::WC;
+}
+template <int NW>
+constexpr bool ins_moves_once() {
+  int n[2][InsWarp<NW>::WC] = {};
+  for (int l = 0; l < 32; ++l)
+    if (ins_moves<NW>(l)) ++n[(l / InsWarp<NW>::WC) & 1][l & (InsWarp<NW>::WC - 1)];
+  for (int c = 0; c < InsWarp<NW>::WC; ++c)
+    if (n[0][c] != 1 || n[1][c] != 1) return false;
+  return true;
+}
+static_assert(ins_moves_once<INS_WARPS>() && ins_moves_once<INS_WARPS_WIDE>(), "each range is moved once");
+
 constexpr int INS_MIN_SPAN = 256;  // smallest group a chain may ask for (tests), in candidates of a whole tile
 
 // Old operator times a tile stages in shared memory: its own cells' and those
@@ -713,7 +731,7 @@ __device__ __forceinline__ void insert_tile(InsSmem<Q, NW> &S, DevChain *__restr
   }
   X.kpre -= X.K;
   staged = __all_sync(0xffffffffu, staged || !valid) && shi > slo;
-  if (staged && valid) {  // ranges from the first staged operator on
+  if (staged && valid && ins_moves<NW>(lane)) {  // ranges from the first staged operator on
     const int n0 = side * (2 * Q - 1);
 #pragma unroll
     for (int k = 0; k < 2 * Q - 1; ++k) {
