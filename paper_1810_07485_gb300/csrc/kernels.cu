@@ -121,7 +121,18 @@ __device__ void block_sums(long long &c, u128 &x, u128 &y, u128 &z) {
   }
 }
 
+// Whether the update has stopped.  The status word may be set while a launch's
+// blocks start: by the launch itself (a chain without room, a wait that ran out,
+// a failed check) and by the kernels of another spin group, which run beside it.
+// Threads that read it one by one may then disagree, and the ones that go on would
+// use shared memory that the others never wrote.  So a kernel whose threads work
+// together takes one answer for the block (a warp, where a warp works alone).  The
+// answer of a single thread is enough where nothing that can set the word runs
+// beside the launch (k_start, k_compact<.., false>, k_sites, k_final) or each thread
+// works alone (k_check_forest).
 __device__ __forceinline__ bool halted(const Scratch &s) { return __ldcg(s.status) != 0; }
+__device__ __forceinline__ bool halted_warp(const Scratch &s) { return __any_sync(0xffffffffu, halted(s)); }
+__device__ __forceinline__ bool halted_block(const Scratch &s) { return __syncthreads_or(halted(s)) != 0; }
 
 // Tile blocks of the vertex-parallel kernels: TPB threads walk the tile's
 // vertices in id order (coalesced).  A launch of few tiles leaves most of the
@@ -233,7 +244,7 @@ __device__ int64_t lb_lookback(unsigned long long *st, int64_t g, int64_t first,
         if (lane == 0) atomicOr(s.status, ST_TIMEOUT);
         return 0;
       }
-      if ((spins & 255) == 0 && halted(s)) return 0;
+      if ((spins & 255) == 0 && halted_warp(s)) return 0;
       __nanosleep(32);
       continue;
     }
@@ -634,10 +645,11 @@ __device__ __forceinline__ void insert_tile(InsSmem<Q, NW> &S, DevChain *__restr
                                             const int2 *__restrict__ tab, int64_t blk0, int group,
                                             Scratch s) {
   constexpr int WC = InsWarp<NW>::WC;
-  if (halted(s)) return;
-  if (threadIdx.x == 0) S.gt = blk0 + (int64_t)atomicAdd(s.tickets + group, 1u);
+  // a ticket, or none if the update has stopped: one answer for the block
+  if (threadIdx.x == 0) S.gt = halted(s) ? -1 : blk0 + (int64_t)atomicAdd(s.tickets + group, 1u);
   __syncthreads();
   const int64_t gt = S.gt;
+  if (gt < 0) return;
   const int2 t = tab[gt];
   DevChain &C = ch[t.x];
   const int cur = C.cur;
@@ -857,7 +869,7 @@ __global__ void __launch_bounds__(1024) k_scan_ops(DevChain *__restrict__ ch, Sc
   // loads are issued before the current chunk's scan.
   __shared__ int64_t sm[33];
   __shared__ int64_t before;
-  if (halted(s)) return;
+  if (halted_block(s)) return;
   DevChain &C = ch[blockIdx.x];
   const int per = (C.ntile + gridDim.y - 1) / gridDim.y;
   const int i0 = min(C.ntile, (int)blockIdx.y * per), nt = min(C.ntile, i0 + per) - i0;
@@ -929,7 +941,7 @@ __global__ void __launch_bounds__(SITE_BLOCK * Q) k_cut(const DevChain *__restri
                                                     Scratch s) {
   __shared__ int slast[SITE_BLOCK * Q];
   __shared__ uint8_t stop_[SITE_BLOCK * Q];
-  if (halted(s)) return;
+  if (halted_block(s)) return;
   const int2 t = tab[blk0 + blockIdx.x];
   const DevChain &C = ch[t.x];
   const int u = t.y * SITE_BLOCK * Q + threadIdx.x, i = u / Q;  // subsite, site
@@ -1158,7 +1170,6 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_link(const DevChain *__restri
   __shared__ int cvp[TILE + 1];
   __shared__ int lp[SMEM_CAP];
   __shared__ uint32_t equeue[NT / 32][64];  // per warp: edges to unite
-  if (halted(s)) return;
   const int2 t = tab[blk0 + blockIdx.x];
   const DevChain &C = ch[t.x];
   const int c0 = t.y * TILE, c1 = min(C.ncell, c0 + TILE), ncl = c1 - c0;
@@ -1186,7 +1197,7 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_link(const DevChain *__restri
     }
     L.own_bj = before_window(C, vp, b, j);
   }
-  __syncthreads();
+  if (halted_block(s)) return;  // so far only cell offsets were read, at places the geometry gives
   const int a = cvp[0], e = cvp[ncl], nv = e - a;
   const bool local = nv <= local_cap(C);
   if (local)
@@ -1319,7 +1330,7 @@ __global__ void __launch_bounds__(TPB_X) k_link_x(const DevChain *__restrict__ c
                                                 const int2 *__restrict__ tab, int64_t ntiles,
                                                 Scratch s) {
   __shared__ int xlist[TPB_X / 32][XLIST];
-  if (halted(s)) return;
+  if (halted_warp(s)) return;
   const int lane = threadIdx.x & 31;
   const int64_t gt = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (gt >= ntiles) return;
@@ -1400,7 +1411,7 @@ __global__ void __launch_bounds__(TPB_X) k_link_xt(const DevChain *__restrict__ 
                                                 Scratch s) {
   __shared__ unsigned short xlist[SMEM_CAP];
   __shared__ int nx;
-  if (halted(s)) return;
+  if (halted_block(s)) return;
   const int2 t = tab[blk0 + blockIdx.x];
   const DevChain &C = ch[t.x];
   const int c0 = t.y * TILE, c1 = min(C.ncell, c0 + TILE);
@@ -1479,7 +1490,7 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_compress(const DevChain *__re
   __shared__ uint32_t ocoin[SMEM_CAP / 32 + 2];  // coins of the outside roots, at the nodes that point there
   __shared__ unsigned short olist[SMEM_CAP];     // those nodes
   __shared__ int nout;
-  if (halted(s)) return;
+  if (halted_block(s)) return;
   const int64_t gt = blk0 + blockIdx.x;
   const int2 t = tab[gt];
   const DevChain &C = ch[t.x];
@@ -1715,7 +1726,7 @@ __global__ void __launch_bounds__(NT, (T ? 1536 : 2048) / NT) k_est(const DevCha
   extern __shared__ long long est_dyn[];
   long long *qv = est_dyn;                   // ticks q(tau) of the tile's vertices
   int2 *ev = (int2 *)(est_dyn + EST_STAGE);  // their phase factors exp(i w1 tau)
-  if (halted(s)) return;
+  if (halted_block(s)) return;
   const int64_t gt = blk0 + blockIdx.x;
   const int2 t = tab[gt];
   const DevChain &C = ch[t.x];
@@ -1936,7 +1947,7 @@ __global__ void __launch_bounds__(TPB, T || SMALL ? 4 : 8) k_compact(DevChain *_
   __shared__ unsigned short olist[NW][32];
   __shared__ ulonglong2 tsum[3];
   const int2 t = SMALL && blockIdx.x >= ntiles ? make_int2(0, 0) : tab[blockIdx.x];
-  if (halted(s)) return;
+  if (SMALL ? halted_block(s) : halted(s)) return;  // SMALL sets the status word itself
   if (SMALL && blockIdx.x >= ntiles) {
     rewrite_sites<0>(ch, site_tab, blockIdx.x - ntiles, s);
     return;

@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_sw_local(SwScratch s) {
   __shared__ uint32_t ob[SW_WORDS];       // local roots of open components
   __shared__ int vbase[SW_WORDS];
   __shared__ int nvert, nopen;
-  if (__ldcg(s.status)) return;
+  const bool stop = __ldcg(s.status) != 0;
   const SwDev &D = *s.dev;
   const int t = blockIdx.x, L = D.L;
   int x0, y0, w, h;
@@ -316,7 +316,9 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_sw_local(SwScratch s) {
       lp[l] = l;
     }
   }
-  __syncthreads();
+  // One answer for the block: a walk that runs out in another block sets the status
+  // word while this one starts, and what follows shares what every warp wrote.
+  if (__syncthreads_or(stop)) return;
   const int tx = t % D.ntx, ty = t / D.ntx;
   const int left = ty * D.ntx + (tx ? tx - 1 : D.ntx - 1), right = ty * D.ntx + (tx + 1 < D.ntx ? tx + 1 : 0);
   const int up = (ty ? ty - 1 : D.nty - 1) * D.ntx + tx, down = (ty + 1 < D.nty ? ty + 1 : 0) * D.ntx + tx;
