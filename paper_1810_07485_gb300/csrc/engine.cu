@@ -798,7 +798,11 @@ int Engine::sync(bool *at_once) {
     CK(cudaStreamSynchronize(st_));
     return LCQMC_OK;
   }
-  for (int guard = 0; guard < 64; ++guard) {
+  // A pass that grew a chain is progress: the chains of a batch may run out of room
+  // at as many different updates as there are chains.  Each growth adds an eighth at
+  // least, so memory or the vertex ids end it.
+  for (int stuck = 0; stuck < 64;) {
+    bool grew = false;
     int status = 0;
     int rc = fetch(&status);
     if (rc) return rc;
@@ -851,7 +855,10 @@ int Engine::sync(bool *at_once) {
     }
     if (status & ST_VTX_OVERFLOW) {
       for (size_t c = 0; c < cs_.size(); ++c)
-        if (hch[c].n > cs_[c]->vcap) cs_[c]->vcap = (hch[c].n + hch[c].n / 8 + 4096 + 127) / 128 * 128;
+        if (hch[c].n > cs_[c]->vcap) {
+          cs_[c]->vcap = (hch[c].n + hch[c].n / 8 + 4096 + 127) / 128 * 128;
+          grew = true;
+        }
       rc = layout();
       if (rc) return rc;
     }
@@ -860,6 +867,7 @@ int Engine::sync(bool *at_once) {
         if (hch[c].n_off_new > hch[c].op_cap) {
           rc = grow_ops(c, hch[c].n_off_new);
           if (rc) return rc;
+          grew = true;
         }
       rc = push_chains();
       if (rc) return rc;
@@ -872,6 +880,7 @@ int Engine::sync(bool *at_once) {
       rc = update(remaining);
       if (rc) return rc;
     }
+    if (!grew) ++stuck;
   }
   set_error("capacity growth did not converge");
   return LCQMC_E_NOMEM;

@@ -88,3 +88,28 @@ def test_served_chains_grow():
     for m, t in zip(mix, tickets):
         assert res[t].status == 0
         _check_against_oracle(res[t], m)
+
+
+def test_many_chains_grow_at_different_updates():
+    # 160 chains whose vertices reach the end of their reserve once in a few dozen
+    # updates: one call stops at more updates than a fixed number of passes covers
+    from paper_1810_07485_gb300 import lcqmc
+    n, specs = 400, [dict(L=2, beta=3494.5 + i * 9.5 / 160, seed=100 + i) for i in range(160)]
+    want, stops = [], set()
+    for sp in specs:
+        ch = lcqmc.Chain(sp["L"], sp["beta"], seed=sp["seed"])
+        for t in range(n):
+            ch.update(1)
+            ch.sync()
+            if ch.geometry().replays:
+                stops.add(t)
+                ch.update(n - t - 1)
+                break
+        want.append((list(ch.measure().sum), ch.records()[-256:]))  # a batch keeps 256 records a chain
+        ch.close()
+    assert len(stops) > 64
+    b = lcqmc.Batch(specs)
+    b.update(n)
+    for i in range(len(specs)):
+        assert list(b.measure(i).sum) == want[i][0] and np.array_equal(b.records(i), want[i][1]), i
+    b.close()
