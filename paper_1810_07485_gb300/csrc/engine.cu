@@ -844,8 +844,9 @@ int Engine::sync(bool *at_once) {
         return LCQMC_E_STATE;
       }
       long long dbg[8] = {0};
-      cudaMemcpy(dbg, s_.dbg, sizeof(dbg), cudaMemcpyDeviceToHost);
-      cudaMemset(s_.dbg, 0, sizeof(dbg));
+      cudaMemcpyAsync(dbg, s_.dbg, sizeof(dbg), cudaMemcpyDeviceToHost, st_);
+      cudaMemsetAsync(s_.dbg, 0, sizeof(dbg), st_);
+      cudaStreamSynchronize(st_);
       char msg[256];
       std::snprintf(msg, sizeof msg,
                     "internal consistency check %lld failed on the device (%lld %lld %lld %lld %lld)",
@@ -1075,9 +1076,12 @@ int Engine::import_config(int64_t c, const uint8_t *s0, const int32_t *op_ptr, c
     drop_graphs();
   }
   const ChainBuf &b = cs_[c]->buf;
-  CK(cudaMemcpy(b.s0[d.cur], s0, d.nsub, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(b.op_ptr[d.cur], op_ptr, 4 * ((size_t)d.ncell + 1), cudaMemcpyHostToDevice));
-  if (n_off > 0) CK(cudaMemcpy(b.op_tau[d.cur], op_tau, 8 * (size_t)n_off, cudaMemcpyHostToDevice));
+  // On the handle's stream (push_chains waits for it): a plain copy from pageable
+  // memory may return before its last bytes have arrived, and the handle's own stream
+  // does not wait for it.
+  CK(cudaMemcpyAsync(b.s0[d.cur], s0, d.nsub, cudaMemcpyHostToDevice, st_));
+  CK(cudaMemcpyAsync(b.op_ptr[d.cur], op_ptr, 4 * ((size_t)d.ncell + 1), cudaMemcpyHostToDevice, st_));
+  if (n_off > 0) CK(cudaMemcpyAsync(b.op_tau[d.cur], op_tau, 8 * (size_t)n_off, cudaMemcpyHostToDevice, st_));
   d.sweep = sweep;
   return push_chains();
 }

@@ -2408,7 +2408,11 @@ int init_kernel_attributes() {
     tab[k] = make_int2((int)std::llrint(std::ldexp(std::cos(ang), 30)),
                        (int)std::llrint(std::ldexp(std::sin(ang), 30)));
   }
-  if (cudaMemcpyToSymbol(g_phase_tab, tab, sizeof(tab)) != cudaSuccess) return -1;
+  // waited for: other streams read the table
+  if (cudaMemcpyToSymbolAsync(g_phase_tab, tab, sizeof(tab), 0, cudaMemcpyHostToDevice, cudaStreamLegacy) !=
+          cudaSuccess ||
+      cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess)
+    return -1;
 #define EST_ATTR_Q(Q)                                                                      \
   if (cudaFuncSetAttribute(k_est<Q, true, TPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                            (int)EST_DYN_SMEM) != cudaSuccess ||                              \

@@ -1010,12 +1010,14 @@ class SwEngine {
       }
     int rc = sync();
     if (rc) return rc;
-    SWCK(cudaMemcpy(s_.bytes, spins, (size_t)h_.N, cudaMemcpyHostToDevice));
+    // On the handle's stream: a plain copy from pageable memory may return before its
+    // last bytes have arrived, and the handle's own stream does not wait for it.
+    SWCK(cudaMemcpyAsync(s_.bytes, spins, (size_t)h_.N, cudaMemcpyHostToDevice, st_));
     k_sw_pack<<<h_.ntile * SW_TY / 8, 256, 0, st_>>>(s_);  // a warp per tile row
     SWCK(cudaGetLastError());
-    SWCK(cudaStreamSynchronize(st_));
-    SWCK(cudaMemcpy((char *)s_.dev + offsetof(SwDev, sweep), &sweep, sizeof(uint32_t),
-                    cudaMemcpyHostToDevice));
+    SWCK(cudaMemcpyAsync((char *)s_.dev + offsetof(SwDev, sweep), &sweep, sizeof(uint32_t),
+                         cudaMemcpyHostToDevice, st_));
+    SWCK(cudaStreamSynchronize(st_));  // the caller's memory is its own again
     return LCQMC_OK;
   }
 
