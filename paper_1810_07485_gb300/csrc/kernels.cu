@@ -2136,6 +2136,7 @@ __device__ __forceinline__ void warp_sums(ChainSums &x) {
 }
 
 constexpr int FINAL_THREADS = 256;
+constexpr int FINAL_BLOCKS = 152 * 16;  // of a launch, when chains are cut in parts
 
 __global__ void __launch_bounds__(FINAL_THREADS) k_final(DevChain *__restrict__ ch, Scratch s) {
   __shared__ ChainSums part[FINAL_THREADS / 32];
@@ -2482,7 +2483,12 @@ void launch_sites(const Launch &L, cudaStream_t st) {
 }
 
 void launch_final(const Launch &L, cudaStream_t st) {
-  const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(L.max_ntile / 512, 64));
+  // Parts of at least 512 tiles, and no more blocks in all than the chip holds a few
+  // times over: every chain gets as many parts as the largest.  One chain of 32768
+  // tiles with 16, 1024, 4096, 12000 chains of 8, 4, 1, 1 tiles, ms per update: 64
+  // parts each 2.78, 3.34, 4.40, 7.47; so limited 2.78, 3.17, 3.50, 4.63.
+  const int parts = (int)std::max<int64_t>(
+      1, std::min<int64_t>(L.max_ntile / 512, std::min<int64_t>(64, FINAL_BLOCKS / L.nchains)));
   k_final<<<dim3(L.nchains, parts), FINAL_THREADS, 0, st>>>(L.ch, L.s);
 }
 
