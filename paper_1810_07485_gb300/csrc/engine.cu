@@ -155,6 +155,28 @@ void Engine::dfree(void *p) {
 }
 
 
+// Page-locked host memory for read-back: whole pages of the process's own, locked in
+// place (7 us, and 10 to release; cudaHostAlloc and cudaFreeHost take 110 and 150, as
+// much again as creating a small chain).
+static cudaError_t staging_alloc(void **p, size_t bytes) {
+  constexpr size_t page = 65536;  // the largest base page of the hosts of these GPUs
+  const size_t n = (bytes + page - 1) / page * page;
+  void *q = std::aligned_alloc(page, n);
+  if (!q) return cudaErrorMemoryAllocation;
+  const cudaError_t e = cudaHostRegister(q, n, cudaHostRegisterPortable);
+  if (e != cudaSuccess) {
+    std::free(q);
+    return e;
+  }
+  *p = q;
+  return cudaSuccess;
+}
+static void staging_free(void *p) {
+  if (!p) return;
+  cudaHostUnregister(p);
+  std::free(p);
+}
+
 #define DALLOC(ptr, type, count)                                                    \
   do {                                                                              \
     ptr = (type *)dalloc(sizeof(type) * (size_t)(count));                           \
@@ -273,8 +295,8 @@ Engine::~Engine() {
   dfree(s_.dbg);
   if (st_) cudaStreamSynchronize(st_);  // stream-ordered frees done
   if (pool_) cudaMemPoolDestroy(pool_);
-  if (stage_) cudaFreeHost(stage_);
-  if (stage_ch_) cudaFreeHost(stage_ch_);
+  staging_free(stage_);
+  staging_free(stage_ch_);
   if (own_stream_ && st_) cudaStreamDestroy(st_);
 }
 
@@ -313,7 +335,7 @@ int Engine::open(void *stream, const lcqmc_allocator *alloc, int ring_cap, bool 
   std::vector<uint64_t> T(KMAX);
   poisson_table(CELL_MEAN, T.data());
   set_full_table(T.data(), st_);
-  CK(cudaHostAlloc((void **)&stage_, sizeof(HostStage), cudaHostAllocDefault));
+  CK(staging_alloc((void **)&stage_, sizeof(HostStage)));
   DALLOC(s_.status, int, 1);
   s_.uf_limit = UF_MAX_ITERS;
   // Tests: the most steps a global union-find walk or retry loop of this
@@ -744,10 +766,10 @@ int Engine::update(int64_t n) {
 int Engine::fetch(int *status) {
   const size_t nc = hch.size();
   if (nc > stage_nch_) {
-    if (stage_ch_) cudaFreeHost(stage_ch_);
+    staging_free(stage_ch_);
     stage_ch_ = nullptr;
     stage_nch_ = 0;
-    CK(cudaHostAlloc((void **)&stage_ch_, sizeof(DevChain) * nc, cudaHostAllocDefault));
+    CK(staging_alloc((void **)&stage_ch_, sizeof(DevChain) * nc));
     stage_nch_ = nc;
   }
   CK(cudaMemcpyAsync(&stage_->status, s_.status, sizeof(int), cudaMemcpyDeviceToHost, st_));
