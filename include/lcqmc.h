@@ -226,7 +226,8 @@ int lcqmc_set_tuning(lcqmc_handle h, const lcqmc_tuning *cfg);
 /* Autotuner: times each candidate with the phase events over
  * updates_per_trial updates (a coordinate search: 128/256 x 2/4/8 for the
  * linking phase, then 64/128 for the compression; 8 trials) and keeps the
- * fastest.  The trial updates are ordinary updates of the chain (records and
+ * fastest; a size that the chain's launches do not use (see above) keeps its
+ * value.  The trial updates are ordinary updates of the chain (records and
  * running sums included).  out (may be NULL) receives the choice. */
 int lcqmc_autotune(lcqmc_handle h, int64_t updates_per_trial, lcqmc_tuning *out);
 int lcqmc_get_phase_times(lcqmc_handle h, double *ms, int nphase);

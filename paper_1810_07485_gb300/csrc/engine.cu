@@ -1202,13 +1202,15 @@ int Engine::set_tuning(const lcqmc_tuning &t) {
 // candidate timed by the phase events over n updates: linking + global unions
 // (phase 2) over link_threads x link_x_warps, then compression (phase 3) over
 // compress_threads.  The trial updates are ordinary updates of every chain;
-// the block sizes do not change any result.
+// the block sizes do not change any result.  A size that the launches do not use
+// keeps its value: its trials differ by noise alone.
 int Engine::autotune(int64_t n, lcqmc_tuning *out) {
   if (n < 1) {
     set_error("autotune needs at least one update per trial");
     return LCQMC_E_INVAL;
   }
   const bool was_timing = timing_;
+  const int used = tunable(L_);
   lcqmc_tuning best;
   get_tuning(&best);
   auto trial = [&](const lcqmc_tuning &t, int phase, double *ms) -> int {
@@ -1231,7 +1233,8 @@ int Engine::autotune(int64_t n, lcqmc_tuning *out) {
       if (rc) return rc;
       if (ms < best_ms) {
         best_ms = ms;
-        best = cur;
+        if (used & TUNE_LINK) best.link_threads = lt;
+        if (used & TUNE_LINK_X) best.link_x_warps = xw;
       }
     }
   best_ms = 1e300;
@@ -1243,7 +1246,7 @@ int Engine::autotune(int64_t n, lcqmc_tuning *out) {
     if (rc) return rc;
     if (ms < best_ms) {
       best_ms = ms;
-      best.compress_threads = ct;
+      if (used & TUNE_COMPRESS) best.compress_threads = ct;
     }
   }
   int rc = set_tuning(best);

@@ -2309,6 +2309,13 @@ static int64_t all_tiles(const Launch &L) {
 // Whether Q group q is launched: the one asked for, or all (only < 0).
 static bool picked(int only, int q) { return only < 0 || only == q; }
 
+int tunable(const Launch &L) {
+  int used = all_tiles(L) <= WIDE_TILES ? 0 : TUNE_LINK | TUNE_COMPRESS;
+  for (int q = 0; q < QMAX; ++q)
+    if (L.ntile[q] > xt_max_tiles(q + 1)) used |= TUNE_LINK_X;
+  return used;
+}
+
 void launch_start(const Launch &L, int64_t ntile, int64_t nw, cudaStream_t st) {
   int64_t nbb = 0;
   for (int q = 0; q < QMAX; ++q) nbb += L.nbondblk[q];

@@ -25,6 +25,10 @@ struct Launch {
   int check_forest = 0;       // verify the loop forest after compression (debug)
 };
 
+// Which of the three block sizes the launches use: TUNE_LINK | TUNE_LINK_X |
+// TUNE_COMPRESS
+enum : int { TUNE_LINK = 1, TUNE_LINK_X = 2, TUNE_COMPRESS = 4 };
+int tunable(const Launch &L);
 void set_full_table(const uint64_t *T, cudaStream_t st);
 int init_kernel_attributes();
 // bond parities; zeroes the look-back words of ntile tiles, the tickets and nw
