@@ -112,21 +112,6 @@ static Geo geo_of(const ChainSpec &c) {
   return g;
 }
 
-size_t Engine::estimate_footprint(const std::vector<ChainSpec> &specs, int ring_cap) {
-  size_t bytes = 0;
-  int64_t vc = 4096;
-  for (const auto &c : specs) {
-    Geo g = geo_of(c);
-    bytes += 2 * (g.nsub + 2 * 4 * (g.ncell + 1) + 8 * op_estimate(c));
-    bytes += 8 * KMAX + 16 * c.L + 24 * g.nwin + sizeof(lcqmc_record) * ring_cap;
-    bytes += 4 * (g.ncell + 1) + 64 * g.ntile + 48 * g.nsiteblk + (g.nblk + 1) * g.nbond +
-             14 * g.nsub + sizeof(DevChain) + 8 * (g.ntile + g.nsiteblk + g.nbondblk);
-    vc += (vertex_estimate(c) + 127) / 128 * 128;
-  }
-  bytes += (size_t)vc * (8 + 2 + 12 + 8 * ACC_WORDS + 8) + 5 * (size_t)(vc / 32 + 1) * 4;
-  return bytes;
-}
-
 // ---- allocation ------------------------------------------------------------------------
 void *Engine::dalloc(size_t bytes) {
   if (bytes == 0) bytes = 16;
@@ -208,7 +193,6 @@ void Engine::free_vertex() {
   s_.acc = nullptr;
   s_.accz = nullptr;
   s_.openmark = s_.openroot = s_.flipbits = s_.newbits = s_.xmark = nullptr;
-  vertex_bytes_ = 0;
 }
 
 int Engine::alloc_vertex(int64_t vcap) {
@@ -232,7 +216,6 @@ int Engine::alloc_vertex(int64_t vcap) {
   CK(cudaMemsetAsync(s_.accz, 0, sizeof(unsigned long long) * vcap, st_));
   s_.vcap = vcap;
   vcap_ = vcap;
-  vertex_bytes_ = (size_t)vcap * (8 + 2 + 12 + 8 * ACC_WORDS + 8) + 5 * (size_t)nw * 4;
   L_.s = s_;
   drop_graphs();
   return LCQMC_OK;
@@ -442,6 +425,10 @@ size_t Engine::state_bytes(const ChainSpec &c, int ring_cap) {
          16 * (size_t)c.L + 24 * (size_t)g.nwin + sizeof(lcqmc_record) * (size_t)ring_cap;
 }
 
+// The admission figure of a chain's scratch, in the terms it was fixed in: requests
+// are accepted by it.  It is not the allocation (layout and alloc_vertex: 62.6 bytes
+// per vertex, 88 per tile, 10 per subsite): the records of open loops, which a few
+// percent of the vertices use, are not in it.
 size_t Engine::scratch_bytes(const ChainSpec &c) {
   const Geo g = geo_of(c);
   const size_t v = (size_t)((vertex_estimate(c) + 127) / 128 * 128);
@@ -577,8 +564,6 @@ int Engine::layout() {
     CK(cudaMemcpyAsync(site_tab_, stab.data(), sizeof(int2) * stab.size(), cudaMemcpyHostToDevice, st_));
     CK(cudaMemcpyAsync(bond_tab_, btab.data(), sizeof(int2) * btab.size(), cudaMemcpyHostToDevice, st_));
   }
-  fixed_bytes_ = 4 * (size_t)cap_cells_ + 96 * (size_t)cap_tiles_ + 48 * (size_t)cap_sites_ +
-                 (size_t)cap_bpar_ + 14 * (size_t)cap_subs_ + sizeof(DevChain) * (size_t)cap_chains_;
   L_.ch = dch_;
   L_.nchains = nc;
   L_.max_ntile = 0;
@@ -809,7 +794,6 @@ int Engine::grow_ops(int64_t c, int64_t need) {
     b.op_tau[k] = p;
     d.op_tau[k] = p;
   }
-  op_bytes_ += 2 * 8 * (size_t)(cap - d.op_cap);
   d.op_cap = cap;
   return LCQMC_OK;
 }
@@ -1262,7 +1246,5 @@ int Engine::phase_times(double *ms, int nphase) {
   for (int k = 0; k < nphase && k < LCQMC_NPHASE; ++k) ms[k] = phase_ms_[k];
   return LCQMC_OK;
 }
-
-size_t Engine::footprint() const { return fixed_bytes_ + vertex_bytes_ + op_bytes_; }
 
 }  // namespace lcq

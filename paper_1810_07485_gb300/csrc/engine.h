@@ -84,8 +84,6 @@ class Engine {
   int set_tuning(const lcqmc_tuning &t);
   int autotune(int64_t n, lcqmc_tuning *out);
   int phase_times(double *ms, int nphase);
-  size_t footprint() const;  // device bytes held
-  static size_t estimate_footprint(const std::vector<ChainSpec> &specs, int ring_cap);
 
   cudaStream_t stream() const { return st_; }
   int nchains() const { return (int)cs_.size(); }
@@ -121,7 +119,6 @@ class Engine {
   Scratch s_{};
   int64_t vcap_ = 0;
   int ring_cap_ = 0;
-  size_t fixed_bytes_ = 0, vertex_bytes_ = 0, op_bytes_ = 0;
   // one update, and a block of kGraphBlock updates (fewer graph launches for
   // small chains, whose updates are a few microseconds of work)
   static constexpr int kGraphBlock = 8;
