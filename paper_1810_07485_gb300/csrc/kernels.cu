@@ -1402,8 +1402,10 @@ __global__ void __launch_bounds__(TPB_X) k_link_x(const DevChain *__restrict__ c
 // update in us, block / warp per tile: S = 1/2, 64 tiles 71.7 / 75.2, 512 122 / 128,
 // 1024 173 / 179, 1280 206 / 208, 1408 217 / 217, 2048 258 / 257, 3000 344 / 342
 // (beta = 4, loops that span few tiles: 2048 140 / 136, 3072 180 / 175); S = 1, 512
-// 140 / 151, 1024 190 / 199, 2048 305 / 306, 3000 411 / 407; S = 2 crosses
-// between 2048 (701 / 773) and 4096 (1224 / 1217).
+// 140 / 151, 1024 190 / 199, 2048 305 / 306, 3000 411 / 407; S = 2,
+// beta = 512: 2048 595 / 662, 3040 793 / 828, 3600 889 / 903, 4096 1026 / 1021.  S = 3/2
+// has S = 2's line, which is on the safe side of its own (3040 609 / 704, 4096 766 / 838,
+// 6000 1041 / 1084).
 constexpr int64_t xt_max_tiles(int Q) { return 152 * (Q == 1 ? 8 : Q == 2 ? 12 : 20); }
 
 __global__ void __launch_bounds__(TPB_X) k_link_xt(const DevChain *__restrict__ ch,

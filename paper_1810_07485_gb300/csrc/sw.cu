@@ -478,13 +478,17 @@ __device__ __forceinline__ int32_t local_root(const SwScratch &s, const SwDev &D
 
 // One thread per edge bond.  Most find the larger local root still its own parent
 // and hang it below the smaller one (L=3000 update 165 -> 154 us, L=8192 899 -> 895,
-// against a search for both global roots first).  Up to SW_WALK_TILES tiles every
-// thread walks once more after its union: the time there is the longest chain of
-// dependent accesses, and all threads' walks halve the same paths for the waiting
-// unions and for k_sw_find (update, us, without / with: L=48 24.2 / 25.0, L=333
-// 34.7 / 34.7, L=1000 50.7 / 49.4, L=1500, 1128 tiles, 70.9 / 68.0, L=3000, 4418
-// tiles, 153.8 / 154.0, L=8192 890 / 890).
-constexpr int SW_WALK_TILES = 2048;
+// against a search for both global roots first).  Between SW_WALK_MIN and
+// SW_WALK_TILES tiles every thread walks once more after its union: the time there
+// is the longest chain of dependent accesses, and all threads' walks halve the same
+// paths for the waiting unions and for k_sw_find.  One update, us, without / with the
+// walk, at K_c: L=48 24.0 / 24.6, L=250 31.4 / 31.6, L=333, 66 tiles, 34.5 / 34.6,
+// L=500, 128 tiles, 35.7 / 35.6, L=700, 242 tiles, 42.4 / 41.6, L=1000 50.6 / 49.2,
+// L=1500, 1128 tiles, 69.4 / 67.5, L=2000 93.1 / 92.3, L=3000, 4418 tiles, 153.8 /
+// 154.0.  The lines are K_c's, where the paths are longest; away from it the walk
+// costs: L=1000, 1500, 2000 at K = 0.3 40.1 / 40.8, 54.9 / 55.6, 75.0 / 75.7, at K =
+// 0.7 40.0 / 41.5, 57.5 / 61.0, 81.8 / 89.0.
+constexpr int SW_WALK_MIN = 152, SW_WALK_TILES = 2048;
 constexpr int SW_EDGE = SW_TX + SW_TY;
 
 __global__ void __launch_bounds__(SW_EDGE) k_sw_merge(SwScratch s) {
@@ -512,7 +516,7 @@ __global__ void __launch_bounds__(SW_EDGE) k_sw_merge(SwScratch s) {
     const int lo = min(a, b), hi = max(a, b), old = atomicCAS(s.par + hi, hi, lo);
     if (old != hi && old != lo) uf_union(s.par, lo, old, s.status);
   }
-  if (D.ntile > SW_WALK_TILES) return;
+  if (D.ntile <= SW_WALK_MIN || D.ntile > SW_WALK_TILES) return;
   const int r = uf_find(s.par, a, s.status);
   if (r != a) s.par[a] = r;
 }
