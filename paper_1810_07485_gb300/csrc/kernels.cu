@@ -126,7 +126,9 @@ __device__ void block_sums(long long &c, u128 &x, u128 &y, u128 &z) {
 // a failed check) and by the kernels of another spin group, which run beside it.
 // Threads that read it one by one may then disagree, and the ones that go on would
 // use shared memory that the others never wrote.  So a kernel whose threads work
-// together takes one answer for the block (a warp, where a warp works alone).  The
+// together takes one answer for the block (a warp, where a warp works alone), behind
+// the loads of the tile's place, whose addresses the geometry gives: the word is on
+// its way meanwhile.  The
 // answer of a single thread is enough where nothing that can set the word runs
 // beside the launch (k_start, k_compact<.., false>, k_sites, k_final) or each thread
 // works alone (k_check_forest).
@@ -1170,6 +1172,7 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_link(const DevChain *__restri
   __shared__ int cvp[TILE + 1];
   __shared__ int lp[SMEM_CAP];
   __shared__ uint32_t equeue[NT / 32][64];  // per warp: edges to unite
+  const bool stop = halted(s);
   const int2 t = tab[blk0 + blockIdx.x];
   const DevChain &C = ch[t.x];
   const int c0 = t.y * TILE, c1 = min(C.ncell, c0 + TILE), ncl = c1 - c0;
@@ -1197,7 +1200,7 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_link(const DevChain *__restri
     }
     L.own_bj = before_window(C, vp, b, j);
   }
-  if (halted_block(s)) return;  // so far only cell offsets were read, at places the geometry gives
+  if (__syncthreads_or(stop)) return;
   const int a = cvp[0], e = cvp[ncl], nv = e - a;
   const bool local = nv <= local_cap(C);
   if (local)
@@ -1413,7 +1416,7 @@ __global__ void __launch_bounds__(TPB_X) k_link_xt(const DevChain *__restrict__ 
                                                 Scratch s) {
   __shared__ unsigned short xlist[SMEM_CAP];
   __shared__ int nx;
-  if (halted_block(s)) return;
+  const bool stop = halted(s);
   const int2 t = tab[blk0 + blockIdx.x];
   const DevChain &C = ch[t.x];
   const int c0 = t.y * TILE, c1 = min(C.ncell, c0 + TILE);
@@ -1421,6 +1424,7 @@ __global__ void __launch_bounds__(TPB_X) k_link_xt(const DevChain *__restrict__ 
   const int a = vp[c0], e = vp[c1];
   const int64_t vb = C.vtx_base;
   int32_t *par = s.parent + vb;
+  if (__syncthreads_or(stop)) return;
   if (e - a > local_cap(C)) {  // every edge of the tile
     for (int w = a + threadIdx.x; w < e; w += TPB_X)
       uf_union(par, s.pl[vb + w], s.pr[vb + w], s.status, s.uf_limit);
@@ -1492,7 +1496,7 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_compress(const DevChain *__re
   __shared__ uint32_t ocoin[SMEM_CAP / 32 + 2];  // coins of the outside roots, at the nodes that point there
   __shared__ unsigned short olist[SMEM_CAP];     // those nodes
   __shared__ int nout;
-  if (halted_block(s)) return;
+  const bool stop = halted(s);
   const int64_t gt = blk0 + blockIdx.x;
   const int2 t = tab[gt];
   const DevChain &C = ch[t.x];
@@ -1501,6 +1505,7 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_compress(const DevChain *__re
   const int a = uniform(vp[c0]), e = uniform(vp[c1]);
   const int64_t vb = C.vtx_base, wb = vb >> 5;
   int32_t *par = s.parent + vb;
+  if (__syncthreads_or(stop)) return;
   const bool oversized = (e - a) > local_cap(C);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int step = blockDim.x, first = (a & ~31) + 32 * wid;  // words of 32 vertices, a warp each
@@ -1728,7 +1733,7 @@ __global__ void __launch_bounds__(NT, (T ? 1536 : 2048) / NT) k_est(const DevCha
   extern __shared__ long long est_dyn[];
   long long *qv = est_dyn;                   // ticks q(tau) of the tile's vertices
   int2 *ev = (int2 *)(est_dyn + EST_STAGE);  // their phase factors exp(i w1 tau)
-  if (halted_block(s)) return;
+  const bool stop = halted(s);
   const int64_t gt = blk0 + blockIdx.x;
   const int2 t = tab[gt];
   const DevChain &C = ch[t.x];
@@ -1738,6 +1743,7 @@ __global__ void __launch_bounds__(NT, (T ? 1536 : 2048) / NT) k_est(const DevCha
   const int64_t vb = C.vtx_base, wb = vb >> 5;
   const int32_t *par = s.parent + vb;
   const uint64_t *vt = (const uint64_t *)s.vtau + vb;
+  if (__syncthreads_or(stop)) return;
   const int F = C.F;
   // Ticks of every vertex of the tile, once: the fragments below a vertex
   // mostly start at vertices of the same tile.
