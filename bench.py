@@ -116,20 +116,20 @@ def phase_bytes(rec, ncell, L):
     no, nn = float(rec["n_off_old"]), float(rec["n_off_new"])
     return {
         # old operator times and offsets in; vertex time/flag/cell and cell
-        # offsets out; four per-vertex bitmaps cleared
-        "insert": 8 * no + 10 * n + 8 * ncell + n / 2,
+        # offsets out; five per-vertex bitmaps cleared
+        "insert": 8 * no + 10.625 * n + 8 * ncell,
         "cut": 16.0 * L,
         # vertex time and cell in, predecessor links and parent forest out,
         # flag read-modify-write, cell offsets
         "link_union": 23 * n + 4 * ncell,
         # parent read, root written, open-mark / open-root / flip bitmaps
         "loop_ids": 8.375 * n,
-        # cell, links, flag read+write, parent, time, flip bits; new-operator
-        # counts per cell
-        "loop_props": 23.125 * n + 4 * ncell,
+        # cell, links, flag, parent, time and flip bits in; new-operator bits out
+        "loop_props": 22.25 * n,
         "op_offsets": 16 * (ncell / 128.0),
-        # flags, new operator times read + written, cell offsets
-        "op_rewrite": n + 16 * nn + 8 * ncell,
+        # new-operator and open-root bits, new operator times read + written,
+        # cell offsets read + written
+        "op_rewrite": 0.25 * n + 16 * nn + 8 * ncell,
         "spin_rewrite": 2.0 * L + 64.0,
     }
 

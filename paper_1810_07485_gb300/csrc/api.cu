@@ -67,8 +67,9 @@ extern "C" {
 const char *lcqmc_last_error(void) { return lcq::last_error(); }
 
 // Host-side check of the integer forms of the method's rounding steps against
-// the C library's fma / llrint (the kernels take the tick conversion's hardware
-// form, compared with the oracle by the GPU tests).
+// the C library's fma / llrint.  The kernels take the tick conversion's hardware form
+// and, for all but the smallest draws, another form of the unit factor: these are
+// compared with the oracle on the device, at their edges too.
 int lcqmc_selftest(int which, int64_t n, uint64_t seed, int64_t *mismatches) {
   if (!mismatches || n < 0) return LCQMC_E_INVAL;
   uint64_t x = seed * 0x9E3779B97F4A7C15ull + 1;

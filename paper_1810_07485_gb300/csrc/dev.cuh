@@ -265,9 +265,8 @@ __device__ __forceinline__ u128 sq_abs(long long v) {
 // loops keep imaginary times as the bit patterns of non-negative doubles
 // (ordered like the doubles themselves when read as int64) and compare those.
 // Two fp64 instructions are left: one fused multiply-add per insertion
-// candidate, and per vertex the conversion of its time to integer ticks (25
-// integer instructions; rounded to nearest, ties to even), with the fp64 pipe
-// otherwise idle.
+// candidate, and per vertex the conversion of its time to integer ticks (rounded
+// to nearest, ties to even).
 
 constexpr uint64_t M52 = (1ull << 52) - 1;
 
@@ -284,10 +283,10 @@ __host__ __device__ __forceinline__ uint64_t unit_bits(uint64_t u53) {
 }
 
 // llrint(ldexp(x, F)) for a non-negative double x given as bits (x 2^F < 2^62).
-// Device: the exponent raised by F and one rounding conversion (25 integer
-// instructions otherwise: k_est 0.82 -> 0.73 ms at L=16384, beta=4096; the fp64
-// pipe stays at a fifth); a denormal x is below half a tick.  Host (self test):
-// the same from the bits.
+// Device: the exponent raised by F and one rounding conversion (the form from the
+// bits took 25 integer instructions: k_est 0.82 -> 0.73 ms at L=16384, beta=4096; the
+// fp64 pipe stays at a fifth); a denormal x is below half a tick.  Host (self test):
+// the form from the bits, which no kernel runs.
 __host__ __device__ __forceinline__ long long q_time(uint64_t x_bits, int F) {
 #ifdef __CUDA_ARCH__
   return (x_bits >> 52) == 0 ? 0 : __double2ll_rn(__longlong_as_double((long long)(x_bits + ((uint64_t)F << 52))));

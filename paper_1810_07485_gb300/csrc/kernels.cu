@@ -210,8 +210,8 @@ __global__ void __launch_bounds__(BOND_BLOCK) k_start(const DevChain *__restrict
 
 // ---- insertion (labeling, rules i-iii) --------------------------------------
 // Imaginary times are handled as the int64 bit patterns of non-negative doubles
-// (same order as the values); a candidate's time is the exact integer form of
-// fma(t_end - t0, u, t0).  No fp64 instruction is issued.
+// (same order as the values); the one fp64 instruction per candidate is the fused
+// multiply-add of its time, fma(t_end - t0, u, t0).
 // Single pass: every tile counts its cells' vertices, publishes the count, and
 // gets the chain-local offset of its first vertex by decoupled look-back over
 // the tiles before it (tile order = order in which blocks took their ticket,
@@ -1309,11 +1309,6 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_link(const DevChain *__restri
   }
 }
 
-// Global unions of the edges that leave their tile (all edges of a tile too
-// large for shared memory), on the forests the tiles stored.  One warp per
-// tile, eight tiles per block: a tile has about 45 words of marks, and the
-// unions are chains of dependent global loads, so many tiles are kept in
-// flight.
 // Union that tries one compare-and-swap on the nodes' parents (tile roots) before
 // it looks for global roots: L=16384, beta=4096 linking + unions 0.688 -> 0.679 ms,
 // S=1, L=4096 0.312 -> 0.305 (no difference in k_link_xt, whose time is the
@@ -1326,6 +1321,11 @@ __device__ __forceinline__ void uf_union_try(int32_t *par, int a, int b, int *st
   if (old != hi && old != lo) uf_union(par, lo, old, status, limit);
 }
 
+// Global unions of the edges that leave their tile (all edges of a tile too
+// large for shared memory), on the forests the tiles stored.  One warp per
+// tile, eight tiles per block: a tile has about 45 words of marks, and the
+// unions are chains of dependent global loads, so many tiles are kept in
+// flight.
 constexpr int TPB_X = 256;
 constexpr int XLIST = 256;  // crossing edges of a tile listed per warp
 
@@ -1941,7 +1941,12 @@ __global__ void __launch_bounds__(SITE_BLOCK) k_sites(const DevChain *__restrict
 // which need nothing of the operator list (with k_start's two parts in one launch:
 // an update of the L=64 chain 55 -> 51 us, of L=1024, beta=256 93 -> 86 us;
 // later steps brought these to 43 and 75).  Longer chains have the two kernels of their own: the code for both
-// in one kernel cost the operator rewrite 4 % at 2^19 tiles (registers).
+// in one kernel cost the operator rewrite 4 % at 2^19 tiles (registers).  The line is
+// set by the chain, not by the launch, and large batches of such chains lose by it:
+// with half the blocks per SM the whole update takes 4 to 7 % more (ms, SMALL / the
+// long chains' kernels: 16 chains of 25 tiles 0.116 / 0.121, 64 of 25 0.219 / 0.221,
+// 4096 of one 0.730 / 0.750; 64 of 100 0.648 / 0.622, 512 of 100 4.56 / 4.29, 4096 of
+// 100 35.8 / 33.6).
 constexpr int OWN_SCAN = 1024;
 
 template <bool T, bool SMALL>
