@@ -62,20 +62,17 @@ KERNELS_PER_SHORT_UPDATE = 9  # chains of at most 1024 tiles of 128 cells: opera
 # L=2^20, beta=2^10, so the full launch's traffic is this figure times its
 # vertex count.  With the temporal moment on, the loop-properties and
 # operator-rewrite kernels differ and have no entry.
-TRAFFIC_PER_VERTEX = {"insert": 13.2, "link_union": 26.5, "loop_ids": 6.6, "loop_props": 23.5,
-                      "op_rewrite": 13.8}
+TRAFFIC_PER_VERTEX = {"insert": 13.2, "link_union": 26.5, "loop_ids": 6.5, "loop_props": 23.6,
+                      "op_rewrite": 13.9}
 TRAFFIC_PER_VERTEX_TEMPORAL = {k: v for k, v in TRAFFIC_PER_VERTEX.items() if k not in ("loop_props", "op_rewrite")}
-# the profiled source, and the current one, which only moves the number of tiles
-# up to which crossing edges take a block per tile (below that of either size)
-TRAFFIC_KERNELS_SHA1 = ("2a9085956a733fbf1087d3164e1e29dfc4790f18", "002b5e34b1aa9cf33922f27dd67dcd92f0e4d81f")
+TRAFFIC_KERNELS_SHA1 = ("797d8a37dcfcac843d22075f3a3d3a2b24b79358",)
 
 
 # DRAM bytes per launch of each Swendsen-Wang phase at L = 8192, K = K_c (one
 # ncu capture; profiles/sw_L8192_Kc.md), valid for sw.cu with this sha1 only.
-SW_TRAFFIC = {"tile_bonds_uf": 323.1e6, "boundary_merge": 175.4e6, "roots_flip": 285.8e6,
-              "open_sizes_record": 20.0e6}
-# the profiled source, and the current one (a comment differs)
-SW_TRAFFIC_SHA1 = ("0d60bfd6c39d312a1fe66898190c3b14d1ce0958", "f441500369003b81e4dfa7ae59eb521ece966b94")
+SW_TRAFFIC = {"tile_bonds_uf": 323.5e6, "boundary_merge": 175.5e6, "roots_flip": 285.8e6,
+              "open_sizes_record": 20.1e6}
+SW_TRAFFIC_SHA1 = ("d3e4adb6175a72c79907fd545ad15e5aad69988d",)
 
 
 def kernels_sha1(name="kernels.cu"):
@@ -701,7 +698,7 @@ def run_sw(args, world, rank, local):
                    "mean_largest_cluster": float(recs["max_cluster"].mean()),
                    "union_find_ms_per_step": uf_ms,
                    "paper_union_find_s_per_step_1_thread": 0.097,
-                   "l2": "inputs larger than L2 (spins, forest and size arrays: 0.6 GB)"},
+                   "l2": "inputs larger than L2 (spins, forest and size arrays: 0.7 GB)"},
         "roofline": roofline,
         "cpu_baseline": cpu,
         "e2e": {"value": units2 / e2e_max, "unit": "site updates/s", "h2d_bytes_per_step": 0,
